@@ -244,6 +244,7 @@ int band_half_sweep_impl(const ising_lattice_t *lat, const Accept &acc, const Ro
     p.acc = acc;
     p.rk = rk;
     p.obs = (long long *)obs;
+    p.overlap = 0;  // each band's half-sweep follows events of other streams
     cudaError_t e = msc4_half_sweep(p, colour, s);
     return e == cudaSuccess ? ISING_OK : cuda_fail(e, "band half-sweep launch");
 }

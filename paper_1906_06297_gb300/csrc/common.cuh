@@ -103,6 +103,7 @@ struct Msc4SweepParams {
     RoundKeys rk;
     long long *obs;       // {sum s, sum bonds} accumulators or nullptr
     int32_t spare_sms = 0;  // host side: SMs the launch leaves without a block
+    int32_t overlap = 1;    // host side: may start beside the kernel before it in the stream
 };
 
 struct Int8SweepParams {
@@ -163,6 +164,37 @@ __device__ __forceinline__ void block_reduce_add2(long long a, long long b, long
     if (warp == 0) {
         a = lane < kWarps ? sa[lane] : 0;
         b = lane < kWarps ? sb[lane] : 0;
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) {
+            a += __shfl_xor_sync(0xffffffffu, a, off);
+            b += __shfl_xor_sync(0xffffffffu, b, off);
+        }
+        if (lane == 0) {
+            atomicAdd(reinterpret_cast<unsigned long long *>(out), (unsigned long long)a);
+            atomicAdd(reinterpret_cast<unsigned long long *>(out + 1), (unsigned long long)b);
+        }
+    }
+}
+
+// The same for any block size of up to 1024 threads.
+__device__ __forceinline__ void block_reduce_add2_any(long long a, long long b, long long *out)
+{
+    __shared__ long long sa[32], sb[32];  // any block size
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+        a += __shfl_xor_sync(0xffffffffu, a, off);
+        b += __shfl_xor_sync(0xffffffffu, b, off);
+    }
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (lane == 0) {
+        sa[warp] = a;
+        sb[warp] = b;
+    }
+    __syncthreads();
+    if (warp == 0) {
+        const int warps = (blockDim.x + 31) >> 5;
+        a = lane < warps ? sa[lane] : 0;
+        b = lane < warps ? sb[lane] : 0;
 #pragma unroll
         for (int off = 16; off > 0; off >>= 1) {
             a += __shfl_xor_sync(0xffffffffu, a, off);

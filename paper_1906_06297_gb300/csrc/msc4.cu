@@ -13,7 +13,8 @@
 // (black on odd rows, white on even rows).  With spins as 0/1 nibbles, the
 // four neighbour words add nibble-wise without carries (each sum is 0..4).
 //
-// Sweep kernel design (GB300, sm_103a):
+// Sweep kernel design for large planes (GB300, sm_103a; small ones take
+// msc4_flat_kernel below):
 //   * Each warp owns a 64-word column chunk (lane l holds words 2l, 2l+1, one
 //     16-byte copy per plane row) and marches down a contiguous range of rows.
 //     Rows i-1, i, i+1 of the source plane, the target row and the next rows
@@ -55,7 +56,7 @@ namespace {
 #endif
 constexpr int kThreads = ISING_MSC4_THREADS;
 constexpr int kWarps = kThreads / 32;
-constexpr int kMinRowsPerWarp = 16;
+constexpr int kMinRowsPerWarp = 4;  // 2048^2: 22.6 us per sweep, 37.0 at 8 and 65.8 at 16 rows
 
 __device__ __forceinline__ void st128(uint64_t *p, uint4 v)
 {
@@ -236,6 +237,143 @@ __global__ void __launch_bounds__(kThreads, ISING_MSC4_MIN_BLOCKS)
     }
 }
 
+// ---------------------------------------------------------------------------
+// Flat sweep kernel: a thread takes HALVES 32-bit half words (8 sites each) of
+// one row at a time, for planes too small for the marching kernel above, whose
+// warps need 64-word chunks and tens of rows each.  A small half-sweep is bound
+// by the latency from one kernel's end to the next one's loads, so the kernel
+// may start beside the one before it in the stream (programmatic launch): it
+// first forms its draws' marks -- nearly all of the arithmetic, and dependent
+// on the keys alone -- then waits for that kernel, loads the target half
+// words, the three source rows and the side half word, decides and stores.
+// One block per SM, each with an equal range of items; at 64 registers two
+// blocks of 512 threads fit on an SM, one of each of two kernels.  (Blocks of
+// 128 threads, as many as there are items: the waiting blocks of the next
+// kernel gather on the SMs that finish first, 17.7 instead of 5.4 us per sweep
+// of 2048^2.)  Measured, us per sweep with the trace, marching kernel (at least
+// 16 rows per warp) / this one: 256^2 66 / 3.6 (the host's launch rate), 2112^2
+// 66.7 / 5.6, 4096^2 67.7 / 16.0, 8192^2 68.0 / 53.6.
+// ---------------------------------------------------------------------------
+constexpr int kFlatThreads = 512;
+
+template <int HALVES>
+struct HalfWords {
+    uint32_t v[HALVES];
+};
+
+template <int HALVES>
+__device__ __forceinline__ HalfWords<HALVES> ld_halves(const uint32_t *p)
+{
+    HalfWords<HALVES> r;
+    if constexpr (HALVES == 4) {
+        const uint4 x = *reinterpret_cast<const uint4 *>(p);
+        r.v[0] = x.x, r.v[1] = x.y, r.v[2] = x.z, r.v[3] = x.w;
+    } else {
+        r.v[0] = *p;
+    }
+    return r;
+}
+
+template <int HALVES>
+__device__ __forceinline__ void st_halves(uint32_t *p, const HalfWords<HALVES> &r)
+{
+    if constexpr (HALVES == 4) *reinterpret_cast<uint4 *>(p) = make_uint4(r.v[0], r.v[1], r.v[2], r.v[3]);
+    else *p = r.v[0];
+}
+
+struct FlatSplit {
+    uint32_t items;  // rows x units per row
+    uint32_t upr;    // units of HALVES half words per row
+    uint32_t per;    // items per block
+};
+
+template <int COLOR, bool OBS, bool ALWAYS, int HALVES>
+__global__ void __launch_bounds__(kFlatThreads, 2)
+    msc4_flat_kernel(const __grid_constant__ Msc4SweepParams p, const __grid_constant__ FlatSplit f)
+{
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    const uint32_t end = min(f.items, (blockIdx.x + 1) * f.per);
+    const DrawCtx dc{p.c2, p.c3, p.acc.T3, p.acc.T4, p.acc.zero};
+    const int64_t stride = 2 * p.stride;  // in half words
+    uint32_t ones = 0, dsum = 0, n = 0;
+    bool waited = false;
+    for (uint32_t e = blockIdx.x * f.per + threadIdx.x; e < end; e += blockDim.x) {
+        const uint32_t row = e / f.upr, u = e - row * f.upr;
+        const uint32_t q = (uint32_t)(p.row0 + row) * (uint32_t)p.qrow + 2 * HALVES * u;
+        uint32_t g[HALVES];
+#pragma unroll
+        for (int h = 0; h < HALVES; ++h) g[h] = ALWAYS ? 0u : half_marks(q + 2 * h, 0u, dc, p.rk);
+        if (!waited) {
+            asm volatile("griddepcontrol.wait;" ::: "memory");
+            waited = true;
+        }
+        const int64_t ru = row == 0 ? p.first_up : (int64_t)row - 1;
+        const int64_t rd = (int64_t)row + 1 == p.wrap_row ? p.wrap_to : (int64_t)row + 1;
+        const uint32_t *src = reinterpret_cast<const uint32_t *>(p.src) + HALVES * u;
+        const uint32_t *crow = src + (int64_t)row * stride;
+        uint32_t *tp = reinterpret_cast<uint32_t *>(p.tgt) + (int64_t)row * stride + HALVES * u;
+        const bool left = ((row + p.row0 + COLOR) & 1) == 0;
+        const int32_t last = (int32_t)f.upr - 1;
+        const int32_t off = left ? (u == 0 ? HALVES * last + HALVES - 1 : -1)
+                                 : ((int32_t)u == last ? -HALVES * last : HALVES);
+        const HalfWords<HALVES> up = ld_halves<HALVES>(src + ru * stride), cur = ld_halves<HALVES>(crow),
+                                dn = ld_halves<HALVES>(src + rd * stride), tg = ld_halves<HALVES>(tp);
+        const uint32_t edge = crow[off];
+        HalfWords<HALVES> ns;
+        uint32_t dacc = 0, n8 = 0;
+#pragma unroll
+        for (int h = 0; h < HALVES; ++h) {
+            const uint32_t prev = h == 0 ? edge : cur.v[h - 1], next = h == HALVES - 1 ? edge : cur.v[h + 1];
+            const uint32_t side = left ? __funnelshift_l(prev, cur.v[h], 4) : __funnelshift_r(cur.v[h], next, 4);
+            ns.v[h] = decide_half<OBS, ALWAYS>(tg.v[h], up.v[h] + dn.v[h] + cur.v[h], side, g[h], dacc);
+            n8 += ns.v[h] + cur.v[h];
+        }
+        st_halves<HALVES>(tp, ns);
+        if (OBS) {
+            // up-spin counts nibble-wise (at most 2 HALVES per nibble), then by bytes
+            const uint32_t sb = (n8 & 0x0F0F0F0Fu) + ((n8 >> 4) & 0x0F0F0F0Fu);
+            ones += (sb * 0x01010101u) >> 24;
+            dsum += (dacc * 0x01010101u) >> 24;
+            n += HALVES;
+        }
+    }
+    // the kernel after this one relies on this one's wait, so every thread waits
+    if (!waited) asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (OBS) {
+        // 8 white and 8 black spins and 32 bonds per half word
+        const long long sum_s = 2 * (long long)ones - 16 * (long long)n;
+        const long long sum_b = 32 * (long long)n - 2 * (long long)dsum;
+        block_reduce_add2_any(sum_s, sum_b, p.obs);
+    }
+}
+
+template <int COLOR, bool OBS, bool ALWAYS, int HALVES>
+cudaError_t launch_flat(const Msc4SweepParams &p, cudaStream_t s)
+{
+    DeviceInfo info;
+    cudaError_t e = device_info(&info);
+    if (e != cudaSuccess) return e;
+    FlatSplit f;
+    f.upr = (uint32_t)(p.L / 16 / HALVES);
+    f.items = (uint32_t)p.rows * f.upr;
+    // one block per SM, equal ranges of items, in as few equal steps as fit
+    const uint32_t sms = (uint32_t)std::max(1, info.sm_count - p.spare_sms);
+    const uint32_t share = (f.items + sms - 1) / sms;
+    const uint32_t steps = (share + kFlatThreads - 1) / kFlatThreads;
+    const uint32_t threads = ((share + steps - 1) / steps + 31) / 32 * 32;
+    f.per = std::max<uint32_t>(share, 32);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((f.items + f.per - 1) / f.per);
+    cfg.blockDim = dim3(threads);
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = p.overlap && p.spare_sms == 0 ? 1 : 0;  // an overlapping kernel would take the spare SMs
+    return cudaLaunchKernelEx(&cfg, msc4_flat_kernel<COLOR, OBS, ALWAYS, HALVES>, p, f);
+}
+
 struct Occupancy {
     std::mutex mu;
     int blocks[64][16] = {};  // per device: colour x obs x always x q64
@@ -276,12 +414,28 @@ cudaError_t launch_sweep(const Msc4SweepParams &p, cudaStream_t s)
     return cudaGetLastError();
 }
 
+// Where the lines lie (us per sweep with the trace): one half word per thread
+// up to 1024 of them per SM, for the shortest chain from a kernel's wait to its
+// stores (1536^2: 4.6 against 5.2 with four), else four (2048^2: 5.4 against
+// 7.0; two are never best); and the marching kernel above 3 million pairs of
+// words (8192^2, 1 million: 53.6 against 59.8 marching; 16384^2, 4.2 million:
+// 212 against 205), and where the Philox counter q = site / 4 of the last row
+// needs more than 32 bits (L above 185363), for which it alone has a form.
+constexpr int64_t kFlatMaxPairs = 3 << 20;
+constexpr int64_t kFlatOneHalf = 1024;
+
 template <int COLOR, bool OBS, bool ALWAYS>
 cudaError_t launch_sweep_q(const Msc4SweepParams &p, cudaStream_t s)
 {
-    // the Philox counter of the last row's blocks fits 32 bits up to L = 185363
     const bool q64 = (uint64_t)(p.row0 + p.rows + 1) * (uint64_t)p.qrow > 0xFFFFFFFFull;
-    return q64 ? launch_sweep<COLOR, OBS, ALWAYS, true>(p, s) : launch_sweep<COLOR, OBS, ALWAYS, false>(p, s);
+    if (q64) return launch_sweep<COLOR, OBS, ALWAYS, true>(p, s);
+    const int64_t pairs = p.rows * (p.wpr / 2);
+    if (pairs > kFlatMaxPairs) return launch_sweep<COLOR, OBS, ALWAYS, false>(p, s);
+    DeviceInfo info;
+    cudaError_t e = device_info(&info);
+    if (e != cudaSuccess) return e;
+    return 4 * pairs <= kFlatOneHalf * info.sm_count ? launch_flat<COLOR, OBS, ALWAYS, 1>(p, s)
+                                                     : launch_flat<COLOR, OBS, ALWAYS, 4>(p, s);
 }
 
 template <int COLOR>

@@ -1,0 +1,71 @@
+"""The kernels that share the work of a sweep call, at the sizes where one
+takes over from another: bit-exact against the oracle or against the same
+lattice swept along another route."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import paper_1906_06297_gb300 as ising
+
+pytestmark = pytest.mark.gpu
+BETA = 0.4406868
+
+
+@pytest.fixture(scope="module", autouse=True)
+def built():
+    ising.build()
+    oracle.build()
+
+
+# 1536 / 1600: one and four half words per thread of the flat kernel (1024 half
+# words per SM of 152); the last row of a block's range is ragged in both
+@pytest.mark.parametrize("L,stride", [(1536, None), (1600, 1600 // 4 + 16)])
+def test_flat_kernel_matches_oracle_at_its_edges(L, stride):
+    lat = ising.Lattice(L, "msc4", row_stride_bytes=stride)
+    ising.ising_init_lattice(lat, ising.ISING_INIT_RANDOM, 7)
+    trace = torch.zeros((2, 2), dtype=torch.int64, device="cuda")
+    ising.ising_sweep(lat, BETA, 2, 7, 5, trace)
+    s = oracle.init(L, oracle.MODE_RANDOM, 7)
+    want = oracle.run(s, BETA, 2, 7, 5)
+    assert np.array_equal(oracle.from_planes_msc4(L, *lat.planes_numpy()), s)
+    assert np.array_equal(trace.cpu().numpy(), want)
+
+
+# 13824^2 / 13888^2 lie on the two sides of the marching kernel's smallest size;
+# slabs of a third of their rows take the flat kernel in both cases
+@pytest.mark.parametrize("L", [13824, 13888])
+def test_flat_and_marching_kernels_agree(L):
+    lat = ising.Lattice(L, "msc4")
+    ising.ising_init_lattice(lat, ising.ISING_INIT_RANDOM, 3)
+    slabs = []
+    for r0, rows in ising.slab_partition(L, 3):
+        sl = ising.Slab(L, r0, rows)
+        ising.ising_slab_init(sl, ising.ISING_INIT_RANDOM, 3)
+        slabs.append(sl)
+    a, b = (torch.zeros((2, 2), dtype=torch.int64, device="cuda") for _ in range(2))
+    ising.ising_sweep(lat, BETA, 2, 3, 0, a)
+    ising.ising_slab_sweep(slabs, BETA, 2, 3, 0, b)
+    assert torch.equal(a, b)
+    for colour in ("black", "white"):
+        assert torch.equal(getattr(lat, colour), torch.cat([getattr(sl, colour)[1:-1] for sl in slabs]))
+
+
+@pytest.mark.parametrize("layout,L,n", [("msc4", 256, 1), ("msc4", 1088, 3), ("int8", 130, 4)])
+def test_captured_sweeps_replay_as_called(layout, L, n):
+    """A sweep call recorded into a CUDA graph and replayed twice equals the
+    same call made twice."""
+    a, b = ising.Lattice(L, layout), ising.Lattice(L, layout)
+    for lat in (a, b):
+        ising.ising_init_lattice(lat, ising.ISING_INIT_RANDOM, 9)
+    ta, tb = (torch.zeros((n, 2), dtype=torch.int64, device="cuda") for _ in range(2))
+    ising.ising_sweep(a, BETA, n, 9, 0, ta)
+    ising.ising_sweep(a, BETA, n, 9, 0, ta)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        ising.ising_sweep(b, BETA, n, 9, 0, tb)
+    graph.replay()
+    graph.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(a.black, b.black) and torch.equal(a.white, b.white) and torch.equal(ta, tb)
