@@ -8,22 +8,278 @@
 // rand < exp(-2 beta nn s).  Here the random number is the site's keyed
 // Philox draw and the test is the exact integer form u < T[a].
 //
-// Each thread owns one Philox block, i.e. 4 consecutive sites of the plane in
-// row-major order (they may straddle a row end when L/2 is not a multiple
-// of 4), so every block is computed exactly once.
+// A thread owns one Philox block (4 consecutive sites of the plane in row-major
+// order, which may straddle a row end when L/2 is not a multiple of 4) or a run of
+// sites of one row.  int8_words_kernel takes planes whose rows are whole aligned
+// 16-byte groups, int8_rows_kernel the other ones, and int8_sweep_kernel what
+// their 32-bit indices do not reach.
 #include <cuda_runtime.h>
 
 #include <algorithm>
 
 #include "common.cuh"
 #include "launch.h"
+#include "sweep_core.cuh"
 
 namespace ising {
 
 namespace {
 
 constexpr int kThreads = 256;
+// Flat kernels: blocks of up to 512 threads at 64 registers, one per SM (so that a
+// block of the next kernel fits beside it), or two from four steps per block on.
+constexpr int kFlatThreads = 512;
 
+// ---------------------------------------------------------------------------
+// Four spins at once, one per byte of a 32-bit word (+1 = 0x01, -1 = 0xFF).
+// Bit 1 of a byte says "down", so the sum of four words masked to that bit is
+// twice the number of down neighbours, y = 2 kd in 0..8, and no carry leaves a
+// byte.  With d the number of anti-aligned neighbours (kd for an up spin, 4 - kd
+// for a down spin) and G the draw's marks (half_marks), the decision is "flip
+// iff d >= G"; per byte 16 + 2 d - 2 G lies in 12..24, and its bit 4 is the flip.
+// ---------------------------------------------------------------------------
+constexpr uint32_t kDown = 0x02020202u;
+
+__device__ __forceinline__ uint32_t byte_signs(uint32_t x)  // 0xFF where the byte's top bit is set
+{
+    uint32_t r;
+    asm("prmt.b32 %0, %1, 0, 0xBA98;" : "=r"(r) : "r"(x));
+    return r;
+}
+
+__device__ __forceinline__ uint32_t block_marks(uint32_t q, const DrawCtx &dc, const RoundKeys &rk)
+{
+    const uint4 u = philox(q, 0u, dc.c2, dc.c3, rk);
+    uint32_t g = 0, unused = 0;
+    mark_ge(g, unused, u.x, dc.T3, dc.T4, 1u << 1);
+    mark_ge(g, unused, u.y, dc.T3, dc.T4, 1u << 9);
+    mark_ge(g, unused, u.z, dc.T3, dc.T4, 1u << 17);
+    mark_ge(g, unused, u.w, dc.T3, dc.T4, 1u << 25);
+    return g;
+}
+
+// New values of the four spins t; with OBS, adds to `down` twice the number of
+// down spins among the new values and the centres and to `anti` twice the
+// anti-aligned counts after the update, both over the bytes of mask `in`.
+template <bool OBS, bool ALWAYS>
+__device__ __forceinline__ uint32_t decide_bytes(uint32_t t, uint32_t up, uint32_t cur, uint32_t dn, uint32_t side,
+                                                 uint32_t g, uint32_t in, uint32_t &down, uint32_t &anti)
+{
+    const uint32_t y = (up & kDown) + (cur & kDown) + (dn & kDown) + (side & kDown);
+    const uint32_t a = y + 0x10101010u, b = 0x18181818u - y;
+    uint32_t nt;
+    if (ALWAYS) {
+        nt = t ^ 0xFEFEFEFEu;
+    } else {
+        const uint32_t m = byte_signs(t);
+        const uint32_t x = ((a & ~m) | (b & m)) - g;
+        nt = t ^ (byte_signs(x << 3) & 0xFEFEFEFEu);
+    }
+    if (OBS) {
+        const uint32_t m = byte_signs(nt);
+        const uint32_t d2 = ((a & ~m) | (b & m)) & (0x0F0F0F0Fu & in);  // 2 d in 0..8
+        down += (((nt & (kDown & in)) + (cur & (kDown & in))) * 0x01010101u) >> 24;
+        anti += (d2 * 0x01010101u) >> 24;
+    }
+    return nt;
+}
+
+struct FlatSplit {
+    uint32_t items, per;  // items of the plane, items per block
+    uint32_t upr;         // units per row (words kernel)
+    int32_t colour;
+};
+
+// Planes whose rows are whole 16-byte groups (L/2, the row stride and the plane
+// addresses multiples of 16).  Bound by Philox's multiplies
+// as the multi-spin-coded kernel is; the byte-wise arithmetic takes about twice
+// its logic instructions per spin.  Launched as msc4_flat_kernel is (one block
+// per SM, marks before the wait for the kernel before it).  2560^2, us per
+// sweep: thread per Philox block with 64-bit site indices and byte accesses
+// 36.9, this kernel 9.3.
+template <bool OBS, bool ALWAYS>
+__global__ void __launch_bounds__(kFlatThreads, 2)
+    int8_words_kernel(const __grid_constant__ Int8SweepParams p, const __grid_constant__ FlatSplit f)
+{
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    const uint32_t end = min(f.items, (blockIdx.x + 1) * f.per);
+    const DrawCtx dc{p.c2, p.c3, p.acc.T3, p.acc.T4, p.acc.zero};
+    constexpr int WORDS = 4;
+    const uint32_t L = (uint32_t)p.L;
+    uint32_t down = 0, anti = 0, n = 0;
+    bool waited = false;
+    for (uint32_t e = blockIdx.x * f.per + threadIdx.x; e < end; e += blockDim.x) {
+        const uint32_t row = e / f.upr, u = e - row * f.upr;
+        uint32_t g[WORDS];
+#pragma unroll
+        for (int h = 0; h < WORDS; ++h) g[h] = ALWAYS ? 0u : block_marks(WORDS * e + h, dc, p.rk);
+        if (!waited) {
+            asm volatile("griddepcontrol.wait;" ::: "memory");
+            waited = true;
+        }
+        const uint32_t ru = row == 0 ? L - 1 : row - 1, rd = row + 1 == L ? 0 : row + 1;
+        const int8_t *col = p.src + 4 * WORDS * u;
+        const uint32_t *crow = reinterpret_cast<const uint32_t *>(col + row * p.stride);
+        const uint32_t *urow = reinterpret_cast<const uint32_t *>(col + ru * p.stride);
+        const uint32_t *drow = reinterpret_cast<const uint32_t *>(col + rd * p.stride);
+        uint32_t *tp = reinterpret_cast<uint32_t *>(p.tgt + row * p.stride + 4 * WORDS * u);
+        const bool left = ((row + f.colour) & 1) == 0;
+        const int32_t last = (int32_t)f.upr - 1;
+        const int32_t off = left ? (u == 0 ? WORDS * last + WORDS - 1 : -1)
+                                 : ((int32_t)u == last ? -WORDS * last : WORDS);
+        const uint4 a = *reinterpret_cast<const uint4 *>(urow), b = *reinterpret_cast<const uint4 *>(crow),
+                    c = *reinterpret_cast<const uint4 *>(drow), d = *reinterpret_cast<const uint4 *>(tp);
+        const uint32_t up[WORDS] = {a.x, a.y, a.z, a.w}, cur[WORDS] = {b.x, b.y, b.z, b.w},
+                       dn[WORDS] = {c.x, c.y, c.z, c.w};
+        uint32_t tg[WORDS] = {d.x, d.y, d.z, d.w};
+        const uint32_t edge = crow[off];
+#pragma unroll
+        for (int h = 0; h < WORDS; ++h) {
+            const uint32_t prev = h == 0 ? edge : cur[h - 1], next = h == WORDS - 1 ? edge : cur[h + 1];
+            const uint32_t side = left ? __funnelshift_l(prev, cur[h], 8) : __funnelshift_r(cur[h], next, 8);
+            tg[h] = decide_bytes<OBS, ALWAYS>(tg[h], up[h], cur[h], dn[h], side, g[h], 0xFFFFFFFFu, down, anti);
+        }
+        *reinterpret_cast<uint4 *>(tp) = make_uint4(tg[0], tg[1], tg[2], tg[3]);
+        n += 4 * WORDS;
+    }
+    if (!waited) asm volatile("griddepcontrol.wait;" ::: "memory");
+    // n white and n black spins, 4 n bonds
+    if (OBS) block_reduce_add2_any(2 * (long long)n - (long long)down, 4 * (long long)n - (long long)anti, p.obs);
+}
+
+// The 4 WORDS bytes from p on, of which the first nv are asked for, from the
+// aligned words that hold any of those (so nothing outside the row's own words
+// is read); the other bytes of x are arbitrary.
+template <int WORDS>
+__device__ __forceinline__ void ld_bytes(const int8_t *p, uint32_t nv, uint32_t (&x)[WORDS])
+{
+    const uint32_t a = (uint32_t)(uintptr_t)p & 3u;
+    const uint32_t *w = reinterpret_cast<const uint32_t *>(p - a);
+    uint32_t v[WORDS + 1];
+#pragma unroll
+    for (int h = 0; h <= WORDS; ++h) v[h] = 4 * h < nv + a ? w[h] : 0u;
+#pragma unroll
+    for (int h = 0; h < WORDS; ++h) x[h] = __funnelshift_r(v[h], v[h + 1], 8 * a);
+}
+
+// Any other plane with fewer than 2^32 sites: a thread takes up to 4 WORDS
+// consecutive sites of one row, at any byte offset.  Their draws start in the
+// middle of a Philox block when row x L/2 is not a multiple of 4: one block
+// more, and the marks are shifted by whole bytes as the spins are.  Only the
+// bytes at the two ends that fill no aligned word are stored singly.  2562^2
+// (L/2 = 1281), us per sweep: general kernel 37.3, a Philox block per thread
+// with its sites' bytes 24.2, this kernel 15.9; 8194^2 305 and 117.
+template <bool OBS, bool ALWAYS, int WORDS>
+__global__ void __launch_bounds__(kFlatThreads, 2)
+    int8_rows_kernel(const __grid_constant__ Int8SweepParams p, const __grid_constant__ FlatSplit f)
+{
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    const uint32_t end = min(f.items, (blockIdx.x + 1) * f.per);
+    const DrawCtx dc{p.c2, p.c3, p.acc.T3, p.acc.T4, p.acc.zero};
+    const uint32_t L = (uint32_t)p.L, half = (uint32_t)p.half;
+    uint32_t down = 0, anti = 0, n = 0;
+    bool waited = false;
+    for (uint32_t e = blockIdx.x * f.per + threadIdx.x; e < end; e += blockDim.x) {
+        const uint32_t row = e / f.upr, j = 4 * WORDS * (e - row * f.upr);
+        const uint32_t nv = min(4u * WORDS, half - j), site = row * half + j, o = site & 3u;
+        uint32_t g[WORDS + 1];
+#pragma unroll
+        for (int h = 0; h < WORDS; ++h) g[h] = ALWAYS ? 0u : block_marks((site >> 2) + h, dc, p.rk);
+        g[WORDS] = 0;
+        if (!ALWAYS && o != 0) g[WORDS] = block_marks((site >> 2) + WORDS, dc, p.rk);
+        if (!waited) {
+            asm volatile("griddepcontrol.wait;" ::: "memory");
+            waited = true;
+        }
+        const uint32_t ru = row == 0 ? L - 1 : row - 1, rd = row + 1 == L ? 0 : row + 1;
+        const int8_t *srow = p.src + row * p.stride;
+        int8_t *tp = p.tgt + row * p.stride + j;
+        const bool left = ((row + f.colour) & 1) == 0;
+        uint32_t up[WORDS], cur[WORDS], dn[WORDS], tg[WORDS];
+        ld_bytes<WORDS>(p.src + ru * p.stride + j, nv, up);
+        ld_bytes<WORDS>(srow + j, nv, cur);
+        ld_bytes<WORDS>(p.src + rd * p.stride + j, nv, dn);
+        ld_bytes<WORDS>(tp, nv, tg);
+        const uint32_t edge = (uint8_t)srow[left ? (j == 0 ? half : j) - 1 : (j + nv == half ? 0 : j + nv)];
+#pragma unroll
+        for (int h = 0; h < WORDS; ++h) {
+            // right: the spin after the last of the row's sites is `edge`
+            uint32_t c = cur[h], next = h + 1 < WORDS ? cur[h + 1] : edge;
+            if ((nv >> 2) == (uint32_t)h) c = (c & ~(0xFFu << (8 * (nv & 3)))) | (edge << (8 * (nv & 3)));
+            if (h + 1 < WORDS && (nv >> 2) == (uint32_t)h + 1 && (nv & 3) == 0) next = edge;
+            const uint32_t prev = h == 0 ? edge << 24 : cur[h - 1];
+            const uint32_t side = left ? __funnelshift_l(prev, cur[h], 8) : __funnelshift_r(c, next, 8);
+            const uint32_t m = 4 * h + 4 <= nv ? 0xFFFFFFFFu : (4 * h >= nv ? 0u : (1u << (8 * (nv & 3))) - 1u);
+            tg[h] = decide_bytes<OBS, ALWAYS>(tg[h], up[h], cur[h], dn[h], side, __funnelshift_r(g[h], g[h + 1], 8 * o), m,
+                                              down, anti);
+        }
+        n += nv;
+        const uint32_t a = (uint32_t)(uintptr_t)tp & 3u;
+        uint32_t *tw = reinterpret_cast<uint32_t *>(tp - a);
+#pragma unroll
+        for (int h = 0; h <= WORDS; ++h) {
+            // bytes 4 h - a .. 4 h - a + 3 of the unit
+            const uint32_t w = __funnelshift_l(h > 0 ? tg[h > 0 ? h - 1 : 0] : 0u, h < WORDS ? tg[h < WORDS ? h : 0] : 0u, 8 * a);
+            if (4 * h >= a && 4 * h + 4 <= nv + a) {
+                tw[h] = w;
+            } else if (4 * h < nv + a) {
+#pragma unroll
+                for (uint32_t k = 0; k < 4; ++k)
+                    if (4 * h + k >= a && 4 * h + k < nv + a) tp[(int)(4 * h + k) - (int)a] = (int8_t)(w >> (8 * k));
+            }
+        }
+    }
+    if (!waited) asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (OBS) block_reduce_add2_any(2 * (long long)n - (long long)down, 4 * (long long)n - (long long)anti, p.obs);
+}
+
+// One block per SM over equal ranges of `items`, which may start beside the
+// kernel before it in the stream (it waits for it itself).
+template <typename K>
+cudaError_t launch_flat(K kernel, const Int8SweepParams &p, int colour, uint32_t items, uint32_t upr, cudaStream_t s)
+{
+    DeviceInfo info;
+    cudaError_t e = device_info(&info);
+    if (e != cudaSuccess) return e;
+    uint32_t blocks = (uint32_t)info.sm_count;
+    if (items > 3 * kFlatThreads * blocks) blocks *= 2;  // see kFlatThreads
+    const uint32_t share = (items + blocks - 1) / blocks, steps = (share + kFlatThreads - 1) / kFlatThreads;
+    FlatSplit f;
+    f.items = items;
+    f.per = std::max<uint32_t>(share, 32);
+    f.upr = upr;
+    f.colour = colour;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((items + f.per - 1) / f.per);
+    cfg.blockDim = dim3(((share + steps - 1) / steps + 31) / 32 * 32);
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, p, f);
+}
+
+// The kernel for a plane, by L/2 and the alignment of its rows; units of one
+// word while one per thread fits (770^2: 4.3 us per sweep against 4.8 with four
+// words, 1026^2, two steps of one word: 6.0 against 4.4).
+template <bool OBS, bool ALWAYS>
+cudaError_t launch_small_index(const Int8SweepParams &p, int colour, cudaStream_t s)
+{
+    const uint64_t align = (uint64_t)p.half | (uint64_t)p.stride | (uintptr_t)p.src | (uintptr_t)p.tgt;
+    if (align % 16 == 0)
+        return launch_flat(int8_words_kernel<OBS, ALWAYS>, p, colour, (uint32_t)(p.nblk / 4), (uint32_t)(p.half / 16), s);
+    DeviceInfo info;
+    cudaError_t e = device_info(&info);
+    if (e != cudaSuccess) return e;
+    const uint32_t u1 = (uint32_t)((p.half + 3) / 4), u4 = (uint32_t)((p.half + 15) / 16);
+    if (p.L * u1 <= kFlatThreads * info.sm_count)
+        return launch_flat(int8_rows_kernel<OBS, ALWAYS, 1>, p, colour, (uint32_t)p.L * u1, u1, s);
+    return launch_flat(int8_rows_kernel<OBS, ALWAYS, 4>, p, colour, (uint32_t)p.L * u4, u4, s);
+}
+
+// The general form: 64-bit indices, any L.
 template <int COLOR, bool OBS>
 __global__ void __launch_bounds__(kThreads) int8_sweep_kernel(const __grid_constant__ Int8SweepParams p)
 {
@@ -127,6 +383,10 @@ cudaError_t int8_half_sweep(const Int8SweepParams &p, int colour, cudaStream_t s
 {
     const unsigned g = grid_for(p.nblk, kThreads, 8);
     const bool obs = p.obs != nullptr;
+    if (p.L * p.half < (int64_t(1) << 32)) {  // 32-bit site indices
+        if (p.acc.always) return obs ? launch_small_index<true, true>(p, colour, s) : launch_small_index<false, true>(p, colour, s);
+        return obs ? launch_small_index<true, false>(p, colour, s) : launch_small_index<false, false>(p, colour, s);
+    }
     if (colour == 0) {
         if (obs) int8_sweep_kernel<0, true><<<g, kThreads, 0, s>>>(p);
         else int8_sweep_kernel<0, false><<<g, kThreads, 0, s>>>(p);

@@ -250,9 +250,11 @@ __global__ void __launch_bounds__(kThreads, ISING_MSC4_MIN_BLOCKS)
 // blocks of 512 threads fit on an SM, one of each of two kernels.  (Blocks of
 // 128 threads, as many as there are items: the waiting blocks of the next
 // kernel gather on the SMs that finish first, 17.7 instead of 5.4 us per sweep
-// of 2048^2.)  Measured, us per sweep with the trace, marching kernel (at least
+// of 2048^2.)  From four steps per block on, where hiding a step's loads counts
+// more than the overlap, two blocks per SM: 4096^2 16.0 -> 15.2 us, 6400^2 35.3
+// -> 33.2 (2 to 3 steps: 3200^2 10.6 -> 13.9).  Measured, us per sweep with the trace, marching kernel (at least
 // 16 rows per warp) / this one: 256^2 66 / 3.6 (the host's launch rate), 2112^2
-// 66.7 / 5.6, 4096^2 67.7 / 16.0, 8192^2 68.0 / 53.6.
+// 66.7 / 5.6, 4096^2 67.7 / 15.2, 8192^2 68.0 / 52.5.
 // ---------------------------------------------------------------------------
 constexpr int kFlatThreads = 512;
 
@@ -357,8 +359,9 @@ cudaError_t launch_flat(const Msc4SweepParams &p, cudaStream_t s)
     f.upr = (uint32_t)(p.L / 16 / HALVES);
     f.items = (uint32_t)p.rows * f.upr;
     // one block per SM, equal ranges of items, in as few equal steps as fit
-    const uint32_t sms = (uint32_t)std::max(1, info.sm_count - p.spare_sms);
-    const uint32_t share = (f.items + sms - 1) / sms;
+    uint32_t blocks = (uint32_t)std::max(1, info.sm_count - p.spare_sms);
+    if (p.spare_sms == 0 && f.items > 3 * kFlatThreads * blocks) blocks *= 2;
+    const uint32_t share = (f.items + blocks - 1) / blocks;
     const uint32_t steps = (share + kFlatThreads - 1) / kFlatThreads;
     const uint32_t threads = ((share + steps - 1) / steps + 31) / 32 * 32;
     f.per = std::max<uint32_t>(share, 32);
@@ -418,7 +421,7 @@ cudaError_t launch_sweep(const Msc4SweepParams &p, cudaStream_t s)
 // up to 1024 of them per SM, for the shortest chain from a kernel's wait to its
 // stores (1536^2: 4.6 against 5.2 with four), else four (2048^2: 5.4 against
 // 7.0; two are never best); and the marching kernel above 3 million pairs of
-// words (8192^2, 1 million: 53.6 against 59.8 marching; 16384^2, 4.2 million:
+// words (8192^2, 1 million: 52.5 against 59.8 marching; 16384^2, 4.2 million:
 // 212 against 205), and where the Philox counter q = site / 4 of the last row
 // needs more than 32 bits (L above 185363), for which it alone has a form.
 constexpr int64_t kFlatMaxPairs = 3 << 20;

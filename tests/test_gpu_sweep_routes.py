@@ -32,6 +32,24 @@ def test_flat_kernel_matches_oracle_at_its_edges(L, stride):
     assert np.array_equal(trace.cpu().numpy(), want)
 
 
+# rows of whole 16-byte and 4-byte words, rows that are neither, and strides
+# that take an aligned row length off its alignment; blocks of 4 sites that
+# straddle row ends, and the largest L/2 that no kernel but the general one takes
+@pytest.mark.parametrize("L,stride", [(6, None), (8, None), (8, 5), (26, None), (30, 17), (32, None), (32, 24),
+                                      (34, None), (40, None), (96, None), (96, 50), (1286, None), (2560, None)])
+@pytest.mark.parametrize("beta", [0.0, BETA, 50.0])
+def test_int8_kernels_match_oracle(L, stride, beta):
+    lat = ising.Lattice(L, "int8", row_stride_bytes=stride)
+    ising.ising_init_lattice(lat, ising.ISING_INIT_RANDOM, 4)
+    n = 3 if L < 1000 else 1
+    trace = torch.zeros((n, 2), dtype=torch.int64, device="cuda")
+    ising.ising_sweep(lat, beta, n, 4, 2, trace)
+    s = oracle.init(L, oracle.MODE_RANDOM, 4)
+    want = oracle.run(s, beta, n, 4, 2)
+    assert np.array_equal(oracle.from_planes_int8(L, *lat.planes_numpy()), s)
+    assert np.array_equal(trace.cpu().numpy(), want)
+
+
 # 13824^2 / 13888^2 lie on the two sides of the marching kernel's smallest size;
 # slabs of a third of their rows take the flat kernel in both cases
 @pytest.mark.parametrize("L", [13824, 13888])
