@@ -473,13 +473,30 @@ ISING_API int ising_sweep(const ising_lattice_t *lat, double beta, int64_t n_swe
     rc = build_accept(beta, &acc, T);
     if (rc) return rc;
     cudaStream_t s = (cudaStream_t)stream;
-    if (trace_dev != nullptr && n_sweeps > 0) {
+    const bool traced = trace_dev != nullptr && n_sweeps > 0;
+    if (traced) {
         rc = check_device_range(trace_dev, (size_t)n_sweeps * 2 * sizeof(int64_t), "trace");
         if (rc) return rc;
+    }
+    const RoundKeys rk = make_round_keys(seed);
+    if (resident_fits(lat->L)) {
+        ResidentSweep p{};
+        p.plane[0] = lat->black;
+        p.plane[1] = lat->white;
+        p.stride = lat->row_stride_bytes;
+        p.L = (int32_t)lat->L;
+        p.bytes = lat->layout == ISING_INT8;
+        p.t0 = sweep_offset;
+        p.acc = acc;
+        p.rk = rk;
+        p.trace = (long long *)trace_dev;
+        cudaError_t e = resident_sweep(p, n_sweeps, s);
+        return e == cudaSuccess ? ISING_OK : cuda_fail(e, "resident sweep launch");
+    }
+    if (traced) {
         cudaError_t e = cudaMemsetAsync(trace_dev, 0, (size_t)n_sweeps * 2 * sizeof(int64_t), s);
         if (e != cudaSuccess) return cuda_fail(e, "trace memset");
     }
-    const RoundKeys rk = make_round_keys(seed);
     for (int64_t k = 0; k < n_sweeps; ++k) {
         const uint64_t t = sweep_offset + (uint64_t)k;
         rc = half_sweep_impl(lat, acc, rk, 0, t, nullptr, s);

@@ -119,6 +119,20 @@ struct Int8SweepParams {
     long long *obs;
 };
 
+// A sweep call of a small lattice in one launch (resident.cu).
+struct ResidentSweep {
+    void *plane[2];     // black, white
+    int64_t stride;     // bytes between rows
+    int32_t L;
+    int32_t hpr;        // half words (8 spins) per plane row; set by resident_sweep
+    int32_t bytes;      // one byte per spin (else MSC4)
+    int32_t n_sweeps;   // set by resident_sweep
+    uint64_t t0;        // index of the first sweep
+    Accept acc;
+    RoundKeys rk;
+    long long *trace;   // {sum s, sum bonds} per sweep or nullptr
+};
+
 constexpr uint32_t kNibbleLsb = 0x11111111u;
 
 // The 16 spins of an MSC4 word as 16 bits (bit k = the low bit of nibble k,

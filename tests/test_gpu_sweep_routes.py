@@ -32,6 +32,32 @@ def test_flat_kernel_matches_oracle_at_its_edges(L, stride):
     assert np.array_equal(trace.cpu().numpy(), want)
 
 
+# whole calls in one cluster: one CTA up to 16, one and two half words per
+# thread, bands of unequal rows, rows with a partial last half word and draws
+# that start inside a Philox block, recorded beyond one block of trace rows, and
+# the largest side of that route and the sides above it
+@pytest.mark.parametrize("layout,L,n,stride", [
+    ("int8", 2, 3, None), ("int8", 4, 2, 3), ("int8", 14, 3, None), ("int8", 34, 3, 20), ("int8", 62, 600, None),
+    ("int8", 130, 5, None), ("int8", 144, 4, None), ("msc4", 64, 520, None), ("msc4", 192, 6, 64), ("msc4", 320, 4, None),
+    ("int8", 398, 3, None), ("int8", 402, 2, None), ("int8", 496, 2, 300), ("msc4", 512, 3, None), ("int8", 512, 2, None),
+    ("msc4", 576, 2, None), ("int8", 766, 2, None), ("int8", 782, 2, None)])
+@pytest.mark.parametrize("beta", [0.0, BETA])
+def test_small_lattice_calls_match_oracle(layout, L, n, stride, beta):
+    lat = ising.Lattice(L, layout, row_stride_bytes=stride)
+    lat.black.fill_(85)
+    lat.white.fill_(85)
+    ising.ising_init_lattice(lat, ising.ISING_INIT_RANDOM, 6)
+    s = oracle.init(L, oracle.MODE_RANDOM, 6)
+    for off in (3, 2**32 - 1):  # the second call's sweep index crosses 32 bits
+        trace = torch.full((n, 2), 77, dtype=torch.int64, device="cuda")
+        ising.ising_sweep(lat, beta, n, 6, off, trace)
+        want = oracle.run(s, beta, n, 6, off)
+        unpack = oracle.from_planes_int8 if layout == "int8" else oracle.from_planes_msc4
+        assert np.array_equal(unpack(L, *lat.planes_numpy()), s)
+        assert np.array_equal(trace.cpu().numpy(), want)
+    assert (lat.black[:, lat.row_bytes:] == 85).all() and (lat.white[:, lat.row_bytes:] == 85).all()
+
+
 # rows of whole 16-byte and 4-byte words, rows that are neither, and strides
 # that take an aligned row length off its alignment; blocks of 4 sites that
 # straddle row ends, and the largest L/2 that no kernel but the general one takes
