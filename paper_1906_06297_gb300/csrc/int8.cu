@@ -58,6 +58,22 @@ __device__ __forceinline__ uint32_t block_marks(uint32_t q, const DrawCtx &dc, c
     return g;
 }
 
+__device__ __forceinline__ uint32_t neighbour_downs(uint32_t up, uint32_t cur, uint32_t dn, uint32_t side)
+{
+    return (up & kDown) + (cur & kDown) + (dn & kDown) + (side & kDown);
+}
+
+// Adds twice the down spins among t and the centres, and twice t's anti-aligned
+// counts given y, over the bytes of mask `in`.
+__device__ __forceinline__ void count_bytes(uint32_t t, uint32_t y, uint32_t cur, uint32_t in, uint32_t &down,
+                                            uint32_t &anti)
+{
+    const uint32_t m = byte_signs(t);
+    const uint32_t d2 = ((y & ~m) | ((0x08080808u - y) & m)) & in;  // 2 d in 0..8
+    down += (((t & (kDown & in)) + (cur & (kDown & in))) * 0x01010101u) >> 24;
+    anti += (d2 * 0x01010101u) >> 24;
+}
+
 // New values of the four spins t; with OBS, adds to `down` twice the number of
 // down spins among the new values and the centres and to `anti` twice the
 // anti-aligned counts after the update, both over the bytes of mask `in`.
@@ -65,22 +81,16 @@ template <bool OBS, bool ALWAYS>
 __device__ __forceinline__ uint32_t decide_bytes(uint32_t t, uint32_t up, uint32_t cur, uint32_t dn, uint32_t side,
                                                  uint32_t g, uint32_t in, uint32_t &down, uint32_t &anti)
 {
-    const uint32_t y = (up & kDown) + (cur & kDown) + (dn & kDown) + (side & kDown);
-    const uint32_t a = y + 0x10101010u, b = 0x18181818u - y;
+    const uint32_t y = neighbour_downs(up, cur, dn, side);
     uint32_t nt;
     if (ALWAYS) {
         nt = t ^ 0xFEFEFEFEu;
     } else {
         const uint32_t m = byte_signs(t);
-        const uint32_t x = ((a & ~m) | (b & m)) - g;
+        const uint32_t x = (((y + 0x10101010u) & ~m) | ((0x18181818u - y) & m)) - g;
         nt = t ^ (byte_signs(x << 3) & 0xFEFEFEFEu);
     }
-    if (OBS) {
-        const uint32_t m = byte_signs(nt);
-        const uint32_t d2 = ((a & ~m) | (b & m)) & (0x0F0F0F0Fu & in);  // 2 d in 0..8
-        down += (((nt & (kDown & in)) + (cur & (kDown & in))) * 0x01010101u) >> 24;
-        anti += (d2 * 0x01010101u) >> 24;
-    }
+    if (OBS) count_bytes(nt, y, cur, in, down, anti);
     return nt;
 }
 
@@ -162,6 +172,24 @@ __device__ __forceinline__ void ld_bytes(const int8_t *p, uint32_t nv, uint32_t 
     for (int h = 0; h < WORDS; ++h) x[h] = __funnelshift_r(v[h], v[h + 1], 8 * a);
 }
 
+// Mask of the bytes of word h of a unit of nv sites that hold one of them.
+__device__ __forceinline__ uint32_t bytes_in(uint32_t h, uint32_t nv)
+{
+    return 4 * h + 4 <= nv ? 0xFFFFFFFFu : (4 * h >= nv ? 0u : (1u << (8 * (nv & 3))) - 1u);
+}
+
+// The side neighbours of word h of a unit of nv centres: the bytes before them, or
+// after them, where `edge` is the one before the first or after the last.
+template <int WORDS>
+__device__ __forceinline__ uint32_t row_side(const uint32_t (&cur)[WORDS], uint32_t edge, bool left, int h, uint32_t nv)
+{
+    const uint32_t prev = h == 0 ? edge << 24 : cur[h > 0 ? h - 1 : 0];
+    uint32_t c = cur[h], next = h + 1 < WORDS ? cur[h + 1 < WORDS ? h + 1 : h] : edge;
+    if ((nv >> 2) == (uint32_t)h) c = (c & ~(0xFFu << (8 * (nv & 3)))) | (edge << (8 * (nv & 3)));
+    if ((nv >> 2) == (uint32_t)h + 1 && (nv & 3) == 0) next = edge;
+    return left ? __funnelshift_l(prev, cur[h], 8) : __funnelshift_r(c, next, 8);
+}
+
 // Any other plane with fewer than 2^32 sites: a thread takes up to 4 WORDS
 // consecutive sites of one row, at any byte offset.  Their draws start in the
 // middle of a Philox block when row x L/2 is not a multiple of 4: one block
@@ -203,13 +231,7 @@ __global__ void __launch_bounds__(kFlatThreads, 2)
         const uint32_t edge = (uint8_t)srow[left ? (j == 0 ? half : j) - 1 : (j + nv == half ? 0 : j + nv)];
 #pragma unroll
         for (int h = 0; h < WORDS; ++h) {
-            // right: the spin after the last of the row's sites is `edge`
-            uint32_t c = cur[h], next = h + 1 < WORDS ? cur[h + 1] : edge;
-            if ((nv >> 2) == (uint32_t)h) c = (c & ~(0xFFu << (8 * (nv & 3)))) | (edge << (8 * (nv & 3)));
-            if (h + 1 < WORDS && (nv >> 2) == (uint32_t)h + 1 && (nv & 3) == 0) next = edge;
-            const uint32_t prev = h == 0 ? edge << 24 : cur[h - 1];
-            const uint32_t side = left ? __funnelshift_l(prev, cur[h], 8) : __funnelshift_r(c, next, 8);
-            const uint32_t m = 4 * h + 4 <= nv ? 0xFFFFFFFFu : (4 * h >= nv ? 0u : (1u << (8 * (nv & 3))) - 1u);
+            const uint32_t side = row_side<WORDS>(cur, edge, left, h, nv), m = bytes_in(h, nv);
             tg[h] = decide_bytes<OBS, ALWAYS>(tg[h], up[h], cur[h], dn[h], side, __funnelshift_r(g[h], g[h + 1], 8 * o), m,
                                               down, anti);
         }
@@ -348,25 +370,51 @@ __global__ void int8_init_kernel(int8_t *plane, int64_t L, int64_t stride, int m
     }
 }
 
-// Thread per white site: s_w * (sum of its 4 black neighbours) visits every
-// bond once; s_w + s_b(i, j) visits every site once.
-__global__ void __launch_bounds__(256) int8_obs_kernel(const int8_t *black, const int8_t *white, int64_t L,
-                                                       int64_t stride, long long *out)
+// Observables without an update: each white site's s (sum of its 4 black
+// neighbours) visits every bond once, s_w + s_b every site once.  A thread takes
+// up to 16 sites of a row, as int8_rows_kernel does; WIDE: its rows are whole
+// aligned 16-byte groups.  16384^2: thread per site 649 us, here 97, WIDE 51.6
+// (5.2 TB/s).
+template <typename I, bool WIDE>
+__global__ void __launch_bounds__(256) int8_obs_kernel(const int8_t *__restrict__ black,
+                                                       const int8_t *__restrict__ white, int64_t L, int64_t stride,
+                                                       long long *out)
 {
-    const int64_t half = L / 2, nsites = L * half;
-    long long sum_s = 0, sum_b = 0;
-    for (int64_t site = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; site < nsites;
-         site += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t i = site / half, j = site - i * half;
-        const int64_t iu = i == 0 ? L - 1 : i - 1, id = i + 1 == L ? 0 : i + 1;
-        const int64_t joff = (i & 1) ? (j == 0 ? half - 1 : j - 1) : (j + 1 == half ? 0 : j + 1);
-        const int centre = black[i * stride + j];
-        const int nn = black[iu * stride + j] + black[id * stride + j] + centre + black[i * stride + joff];
-        const int s = white[i * stride + j];
-        sum_s += s + centre;
-        sum_b += s * nn;
+    const uint32_t half = (uint32_t)(L / 2);
+    const I upr = (I)((half + 15) / 16), items = (I)L * upr, step = (I)gridDim.x * 256;
+    long long n = 0, down_sum = 0, anti_sum = 0;
+    for (I e = (I)blockIdx.x * 256 + threadIdx.x; e < items; e += step) {
+        const I row = e / upr;
+        const uint32_t j = 16 * (uint32_t)(e - row * upr), nv = WIDE ? 16u : min(16u, half - j);
+        const I ru = row == 0 ? (I)L - 1 : row - 1, rd = row + 1 == (I)L ? 0 : row + 1;
+        const int8_t *srow = black + (int64_t)row * stride;
+        const bool left = (row & 1) != 0;
+        uint32_t up[4], cur[4], dn[4], t[4];
+        auto load = [&](const int8_t *p, uint32_t (&x)[4]) {
+            if constexpr (WIDE) {
+                const uint4 v = *reinterpret_cast<const uint4 *>(p);
+                x[0] = v.x, x[1] = v.y, x[2] = v.z, x[3] = v.w;
+            } else {
+                ld_bytes<4>(p, nv, x);
+            }
+        };
+        load(black + (int64_t)ru * stride + j, up);
+        load(srow + j, cur);
+        load(black + (int64_t)rd * stride + j, dn);
+        load(white + (int64_t)row * stride + j, t);
+        const uint32_t edge = (uint8_t)srow[left ? (j == 0 ? half : j) - 1 : (j + nv == half ? 0 : j + nv)];
+        uint32_t down = 0, anti = 0;
+#pragma unroll
+        for (int h = 0; h < 4; ++h) {
+            const uint32_t m = bytes_in(h, nv);
+            const uint32_t side = row_side<4>(cur, edge, left, h, nv);
+            count_bytes(t[h], neighbour_downs(up[h], cur[h], dn[h], side), cur[h], m, down, anti);
+        }
+        n += nv;
+        down_sum += down;
+        anti_sum += anti;
     }
-    block_reduce_add2<256>(sum_s, sum_b, out);
+    block_reduce_add2<256>(2 * n - down_sum, 4 * n - anti_sum, out);
 }
 
 unsigned grid_for(int64_t n, int threads, int per_sm)
@@ -410,7 +458,12 @@ cudaError_t int8_init(int8_t *plane, int colour, int64_t L, int64_t stride, int 
 cudaError_t int8_observables(const int8_t *black, const int8_t *white, int64_t L, int64_t stride, long long *out,
                              cudaStream_t s)
 {
-    int8_obs_kernel<<<grid_for(L * (L / 2), 256, 8), 256, 0, s>>>(black, white, L, stride, out);
+    const int64_t items = L * ((L / 2 + 15) / 16);
+    const unsigned g = grid_for(items, 256, 8);
+    const bool wide = ((uint64_t)(L / 2) | (uint64_t)stride | (uintptr_t)black | (uintptr_t)white) % 16 == 0;
+    auto go = [&](auto kernel) { kernel<<<g, 256, 0, s>>>(black, white, L, stride, out); };
+    if (items < (int64_t(1) << 31)) wide ? go(int8_obs_kernel<uint32_t, true>) : go(int8_obs_kernel<uint32_t, false>);
+    else wide ? go(int8_obs_kernel<uint64_t, true>) : go(int8_obs_kernel<uint64_t, false>);
     return cudaGetLastError();
 }
 

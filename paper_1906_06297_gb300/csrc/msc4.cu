@@ -450,102 +450,150 @@ cudaError_t launch_sweep_colour(const Msc4SweepParams &p, cudaStream_t s)
 }
 
 // ---------------------------------------------------------------------------
-// Initial state: thread per word.  Random: spin n of word (i, w) has plane site
-// i*L/2 + 16w + n and is +1 iff its purpose-1 draw at t = 0 is below 2^31.
+// Passes over a whole plane: initial state, observables, layout conversion.  A
+// thread takes a pair of words (16 bytes), and I, the index type, is 32-bit
+// where the plane's pairs fit it: a 64-bit division per word took longer than
+// its memory traffic.
 // ---------------------------------------------------------------------------
-__global__ void msc4_init_kernel(uint64_t *plane, int64_t L, int64_t rows, int64_t row0, int64_t stride, int mode,
-                                 uint32_t c3, const __grid_constant__ RoundKeys rk)
+constexpr int kPassThreads = 256;
+
+__device__ __forceinline__ uint32_t up_bit(uint32_t u, uint32_t bit) { return (int32_t)u >= 0 ? bit : 0u; }
+
+// Random: spin n of word (i, w) has plane site i*L/2 + 16w + n and is +1 iff its
+// purpose-1 draw at t = 0 is below 2^31.  Bound by Philox; the eight blocks of a
+// pair share the rounds' common products.  16384^2, us per plane: thread per
+// word 101.9, here 89.4 (Philox alone: 74).
+template <typename I>
+__global__ void __launch_bounds__(kPassThreads, 4) msc4_init_kernel(uint64_t *plane, int64_t L, int64_t rows, int64_t row0,
+                                                                 int64_t stride, int mode, uint32_t c3,
+                                                                 const __grid_constant__ RoundKeys rk)
 {
-    const int64_t wpr = L / 32, qrow = L / 8;
-    const int64_t n = rows * wpr;
-    for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < n;
-         idx += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t i = idx / wpr, w = idx - i * wpr;  // local row i = global row row0 + i
-        uint64_t word;
-        if (mode == 1) {
-            word = 0x1111111111111111ull;
-        } else if (mode == 2) {
-            word = 0;
-        } else {
-            word = 0;
-            const uint64_t q0 = (uint64_t)(row0 + i) * qrow + 4 * (uint64_t)w;
+    const I ppr = (I)(L / 64), n = (I)rows * ppr, step = (I)gridDim.x * kPassThreads;
+    for (I idx = (I)blockIdx.x * kPassThreads + threadIdx.x; idx < n; idx += step) {
+        const I i = idx / ppr, w = 2 * (idx - i * ppr);  // local row i = global row row0 + i
+        uint32_t h[4];
+        if (mode != 0) {
 #pragma unroll
-            for (int b = 0; b < 4; ++b) {
-                const uint4 u = philox((uint32_t)q0 + b, (uint32_t)(q0 >> 32), 0u, c3, rk);
-                const int sh = 16 * b;
-                word |= ((uint64_t)(u.x < 0x80000000u) << sh) | ((uint64_t)(u.y < 0x80000000u) << (sh + 4)) |
-                        ((uint64_t)(u.z < 0x80000000u) << (sh + 8)) | ((uint64_t)(u.w < 0x80000000u) << (sh + 12));
+            for (int k = 0; k < 4; ++k) h[k] = mode == 1 ? kNibbleLsb : 0u;
+        } else {
+            const uint64_t q0 = (uint64_t)(row0 + i) * (uint64_t)(L / 8) + 4 * (uint64_t)w;  // a multiple of 8
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                h[k] = 0;
+#pragma unroll
+                for (int b = 0; b < 2; ++b) {
+                    const uint4 u = philox((uint32_t)q0 | (2 * k + b), (uint32_t)(q0 >> 32), 0u, c3, rk);
+                    h[k] |= up_bit(u.x, 1u << (16 * b)) | up_bit(u.y, 0x10u << (16 * b)) | up_bit(u.z, 0x100u << (16 * b)) |
+                            up_bit(u.w, 0x1000u << (16 * b));
+                }
             }
         }
-        plane[i * stride + w] = word;
+        st128(plane + (int64_t)i * stride + w, make_uint4(h[0], h[1], h[2], h[3]));
     }
 }
 
-// ---------------------------------------------------------------------------
-// Observables without an update: thread per white word.  Same neighbour rule
-// as the white half-sweep; each white site contributes s * (sum of its black
-// neighbours) = 4 - 2d (d = anti-aligned count), each site its spin.
-// ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) msc4_obs_kernel(const uint64_t *black, const uint64_t *white, int64_t L,
-                                                       int64_t stride, long long *out)
+// Observables without an update.  Same neighbour rule as the white half-sweep;
+// each white site contributes s * (sum of its black neighbours) = 4 - 2d (d =
+// anti-aligned count), each site its spin.  Bound by memory: four loads per pair,
+// two of them of rows that a neighbour in the grid loads too (L1, L2).  16384^2:
+// thread per word 70.2 us, here 25.1 (5.3 TB/s).
+template <typename I>
+__global__ void __launch_bounds__(kPassThreads) msc4_obs_kernel(const uint64_t *__restrict__ black,
+                                                                const uint64_t *__restrict__ white, int64_t L,
+                                                                int64_t stride, long long *out)
 {
-    const int64_t wpr = L / 32;
-    const int64_t n = L * wpr;
+    const I ppr = (I)(L / 64), n = (I)L * ppr, step = (I)gridDim.x * kPassThreads;
     long long ones = 0, dsum = 0, cnt = 0;
-    for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < n;
-         idx += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t i = idx / wpr, w = idx - i * wpr;
-        const int64_t iu = i == 0 ? L - 1 : i - 1, id = i + 1 == L ? 0 : i + 1;
-        const uint64_t C = black[i * stride + w];
-        uint64_t side;
-        if ((i & 1) == 1) {  // white, odd row: left word
-            const uint64_t W = black[i * stride + (w == 0 ? wpr - 1 : w - 1)];
-            side = (C << 4) | (W >> 60);
-        } else {
-            const uint64_t E = black[i * stride + (w + 1 == wpr ? 0 : w + 1)];
-            side = (C >> 4) | (E << 60);
-        }
-        const uint64_t k = black[iu * stride + w] + black[id * stride + w] + C + side;
-        const uint64_t s = white[i * stride + w];
-        const uint64_t m = s * 15ull;
-        const uint64_t d = (k & ~m) | ((0x4444444444444444ull - k) & m);
-        const uint64_t nib = (d & 0x0F0F0F0F0F0F0F0Full) + ((d >> 4) & 0x0F0F0F0F0F0F0F0Full);
-        dsum += (long long)((nib * 0x0101010101010101ull) >> 56);
-        ones += __popcll(s) + __popcll(C);
+    for (I idx = (I)blockIdx.x * kPassThreads + threadIdx.x; idx < n; idx += step) {
+        const I i = idx / ppr, u = idx - i * ppr;
+        const I iu = i == 0 ? (I)L - 1 : i - 1, id = i + 1 == (I)L ? 0 : i + 1;
+        const uint64_t *row = black + (int64_t)i * stride;
+        const bool left = (i & 1) == 1;  // white, odd row: left word
+        const uint4 c = *reinterpret_cast<const uint4 *>(row + 2 * u);
+        const uint4 a = *reinterpret_cast<const uint4 *>(black + (int64_t)iu * stride + 2 * u);
+        const uint4 b = *reinterpret_cast<const uint4 *>(black + (int64_t)id * stride + 2 * u);
+        const uint4 s = *reinterpret_cast<const uint4 *>(white + (int64_t)i * stride + 2 * u);
+        const uint32_t *half = reinterpret_cast<const uint32_t *>(row);
+        const uint32_t edge = left ? half[4 * (u == 0 ? ppr : u) - 1] : half[u + 1 == ppr ? 0 : 4 * (u + 1)];
+        uint4 sd;
+        if (left)
+            sd = make_uint4(__funnelshift_l(edge, c.x, 4), __funnelshift_l(c.x, c.y, 4), __funnelshift_l(c.y, c.z, 4),
+                            __funnelshift_l(c.z, c.w, 4));
+        else
+            sd = make_uint4(__funnelshift_r(c.x, c.y, 4), __funnelshift_r(c.y, c.z, 4), __funnelshift_r(c.z, c.w, 4),
+                            __funnelshift_r(c.w, edge, 4));
+        auto anti = [](uint32_t t, uint32_t sp) {  // anti-aligned counts of 8 sites, by bytes
+            const uint32_t m = sp * 15u;
+            const uint32_t d = (t & ~m) | ((0x44444444u - t) & m);
+            return (d & 0x0F0F0F0Fu) + ((d >> 4) & 0x0F0F0F0Fu);
+        };
+        const uint32_t d = anti(a.x + b.x + c.x + sd.x, s.x) + anti(a.y + b.y + c.y + sd.y, s.y) +
+                           anti(a.z + b.z + c.z + sd.z, s.z) + anti(a.w + b.w + c.w + sd.w, s.w);
+        const uint32_t n8 = s.x + s.y + s.z + s.w + c.x + c.y + c.z + c.w;  // up spins, at most 8 per nibble
+        const uint32_t o = (n8 & 0x0F0F0F0Fu) + ((n8 >> 4) & 0x0F0F0F0Fu);
+        dsum += (d * 0x01010101u) >> 24;
+        ones += (o * 0x01010101u) >> 24;
         cnt += 1;
     }
-    block_reduce_add2<256>(2 * ones - 32 * cnt, 64 * cnt - 2 * dsum, out);
+    // 32 white and 32 black spins and 128 bonds per pair of words
+    block_reduce_add2<kPassThreads>(2 * ones - 64 * cnt, 128 * cnt - 2 * dsum, out);
 }
 
-// ---------------------------------------------------------------------------
-// Layout conversion: thread per word; int8 column j <-> word j/16, nibble j%16.
-// ---------------------------------------------------------------------------
-__global__ void msc4_pack_kernel(const int8_t *src, int64_t sstride, uint64_t *dst, int64_t dstride, int64_t L)
+// Layout conversion: int8 column j <-> word j/16, nibble j%16; thread per word.
+// WIDE: the bytes' rows are 16-byte aligned, so 16 of them are one access (a
+// thread's bytes one at a time: 371 us per plane of 16384^2 to unpack and 63 to
+// pack, here 30.4 and 31.0, 6.6 TB/s).
+template <typename I, bool WIDE>
+__global__ void __launch_bounds__(kPassThreads) msc4_pack_kernel(const int8_t *__restrict__ src, int64_t sstride,
+                                                                 uint64_t *__restrict__ dst, int64_t dstride, int64_t L)
 {
-    const int64_t wpr = L / 32, n = L * wpr;
-    for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < n;
-         idx += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t i = idx / wpr, w = idx - i * wpr;
-        const int8_t *row = src + i * sstride + 16 * w;
-        uint64_t word = 0;
+    const I wpr = (I)(L / 32), n = (I)L * wpr, step = (I)gridDim.x * kPassThreads;
+    for (I idx = (I)blockIdx.x * kPassThreads + threadIdx.x; idx < n; idx += step) {
+        const I i = idx / wpr, w = idx - i * wpr;
+        const int8_t *row = src + (int64_t)i * sstride + 16 * (int64_t)w;
+        if constexpr (WIDE) {
+            const uint4 v = *reinterpret_cast<const uint4 *>(row);
+            auto nibbles = [](uint32_t lo, uint32_t hi) {
+                lo = __vcmpgts4(lo, 0u) & 0x01010101u;
+                hi = __vcmpgts4(hi, 0u) & 0x01010101u;
+                return __byte_perm(lo, hi, 0x6420) | (__byte_perm(lo, hi, 0x7531) << 4);
+            };
+            dst[(int64_t)i * dstride + w] = (uint64_t)nibbles(v.x, v.y) | ((uint64_t)nibbles(v.z, v.w) << 32);
+        } else {
+            uint64_t word = 0;
 #pragma unroll
-        for (int t = 0; t < 16; ++t) word |= (uint64_t)(row[t] > 0) << (4 * t);
-        dst[i * dstride + w] = word;
+            for (int t = 0; t < 16; ++t) word |= (uint64_t)(row[t] > 0) << (4 * t);
+            dst[(int64_t)i * dstride + w] = word;
+        }
     }
 }
 
-__global__ void msc4_unpack_kernel(const uint64_t *src, int64_t sstride, int8_t *dst, int64_t dstride, int64_t L)
+template <typename I, bool WIDE>
+__global__ void __launch_bounds__(kPassThreads) msc4_unpack_kernel(const uint64_t *__restrict__ src, int64_t sstride,
+                                                                   int8_t *__restrict__ dst, int64_t dstride, int64_t L)
 {
-    const int64_t wpr = L / 32, n = L * wpr;
-    for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < n;
-         idx += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t i = idx / wpr, w = idx - i * wpr;
-        const uint64_t word = src[i * sstride + w];
-        int8_t *row = dst + i * dstride + 16 * w;
+    const I wpr = (I)(L / 32), n = (I)L * wpr, step = (I)gridDim.x * kPassThreads;
+    for (I idx = (I)blockIdx.x * kPassThreads + threadIdx.x; idx < n; idx += step) {
+        const I i = idx / wpr, w = idx - i * wpr;
+        const uint64_t word = src[(int64_t)i * sstride + w];
+        int8_t *row = dst + (int64_t)i * dstride + 16 * (int64_t)w;
+        if constexpr (WIDE) {
+            auto bytes = [](uint32_t h, uint32_t sel) {  // four nibbles to +1 (0x01) or -1 (0xFF)
+                const uint32_t v = __byte_perm(h & 0x01010101u, (h >> 4) & 0x01010101u, sel);
+                return 0xFFFFFFFFu ^ (v * 0xFEu);
+            };
+            const uint32_t lo = (uint32_t)word, hi = (uint32_t)(word >> 32);
+            *reinterpret_cast<uint4 *>(row) =
+                make_uint4(bytes(lo, 0x5140), bytes(lo, 0x7362), bytes(hi, 0x5140), bytes(hi, 0x7362));
+        } else {
 #pragma unroll
-        for (int t = 0; t < 16; ++t) row[t] = ((word >> (4 * t)) & 1) ? 1 : -1;
+            for (int t = 0; t < 16; ++t) row[t] = ((word >> (4 * t)) & 1) ? 1 : -1;
+        }
     }
 }
+
+// Items below which a pass and its last step over the end stay within 32 bits.
+constexpr int64_t kIndex32 = int64_t(1) << 31;
 
 unsigned grid_for(int64_t n, int threads)
 {
@@ -566,9 +614,14 @@ cudaError_t msc4_init(uint64_t *plane, int colour, int64_t L, int64_t rows, int6
                       int mode, uint64_t seed, cudaStream_t s)
 {
     const RoundKeys rk = make_round_keys(seed);
-    const int64_t n = rows * (L / 32);
-    msc4_init_kernel<<<grid_for(n, 256), 256, 0, s>>>(plane, L, rows, row0, stride_words, mode,
-                                                      counter_word3(colour, kPurposeInit, 0), rk);
+    const int64_t n = rows * (L / 64);
+    const uint32_t c3 = counter_word3(colour, kPurposeInit, 0);
+    if (n < kIndex32)
+        msc4_init_kernel<uint32_t><<<grid_for(n, kPassThreads), kPassThreads, 0, s>>>(plane, L, rows, row0, stride_words,
+                                                                                      mode, c3, rk);
+    else
+        msc4_init_kernel<uint64_t><<<grid_for(n, kPassThreads), kPassThreads, 0, s>>>(plane, L, rows, row0, stride_words,
+                                                                                      mode, c3, rk);
     return cudaGetLastError();
 }
 
@@ -593,8 +646,10 @@ cudaError_t msc4_copy_rows(const HaloCopy &c, int n, int64_t words, cudaStream_t
 cudaError_t msc4_observables(const uint64_t *black, const uint64_t *white, int64_t L, int64_t stride_words,
                              long long *out, cudaStream_t s)
 {
-    const int64_t n = L * (L / 32);
-    msc4_obs_kernel<<<grid_for(n, 256), 256, 0, s>>>(black, white, L, stride_words, out);
+    const int64_t n = L * (L / 64);
+    const unsigned g = grid_for(n, kPassThreads);
+    if (n < kIndex32) msc4_obs_kernel<uint32_t><<<g, kPassThreads, 0, s>>>(black, white, L, stride_words, out);
+    else msc4_obs_kernel<uint64_t><<<g, kPassThreads, 0, s>>>(black, white, L, stride_words, out);
     return cudaGetLastError();
 }
 
@@ -602,7 +657,11 @@ cudaError_t msc4_pack(const int8_t *src, int64_t src_stride, uint64_t *dst, int6
                       cudaStream_t s)
 {
     const int64_t n = L * (L / 32);
-    msc4_pack_kernel<<<grid_for(n, 256), 256, 0, s>>>(src, src_stride, dst, dst_stride_words, L);
+    const unsigned g = grid_for(n, kPassThreads);
+    const bool wide = ((uintptr_t)src | (uint64_t)src_stride) % 16 == 0;
+    auto go = [&](auto kernel) { kernel<<<g, kPassThreads, 0, s>>>(src, src_stride, dst, dst_stride_words, L); };
+    if (n < kIndex32) wide ? go(msc4_pack_kernel<uint32_t, true>) : go(msc4_pack_kernel<uint32_t, false>);
+    else wide ? go(msc4_pack_kernel<uint64_t, true>) : go(msc4_pack_kernel<uint64_t, false>);
     return cudaGetLastError();
 }
 
@@ -610,7 +669,11 @@ cudaError_t msc4_unpack(const uint64_t *src, int64_t src_stride_words, int8_t *d
                         cudaStream_t s)
 {
     const int64_t n = L * (L / 32);
-    msc4_unpack_kernel<<<grid_for(n, 256), 256, 0, s>>>(src, src_stride_words, dst, dst_stride, L);
+    const unsigned g = grid_for(n, kPassThreads);
+    const bool wide = ((uintptr_t)dst | (uint64_t)dst_stride) % 16 == 0;
+    auto go = [&](auto kernel) { kernel<<<g, kPassThreads, 0, s>>>(src, src_stride_words, dst, dst_stride, L); };
+    if (n < kIndex32) wide ? go(msc4_unpack_kernel<uint32_t, true>) : go(msc4_unpack_kernel<uint32_t, false>);
+    else wide ? go(msc4_unpack_kernel<uint64_t, true>) : go(msc4_unpack_kernel<uint64_t, false>);
     return cudaGetLastError();
 }
 

@@ -113,3 +113,24 @@ def test_captured_sweeps_replay_as_called(layout, L, n):
     graph.replay()
     torch.cuda.synchronize()
     assert torch.equal(a.black, b.black) and torch.equal(a.white, b.white) and torch.equal(ta, tb)
+
+
+# one-byte rows on and off 16-byte boundaries: the wide and the byte-wise conversions
+@pytest.mark.parametrize("L,stride", [(64, None), (192, None), (192, 97), (448, 240)])
+def test_conversions_at_any_row_alignment(L, stride):
+    a, b = ising.Lattice(L, "int8", row_stride_bytes=stride), ising.Lattice(L, "int8", row_stride_bytes=stride)
+    m = ising.Lattice(L, "msc4")
+    for lat in (a, b):
+        lat.black.fill_(85)
+        lat.white.fill_(85)
+    ising.ising_init_lattice(a, ising.ISING_INIT_RANDOM, 8)
+    s = oracle.init(L, oracle.MODE_RANDOM, 8)
+    ising.ising_pack(a, m)
+    assert np.array_equal(oracle.from_planes_msc4(L, *m.planes_numpy()), s)
+    ising.ising_unpack(m, b)
+    assert torch.equal(a.black, b.black) and torch.equal(a.white, b.white)
+    obs = torch.zeros((2, 2), dtype=torch.int64, device="cuda")
+    ising.ising_observables(a, obs[0])
+    ising.ising_observables(m, obs[1])
+    want = [int(s.sum()), int((s.astype(int) * (np.roll(s, -1, 0) + np.roll(s, -1, 1))).sum())]
+    assert obs.tolist() == [want, want]
