@@ -19,11 +19,16 @@
 // The exchange draw of slot pair (k, k+1) of ladder l at sweep t is the
 // purpose-2 draw of site k in stream l.
 //
-// Schedule (one cooperative launch, grid-wide barriers between phases):
+// Schedule (one cooperative launch):
 //   for each sweep t:  black half-sweep | barrier | white half-sweep
 //   (with per-lattice observables when t is a record sweep) | barrier |
 //   on record sweeps: record and exchange | barrier.
-// Every barrier wait is bounded: after `timeout_cycles` the block sets the
+// Where whole lattices can be dealt to the SMs (or pairs or quads of SMs, as
+// thread-block clusters) evenly enough, each of these owners sweeps its own
+// lattices, the barriers between half-sweeps are the block's (the cluster's)
+// own, and only the two around an exchange are grid-wide; else every half-sweep
+// is shared by the whole grid and every barrier is grid-wide (see pick_owners).
+// Every grid-wide wait is bounded: after `timeout_cycles` the block sets the
 // error flag to ISING_ETIMEOUT and the whole grid returns.
 #include <cuda_runtime.h>
 
@@ -51,16 +56,16 @@ namespace {
 
 constexpr int kMaxGroups = 16;
 constexpr int kMarchMinL = 128;  // smallest side of the row-marching path
+constexpr int kMaxOwners = 160;
 
 struct BatchGroup {
     int64_t first;        // first lattice id of the group
     int64_t count;        // lattices in the group
     int64_t word_base;    // word offset of the first lattice's plane
-    int64_t chunk_begin;  // first chunk (32 items) of the group
     int64_t items;        // items per lattice = L * wpr / wpt
-    int64_t weight_begin; // cumulative work weight of the groups before this one
     int32_t L, wpr, wpt, gpr;  // side, words per row, words per item, items per row
-    int32_t weight;       // work weight of one chunk: wpt + kappa
+    int32_t weight;       // work weight of one chunk
+    int32_t log2L;        // of a march group
     int32_t march;        // 1: rows marched by lane groups (side a power of two, 128 .. 2048)
 };
 
@@ -71,68 +76,120 @@ struct BatchParams {
     int32_t S;            // ladder size
     int64_t n;            // lattices
     int64_t n_ladders;
-    int64_t n_chunks;
-    int64_t plane_words;  // words of one colour plane over all lattices
-    int64_t total_weight; // sum of the chunk weights
     int32_t *slot_of;     // [n] slot of each lattice
     int32_t *lattice_at;  // [n_ladders * S] lattice at each (ladder, slot)
     const uint32_t *thr;  // [S][2] (T3, T4) of each slot's beta
     const int64_t *swap_off, *swap_len;  // [S - 1] exchange threshold tables
     const uint64_t *swap_tab;
     long long *acc;       // [n][2] observables accumulators
+    long long *acc2;      // owners: the accumulators and the ladders' state of every
+    int32_t *lattice_at2; // other event (nullptr: the grid must share every lattice)
     long long *trace;     // [events][n][2] or nullptr
-    unsigned *bar;        // [0] arrivals, [1] generation
-    int *err;
+    unsigned *bar;        // the grid barrier's word, 8-byte aligned
+    int *err;             // error flag, the word after it
     int64_t n_sweeps;
     uint64_t t0;
     int64_t event_first;
     int32_t record_every, swaps;
     long long timeout_cycles;
     int32_t expect_blocks;  // blocks a barrier waits for (gridDim.x; larger only in the self-test)
+    int32_t cs;             // blocks per owner; 0: the grid shares every lattice
+    int32_t sync_every;     // owners: sweeps after which they meet without a record
+    uint32_t part[kMaxGroups][kMaxOwners + 1];  // owner o sweeps lattices part[g][o] .. part[g][o + 1] - 1 of group g
     RoundKeys rk;
 };
 
 // ---------------------------------------------------------------------------
-// Grid-wide barrier with a bounded wait.  Thread 0 of each block arrives on a
-// counter; the last arrival resets it and bumps the generation word, which
-// the others poll.  Returns false (in every thread) once any block has set
-// the error flag; the caller then returns.
+// Grid-wide barrier with a bounded wait.  Thread 0 of each block adds to one
+// counter word: 1, or for block 0 what brings the sum of all blocks to 2^31, so
+// the word's top bit flips when the last block arrives and its other bits are 0
+// again.  The others poll the word together with the error flag beside it (one
+// 64-bit load).  Returns false (in every thread) once any block has set the
+// error flag; the caller then returns.  (An arrival counter that the last block
+// resets beside a generation word, polled with sleeps of 128 ns: 0.7 us
+// more per record of a batch of 384 lattices and 1.1 per half-sweep of 4 of 640^2.)
 // ---------------------------------------------------------------------------
 __device__ bool grid_sync(const BatchParams &p)
 {
     __shared__ int s_ok;
     __syncthreads();
     if (threadIdx.x == 0) {
-        volatile unsigned *gen = p.bar + 1;
-        volatile int *err = p.err;
-        const unsigned g0 = *gen;
         __threadfence();
-        const unsigned arrived = atomicAdd(p.bar, 1u) + 1;
-        if (arrived == (unsigned)p.expect_blocks) {
-            atomicExch(p.bar, 0u);
-            __threadfence();
-            atomicAdd(p.bar + 1, 1u);
-        } else {
-            const long long start = clock64();
-            while (*gen == g0) {
-                if (*err != 0) break;
-                if (clock64() - start > p.timeout_cycles) {
-                    atomicCAS(p.err, 0, (int)ISING_ETIMEOUT);
-                    break;
-                }
-                __nanosleep(128);
+        const unsigned old = atomicAdd(p.bar, blockIdx.x == 0 ? 0x80000000u - (unsigned)(p.expect_blocks - 1) : 1u);
+        const long long start = clock64();
+        unsigned err;
+        for (;;) {
+            unsigned long long v;
+            asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p.bar) : "memory");
+            err = (unsigned)(v >> 32);
+            if (((old ^ (unsigned)v) >> 31) || err) break;
+            if (clock64() - start > p.timeout_cycles) {
+                atomicCAS(p.err, 0, (int)ISING_ETIMEOUT);
+                err = (unsigned)ISING_ETIMEOUT;
+                break;
             }
         }
         __threadfence();
-        s_ok = (*err == 0);
+        s_ok = err == 0;
     }
     __syncthreads();
     return s_ok != 0;
 }
 
+// The chunks that a block's owner (the whole grid, or the block's cluster) has to
+// sweep, numbered through its lattices of all groups, and a warp's share of them:
+// the contiguous chunks whose starting weight lies in [w W / nw, (w + 1) W / nw) of
+// the total weight W, for warp w of the owner's nw.
+struct Split {
+    int64_t chunk[kMaxGroups + 1];  // the owner's first chunk of each group; [n_groups]: all of them
+    int64_t shift[kMaxGroups];      // what leads from there to the chunk's number in its group
+};
+
+__device__ void fill_split(const BatchParams &p, Split &sp, int64_t &cb, int64_t &ce)
+{
+    __shared__ int64_t weight[kMaxGroups + 1];
+    if (threadIdx.x == 0) {
+        const int o = p.cs > 0 ? (int)blockIdx.x / p.cs : 0;
+        int64_t c = 0, w = 0;
+        for (int g = 0; g < p.n_groups; ++g) {
+            const BatchGroup &G = p.g[g];
+            const int64_t per = G.items / 32;  // chunks per lattice
+            const int64_t first = p.cs > 0 ? p.part[g][o] : 0, count = p.cs > 0 ? p.part[g][o + 1] - first : G.count;
+            sp.chunk[g] = c;
+            sp.shift[g] = first * per - c;
+            weight[g] = w;
+            c += count * per;
+            w += count * per * G.weight;
+        }
+        sp.chunk[p.n_groups] = c;
+        weight[p.n_groups] = w;
+    }
+    __syncthreads();
+    const int64_t W = weight[p.n_groups];
+    const int wpb = (int)(blockDim.x >> 5);
+    // consecutive shares go to the warps of one scheduler (warp % 4): shares differ
+    // by a chunk in a regular pattern, which dealt to the warps in their order gave
+    // one scheduler all the long ones
+    const int wb = threadIdx.x >> 5, share = (wb & 3) * (wpb >> 2) + (wb >> 2);
+    const int64_t warp = (int64_t)(p.cs > 0 ? (int)blockIdx.x % p.cs : (int)blockIdx.x) * wpb + share;
+    const int64_t nw = (int64_t)(p.cs > 0 ? p.cs : (int)gridDim.x) * wpb;
+    auto chunk_at = [&](int64_t w) -> int64_t {
+        if (w >= W) return sp.chunk[p.n_groups];
+        int g = 0;
+        while (g + 1 < p.n_groups && weight[g + 1] <= w) ++g;
+        const int64_t per = p.g[g].weight;
+        return sp.chunk[g] + (w - weight[g] + per - 1) / per;
+    };
+    cb = chunk_at(warp * W / nw);
+    ce = chunk_at((warp + 1) * W / nw);
+}
+
+// Between two half-sweeps of an owner's lattices.
+__device__ bool phase_sync(const BatchParams &p);
+
 // One work item: `WPT` consecutive words of row r of one lattice.
 template <int WPT, bool OBS>
-__device__ __forceinline__ void sweep_item(const uint64_t *__restrict__ src, uint64_t *__restrict__ tgt, int L,
+__device__ __forceinline__ void sweep_item(const uint64_t *src, uint64_t *tgt, int L,
                                            int wpr, int r, int w0, int colour, uint32_t stream, const DrawCtx &dc,
                                            const RoundKeys &rk, uint32_t &ones, uint32_t &dsum)
 {
@@ -174,6 +231,18 @@ __device__ __forceinline__ void sweep_item(const uint64_t *__restrict__ src, uin
     if (OBS) dsum += (dacc & 0xFFu) + ((dacc >> 8) & 0xFFu) + ((dacc >> 16) & 0xFFu) + (dacc >> 24);
 }
 
+__device__ bool phase_sync(const BatchParams &p)
+{
+    if (p.cs == 0) return grid_sync(p);
+    if (p.cs == 1) {
+        __syncthreads();
+    } else {
+        asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+        asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    }
+    return true;
+}
+
 // ---------------------------------------------------------------------------
 // Row-marching path for lattices whose side L is a power of two from 128 to
 // 2048.  A row of L/32 words is held whole by a group of L/64 lanes, 2 words
@@ -210,7 +279,7 @@ __device__ __forceinline__ void cp_wait_all() { asm volatile("cp.async.wait_grou
 // Adds a lane group's observables of one lattice: per lane and row 32 white
 // sites (4 bonds each) and 32 black centres were counted, `ones` of them up.
 template <bool OBS>
-__device__ __forceinline__ void march_flush(const BatchParams &p, int64_t lat, unsigned gmask, int lpr, int j,
+__device__ __forceinline__ void march_flush(long long *acc, int64_t lat, unsigned gmask, int lpr, int j,
                                             uint32_t &ones, uint32_t &dsum, uint32_t &nrows)
 {
     if (!OBS) return;
@@ -221,8 +290,8 @@ __device__ __forceinline__ void march_flush(const BatchParams &p, int64_t lat, u
         c += __shfl_xor_sync(gmask, c, off);
     }
     if (j == 0 && c > 0) {
-        atomicAdd(reinterpret_cast<unsigned long long *>(p.acc + 2 * lat), (unsigned long long)(2 * a - 64 * c));
-        atomicAdd(reinterpret_cast<unsigned long long *>(p.acc + 2 * lat + 1), (unsigned long long)(128 * c - 2 * b));
+        atomicAdd(reinterpret_cast<unsigned long long *>(acc + 2 * lat), (unsigned long long)(2 * a - 64 * c));
+        atomicAdd(reinterpret_cast<unsigned long long *>(acc + 2 * lat + 1), (unsigned long long)(128 * c - 2 * b));
     }
     ones = dsum = nrows = 0;
 }
@@ -232,7 +301,7 @@ __device__ __forceinline__ void march_flush(const BatchParams &p, int64_t lat, u
 // n = c1 - c0 rows, run k for lane group k.
 template <bool OBS>
 __device__ void march_rows(const BatchParams &p, const BatchGroup &G, int64_t c0, int64_t c1, int colour,
-                           uint64_t t, MarchRing &ring)
+                           uint64_t t, long long *acc, MarchRing &ring)
 {
     const int lane = threadIdx.x & 31;
     const int lpr = G.gpr;  // lanes per row
@@ -242,8 +311,8 @@ __device__ void march_rows(const BatchParams &p, const BatchGroup &G, int64_t c0
     const int n = (int)(c1 - c0);
     const int L = G.L, wpr = G.wpr;
     const int64_t rho = c0 * P + (int64_t)grp * n;  // first row of this lane group's run
-    int64_t li = rho / L;
-    int r = (int)(rho - li * L);
+    int64_t li = rho >> G.log2L;
+    int r = (int)rho & (L - 1);
     const int64_t lat_words = (int64_t)L * wpr;
     const uint64_t *src_all = (colour == 0 ? p.white : p.black) + G.word_base + 2 * j;
     uint64_t *tgt_all = (colour == 0 ? p.black : p.white) + G.word_base + 2 * j;
@@ -328,35 +397,31 @@ __device__ void march_rows(const BatchParams &p, const BatchGroup &G, int64_t c0
         q += qrow;
         src2 = r + 2 == L ? src : src2 + wpr;
         if (last_row) {
-            march_flush<OBS>(p, lat, gmask, lpr, j, ones, dsum, nrows);
+            march_flush<OBS>(acc, lat, gmask, lpr, j, ones, dsum, nrows);
             ++li;
             r = 0;
             if (more) enter(s + 1);
         }
     }
-    if (n > 0 && r != 0) march_flush<OBS>(p, lat, gmask, lpr, j, ones, dsum, nrows);
+    if (OBS) {
+        // the warp's lane groups often end in the same lattice: one pair of atomics then
+        const bool some = n > 0 && r != 0;
+        const int64_t lat0 = __shfl_sync(0xffffffffu, lat, 0);  // by every lane, whatever `some` says
+        if (__all_sync(0xffffffffu, some && lat == lat0))
+            march_flush<OBS>(acc, lat, 0xffffffffu, 32, lane, ones, dsum, nrows);
+        else if (some)
+            march_flush<OBS>(acc, lat, gmask, lpr, j, ones, dsum, nrows);
+    }
     cp_wait_all();
 }
 
-// One half-sweep of every lattice.  Each chunk carries a work weight wpt +
-// kappa (its words plus a fixed per-chunk cost, kappa chosen by the
-// autotuner); warp gw owns the contiguous chunks whose starting weight lies in
-// [gw * W / nw, (gw + 1) * W / nw) of the total W.  Observables are flushed
-// with one pair of atomics whenever the warp moves to another lattice.
+// The warp's chunks [cb, ce) of one half-sweep.  Observables are flushed with one
+// pair of atomics whenever the warp moves to another lattice.
 template <bool OBS>
-__device__ void batch_half(const BatchParams &p, int colour, uint64_t t, MarchRing &ring)
+__device__ void batch_half(const BatchParams &p, const Split &sp, int64_t cb, int64_t ce, int colour, uint64_t t,
+                           long long *acc, MarchRing &ring)
 {
     const int lane = threadIdx.x & 31;
-    const int64_t gw = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    auto chunk_at = [&](int64_t w) -> int64_t {
-        if (w >= p.total_weight) return p.n_chunks;
-        int g = 0;
-        while (g + 1 < p.n_groups && p.g[g + 1].weight_begin <= w) ++g;
-        const int64_t per = p.g[g].weight;
-        return p.g[g].chunk_begin + (w - p.g[g].weight_begin + per - 1) / per;
-    };
-    const int64_t cb = chunk_at(gw * p.total_weight / nw), ce = chunk_at((gw + 1) * p.total_weight / nw);
     const uint64_t *src = colour == 0 ? p.white : p.black;
     uint64_t *tgt = colour == 0 ? p.black : p.white;
     DrawCtx dc{(uint32_t)t, counter_word3(colour, kPurposeMetropolis, t), 0u, 0u, 0u};
@@ -376,9 +441,9 @@ __device__ void batch_half(const BatchParams &p, int colour, uint64_t t, MarchRi
             if (lane == 0) {
                 // c white sites and c black centres were counted, a of them up;
                 // each white site adds 4 - 2d over its 4 bonds
-                atomicAdd(reinterpret_cast<unsigned long long *>(p.acc + 2 * cur_lat),
+                atomicAdd(reinterpret_cast<unsigned long long *>(acc + 2 * cur_lat),
                           (unsigned long long)(2 * a - 2 * c));
-                atomicAdd(reinterpret_cast<unsigned long long *>(p.acc + 2 * cur_lat + 1),
+                atomicAdd(reinterpret_cast<unsigned long long *>(acc + 2 * cur_lat + 1),
                           (unsigned long long)(4 * c - 2 * b));
             }
         }
@@ -392,22 +457,22 @@ __device__ void batch_half(const BatchParams &p, int colour, uint64_t t, MarchRi
     int64_t li = 0;
     int r = 0, q = 0, dr = 0, dq = 0;
     for (int64_t c = cb; c < ce; ++c) {
-        while (gi + 1 < p.n_groups && c >= p.g[gi + 1].chunk_begin) ++gi;
+        while (gi + 1 < p.n_groups && c >= sp.chunk[gi + 1]) ++gi;
         const BatchGroup &G = p.g[gi];
         if (G.march) {
             // this warp's chunks of the group, all at once (warp-uniform)
-            const int64_t gend = gi + 1 < p.n_groups ? p.g[gi + 1].chunk_begin : p.n_chunks;
+            const int64_t gend = sp.chunk[gi + 1];
             const int64_t c1 = ce < gend ? ce : gend;
             flush();
             cur_lat = -1;
-            march_rows<OBS>(p, G, c - G.chunk_begin, c1 - G.chunk_begin, colour, t, ring);
+            march_rows<OBS>(p, G, c + sp.shift[gi], c1 + sp.shift[gi], colour, t, acc, ring);
             c = c1 - 1;
             cur_g = -1;
             continue;
         }
         if (gi != cur_g) {
             cur_g = gi;
-            const int64_t item = (c - G.chunk_begin) * 32 + lane;
+            const int64_t item = (c + sp.shift[gi]) * 32 + lane;
             li = item / G.items;
             const int64_t within = item - li * G.items;
             r = (int)(within / G.gpr);
@@ -449,6 +514,62 @@ __device__ void batch_half(const BatchParams &p, int colour, uint64_t t, MarchRi
     flush();
 }
 
+// Whether slots k and k + 1 of ladder l, held by lattices a and b, exchange at
+// sweep t.
+__device__ __forceinline__ bool pair_swaps(const BatchParams &p, const long long *acc, int64_t l, int k, int32_t a,
+                                           int32_t b, uint64_t t)
+{
+    const long long D = acc[2 * a + 1] - acc[2 * b + 1];  // E_b - E_a
+    if (D >= 0) return true;
+    if ((D & 3) != 0) atomicCAS(p.err, 0, (int)ISING_EINVAL);
+    const int64_t m = -D;
+    const uint64_t TS = m < p.swap_len[k] ? p.swap_tab[p.swap_off[k] + m] : 0ull;
+    const uint32_t site = (uint32_t)k;
+    const uint4 u4 = philox(site >> 2, (uint32_t)l, (uint32_t)t, counter_word3(0, kPurposeExchange, t), p.rk);
+    const uint32_t w = (site & 3) == 0 ? u4.x : (site & 3) == 1 ? u4.y : (site & 3) == 2 ? u4.z : u4.w;
+    return (uint64_t)w < TS;
+}
+
+// The owners' form of record and exchange, without a barrier behind it: a thread
+// takes one of its owner's lattices, records it and decides its pair itself (its
+// partner's thread comes to the same answer), from the state `at` that event left
+// by the last one; the new state goes to the other buffer, `at_next`.  The sums
+// read here are cleared at the next event, when every thread has read them.
+__device__ void owner_exchange(const BatchParams &p, uint64_t t, const int32_t *at, int32_t *at_next,
+                               const long long *acc, long long *acc_next)
+{
+    const int o = (int)blockIdx.x / p.cs, rank = (int)blockIdx.x % p.cs;
+    const int64_t e = (int64_t)((t + 1) / (uint64_t)p.record_every) - 1;
+    const uint32_t S = (uint32_t)p.S;
+    for (int g = 0; g < p.n_groups; ++g) {
+        const int64_t first = p.part[g][o], last = p.part[g][o + 1];
+        for (int64_t i = first + rank + (int64_t)p.cs * threadIdx.x; i < last; i += (int64_t)p.cs * blockDim.x) {
+            const int32_t x = (int32_t)(p.g[g].first + i);
+            const uint32_t l = (uint32_t)x / S;
+            int k = p.slot_of[x];
+            if (p.trace != nullptr) {
+                long long *row = p.trace + 2 * ((e - p.event_first) * p.n + (int64_t)l * S + k);
+                row[0] = acc[2 * x];
+                row[1] = acc[2 * x + 1];
+            }
+            if (p.swaps) {
+                const bool lower = ((k ^ (int)e) & 1) == 0;  // x holds the lower slot of its pair
+                const int pk = lower ? k + 1 : k - 1;
+                if (pk >= 0 && pk < (int)S) {
+                    const int32_t y = at[(int64_t)l * S + pk];
+                    if (pair_swaps(p, acc, l, lower ? k : pk, lower ? x : y, lower ? y : x, t)) {
+                        k = pk;
+                        p.slot_of[x] = k;
+                    }
+                }
+            }
+            at_next[(int64_t)l * S + k] = x;
+            acc_next[2 * x] = 0;
+            acc_next[2 * x + 1] = 0;
+        }
+    }
+}
+
 // Record and exchange: warp gw handles ladders gw, gw + nw, ...
 __device__ void batch_exchange(const BatchParams &p, uint64_t t)
 {
@@ -470,18 +591,7 @@ __device__ void batch_exchange(const BatchParams &p, uint64_t t)
         if (p.swaps) {
             for (int k = (int)(e & 1) + 2 * lane; k + 1 < p.S; k += 64) {
                 const int32_t a = at[k], b = at[k + 1];
-                const long long D = p.acc[2 * a + 1] - p.acc[2 * b + 1];  // E_b - E_a
-                bool swap = D >= 0;
-                if (!swap) {
-                    if ((D & 3) != 0) atomicCAS(p.err, 0, (int)ISING_EINVAL);
-                    const int64_t m = -D;
-                    const uint64_t TS = m < p.swap_len[k] ? p.swap_tab[p.swap_off[k] + m] : 0ull;
-                    const uint32_t site = (uint32_t)k;
-                    const uint4 u4 = philox(site >> 2, (uint32_t)l, (uint32_t)t,
-                                            counter_word3(0, kPurposeExchange, t), p.rk);
-                    const uint32_t w = (site & 3) == 0 ? u4.x : (site & 3) == 1 ? u4.y : (site & 3) == 2 ? u4.z : u4.w;
-                    swap = (uint64_t)w < TS;
-                }
+                const bool swap = pair_swaps(p, p.acc, l, k, a, b, t);
                 if (swap) {
                     at[k] = b;
                     at[k + 1] = a;
@@ -508,19 +618,42 @@ __global__ void __launch_bounds__(512, 1) batch_kernel(const __grid_constant__ B
     // one MarchRing per warp (dynamic shared memory)
     extern __shared__ __align__(16) unsigned char batch_smem[];
     MarchRing &ring = reinterpret_cast<MarchRing *>(batch_smem)[threadIdx.x >> 5];
+    __shared__ Split sp;
+    int64_t cb, ce;
+    fill_split(p, sp, cb, ce);
+    int events = 0;  // of this launch
     for (int64_t s = 0; s < p.n_sweeps; ++s) {
         const uint64_t t = p.t0 + (uint64_t)s;
         const bool rec = p.record_every > 0 && (t + 1) % (uint64_t)p.record_every == 0;
-        batch_half<false>(p, 0, t, ring);
-        if (!grid_sync(p)) return;
-        if (rec)
-            batch_half<true>(p, 1, t, ring);
-        else
-            batch_half<false>(p, 1, t, ring);
-        if (!grid_sync(p)) return;
+        batch_half<false>(p, sp, cb, ce, 0, t, nullptr, ring);
+        if (!phase_sync(p)) return;
         if (rec) {
-            batch_exchange(p, t);
+            const bool odd = p.cs > 0 && (events & 1);
+            batch_half<true>(p, sp, cb, ce, 1, t, odd ? p.acc2 : p.acc, ring);
             if (!grid_sync(p)) return;
+            if (p.cs > 0) {
+                owner_exchange(p, t, odd ? p.lattice_at2 : p.lattice_at, odd ? p.lattice_at : p.lattice_at2,
+                               odd ? p.acc2 : p.acc, odd ? p.acc : p.acc2);
+                ++events;
+                phase_sync(p);
+            } else {
+                batch_exchange(p, t);
+                if (!grid_sync(p)) return;
+            }
+        } else {
+            batch_half<false>(p, sp, cb, ce, 1, t, nullptr, ring);
+            if (p.cs > 0 && (s + 1) % p.sync_every == 0 ? !grid_sync(p) : !phase_sync(p)) return;
+        }
+    }
+    if (events > 0) {
+        // the state back to where the caller has it, the last event's sums cleared
+        if (!grid_sync(p)) return;
+        const bool odd = (events - 1) & 1;
+        for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < p.n; i += (int64_t)gridDim.x * blockDim.x) {
+            if (!odd) p.lattice_at[i] = p.lattice_at2[i];
+            long long *acc = odd ? p.acc2 : p.acc;
+            acc[2 * i] = 0;
+            acc[2 * i + 1] = 0;
         }
     }
 }
@@ -572,6 +705,8 @@ __global__ void batch_reset_kernel(const __grid_constant__ BatchParams p)
         p.lattice_at[i] = (int32_t)i;
         p.acc[2 * i] = 0;
         p.acc[2 * i + 1] = 0;
+        p.acc2[2 * i] = 0;
+        p.acc2[2 * i + 1] = 0;
     }
 }
 
@@ -584,6 +719,8 @@ size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
 // ---------------------------------------------------------------------------
 // Host side: the handle, the workspace layout, graph capture and autotuning.
 // ---------------------------------------------------------------------------
+constexpr int32_t kMeasuredWeights = -1;  // ising_batch::kappa: chunk weights as measured
+
 struct ising_batch {
     int64_t n = 0;
     int32_t S = 0;
@@ -593,17 +730,20 @@ struct ising_batch {
     size_t ws_bytes = 0;
     size_t plane_words = 0;
     // workspace offsets
-    size_t o_black, o_white, o_slot, o_at, o_thr, o_soff, o_slen, o_stab, o_acc, o_bar, o_tune, total;
+    size_t o_black, o_white, o_slot, o_at, o_at2, o_thr, o_soff, o_slen, o_stab, o_acc, o_acc2, o_bar, o_tune, total;
     std::vector<int64_t> swap_len;
     int32_t threads = 512;
     int32_t wpt_max = 4;
-    int32_t kappa = 4;
+    int32_t kappa = kMeasuredWeights;
     int device = 0;
     // captured graph of the persistent launch
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
     cudaGraphNode_t node = nullptr;
-    int32_t graph_threads = 0, graph_blocks = 0;
+    int32_t graph_threads = 0, graph_blocks = 0, graph_cs = 0;
+    // pick_owners' answer for a grid of `owners_blocks` blocks and this wpt_max
+    std::vector<uint32_t> owners;
+    int32_t owners_blocks = 0, owners_wpt = 0, owners_cs = 0, owners_sync = 1, owners_grid = 0;
 };
 
 namespace ising {
@@ -662,16 +802,31 @@ int layout(ising_batch_t *b)
     b->o_slen = take((size_t)std::max(1, b->S - 1) * 8);
     b->o_stab = take(std::max<size_t>(1, ntab) * 8);
     b->o_acc = take((size_t)b->n * 16);
+    b->o_acc2 = take((size_t)b->n * 16);
+    b->o_at2 = take((size_t)b->n * 4);
     b->o_bar = take(64);
     b->o_tune = take(2 * b->plane_words * 8);
     b->total = o;
     return ISING_OK;
 }
 
+// Time of a chunk (32 items) relative to a chunk of marched rows (1024 sites,
+// 100), from the rates at 1.3e8 spins: march 1254-1296 flips/ns, items of 4 words
+// 1153-1169, of 2 words 1076-1084, of 1 word 871-884.
+int32_t chunk_cost(const BatchGroup &G) { return G.march ? 100 : G.wpt == 4 ? 220 : G.wpt == 2 ? 117 : 72; }
+// The same for the split of an owner's chunks among its warps.  Beside marching
+// warps on the same SM an item path is held up by its loads, not by the
+// multipliers: with chunk_cost here the replica-exchange batch of 4096 lattices
+// takes 238 us per sweep, with these weights 218.
+int32_t warp_cost(const BatchGroup &G) { return G.march ? 100 : G.wpt == 4 ? 250 : G.wpt == 2 ? 170 : 100; }
+
+// What a barrier costs in the same unit (1024 sites take an SM 0.11 us): see
+// pick_owners.
+constexpr int64_t kGridSync = 2500, kClusterSync = 500, kBlockSync = 100;
+
 int build_groups(const ising_batch_t *b, int wpt_max, int kappa, BatchParams &p)
 {
     int ng = 0;
-    int64_t chunk = 0, weight = 0;
     for (int64_t i = 0; i < b->n;) {
         int64_t j = i;
         while (j < b->n && b->L[j] == b->L[i]) ++j;
@@ -698,18 +853,113 @@ int build_groups(const ising_batch_t *b, int wpt_max, int kappa, BatchParams &p)
         }
         G.gpr = G.wpr / G.wpt;
         G.items = (int64_t)G.L * G.gpr;
-        G.chunk_begin = chunk;
-        G.weight = G.wpt + kappa;
-        G.weight_begin = weight;
-        chunk += G.count * G.items / 32;
-        weight += G.count * G.items / 32 * G.weight;
+        G.log2L = 0;
+        while (G.march && (1 << G.log2L) < G.L) ++G.log2L;
+        G.weight = kappa == kMeasuredWeights ? warp_cost(G) : G.wpt + kappa;
         i = j;
     }
     p.n_groups = ng;
-    p.n_chunks = chunk;
-    p.plane_words = b->word_off[b->n];
-    p.total_weight = weight;
+    p.cs = 0;
     return ISING_OK;
+}
+
+// Deals the lattices of every group to `owners` so that the most loaded one has as
+// little as the greedy rule gives (largest lattices first, each to the least
+// loaded owner), and returns that load in chunk_cost units per half-sweep.  All
+// lattices of a group weigh the same, so an owner's share of it is a count, and
+// the counts are found by raising a common level instead of one by one.
+int64_t deal(BatchParams &p, int owners)
+{
+    int64_t load[kMaxOwners] = {};
+    int order[kMaxGroups];
+    for (int g = 0; g < p.n_groups; ++g) order[g] = g;
+    std::sort(order, order + p.n_groups, [&](int a, int b) { return p.g[a].L > p.g[b].L; });
+    for (int k = 0; k < p.n_groups; ++k) {
+        const BatchGroup &G = p.g[order[k]];
+        const int64_t w = G.items / 32 * chunk_cost(G);
+        auto room = [&](int o, int64_t level) { return level <= load[o] ? int64_t(0) : (level - load[o]) / w; };
+        // the largest level that does not take more than the group has
+        int64_t lo = 0, hi = *std::max_element(load, load + owners) + (G.count + 1) * w;
+        while (hi - lo > 1) {
+            const int64_t mid = lo + (hi - lo) / 2;
+            int64_t n = 0;
+            for (int o = 0; o < owners && n <= G.count; ++o) n += room(o, mid);
+            (n <= G.count ? lo : hi) = mid;
+        }
+        int64_t take[kMaxOwners], left = G.count;
+        for (int o = 0; o < owners; ++o) left -= take[o] = room(o, lo);
+        for (int o = 0; o < owners; ++o) load[o] += take[o] * w;
+        for (; left > 0; --left) {
+            const int o = (int)(std::min_element(load, load + owners) - load);
+            ++take[o];
+            load[o] += w;
+        }
+        uint32_t *part = p.part[order[k]];
+        part[0] = 0;
+        for (int o = 0; o < owners; ++o) part[o + 1] = part[o] + (uint32_t)take[o];
+    }
+    return *std::max_element(load, load + owners);
+}
+
+// Dynamic shared memory of a launch: one MarchRing per warp.
+size_t smem_for(int threads) { return (size_t)(threads / 32) * sizeof(MarchRing); }
+
+// Clusters of cs blocks of 512 threads that are resident together, 0 if none are
+// (a graphics processing cluster's SMs need not be a multiple of cs).
+int resident_clusters(int cs)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)cs);
+    cfg.blockDim = dim3(512);
+    cfg.dynamicSmemBytes = smem_for(512);
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)cs;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    int n = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, batch_kernel, &cfg) != cudaSuccess) {
+        cudaGetLastError();
+        return 0;
+    }
+    return n;
+}
+
+// Who sweeps what, for a launch of `blocks` blocks of 512 threads, one per SM:
+// the grid, or one, two or four SMs per share of whole lattices, whichever has the
+// shortest half-sweep by chunk_cost and the cost of its barrier.  Owners meet at
+// least every sync_every sweeps (a quarter of a second or so), so that the
+// bounded wait of one that is early never runs out.
+void pick_owners(BatchParams &p, int blocks)
+{
+    p.cs = 0;
+    p.sync_every = 1;
+    if (blocks > kMaxOwners || p.acc2 == nullptr) return;
+    int64_t total = 0;
+    for (int g = 0; g < p.n_groups; ++g) {
+        if (p.g[g].count > (int64_t(1) << 31)) return;
+        total += p.g[g].count * (p.g[g].items / 32) * chunk_cost(p.g[g]);
+    }
+    int64_t best = total / blocks + kGridSync;
+    int pick = 0;
+    for (int cs : {1, 2, 4}) {
+        const int owners = cs == 1 ? blocks : resident_clusters(cs);
+        if (owners < 1 || owners > kMaxOwners) continue;
+        const int64_t cost = deal(p, owners) / cs + (cs == 1 ? kBlockSync : kClusterSync);
+        if (cost < best) {
+            best = cost;
+            pick = cs;
+        }
+    }
+    if (pick > 0) {
+        const int owners = pick == 1 ? blocks : resident_clusters(pick);
+        deal(p, owners);
+        p.expect_blocks = owners * pick;
+    }
+    p.cs = pick;
+    p.sync_every = (int32_t)std::min<int64_t>(1 << 20, std::max<int64_t>(1, 100000000 / best));
 }
 
 BatchParams base_params(const ising_batch_t *b)
@@ -728,13 +978,12 @@ BatchParams base_params(const ising_batch_t *b)
     p.swap_len = (const int64_t *)(b->ws + b->o_slen);
     p.swap_tab = (const uint64_t *)(b->ws + b->o_stab);
     p.acc = (long long *)(b->ws + b->o_acc);
+    p.acc2 = (long long *)(b->ws + b->o_acc2);
+    p.lattice_at2 = (int32_t *)(b->ws + b->o_at2);
     p.bar = (unsigned *)(b->ws + b->o_bar);
-    p.err = (int *)(b->ws + b->o_bar + 16);
+    p.err = (int *)(p.bar + 1);
     return p;
 }
-
-// Dynamic shared memory of a launch: one MarchRing per warp.
-size_t smem_for(int threads) { return (size_t)(threads / 32) * sizeof(MarchRing); }
 
 int blocks_for(int threads, int *blocks)
 {
@@ -751,6 +1000,18 @@ int blocks_for(int threads, int *blocks)
     return ISING_OK;
 }
 
+// The launch as attributes: cooperative, and in clusters of p.cs blocks.
+int launch_attrs(const BatchParams &p, cudaLaunchAttribute (&attr)[2])
+{
+    attr[0].id = cudaLaunchAttributeCooperative;
+    attr[0].val.cooperative = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = (unsigned)std::max(1, p.cs);
+    attr[1].val.clusterDim.y = 1;
+    attr[1].val.clusterDim.z = 1;
+    return p.cs > 1 ? 2 : 1;
+}
+
 cudaError_t launch_coop(const BatchParams &p, int blocks, int threads, cudaStream_t s)
 {
     cudaLaunchConfig_t cfg = {};
@@ -758,11 +1019,9 @@ cudaError_t launch_coop(const BatchParams &p, int blocks, int threads, cudaStrea
     cfg.blockDim = dim3((unsigned)threads);
     cfg.dynamicSmemBytes = smem_for(threads);
     cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeCooperative;
-    attr[0].val.cooperative = 1;
+    cudaLaunchAttribute attr[2];
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = (unsigned)launch_attrs(p, attr);
     return cudaLaunchKernelEx(&cfg, batch_kernel, p);
 }
 
@@ -949,11 +1208,28 @@ static int run_impl(ising_batch_t *b, uint64_t *black, uint64_t *white, int64_t 
     if (rc) return rc;
     p.expect_blocks = blocks;
     if (n_sweeps == 0) return ISING_OK;
+    if (b->threads == 512) {
+        if (b->owners_blocks != blocks || b->owners_wpt != b->wpt_max) {
+            pick_owners(p, blocks);
+            b->owners.assign(&p.part[0][0], &p.part[0][0] + sizeof(p.part) / sizeof(uint32_t));
+            b->owners_cs = p.cs;
+            b->owners_sync = p.sync_every;
+            b->owners_grid = p.expect_blocks;
+            b->owners_blocks = blocks;
+            b->owners_wpt = b->wpt_max;
+        } else {
+            memcpy(p.part, b->owners.data(), sizeof(p.part));
+            p.cs = b->owners_cs;
+            p.sync_every = b->owners_sync;
+            p.expect_blocks = b->owners_grid;
+        }
+        blocks = p.expect_blocks;
+    }
     if (!use_graph) {
         cudaError_t e = launch_coop(p, blocks, b->threads, s);
         return e == cudaSuccess ? ISING_OK : bfail(ISING_ECUDA, cudaGetErrorString(e));
     }
-    if (b->exec == nullptr || b->graph_threads != b->threads || b->graph_blocks != blocks) {
+    if (b->exec == nullptr || b->graph_threads != b->threads || b->graph_blocks != blocks || b->graph_cs != p.cs) {
         if (b->exec) cudaGraphExecDestroy(b->exec);
         if (b->graph) cudaGraphDestroy(b->graph);
         b->exec = nullptr;
@@ -979,6 +1255,7 @@ static int run_impl(ising_batch_t *b, uint64_t *black, uint64_t *white, int64_t 
         b->node = node;
         b->graph_threads = b->threads;
         b->graph_blocks = blocks;
+        b->graph_cs = p.cs;
     }
     cudaKernelNodeParams kp = {};
     void *args[1] = {&p};
@@ -1015,7 +1292,7 @@ ISING_API int ising_batch_check(ising_batch_t *b, ising_stream_t stream)
     cudaError_t e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) return bfail(ISING_ECUDA, cudaGetErrorString(e));
     int err = 0;
-    e = cudaMemcpy(&err, b->ws + b->o_bar + 16, sizeof(int), cudaMemcpyDeviceToHost);
+    e = cudaMemcpy(&err, b->ws + b->o_bar + 4, sizeof(int), cudaMemcpyDeviceToHost);
     if (e != cudaSuccess) return bfail(ISING_ECUDA, cudaGetErrorString(e));
     if (err != 0) {
         cudaMemset(b->ws + b->o_bar, 0, 64);
@@ -1085,7 +1362,7 @@ ISING_API int ising_batch_autotune(ising_batch_t *b, int64_t n_sweeps, ising_str
     b->wpt_max = bw;
     // then the per-chunk weight of the work split
     int32_t bk = b->kappa;
-    for (int32_t kap : {0, 1, 2, 4, 8, 1 << 20}) {
+    for (int32_t kap : {kMeasuredWeights, 0, 1, 2, 4, 8, 1 << 20}) {
         b->kappa = kap;
         int rc = run_impl(b, tb, tw, 1, 0x5eed, 0, 0, 0, nullptr, 0, s);
         if (rc == ISING_OK) {
@@ -1225,6 +1502,9 @@ extern "C" ISING_API int ising_batch_run_noalloc(int64_t n, const int64_t *L, in
     const size_t s_thr = take(thr.size() * 4), s_off = take(std::max<size_t>(1, off.size()) * 8),
                  s_len = take(std::max<size_t>(1, len.size()) * 8), s_tab = take(std::max<size_t>(1, tab.size()) * 8),
                  s_acc = take((size_t)n * 16), s_bar = take(64);
+    // the owners' second buffers where there is room for them
+    const size_t s_acc2 = o, s_at2 = align256(s_acc2 + (size_t)n * 16);
+    const bool owners = s_at2 + (size_t)n * 4 <= (size_t)ISING_NOALLOC_SCRATCH_BYTES;
     if (o > (size_t)ISING_NOALLOC_SCRATCH_BYTES) {
         char msg[160];
         snprintf(msg, sizeof(msg), "needs %zu bytes of scratch; the allocation-free entry point holds %zu",
@@ -1281,14 +1561,14 @@ extern "C" ISING_API int ising_batch_run_noalloc(int64_t n, const int64_t *L, in
         e = cudaMemcpyAsync(sc + s_len, len.data(), len.size() * 8, cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess && !tab.empty())
         e = cudaMemcpyAsync(sc + s_tab, tab.data(), tab.size() * 8, cudaMemcpyHostToDevice, s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(sc + s_acc, 0, (s_bar + 64) - s_acc, s);
+    if (e == cudaSuccess) e = cudaMemsetAsync(sc + s_acc, 0, (owners ? s_at2 : s_bar + 64) - s_acc, s);
     if (e != cudaSuccess) return bfail(ISING_ECUDA, cudaGetErrorString(e));
 
     BatchParams p;
     memset(&p, 0, sizeof(p));
     p.black = (uint64_t *)black_dev;
     p.white = (uint64_t *)white_dev;
-    rc = build_groups(&lay, 4, 4, p);
+    rc = build_groups(&lay, 4, kMeasuredWeights, p);
     if (rc) return rc;
     p.S = ladder_size;
     p.n = n;
@@ -1300,8 +1580,12 @@ extern "C" ISING_API int ising_batch_run_noalloc(int64_t n, const int64_t *L, in
     p.swap_len = (const int64_t *)(sc + s_len);
     p.swap_tab = (const uint64_t *)(sc + s_tab);
     p.acc = (long long *)(sc + s_acc);
+    if (owners) {
+        p.acc2 = (long long *)(sc + s_acc2);
+        p.lattice_at2 = (int32_t *)(sc + s_at2);
+    }
     p.bar = (unsigned *)(sc + s_bar);
-    p.err = (int *)(sc + s_bar + 16);
+    p.err = (int *)(p.bar + 1);
     p.n_sweeps = n_sweeps;
     p.t0 = sweep_offset;
     p.record_every = record_every;
@@ -1315,14 +1599,15 @@ extern "C" ISING_API int ising_batch_run_noalloc(int64_t n, const int64_t *L, in
     if (rc) return rc;
     p.expect_blocks = blocks;
     if (n_sweeps > 0) {
-        e = launch_coop(p, blocks, 512, s);
+        pick_owners(p, blocks);
+        e = launch_coop(p, p.expect_blocks, 512, s);
         if (e != cudaSuccess) return bfail(ISING_ECUDA, cudaGetErrorString(e));
     }
     // synchronous: report a timed-out barrier wait before returning
     e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) return bfail(ISING_ECUDA, cudaGetErrorString(e));
     int err = 0;
-    e = cudaMemcpy(&err, sc + s_bar + 16, sizeof(int), cudaMemcpyDeviceToHost);
+    e = cudaMemcpy(&err, sc + s_bar + 4, sizeof(int), cudaMemcpyDeviceToHost);
     if (e != cudaSuccess) return bfail(ISING_ECUDA, cudaGetErrorString(e));
     if (err != 0) return bfail(err, err == ISING_ETIMEOUT ? "a grid barrier wait timed out" : "device-side check failed");
     return ISING_OK;
