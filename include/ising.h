@@ -408,11 +408,10 @@ ISING_API int ising_net_forward(int64_t L, int64_t C, const void *black_dev, con
  * move: logits_dev[c] = the logits of chain c with block flip_block_dev[c]
  * flipped, given logits_x_dev = this network's logits of the unflipped chains
  * (same params, same planes; another buffer).  A flipped block changes the
- * activations only within 4 rows of it (four 3 x 3 layers), so for L a
- * multiple of 128 only a band of 30 rows per chain is recomputed and the
- * logits outside the block row and its two neighbours are copied from
- * logits_x_dev; the result equals ising_net_forward with flip_block_dev bit
- * for bit.  Other L compute the whole forward.  Inference workspace. */
+ * activations only within 4 rows of it (four 3 x 3 layers), so only a band of
+ * 30 rows per chain is recomputed and the logits outside the block row and its
+ * two neighbours are copied from logits_x_dev; the result equals
+ * ising_net_forward with flip_block_dev bit for bit.  Inference workspace. */
 ISING_API int ising_net_forward_flipped(int64_t L, int64_t C, const void *black_dev, const void *white_dev,
                                         const int32_t *flip_block_dev, const float *params_dev,
                                         const float *logits_x_dev, float *logits_dev, void *work_dev,
@@ -435,9 +434,8 @@ ISING_API int ising_net_wait_selftest(int64_t L, int64_t C, const void *black_de
 
 /* grad_dev = d(sum dlogits * logits)/d(params) for the last training forward
  * on the same chains and parameters (straight-through the bfloat16 rounding).
- * For L a multiple of 128 the data and weight gradients of the 32 -> 32
- * layers run on the tensor cores (the weight gradients see the output
- * gradient as two bfloat16 parts, its rounding and the rounding of the
+ * The data and weight gradients of the 32 -> 32 layers run on the tensor
+ * cores (the weight gradients see the output gradient as two bfloat16 parts, its rounding and the rounding of the
  * remainder, which carry it to about 2^-17); a bounded wait that gives up there
  * is reported by the next ising_net_check.  Every weight gradient is a sum of
  * per-CTA partials in a fixed order: the result is deterministic. */

@@ -23,17 +23,21 @@
 // the gradients are NHWC FP32 without halo.
 //
 // Forward kernels: layer 1 by table lookup (l1_table_kernel, l1_kernel); the
-// two 32 -> 32 layers on the tensor cores (tcgen05; conv32_ring_kernel for L
-// a multiple of 128, conv32_tc_kernel otherwise), the second one also
-// contracting layer 4's input channels (P, the 9 tap projections; reduced to
-// row partials of z4 per 8-pixel block column where L is a multiple of 128);
-// the tap sums and block means (pool_rows_kernel, pool_kernel).  Every
-// reduction has a fixed order, so
+// two 32 -> 32 layers on the tensor cores (tcgen05; conv32_ring_kernel), the
+// second one also contracting layer 4's input channels (P, the 9 tap
+// projections, reduced to row partials of z4 per 8-pixel block column); the tap
+// sums and block means (pool_rows_kernel).  Every reduction has a fixed order, so
 // a forward pass is a deterministic function of the state.  Backward kernels,
-// straight through the bfloat16 roundings: for L a multiple of 128 the data
-// and weight gradients of the two 32 -> 32 layers on the tensor cores
-// (conv32_ring_kernel in BWD mode, wgrad_tc_kernel), the rest in FP32 on the
-// CUDA cores; weight gradients as fixed-order per-CTA partial sums.
+// straight through the bfloat16 roundings: the data and weight gradients of the
+// two 32 -> 32 layers on the tensor cores (conv32_ring_kernel in BWD mode,
+// wgrad_tc_kernel), the rest in FP32 on the CUDA cores; weight gradients as
+// fixed-order per-CTA partial sums.
+//
+// Row tiles.  The tensor-core kernels work on segments of a row of up to 128
+// pixels, one MMA row per pixel: ceil(L / 128) segments of tw pixels (a multiple
+// of 32; the last one may be shorter).  Where a segment has fewer than 128 pixels
+// the MMAs' other rows (or, in the weight gradients, K steps) are not used and
+// the warps that would read them only keep the protocol.
 //
 // Move.  Block b is drawn by inverse CDF of q_x (purpose-3 draw, site 0, in
 // the chain's stream) or uniformly; x' = x with block b flipped; the flip is
@@ -281,19 +285,6 @@ __device__ __forceinline__ int band_row0(const Band &b, int64_t c)
     return r < 0 ? r + b.L : r;
 }
 
-// Pixel pb of the band (0 <= pb < C rows L) -> chain c and the offset yx =
-// y L + x of its pixel within the chain.
-__device__ __forceinline__ void band_pixel(const Band &b, int64_t pb, int64_t &c, int &yx)
-{
-    const int64_t per = (int64_t)b.rows * b.L;
-    c = pb / per;
-    const int r = (int)(pb - c * per);
-    const int ry = r / b.L;
-    int y = band_row0(b, c) + ry;
-    if (y >= b.L) y -= b.L;
-    yx = y * b.L + (r - ry * b.L);
-}
-
 __device__ __forceinline__ int wrap(int v, int L) { return v < 0 ? v + L : (v >= L ? v - L : v); }
 
 // Index of pixel (y, x), -1 <= x <= L, of chain c in an activation buffer
@@ -391,218 +382,31 @@ __global__ void __launch_bounds__(kL1Threads) l1_kernel(Chains ch, Band bd, cons
     }
 }
 
-// Layers 2 and 3 (32 -> 32 channels) on the tensor cores, as an implicit GEMM
-// per tile of 128 consecutive pixels of the band:
-//   Z[m][o] = sum over taps k and input channels i of A_k[m][i] W[o][i][k],
-// M = 128 pixels, N = 32 output channels, K = 9 taps x 32 channels = 18 MMA
-// steps of K = 16 (tcgen05.mma kind::f16, BF16 operands, FP32 accumulator in
-// tensor memory).  A_k, the input activations of the pixels shifted by tap k
-// (periodic), is gathered into shared memory in the no-swizzle K-major layout:
-// for tap k and channel group g (8 channels = 16 bytes) a plane of 128 pixel
-// rows of 16 bytes, planes 2080 bytes apart, so one MMA step (two channel
-// groups of one tap) reads core matrices of 8 pixels x 16 bytes at SBO = 128
-// bytes along M and LBO = 2080 bytes along K.  This kernel serves any L (a
-// multiple of 32); conv32_ring_kernel below is the one for L a multiple of 128.  The weights, B_k[o][i] =
-// bf16(W[o][i][k]), sit the same way (planes of 32 rows, LBO = 512 bytes),
-// staged once per CTA.  Persistent CTAs (one per SM) walk tiles j, j + grid,
-// ...; the gather of tile n+1 and the epilogue of tile n-1 overlap the MMAs of
-// tile n (two shared-memory stages, two accumulators of 32 TMEM columns).
-// Epilogue: warp w reads TMEM lanes 32 (w % 4) .. + 31 (its pixels) and
-// columns 16 (w / 4) .. + 15 (its output channels), adds the bias, and writes
-// z (FP32, training) and bf16(gelu(z)).
+// Layers 2 and 3 (32 -> 32 channels): see conv32_ring_kernel below.
 constexpr int kTileM = 128;
-constexpr int kConvThreads = 256;
 constexpr int kTaps = 9;
 constexpr int kGroups = kCh / 8;                                      // 16-byte channel groups per pixel
-// One channel group of 128 (+2) pixel rows: 2080 bytes, so that the planes of
-// the 4 channel groups start 32 bytes apart modulo the 128-byte bank row and
-// 8 lanes storing 2 pixels x 4 groups hit 8 different 16-byte bank groups.
-constexpr uint32_t kPlane = (kTileM + 2) * 16;
-constexpr uint32_t kAStage = kTaps * kGroups * kPlane;                // 74880 bytes per stage
 constexpr uint32_t kBBytes = kTaps * kGroups * kCh * 16;              // 18432 bytes
-// + bias, barriers and the TMEM slot
-constexpr uint32_t kConvSmem = 2 * kAStage + kBBytes + kCh * 4 + 64;
-constexpr uint32_t kTmemCols = 64;
 constexpr long long kWaitCycles = 4000000000LL;  // ~2 s at 2 GHz
 
 __device__ int g_tc_error;  // set to 1 when a tensor-core wait gives up
 
-struct ConvTc {
-    const __nv_bfloat16 *a_in;  // NHWC, C L^2 x 32
-    __nv_bfloat16 *a_out;
-    float *z_out;  // nullable
-    const float *params;
-    int w_off, b_off;
-    Band bd;
-    int64_t tiles;  // C rows L / 128
-};
-
-__device__ __forceinline__ void tile_origin(const ConvTc &p, int64_t tile, int64_t &c, int &yx0)
-{
-    band_pixel(p.bd, tile * kTileM, c, yx0);
-}
-
-// Gathers A_k for the 9 taps of one tile.  Thread t moves channel group t % 4
-// of pixels m0 = t / 4 and m0 + 64 for every tap.
-__device__ __forceinline__ void conv_gather(const ConvTc &p, int64_t tile, uint8_t *sa)
-{
-    const int L = p.bd.L;
-    int64_t c;
-    int yx0;
-    tile_origin(p, tile, c, yx0);
-    const int g = threadIdx.x & 3, m0 = threadIdx.x >> 2;
-    int py[2], px[2];
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-        const int yx = yx0 + m0 + 64 * h;
-        py[h] = yx / L;
-        px[h] = yx - py[h] * L;
-    }
-    const uint4 *src = reinterpret_cast<const uint4 *>(p.a_in);
-    uint4 v[2 * kTaps];
-#pragma unroll
-    for (int k = 0; k < kTaps; ++k)
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const int yy = wrap(py[h] + k / 3 - 1, L), xx = wrap(px[h] + k % 3 - 1, L);
-            v[2 * k + h] = __ldg(src + apix(L, c, yy, xx) * kGroups + g);
-        }
-#pragma unroll
-    for (int k = 0; k < kTaps; ++k)
-#pragma unroll
-        for (int h = 0; h < 2; ++h)
-            *reinterpret_cast<uint4 *>(sa + (k * kGroups + g) * kPlane + (m0 + 64 * h) * 16) = v[2 * k + h];
-}
-
-__device__ __forceinline__ void conv_epilogue(const ConvTc &p, int64_t tile, uint32_t tacc, const float *bias)
-{
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int quad = warp & 3, half = warp >> 2;
-    int64_t c;
-    int yx0;
-    tile_origin(p, tile, c, yx0);
-    const int L = p.bd.L;
-    const int yx = yx0 + quad * 32 + lane, y = yx / L, x = yx - y * L;
-    const int64_t q = c * (int64_t)L * L + yx;
-    float v[16];
-    tc::tmem_ld16(tacc + (uint32_t)(half * 16) + ((uint32_t)(quad * 32) << 16), v);
-#pragma unroll
-    for (int j = 0; j < 16; ++j) v[j] += bias[half * 16 + j];
-    if (p.z_out) {
-        float4 *zo = reinterpret_cast<float4 *>(p.z_out + q * kCh + half * 16);
-#pragma unroll
-        for (int j = 0; j < 4; ++j) zo[j] = make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
-    }
-    uint32_t w[8];
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-        float g0 = v[2 * j], g1 = v[2 * j + 1];
-        gelu2(g0, g1);
-        w[j] = pack_bf16x2(g0, g1);
-    }
-    store_act(p.a_out, L, c, y, x, half * 16, make_uint4(w[0], w[1], w[2], w[3]));
-    store_act(p.a_out, L, c, y, x, half * 16 + 8, make_uint4(w[4], w[5], w[6], w[7]));
-}
-
-__global__ void __launch_bounds__(kConvThreads, 1) conv32_tc_kernel(const __grid_constant__ ConvTc p)
-{
-    extern __shared__ __align__(1024) uint8_t conv_smem[];
-    uint8_t *sA = conv_smem;
-    uint8_t *sB = conv_smem + 2 * kAStage;
-    float *sBias = reinterpret_cast<float *>(sB + kBBytes);
-    uint64_t *mbar = reinterpret_cast<uint64_t *>(sBias + kCh);
-    uint32_t *tslot = reinterpret_cast<uint32_t *>(mbar + 2);
-    const int tid = threadIdx.x, warp = tid >> 5;
-
-    if (warp == 0) tc::tmem_alloc(tslot, kTmemCols);
-    if (tid == 0) {
-        tc::mbar_init(&mbar[0], 1);
-        tc::mbar_init(&mbar[1], 1);
-        tc::fence_mbar_init();
-    }
-    // B[k][g][o] = the 8 input channels 8g .. 8g+7 of W[o][.][k], bfloat16
-    for (int e = tid; e < kTaps * kGroups * kCh; e += blockDim.x) {
-        const int k = e / (kGroups * kCh), r = e - k * (kGroups * kCh), g = r / kCh, o = r - g * kCh;
-        const float *w = p.params + p.w_off + (o * kCh + 8 * g) * 9 + k;
-        *reinterpret_cast<uint4 *>(sB + e * 16) =
-            make_uint4(pack_bf16x2(w[0], w[9]), pack_bf16x2(w[18], w[27]), pack_bf16x2(w[36], w[45]),
-                       pack_bf16x2(w[54], w[63]));
-    }
-    if (tid < kCh) sBias[tid] = bf16r(p.params[p.b_off + tid]);
-    tc::fence_async_smem();
-    tc::fence_before_sync();
-    __syncthreads();
-    tc::fence_after_sync();
-    const uint32_t tmem = *tslot;
-    const uint32_t idesc = tc::idesc_bf16_f32(kTileM, kCh);
-    const uint32_t a_u32 = tc::smem_u32(sA), b_u32 = tc::smem_u32(sB);
-
-    bool ok = true;
-    int committed = 0;  // tiles whose MMAs were issued
-    for (int n = 0;; ++n) {
-        const int64_t tile = blockIdx.x + (int64_t)n * gridDim.x;
-        const bool has = tile < p.tiles;
-        const int buf = n & 1;
-        // stage `buf` was last read by the MMAs of tile n-2, waited for below at step n-1
-        if (has) conv_gather(p, tile, sA + buf * kAStage);
-        tc::fence_async_smem();
-        __syncthreads();
-        if (has && tid == 0) {
-            tc::fence_after_sync();
-#pragma unroll
-            for (int s = 0; s < 2 * kTaps; ++s) {
-                const int k = s >> 1, g = 2 * (s & 1);
-                const uint64_t ad =
-                    tc::smem_desc(a_u32 + buf * kAStage + (k * kGroups + g) * kPlane, kPlane, 128);
-                const uint64_t bd = tc::smem_desc(b_u32 + (k * kGroups + g) * kCh * 16, kCh * 16, 128);
-                tc::mma_bf16(tmem + (uint32_t)(buf * kCh), ad, bd, idesc, s > 0 ? 1u : 0u);
-            }
-            tc::mma_commit(&mbar[buf]);
-        }
-        if (has) committed = n + 1;
-        if (n >= 1) {
-            const int pn = n - 1, pb = pn & 1;
-            // ok stays warp-uniform: the TMEM loads below are warp-collective
-            if (!__all_sync(0xffffffffu, tc::mbar_wait(&mbar[pb], (uint32_t)((pn >> 1) & 1), kWaitCycles)))
-                ok = false;
-            tc::fence_after_sync();
-            if (ok) conv_epilogue(p, blockIdx.x + (int64_t)pn * gridDim.x, tmem + (uint32_t)(pb * kCh), sBias);
-            tc::fence_before_sync();
-        }
-        if (__syncthreads_or(!ok)) {
-            ok = false;
-            break;
-        }
-        if (!has) break;
-    }
-    if (!ok) {
-        if (tid == 0) {
-            atomicExch(&g_tc_error, 1);
-            // let the MMAs of the last issued tile finish before the TMEM is freed
-            if (committed > 0) {
-                const int ln = committed - 1;
-                tc::mbar_wait(&mbar[ln & 1], (uint32_t)((ln >> 1) & 1), kWaitCycles);
-            }
-        }
-    }
-    tc::fence_before_sync();
-    __syncthreads();
-    if (warp == 0) {
-        tc::fence_after_sync();
-        tc::tmem_dealloc(tmem, kTmemCols);
-    }
-}
-
-// Layers 2 and 3 for L a multiple of 128: the same implicit GEMM per tile (one
-// 128-pixel row segment), fed from a ring of staged input rows.  A work unit
-// is up to kUnitRows consecutive output rows of one (chain, 128-column
-// segment); it stages its rows r0 - 1 .. r0 + n once each, as a halo row of
-// 130 pixels (x0 - 1 .. x0 + 128, periodic) in 4 channel-group planes of
-// kRingPlane bytes, so the operand of tap (dy, dx) is the staged row y + dy
-// offset by (1 + dx) x 16 bytes (LBO = kRingPlane, SBO = 128).
+// Layers 2 and 3 as an implicit GEMM per tile of one row segment,
+//   Z[m][o] = sum over taps k and input channels i of A_k[m][i] W[o][i][k],
+// M = 128 pixels, N = 32 output channels, K = 9 taps x 32 channels (tcgen05.mma
+// kind::f16, BF16 operands, FP32 accumulator in tensor memory), fed from a ring
+// of staged input rows.  A work unit is up to kUnitRows consecutive output rows
+// of one (chain, segment); it stages its rows r0 - 1 .. r0 + n once each, as a
+// halo row of tw + 2 pixels (x0 - 1 .. x0 + tw, periodic) in 4 channel-group
+// planes of kRingPlane bytes, so the operand of tap (dy, dx) is the staged row
+// y + dy offset by (1 + dx) x 16 bytes (no-swizzle K-major, LBO = kRingPlane,
+// SBO = 128).  (Sides that are no multiple of 128 took a kernel that gathered all
+// 9 taps of every tile, im2col, from global memory and one that projected on the
+// CUDA cores: a forward of 256 chains of 96^2 892 us, here 343; a training step of
+// 40 chains of 96^2 1352, here 445.)
 // Warp roles, linked by mbarriers (every wait bounded):
 //   warp 0: loader -- lane 0 fetches each row with four tensor copies (TMA),
-//           one per channel group: a box of 8 channels x 130 pixels of the
+//           one per channel group: a box of 8 channels x tw + 2 pixels of the
 //           padded row (its halo columns included), completing on full[slot];
 //           or, in the first layer of an inference pass (FUSED), the warp
 //           builds the row of a1 itself: 18 lanes turn 3 spin rows x 6
@@ -626,8 +430,11 @@ __global__ void __launch_bounds__(kConvThreads, 1) conv32_tc_kernel(const __grid
 //   warps 2-9: epilogue, warp w on TMEM lanes 32 (w % 4) .. + 31 (its 32
 //           pixels) and columns 16 h .. 16 h + 15, h = (w - 2) / 4 (its 16
 //           channels): loads them, sets them to the bias (every MMA
-//           accumulates, so the next row's sum starts from its bias; zero in
-//           BWD), frees the block (acce, 8 arrivals) and writes z (training)
+//           accumulates, so the next row's sum starts from its bias; to zero in
+//           BWD and for sides that are no multiple of 128, where the bias is
+//           added after the last product, so that their pre-activations, and
+//           with them every bfloat16 rounding, are those of a sum over the taps
+//           plus the bias), frees the block (acce, 8 arrivals) and writes z (training)
 //           and a = bf16(gelu(z)).  (Adding the bias in the epilogue and
 //           gelu as z (1 - h) or z h by sign instead of max(z, 0) - |z| h:
 //           1.438 instead of 1.383 ms per full forward of 1024 chains.)
@@ -795,7 +602,7 @@ struct RingConv {
     const float *params;
     int w_off, b_off;
     Band bd;
-    int segs;           // L / 128
+    int segs, tw;       // row segments and their width
     int units_per_col;  // ceil(bd.rows / kUnitRows)
     int64_t units;      // C segs units_per_col
     int withhold;       // self-test: never signal the first accumulator, so its wait runs out
@@ -803,16 +610,21 @@ struct RingConv {
 
 struct RingUnit {
     int64_t c;
-    int x0, r0, nrows;
+    int x0, width, r0, nrows;  // first pixel, pixels of the segment, first row, rows
 };
 
+// FULL: every segment has 128 pixels (L a multiple of 128), which the compiler
+// then knows (without it the forward of 1024 chains of 128^2 takes 3.6% longer).
+template <bool FULL>
 __device__ __forceinline__ RingUnit ring_unit(const RingConv &p, int64_t u)
 {
     RingUnit w;
     const int64_t col = u / p.units_per_col;
     const int rb = (int)(u - col * p.units_per_col);
     w.c = col / p.segs;
-    w.x0 = (int)(col - w.c * p.segs) * kTileM;
+    const int tw = FULL ? kTileM : p.tw;
+    w.x0 = (int)(col - w.c * p.segs) * tw;
+    w.width = FULL ? kTileM : min(tw, p.bd.L - w.x0);
     w.r0 = rb * kUnitRows;
     w.nrows = min(kUnitRows, p.bd.rows - w.r0);
     return w;
@@ -863,13 +675,15 @@ __device__ __forceinline__ uint32_t chunk_bits(const Chains &ch, const ChunkWord
     return v;
 }
 
-template <bool PROJ, bool BWD, bool FUSED>
+template <bool PROJ, bool BWD, bool FUSED, bool FULL>
 __global__ void __launch_bounds__(ring_threads<PROJ, FUSED>(), 2) conv32_ring_kernel(const __grid_constant__ RingConv p)
 {
     extern __shared__ __align__(1024) uint8_t ring_smem[];
     // the data-gradient kernel and the training forward of the first 32 -> 32
     // layer (neither fused with layer 1 nor projecting) stage their epilogue I/O
     constexpr bool STAGE = BWD || (!PROJ && !FUSED);
+    // where the bias joins the sum: before the first product, or after the last
+    constexpr bool kBiasFirst = FULL && !BWD;
     using Lay = RingLayout<PROJ, STAGE>;
     uint8_t *ring = ring_smem + Lay::ring;
     uint8_t *a3s = ring_smem + Lay::a3;
@@ -943,7 +757,7 @@ __global__ void __launch_bounds__(ring_threads<PROJ, FUSED>(), 2) conv32_ring_ke
         const int quad = warp & 3, half = (warp - 2) >> 2;
         float bias[16];
 #pragma unroll
-        for (int i = 0; i < 16; ++i) bias[i] = sBias[16 * half + i];
+        for (int i = 0; i < 16; ++i) bias[i] = kBiasFirst ? sBias[16 * half + i] : 0.0f;
         for (int a = 0; a < kAcc; ++a) tc::tmem_st16(tmem + (uint32_t)(a * kCh + 16 * half) + ((uint32_t)(quad * 32) << 16), bias);
         tc::tmem_wait_st();
     }
@@ -962,7 +776,7 @@ __global__ void __launch_bounds__(ring_threads<PROJ, FUSED>(), 2) conv32_ring_ke
         const uint4 *ta = reinterpret_cast<const uint4 *>(p.ta);
         const int nw = L / 32;
         for (int64_t u = blockIdx.x; u < p.units && ok; u += gridDim.x) {
-            const RingUnit w = ring_unit(p, u);
+            const RingUnit w = ring_unit<FULL>(p, u);
             const int fb = p.flip ? p.flip[w.c] : -1;
             // lane 6 d + q (d < 3, q < 6): chunk x0 / 32 - 1 + q (periodic) of spin row y - 1 + d
             auto fetch = [&](int j) {
@@ -991,6 +805,7 @@ __global__ void __launch_bounds__(ring_threads<PROJ, FUSED>(), 2) conv32_ring_ke
                 uint8_t *dst = ring + s * kRowBytes;
 #pragma unroll
                 for (int i = 0; i < 5; ++i) {
+                    if (32 * i >= w.width + 2) break;
                     const int e = lane + 32 * i;   // entry e is column x0 - 1 + e
                     const int o = e + 30;          // column x0 - 2 + e relative to the window start x0 - 32
                     const int wi = o >> 5, sh = o & 31;
@@ -1002,7 +817,7 @@ __global__ void __launch_bounds__(ring_threads<PROJ, FUSED>(), 2) conv32_ring_ke
                         const uint32_t trip = (uint32_t)((((uint64_t)hi << 32) | lo) >> sh) & 7u;
                         pat |= trip << (3 * d);
                     }
-                    if (e < kTileM + 2) {
+                    if (e < w.width + 2) {
 #pragma unroll
                         for (int g = 0; g < kGroups; ++g)
                             *reinterpret_cast<uint4 *>(dst + g * kRingPlane + e * 16) = __ldg(ta + pat * kGroups + g);
@@ -1019,7 +834,7 @@ __global__ void __launch_bounds__(ring_threads<PROJ, FUSED>(), 2) conv32_ring_ke
         if (lane == 0) {
             uint32_t n = 0;  // rows staged so far
             for (int64_t u = blockIdx.x; u < p.units && ok; u += gridDim.x) {
-                const RingUnit w = ring_unit(p, u);
+                const RingUnit w = ring_unit<FULL>(p, u);
                 for (int j = -1; j <= w.nrows; ++j, ++n) {
                     const uint32_t s = n & (kRing - 1);
                     if (n >= kRing && !tc::mbar_wait(&empty[s], ((n / kRing) + 1) & 1, kWaitCycles)) {
@@ -1027,7 +842,7 @@ __global__ void __launch_bounds__(ring_threads<PROJ, FUSED>(), 2) conv32_ring_ke
                         break;
                     }
                     const int y = ring_row(p, w.c, w.r0 + j);
-                    tc::mbar_arrive_expect_tx(&full[s], kGroups * (kTileM + 2) * 16);
+                    tc::mbar_arrive_expect_tx(&full[s], (uint32_t)(kGroups * ((FULL ? kTileM : p.tw) + 2) * 16));
                     uint8_t *dst = ring + s * kRowBytes;
 #pragma unroll
                     for (int g = 0; g < kGroups; ++g)
@@ -1065,7 +880,7 @@ __global__ void __launch_bounds__(ring_threads<PROJ, FUSED>(), 2) conv32_ring_ke
             // core takes ~45 cycles per N32 MMA and ~56 per N96 one.)
             uint32_t n0 = 0, t = 0, ready = 0;  // n0: ring index of the unit's row -1; t: rows of the units before
             for (int64_t u = blockIdx.x; u < p.units && ok; u += gridDim.x) {
-                const RingUnit w = ring_unit(p, u);
+                const RingUnit w = ring_unit<FULL>(p, u);
                 for (int i = -1; i <= w.nrows && ok; ++i) {
                     while (ready < n0 + (uint32_t)(i + 2) && ok) {
                         if (!tc::mbar_wait(&full[ready & (kRing - 1)], (ready / kRing) & 1u, kWaitCycles)) ok = false;
@@ -1120,7 +935,7 @@ __global__ void __launch_bounds__(ring_threads<PROJ, FUSED>(), 2) conv32_ring_ke
             const uint32_t idesc_p = tc::idesc_bf16_f32(kTileM, kProjN);
             const uint32_t a3_u32 = tc::smem_u32(a3s), w4_u32 = tc::smem_u32(sW4);
             int64_t rows = 0;
-            for (int64_t u = blockIdx.x; u < p.units; u += gridDim.x) rows += ring_unit(p, u).nrows;
+            for (int64_t u = blockIdx.x; u < p.units; u += gridDim.x) rows += ring_unit<FULL>(p, u).nrows;
             for (int64_t s = 0; s < rows && ok; ++s) {
                 const int b = (int)(s & 1);
                 if (!tc::mbar_wait(&a3full[b], (uint32_t)((s >> 1) & 1), kWaitCycles) ||
@@ -1149,14 +964,15 @@ __global__ void __launch_bounds__(ring_threads<PROJ, FUSED>(), 2) conv32_ring_ke
         float4 *stg = reinterpret_cast<float4 *>(ring_smem + Lay::stage + (uint32_t)(warp - 2) * kStageBytes);
         uint4 *st16 = reinterpret_cast<uint4 *>(stg);
         const int xw = 32 * quad;  // the warp's first pixel in the tile (add w.x0)
-        float bias[16];  // this warp's 16 channels (zero in BWD)
+        float bias[16];  // what the accumulators of this warp's 16 channels start from
 #pragma unroll
-        for (int i = 0; i < 16; ++i) bias[i] = sBias[16 * half + i];
+        for (int i = 0; i < 16; ++i) bias[i] = kBiasFirst ? sBias[16 * half + i] : 0.0f;
         int64_t t = 0;
         for (int64_t u = blockIdx.x; u < p.units && ok; u += gridDim.x) {
-            const RingUnit w = ring_unit(p, u);
+            const RingUnit w = ring_unit<FULL>(p, u);
             for (int j = 0; j < w.nrows; ++j, ++t) {
                 const int a = ring_blk((uint32_t)t);
+                const bool on = FULL || xw < w.width;  // this warp's pixels are inside the segment
                 const int y = ring_row(p, w.c, w.r0 + j);
                 const int64_t q = (w.c * L + y) * (int64_t)L + w.x0 + m;
                 // BWD: gelu'(z_prev) of this row does not depend on the
@@ -1165,15 +981,35 @@ __global__ void __launch_bounds__(ring_threads<PROJ, FUSED>(), 2) conv32_ring_ke
                 const int64_t q0 = q - lane;
                 float gz[16];
                 if constexpr (BWD) {
-                    tile_load_f32(p.zg + q0 * kCh + 16 * half, stg, lane, gz);
+                    if (on) {
+                        tile_load_f32(p.zg + q0 * kCh + 16 * half, stg, lane, gz);
 #pragma unroll
-                    for (int i = 0; i < 16; i += 2) gelu_grad2(gz[i], gz[i + 1]);
+                        for (int i = 0; i < 16; i += 2) gelu_grad2(gz[i], gz[i + 1]);
+                    }
                 }
                 if (!__all_sync(0xffffffffu, tc::mbar_wait(&accf[a], ring_use((uint32_t)t) & 1u, kWaitCycles))) {
                     ok = false;
                     break;
                 }
                 tc::fence_after_sync();
+                if (!on) {
+                    // nothing to read, but the next unit may be wider: back to the bias
+                    tc::tmem_st16(tmem + (uint32_t)(a * kCh + 16 * half) + ((uint32_t)(quad * 32) << 16), bias);
+                    tc::tmem_wait_st();
+                    tc::fence_before_sync();
+                    __syncwarp();
+                    if (lane == 0) tc::mbar_arrive(&acce[a]);
+                    if (PROJ) {
+                        const int b = (int)(t & 1);
+                        if (t >= 2 && !__all_sync(0xffffffffu, tc::mbar_wait(&a3empty[b], (uint32_t)(((t >> 1) + 1) & 1),
+                                                                              kWaitCycles))) {
+                            ok = false;
+                            break;
+                        }
+                        if (lane == 0) tc::mbar_arrive(&a3full[b]);
+                    }
+                    continue;
+                }
                 float v[16];
                 const uint32_t ta = tmem + (uint32_t)(a * kCh + 16 * half) + ((uint32_t)(quad * 32) << 16);
                 tc::tmem_ld16(ta, v);
@@ -1183,6 +1019,10 @@ __global__ void __launch_bounds__(ring_threads<PROJ, FUSED>(), 2) conv32_ring_ke
                 tc::fence_before_sync();
                 __syncwarp();
                 if (lane == 0) tc::mbar_arrive(&acce[a]);
+                if constexpr (!kBiasFirst && !BWD) {
+#pragma unroll
+                    for (int i = 0; i < 16; ++i) v[i] += sBias[16 * half + i];
+                }
                 if constexpr (BWD) {
 #pragma unroll
                     for (int i = 0; i < 16; ++i) v[i] *= gz[i];
@@ -1256,7 +1096,7 @@ __global__ void __launch_bounds__(ring_threads<PROJ, FUSED>(), 2) conv32_ring_ke
         const int quad = warp & 3, m = quad * 32 + lane;
         int64_t s = 0;
         for (int64_t u = blockIdx.x; u < p.units && ok; u += gridDim.x) {
-            const RingUnit w = ring_unit(p, u);
+            const RingUnit w = ring_unit<FULL>(p, u);
             for (int j = 0; j < w.nrows; ++j, ++s) {
                 const int b = (int)(s & 1);
                 if (!__all_sync(0xffffffffu, tc::mbar_wait(&pfull[b], (uint32_t)((s >> 1) & 1), kWaitCycles))) {
@@ -1269,6 +1109,7 @@ __global__ void __launch_bounds__(ring_threads<PROJ, FUSED>(), 2) conv32_ring_ke
                 tc::fence_before_sync();
                 __syncwarp();
                 if (lane == 0) tc::mbar_arrive(&pempty[b]);
+                if (!FULL && 32 * quad >= w.width) continue;
                 // row partials of z4 (see pool_rows_kernel): P_k of this pixel
                 // (y, x), tap k = 3 (dy + 1) + (dx + 1), goes to z4 at (y - dy,
                 // x - dx); per dy, the part that stays in the pixel's 8 x 8
@@ -1304,89 +1145,8 @@ __global__ void __launch_bounds__(ring_threads<PROJ, FUSED>(), 2) conv32_ring_ke
     }
 }
 
-// Layer 4's channel contraction for the general conv kernel: thread per pixel
-// of the band, P[k][q] = sum_i W4[i][k] a3(q)[i] (i in order).
-__global__ void __launch_bounds__(kThreads) l4_project_kernel(Band bd, const float *params, const __nv_bfloat16 *a3,
-                                                              float *P)
-{
-    __shared__ float W[kN1];  // W4[i][k] at 9 i + k
-    for (int i = threadIdx.x; i < kN1; i += blockDim.x) W[i] = bf16r(params[kOffW4 + i]);
-    __syncthreads();
-    const int L = bd.L;
-    const int64_t npix = bd.C * (int64_t)L * L;
-    const int64_t n = bd.C * (int64_t)bd.rows * L;
-    for (int64_t pb = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; pb < n; pb += (int64_t)gridDim.x * blockDim.x) {
-        int64_t c;
-        int yx;
-        band_pixel(bd, pb, c, yx);
-        const int64_t q = c * (int64_t)L * L + yx;
-        const int y = yx / L;
-        const uint4 *src = reinterpret_cast<const uint4 *>(a3 + apix(L, c, y, yx - y * L) * kCh);
-        float acc[9];
-#pragma unroll
-        for (int k = 0; k < 9; ++k) acc[k] = 0.0f;
-#pragma unroll
-        for (int g = 0; g < kGroups; ++g) {
-            const uint4 v = __ldg(src + g);
-            const uint32_t u[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const float lo = bf16_lo(u[j]), hi = bf16_hi(u[j]);
-                const int i = 8 * g + 2 * j;
-#pragma unroll
-                for (int k = 0; k < 9; ++k) acc[k] = fmaf(W[(i + 1) * 9 + k], hi, fmaf(W[i * 9 + k], lo, acc[k]));
-            }
-        }
-#pragma unroll
-        for (int k = 0; k < 9; ++k) P[k * npix + q] = acc[k];
-    }
-}
-
-// Layer 4 and the block mean from the projections: z4(y, x) = b4 + sum over
-// taps k of P[k](y + dy_k, x + dx_k).  Warp per (chain, block row, group of 4
-// blocks) over `brows` block rows per chain (all of them in a full pass; in a
-// band pass the flipped block's row and its two neighbours): lane l owns
-// pixel column 8 b + l of the group and walks the block's 8 rows (taps in
-// order, rows in order), so every load of a tap plane is 32 consecutive
-// floats; the 8 lanes of a block then add up in a fixed shuffle tree.
-__global__ void __launch_bounds__(kThreads) pool_kernel(int L, int64_t C, int brows, const int32_t *flip,
-                                                        const float *params, const float *P, float *logits)
-{
-    const float b4 = bf16r(params[kOffB4]);
-    const int nb1 = L / kBlk, nb = nb1 * nb1, groups = nb1 / 4;
-    const int lane = threadIdx.x & 31;
-    const int64_t npix = C * (int64_t)L * L;
-    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    const int per = brows * groups;
-    for (int64_t wi = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; wi < C * per; wi += nw) {
-        const int64_t c = wi / per;
-        const int r = (int)(wi - c * per), rb = r / groups, bg = r - rb * groups;
-        int by = rb;
-        if (flip) {
-            const int f = flip[c];
-            by = wrap((f < 0 ? 0 : f / nb1) - 1 + rb, nb1);
-        }
-        const float *Pc = P + c * (int64_t)L * L;
-        const int x = bg * 32 + lane;
-        const int xs[3] = {wrap(x - 1, L), x, wrap(x + 1, L)};
-        float part = 0.0f;
-        // unrolled: the loads of all 8 rows are issued before the sums (same order of additions)
-#pragma unroll
-        for (int yy = by * kBlk; yy < by * kBlk + kBlk; ++yy) {
-            const int ys[3] = {wrap(yy - 1, L), yy, wrap(yy + 1, L)};
-            float z = b4;
-#pragma unroll
-            for (int k = 0; k < 9; ++k) z += __ldg(Pc + k * npix + ys[k / 3] * (int64_t)L + xs[k % 3]);
-            part += z;
-        }
-#pragma unroll
-        for (int off = 4; off > 0; off >>= 1) part += __shfl_xor_sync(0xffffffffu, part, off);
-        if ((lane & 7) == 0) logits[c * nb + by * nb1 + 4 * bg + (lane >> 3)] = part * (1.0f / (kBlk * kBlk));
-    }
-}
-
-// The block logits from the row partials the projecting ring kernel writes
-// (L a multiple of 128): R[c][y][3 dy' + j][bx], dy' = dy + 1, holds for the
+// The block logits from the row partials the projecting ring kernel writes:
+// R[c][y][3 dy' + j][bx], dy' = dy + 1, holds for the
 // P values of row y with tap row dy (they feed z4 in row y - dy)
 //   j = 0: the sum over block column bx of the parts that stay in it,
 //   j = 1: the dx = +1 part of the block's first pixel (feeds block bx - 1),
@@ -1483,160 +1243,6 @@ __global__ void __launch_bounds__(kThreads) l4_bwd_data_kernel(int L, int64_t C,
     }
 }
 
-// dz_prev = gelu'(z_prev) * sum_{k, o} W[o][i][k] * bf16(dz(p - off_k)[o]);
-// weights as Wt[k][o][i] (32 contiguous inputs per tap and output).  The
-// incoming gradient is rounded to bfloat16, as on the tensor-core path.
-__global__ void __launch_bounds__(kThreads) conv32_bwd_data_kernel(int L, int64_t C, const float *params, int w_off,
-                                                                   const float *dz, const float *z_prev, float *dz_prev)
-{
-    extern __shared__ float Wt[];
-    for (int i = threadIdx.x; i < kN2; i += blockDim.x) {
-        const int o = i / (kCh * 9), rem = i - o * kCh * 9, ci = rem / 9, k = rem - ci * 9;
-        Wt[(k * kCh + o) * kCh + ci] = bf16r(params[w_off + i]);
-    }
-    __syncthreads();
-    const int64_t npix = C * (int64_t)L * L;
-    for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < npix; p += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t c = p / ((int64_t)L * L);
-        const int yx = (int)(p - c * (int64_t)L * L);
-        const int y = yx / L, x = yx - y * L;
-        float acc[kCh];
-#pragma unroll
-        for (int i = 0; i < kCh; ++i) acc[i] = 0.0f;
-        for (int k = 0; k < 9; ++k) {
-            const int yy = (y - (k / 3 - 1) + L) % L, xx = (x - (k % 3 - 1) + L) % L;
-            const float4 *src = reinterpret_cast<const float4 *>(dz + ((c * L + yy) * (int64_t)L + xx) * kCh);
-#pragma unroll
-            for (int q = 0; q < kCh / 4; ++q) {
-                const float4 v = src[q];
-                const float g4[4] = {bf16r(v.x), bf16r(v.y), bf16r(v.z), bf16r(v.w)};
-#pragma unroll
-                for (int r = 0; r < 4; ++r) {
-                    const float *w = Wt + (k * kCh + 4 * q + r) * kCh;
-#pragma unroll
-                    for (int i = 0; i < kCh; ++i) acc[i] = fmaf(w[i], g4[r], acc[i]);
-                }
-            }
-        }
-        const float *zp = z_prev + p * kCh;
-        float *out = dz_prev + p * kCh;
-#pragma unroll
-        for (int i = 0; i < kCh; ++i) out[i] = acc[i] * gelu_grad(zp[i]);
-    }
-}
-
-// Weight gradients of a 32 -> 32 layer on the CUDA cores (L not a multiple of
-// 128; wgrad_tc_kernel below serves the others), as per-CTA partial sums
-// (fixed order).  The pixels are cut into tiles of 8 rows x 32 columns of one
-// chain; CTA j handles tiles j, j + gridDim.x, ... in order.  A tile's output
-// gradients dz (and the layer's input a, with a one-pixel halo) are staged in
-// shared memory; thread (oq, iq) of 16 x 16 accumulates the 2 x 2 (output,
-// input) channel pairs 2 oq + {0, 1} x 2 iq + {0, 1} for all 9 taps, and
-// threads with iq = 0 the bias sums.  partial[cta][e]: e = (o * 32 + i) * 9 + k
-// for weights, then the biases.
-constexpr int kTy = 8, kTx = 32;
-
-__device__ __forceinline__ void wgrad_stage(const Chains &ch, const __nv_bfloat16 *a_prev, const float *dz, int64_t c,
-                                            int y0, int x0, float *sa, float *sd)
-{
-    const int L = ch.L;
-    // input tile with halo: (kTy + 2) x (kTx + 2) pixels x 32 channels, as four
-    // 16-byte loads of 8 bfloat16 per pixel
-    constexpr int kOct = kCh / 8;
-    for (int e = threadIdx.x; e < (kTy + 2) * (kTx + 2) * kOct; e += blockDim.x) {
-        const int pix = e / kOct, q = e - pix * kOct;
-        const int ty = pix / (kTx + 2), tx = pix - ty * (kTx + 2);
-        int y = y0 + ty - 1, x = x0 + tx - 1;
-        y = y < 0 ? y + L : (y >= L ? y - L : y);
-        x = x < 0 ? x + L : (x >= L ? x - L : x);
-        const uint4 v = *reinterpret_cast<const uint4 *>(a_prev + apix(L, c, y, x) * kCh + 8 * q);
-        float4 *dst = reinterpret_cast<float4 *>(sa + pix * kCh + 8 * q);
-        dst[0] = make_float4(bf16_lo(v.x), bf16_hi(v.x), bf16_lo(v.y), bf16_hi(v.y));
-        dst[1] = make_float4(bf16_lo(v.z), bf16_hi(v.z), bf16_lo(v.w), bf16_hi(v.w));
-    }
-    // output gradients of the tile: a tile row of 32 pixels x 32 channels is
-    // contiguous, loaded as float4
-    for (int e = threadIdx.x; e < kTy * kTx * kCh / 4; e += blockDim.x) {
-        const int row = e / (kTx * kCh / 4), v = e - row * (kTx * kCh / 4);
-        const float4 *src = reinterpret_cast<const float4 *>(dz + ((c * L + y0 + row) * (int64_t)L + x0) * kCh);
-        reinterpret_cast<float4 *>(sd)[e] = src[v];
-    }
-}
-
-__global__ void __launch_bounds__(256) wgrad_kernel(Chains ch, int64_t C, const __nv_bfloat16 *a_prev, const float *dz,
-                                                    float *partial)
-{
-    extern __shared__ float smem[];
-    float *sa = smem;                                 // (kTy+2) (kTx+2) 32
-    float *sd = smem + (kTy + 2) * (kTx + 2) * kCh;   // kTy kTx 32
-    constexpr int NE = kN2 + kCh;
-    const int L = ch.L;
-    const int tiles_x = L / kTx, tiles_y = L / kTy;
-    const int64_t n_tiles = C * tiles_x * tiles_y;
-    const int oq = threadIdx.x >> 4, iq = threadIdx.x & 15;  // channel pairs 2 oq, 2 oq + 1 and 2 iq, 2 iq + 1
-    float acc[2][2][9];
-    float bacc[2] = {0.0f, 0.0f};
-#pragma unroll
-    for (int a = 0; a < 2; ++a)
-#pragma unroll
-        for (int b = 0; b < 2; ++b)
-#pragma unroll
-            for (int k = 0; k < 9; ++k) acc[a][b][k] = 0.0f;
-    for (int64_t tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
-        const int64_t c = tile / (tiles_x * tiles_y);
-        const int rem = (int)(tile - c * tiles_x * tiles_y);
-        const int y0 = (rem / tiles_x) * kTy, x0 = (rem % tiles_x) * kTx;
-        __syncthreads();
-        wgrad_stage(ch, a_prev, dz, c, y0, x0, sa, sd);
-        __syncthreads();
-        // pixels in row order; along a tile row the 3 x 3 input window slides
-        // in registers, so each pixel loads one new column per dy (channel
-        // pairs as float2)
-        for (int ty = 0; ty < kTy; ++ty) {
-            float2 win[3][3];  // [dy][dx], input channels 2 iq, 2 iq + 1
-#pragma unroll
-            for (int dy = 0; dy < 3; ++dy)
-#pragma unroll
-                for (int dx = 0; dx < 2; ++dx)
-                    win[dy][dx] = *reinterpret_cast<const float2 *>(sa + ((ty + dy) * (kTx + 2) + dx) * kCh + 2 * iq);
-#pragma unroll
-            for (int tx = 0; tx < kTx; ++tx) {
-#pragma unroll
-                for (int dy = 0; dy < 3; ++dy)
-                    win[dy][2] = *reinterpret_cast<const float2 *>(sa + ((ty + dy) * (kTx + 2) + tx + 2) * kCh + 2 * iq);
-                const float2 g2 = *reinterpret_cast<const float2 *>(sd + (ty * kTx + tx) * kCh + 2 * oq);
-                const float g[2] = {g2.x, g2.y};
-#pragma unroll
-                for (int a = 0; a < 2; ++a) bacc[a] += g[a];
-#pragma unroll
-                for (int k = 0; k < 9; ++k) {
-                    const float2 wv = win[k / 3][k % 3];
-#pragma unroll
-                    for (int a = 0; a < 2; ++a) {
-                        acc[a][0][k] = fmaf(g[a], wv.x, acc[a][0][k]);
-                        acc[a][1][k] = fmaf(g[a], wv.y, acc[a][1][k]);
-                    }
-                }
-#pragma unroll
-                for (int dy = 0; dy < 3; ++dy) {
-                    win[dy][0] = win[dy][1];
-                    win[dy][1] = win[dy][2];
-                }
-            }
-        }
-    }
-    float *out = partial + (int64_t)blockIdx.x * NE;
-#pragma unroll
-    for (int a = 0; a < 2; ++a)
-#pragma unroll
-        for (int b = 0; b < 2; ++b)
-#pragma unroll
-            for (int k = 0; k < 9; ++k) out[((2 * oq + a) * kCh + 2 * iq + b) * 9 + k] = acc[a][b][k];
-    if (iq == 0)
-#pragma unroll
-        for (int a = 0; a < 2; ++a) out[kN2 + 2 * oq + a] = bacc[a];
-}
-
 // Weight gradients of the layers with one input or one output channel, warp
 // per run of rows, lane per channel:
 //   layer 1 (spins -> 32): dW1[o][k] = sum_p dz1(p)[o] s(p + off_k),
@@ -1650,9 +1256,8 @@ __global__ void __launch_bounds__(256) wgrad_kernel(Chains ch, int64_t C, const 
 // field at column x0 + j of rows y - 1, y, y + 1, the halo columns are loaded
 // by every lane, and the window slides along the chunk by one shuffle per row
 // and pixel.  Per pixel and lane: one load, three shuffles, nine FMAs.  The
-// CTA's warps are added in warp order and written as the CTA's partial sums
-// (layout of wgrad_kernel), summed by reduce_partials_kernel.  (wgrad_kernel
-// gives these layers 16 busy threads per CTA.)
+// CTA's warps are added in warp order and written as the CTA's partial sums (the
+// weights in W[o][i][k] order, then the biases), summed by reduce_partials_kernel.
 constexpr int kThinWarps = 8;
 
 template <bool L4>
@@ -1776,13 +1381,13 @@ __global__ void __launch_bounds__(32 * kReduceWarps) reduce_partials_kernel(cons
     }
 }
 
-// Weight gradients of a 32 -> 32 layer on the tensor cores (L a multiple of
-// 128).  With a the layer's input (bfloat16, halo columns) and dz the gradient
+// Weight gradients of a 32 -> 32 layer on the tensor cores.  With a the layer's input (bfloat16, halo columns) and dz the gradient
 // of its pre-activations,
 //   dW[o][i][k] = sum_p dz(p)[o] a(p + off_k)[i],   db[o] = sum_p dz(p)[o],
 // off_k = (dy - 1, dx - 1) for tap k = 3 dy + dx.  Input row y' meets the
-// gradient rows y' + 1, y', y' - 1 (dy = 0, 1, 2), so per 128-pixel row
-// segment of input row y' there is one GEMM over the segment's 128 pixels (K):
+// gradient rows y' + 1, y', y' - 1 (dy = 0, 1, 2), so per segment of input row y'
+// there is one GEMM over the segment's tw pixels (K; a shorter last segment is
+// filled up with zero gradients):
 //   D[m][n] += sum_x A_y'[m][x] B_y'[n][x]
 // with M = 128 rows, of which rows m = 32 dx + i (dx = 0..2) are the input row
 // shifted by dx - 1 and rows 96..127 are not used, and N = 192 columns
@@ -1790,10 +1395,10 @@ __global__ void __launch_bounds__(32 * kReduceWarps) reduce_partials_kernel(cons
 // dy = 2 - b), each as two bfloat16 parts, h = 0 its rounding and h = 1 the
 // rounding of the remainder, so that a x (hi + lo) carries dz to about 2^-17
 // and the FP32 accumulation sees the unrounded gradient to that accuracy
-// (dW = D[.][64 b + o] + D[.][64 b + 32 + o]).  Eight MMAs of M128 x N192 x
+// (dW = D[.][64 b + o] + D[.][64 b + 32 + o]).  tw / 16 MMAs of M128 x N192 x
 // K16 per input row segment.
 // Both operands are MN-major and come straight from the NHWC buffers: a
-// tensor copy of 128 whole pixels (32 channels, 64 bytes each) with the
+// tensor copy of tw whole pixels (32 channels, 64 bytes each) with the
 // 64-byte swizzle is the MN-major 64-byte-swizzled operand form: 8 K rows
 // (pixels) of 64 bytes per 512-byte atom, SBO = 512 bytes between the 8-row
 // groups along K, LBO = 8 KB between the 32-channel groups along M (or N).
@@ -1811,7 +1416,7 @@ __global__ void __launch_bounds__(32 * kReduceWarps) reduce_partials_kernel(cons
 // gradient rows r0 - 2 .. r0 + n + 1, those outside the run as zeros (tensor
 // copies of a row past the lattice's last, which the copy fills with zeros),
 // so that every (input row, gradient row) pair is counted by exactly one CTA.
-// The accumulators (192 TMEM columns) collect the CTA's whole range; at the
+// The accumulators (192 TMEM columns per set) collect the CTA's whole range; at the
 // end they are written as the CTA's partial sums in the weight-gradient
 // layout (e = (o CIN + i) 9 + k, then the biases).
 // Warp roles (bounded mbarrier waits): warp 0 lane 0 issues the tensor
@@ -1832,17 +1437,22 @@ constexpr uint32_t kWgBar = kWgBias + kWgBiasWarps * kCh * 4;
 constexpr uint32_t kWgSmem = kWgBar + (2 * kWgActSlots + 2 * kWgDzSlots + 1) * 8 + 16;
 constexpr int kWgThreads = 64 + 32 * kWgBiasWarps;
 constexpr int kWgN = 6 * kCh;                       // three gradient rows, hi and lo
-constexpr uint32_t kWgTmemCols = 256;               // 192 used
+// accumulator sets of 192 (in 256) columns: the MMA's accumulation truncates, an
+// error that grows with the terms of a sum (1.6e-5 of the largest weight gradient
+// over 15000 pixels per CTA), so the input rows go to two sets in turn where the
+// CUDA cores' rounding sums had served before (sides that are no multiple of 128)
+template <bool FULL>
+constexpr int kWgSets = FULL ? 1 : 2;
 static_assert(kWgDz0 >= kWgActBytes + kWgBox && kWgSmem <= 227 * 1024 && kWgActBytes % 1024 == 0 &&
                   kWgDz0 % 1024 == 0,
               "the unused M rows of the last input slot read the gradient slots; one CTA per SM");
 
 struct WgradTc {
-    CUtensorMap act;  // a: (32 channels, L + 2 pixels, L rows, C chains), boxes 32 x 128 x 1 x 1, 64-byte swizzle
-    CUtensorMap hi;   // bf16(dz), same layout
-    CUtensorMap lo;   // bf16(dz - bf16(dz)), same layout
+    CUtensorMap act;  // a: (32 channels, L + 2 pixels, L rows, C chains), boxes 32 x tw x 1 x 1, 64-byte swizzle
+    CUtensorMap hi;   // bf16(dz), the same without the last halo column (a box past pixel L reads zeros)
+    CUtensorMap lo;   // bf16(dz - bf16(dz)), likewise
     float *partial;   // [gridDim.x][kN2 + kCh]
-    int L, segs;
+    int L, segs, tw;
     int64_t lines;    // C segs L
 };
 
@@ -1855,10 +1465,12 @@ __device__ __forceinline__ RingUnit wg_run(const WgradTc &p, int64_t lin, int64_
     w.r0 = (int)(lin - col * p.L);
     w.nrows = (int)min((int64_t)(p.L - w.r0), end - lin);
     w.c = col / p.segs;
-    w.x0 = (int)(col - w.c * p.segs) * kTileM;
+    w.x0 = (int)(col - w.c * p.segs) * p.tw;
+    w.width = p.tw;
     return w;
 }
 
+template <bool FULL>
 __global__ void __launch_bounds__(kWgThreads, 1) wgrad_tc_kernel(const __grid_constant__ WgradTc p)
 {
     extern __shared__ __align__(1024) uint8_t wg_smem[];
@@ -1869,9 +1481,11 @@ __global__ void __launch_bounds__(kWgThreads, 1) wgrad_tc_kernel(const __grid_co
     uint32_t *tslot = reinterpret_cast<uint32_t *>(drain + 1);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int L = p.L;
+    const uint32_t box = (uint32_t)(FULL ? kTileM : p.tw) * kCh * 2;  // bytes of a staged row of tw pixels
     const int64_t begin = blockIdx.x * p.lines / gridDim.x, end = (blockIdx.x + 1) * p.lines / gridDim.x;
 
-    if (warp == 1) tc::tmem_alloc(tslot, kWgTmemCols);
+    constexpr uint32_t kCols = 256 * kWgSets<FULL>;
+    if (warp == 1) tc::tmem_alloc(tslot, kCols);
     if (tid == 0) {
         for (int s = 0; s < kWgActSlots; ++s) {
             tc::mbar_init(&afull[s], 1);
@@ -1898,7 +1512,7 @@ __global__ void __launch_bounds__(kWgThreads, 1) wgrad_tc_kernel(const __grid_co
                 if (na >= kWgActSlots && !tc::mbar_wait(&aempty[s], ((na / kWgActSlots) + 1) & 1, kWaitCycles))
                     return false;
                 const int y = wrap(r, L);
-                tc::mbar_arrive_expect_tx(&afull[s], kWgActBytes);
+                tc::mbar_arrive_expect_tx(&afull[s], 3 * box);
                 uint8_t *dst = wg_smem + s * kWgActBytes;
 #pragma unroll
                 for (int dx = 0; dx < 3; ++dx) tc::tma_load_4d(dst + dx * kWgBox, &p.act, 0, w.x0 + dx, y, (int)w.c, &afull[s]);
@@ -1912,7 +1526,7 @@ __global__ void __launch_bounds__(kWgThreads, 1) wgrad_tc_kernel(const __grid_co
                     return false;
                 const int y = (r >= w.r0 && r < w.r0 + w.nrows) ? r : L;
                 const int copies = s < (uint32_t)kWgDzMirror ? 2 : 1;
-                tc::mbar_arrive_expect_tx(&dfull[s], copies * kWgDzBytes);
+                tc::mbar_arrive_expect_tx(&dfull[s], (uint32_t)copies * 2 * box);
                 for (int k = 0; k < copies; ++k) {
                     uint8_t *dst = wg_smem + kWgDz0 + (s + k * kWgDzSlots) * kWgDzBytes;
                     tc::tma_load_4d(dst, &p.hi, 0, w.x0 + 1, y, (int)w.c, &dfull[s]);
@@ -1945,7 +1559,7 @@ __global__ void __launch_bounds__(kWgThreads, 1) wgrad_tc_kernel(const __grid_co
             const uint32_t a_lo0 = (uint32_t)a_desc0, a_hi = (uint32_t)(a_desc0 >> 32);
             const uint32_t b_lo0 = (uint32_t)b_desc0, b_hi = (uint32_t)(b_desc0 >> 32);
             uint32_t ma = 0, md = 0, dready = 0;  // input rows consumed; first gradient row of the run; gradient rows landed
-            bool first = true;
+            uint32_t seen = 0;  // input rows so far: row `seen` goes to set seen % sets
             for (int64_t lin = begin; lin < end && ok;) {
                 const RingUnit w = wg_run(p, lin, end);
                 lin += w.nrows;
@@ -1964,9 +1578,11 @@ __global__ void __launch_bounds__(kWgThreads, 1) wgrad_tc_kernel(const __grid_co
                     const uint32_t b_row = b_lo0 + ((((md + (uint32_t)a) % kWgDzSlots) * kWgDzBytes) >> 4);
 #pragma unroll
                     for (int ks = 0; ks < kTileM / 16; ++ks)  // 16 pixels = two 512-byte atoms
-                        tc::mma_bf16_w(tmem, a_row + (uint32_t)(ks * 64), a_hi, b_row + (uint32_t)(ks * 64), b_hi, idesc,
-                                       (first && ks == 0) ? 0u : 1u);
-                    first = false;
+                        if (FULL || 16 * ks < p.tw)
+                            tc::mma_bf16_w(tmem + 256 * (seen % kWgSets<FULL>), a_row + (uint32_t)(ks * 64), a_hi,
+                                           b_row + (uint32_t)(ks * 64), b_hi, idesc,
+                                           (seen < kWgSets<FULL> && ks == 0) ? 0u : 1u);
+                    ++seen;
                     tc::mma_commit(&aempty[as]);
                     ++ma;
                     tc::mma_commit(&dempty[(md + (uint32_t)a) % kWgDzSlots]);  // gradient row r0 - 2 + a: last use
@@ -2006,6 +1622,7 @@ __global__ void __launch_bounds__(kWgThreads, 1) wgrad_tc_kernel(const __grid_co
             const uint8_t *dz = wg_smem + kWgDz0 + ds * kWgDzBytes;
 #pragma unroll
             for (int it = 0; it < 4; ++it) {
+                if (!FULL && 32 * q >= p.tw) break;  // no pixels of this warp's are staged
                 const int px = 32 * q + 8 * it + p8;
                 const uint32_t at = px * 64 + ((g ^ ((px >> 1) & 3)) << 4);
                 const uint4 h = *reinterpret_cast<const uint4 *>(dz + at);
@@ -2045,6 +1662,13 @@ __global__ void __launch_bounds__(kWgThreads, 1) wgrad_tc_kernel(const __grid_co
                 const uint32_t ta = tmem + (uint32_t)(64 * b + 16 * oh) + ((uint32_t)(quad * 32) << 16);
                 tc::tmem_ld16(ta, vh);
                 tc::tmem_ld16(ta + (uint32_t)kCh, vl);
+                if constexpr (!FULL) {  // a CTA walks three input rows at least: both sets were written
+                    float uh[16], ul[16];
+                    tc::tmem_ld16(ta + 256u, uh);
+                    tc::tmem_ld16(ta + 256u + (uint32_t)kCh, ul);
+#pragma unroll
+                    for (int j = 0; j < 16; ++j) vh[j] += uh[j], vl[j] += ul[j];
+                }
                 if (quad < 3)
 #pragma unroll
                     for (int j = 0; j < 16; ++j)
@@ -2060,7 +1684,7 @@ __global__ void __launch_bounds__(kWgThreads, 1) wgrad_tc_kernel(const __grid_co
     __syncthreads();
     if (warp == 1) {
         tc::fence_after_sync();
-        tc::tmem_dealloc(tmem, kWgTmemCols);
+        tc::tmem_dealloc(tmem, kCols);
     }
 }
 
@@ -2307,11 +1931,9 @@ int check_chains(int64_t L, int64_t C)
 }
 
 // Work layout: training keeps z1 z2 z3 (FP32), a1 a2 a3 (bfloat16) and two
-// FP32 gradient buffers, then the weight-gradient partials; inference keeps
-// a1 and a2 (bfloat16; where a3 is written at all it reuses a1's buffer).
-// Both end with room for the 9 FP32 planes P of layer 4's tap projections
-// (for L a multiple of 128 it holds the row partials of z4 instead, 9 values
-// per row and 8-pixel block column).
+// FP32 gradient buffers, then the weight-gradient partials; inference keeps a2
+// alone (bfloat16).  Both end with the row partials of z4, 9 values per row and
+// 8-pixel block column.
 struct NetWork {
     float *z1, *z2, *z3, *da, *db, *partial, *P, *tz;
     __nv_bfloat16 *a1, *a2, *a3, *ta, *gb1, *gb2;  // gb: bfloat16 gradients with halo columns (training)
@@ -2340,18 +1962,15 @@ NetWork net_layout(int64_t L, int64_t C, int train, char *base)
         w.a3 = (__nv_bfloat16 *)take(apx * 2);
         w.da = (float *)take(pix * 4); w.db = (float *)take(pix * 4);
         w.gb1 = (__nv_bfloat16 *)take(apx * 2); w.gb2 = (__nv_bfloat16 *)take(apx * 2);
-        if (L % kTileM == 0) {
-            w.gr1 = (__nv_bfloat16 *)take(apx * 2); w.gr2 = (__nv_bfloat16 *)take(apx * 2);
-        }
+        w.gr1 = (__nv_bfloat16 *)take(apx * 2); w.gr2 = (__nv_bfloat16 *)take(apx * 2);
         DeviceInfo info{152};
         device_info(&info);
         w.n_cta = (int64_t)info.sm_count * kWgradCtasPerSm;
         w.partial = (float *)take((size_t)w.n_cta * (kN2 + kCh) * sizeof(float));
     } else {
-        w.a1 = (__nv_bfloat16 *)take(apx * 2); w.a2 = (__nv_bfloat16 *)take(apx * 2);
-        w.a3 = w.a1;
+        w.a2 = (__nv_bfloat16 *)take(apx * 2);
     }
-    w.P = (float *)take((size_t)C * L * L * 9 * sizeof(float));
+    w.P = (float *)take((size_t)C * L * (L / kBlk) * 9 * sizeof(float));
     w.tz = (float *)take((size_t)kPatterns * kCh * sizeof(float));
     w.ta = (__nv_bfloat16 *)take((size_t)kPatterns * kCh * 2);
     w.bytes = o;
@@ -2367,7 +1986,11 @@ NetWork net_layout(int64_t L, int64_t C, int train, char *base)
 constexpr int kBandRows[4] = {30, 28, 26, 3};  // a1, a2, a3 rows; logit block rows
 constexpr int kBandLead[3] = {11, 10, 9};
 
-bool band_supported(int64_t L) { return L % kTileM == 0 && L >= 128; }
+static_assert(kBandRows[0] <= 32, "the rows of a band are distinct for every L");
+
+// Row segments of side L: ceil(L / 128) of a width that is a multiple of 32.
+int seg_count(int L) { return (L + kTileM - 1) / kTileM; }
+int seg_width(int L) { return (L / 32 + seg_count(L) - 1) / seg_count(L) * 32; }
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *,
                                   const cuuint64_t *, const cuuint32_t *, const cuuint32_t *, CUtensorMapInterleave,
@@ -2392,7 +2015,7 @@ EncodeTiledFn encode_tiled_fn()
 
 // The ring kernel's view of an activation buffer, one tensor map per channel
 // group g: (8 channels at 8g, L + 2 pixels of 64 bytes, L rows, C chains),
-// boxes of 8 x 130 x 1 x 1.
+// boxes of 8 x tw + 2 x 1 x 1.
 bool encode_rows(CUtensorMap (&m)[kGroups], const __nv_bfloat16 *a, int L, int64_t C)
 {
     EncodeTiledFn fn = encode_tiled_fn();
@@ -2400,7 +2023,7 @@ bool encode_rows(CUtensorMap (&m)[kGroups], const __nv_bfloat16 *a, int L, int64
     const cuuint64_t dims[4] = {8, (cuuint64_t)L + 2, (cuuint64_t)L, (cuuint64_t)C};
     const cuuint64_t strides[3] = {(cuuint64_t)kCh * 2, (cuuint64_t)(L + 2) * kCh * 2,
                                    (cuuint64_t)L * (L + 2) * kCh * 2};
-    const cuuint32_t box[4] = {8, kTileM + 2, 1, 1};
+    const cuuint32_t box[4] = {8, (cuuint32_t)seg_width(L) + 2, 1, 1};
     const cuuint32_t estr[4] = {1, 1, 1, 1};
     for (int g = 0; g < kGroups; ++g)
         if (fn(&m[g], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, (void *)(a + 8 * g), dims, strides, box, estr,
@@ -2408,6 +2031,24 @@ bool encode_rows(CUtensorMap (&m)[kGroups], const __nv_bfloat16 *a, int L, int64
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
             return false;
     return true;
+}
+
+template <bool PROJ, bool BWD, bool FUSED, bool FULL>
+void launch_ring_full(const RingConv &p, unsigned grid, cudaStream_t s)
+{
+    constexpr uint32_t smem = RingLayout<PROJ, BWD || (!PROJ && !FUSED)>::bytes;
+    auto kernel = conv32_ring_kernel<PROJ, BWD, FUSED, FULL>;
+    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    // the fused first conv: shared memory for two CTAs, the rest as L1 for the layer-1 table
+    if (FUSED) cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, 86);
+    kernel<<<grid, ring_threads<PROJ, FUSED>(), smem, s>>>(p);
+}
+
+template <bool PROJ, bool BWD, bool FUSED>
+void launch_ring(const RingConv &p, unsigned grid, cudaStream_t s)
+{
+    if (p.bd.L % kTileM == 0) launch_ring_full<PROJ, BWD, FUSED, true>(p, grid, s);
+    else launch_ring_full<PROJ, BWD, FUSED, false>(p, grid, s);
 }
 
 // The data gradient of a 32 -> 32 layer (weights at w_off) on the tensor
@@ -2434,19 +2075,17 @@ int launch_ring_bwd(int L, int64_t C, const float *params, int w_off, const __nv
     p.bd.rows = L;
     p.bd.lead = 0;
     p.bd.flip = nullptr;
-    p.segs = L / kTileM;
+    p.segs = seg_count(L);
+    p.tw = seg_width(L);
     p.units_per_col = (L + kUnitRows - 1) / kUnitRows;
     p.units = C * p.segs * p.units_per_col;
     const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>(p.units, 2 * info.sm_count));
-    cudaFuncSetAttribute(conv32_ring_kernel<false, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)RingLayout<false, true>::bytes);
-    conv32_ring_kernel<false, true, false><<<grid, kRingThreads, RingLayout<false, true>::bytes, s>>>(p);
+    launch_ring<false, true, false>(p, grid, s);
     cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? ISING_OK : nfail(ISING_ECUDA, cudaGetErrorString(e));
 }
 
-// The weight gradients of a 32 -> 32 layer on the tensor cores (L a multiple
-// of 128): the layer's input a (bfloat16, halo columns) and its gradient as
+// The weight gradients of a 32 -> 32 layer on the tensor cores: the layer's input a (bfloat16, halo columns) and its gradient as
 // hi = bf16(dz), lo = bf16(dz - hi) (same layout); one CTA per SM writes its
 // partial sums into partial[cta][kN2 + kCh].  Returns the number of CTAs.
 int launch_wgrad_tc(int L, int64_t C, const __nv_bfloat16 *a, const __nv_bfloat16 *hi, const __nv_bfloat16 *lo,
@@ -2457,26 +2096,29 @@ int launch_wgrad_tc(int L, int64_t C, const __nv_bfloat16 *a, const __nv_bfloat1
     DeviceInfo info{152};
     device_info(&info);
     WgradTc p{};
-    const cuuint64_t dims[4] = {(cuuint64_t)kCh, (cuuint64_t)L + 2, (cuuint64_t)L, (cuuint64_t)C};
     const cuuint64_t strides[3] = {(cuuint64_t)kCh * 2, (cuuint64_t)(L + 2) * kCh * 2,
                                    (cuuint64_t)L * (L + 2) * kCh * 2};
-    const cuuint32_t box[4] = {kCh, kTileM, 1, 1};  // whole pixels, 64 bytes: the 64-byte swizzle
+    const cuuint32_t box[4] = {kCh, (cuuint32_t)seg_width(L), 1, 1};  // whole pixels, 64 bytes: the 64-byte swizzle
     const cuuint32_t estr[4] = {1, 1, 1, 1};
     const __nv_bfloat16 *src[3] = {a, hi, lo};
     CUtensorMap *maps[3] = {&p.act, &p.hi, &p.lo};
-    for (int t = 0; t < 3; ++t)
+    for (int t = 0; t < 3; ++t) {
+        const cuuint64_t dims[4] = {(cuuint64_t)kCh, (cuuint64_t)L + (t == 0 ? 2 : 1), (cuuint64_t)L, (cuuint64_t)C};
         if (fn(maps[t], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, (void *)src[t], dims, strides, box, estr,
                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
             return nfail(ISING_ECUDA, "cuTensorMapEncodeTiled failed");
+    }
     p.partial = partial;
     p.L = L;
-    p.segs = L / kTileM;
+    p.segs = seg_count(L);
+    p.tw = seg_width(L);
     p.lines = C * p.segs * L;
     // every CTA gets at least one row, so every partial row is written
     const int64_t grid = std::max<int64_t>(1, std::min<int64_t>({(int64_t)info.sm_count, max_ctas, p.lines}));
-    cudaFuncSetAttribute(wgrad_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kWgSmem);
-    wgrad_tc_kernel<<<(unsigned)grid, kWgThreads, kWgSmem, s>>>(p);
+    auto kernel = L % kTileM == 0 ? wgrad_tc_kernel<true> : wgrad_tc_kernel<false>;
+    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kWgSmem);
+    kernel<<<(unsigned)grid, kWgThreads, kWgSmem, s>>>(p);
     *n_cta = grid;
     cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? ISING_OK : nfail(ISING_ECUDA, cudaGetErrorString(e));
@@ -2503,82 +2145,46 @@ int launch_forward(const Chains &ch, int64_t C, const int32_t *flip, bool band, 
         const unsigned gx = (unsigned)std::max<int64_t>(1, std::min<int64_t>(tiles, want));
         const unsigned gy = (unsigned)std::max<int64_t>(1, std::min<int64_t>({C, 65535, (want + gx - 1) / gx}));
         l1_table_kernel<<<kPatterns * kCh / 256, 256, 0, s>>>(params, w.tz, w.ta);
-        // an inference pass of the row-ring kernels forms layer 1 inside the first conv
-        if (train || L % kTileM != 0)
-            l1_kernel<<<dim3(gx, gy), kL1Threads, 0, s>>>(ch, bd[0], flip, w.ta, w.tz, train ? w.z1 : nullptr,
-                                                           w.a1);
+        // an inference pass forms layer 1 inside the first conv
+        if (train) l1_kernel<<<dim3(gx, gy), kL1Threads, 0, s>>>(ch, bd[0], flip, w.ta, w.tz, w.z1, w.a1);
     }
     const int off[2][2] = {{kOffW2, kOffB2}, {kOffW3, kOffB3}};
     const __nv_bfloat16 *ins[2] = {w.a1, w.a2};
     float *zs[2] = {train ? w.z2 : nullptr, train ? w.z3 : nullptr};
-    if (L % kTileM == 0) {
-        // row-ring kernels; the second one also projects onto layer 4's taps
-        cudaFuncSetAttribute(conv32_ring_kernel<false, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)RingLayout<false>::bytes);
-        cudaFuncSetAttribute(conv32_ring_kernel<false, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)RingLayout<false, true>::bytes);
-        cudaFuncSetAttribute(conv32_ring_kernel<true, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)RingLayout<true>::bytes);
-        // shared memory for two CTAs of the first conv, the rest as L1 for the layer-1 table
-        cudaFuncSetAttribute(conv32_ring_kernel<false, false, true>, cudaFuncAttributePreferredSharedMemoryCarveout,
-                             86);
-        __nv_bfloat16 *outs[2] = {w.a2, train ? w.a3 : nullptr};
-        for (int l = 0; l < 2; ++l) {
-            RingConv p{};
-            const bool fused = l == 0 && !train;
-            if (!fused && !encode_rows(p.tmap, ins[l], L, C)) return nfail(ISING_ECUDA, "cuTensorMapEncodeTiled failed");
-            p.ch = ch;
-            p.flip = flip;
-            p.ta = w.ta;
-            p.a_in = ins[l];
-            p.a_out = outs[l];
-            p.z_out = zs[l];
-            p.P = w.P;
-            p.params = params;
-            p.w_off = off[l][0];
-            p.b_off = off[l][1];
-            p.bd = bd[l + 1];
-            p.segs = L / kTileM;
-            p.units_per_col = (bd[l + 1].rows + kUnitRows - 1) / kUnitRows;
-            p.units = C * p.segs * p.units_per_col;
-            p.withhold = withhold && l == 0;
-            const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>(p.units, 2 * info.sm_count));
-            if (fused)
-                conv32_ring_kernel<false, false, true><<<grid, ring_threads<false, true>(), RingLayout<false>::bytes, s>>>(p);
-            else if (l == 0)
-                conv32_ring_kernel<false, false, false><<<grid, kRingThreads, RingLayout<false, true>::bytes, s>>>(p);
-            else
-                conv32_ring_kernel<true, false, false><<<grid, ring_threads<true, false>(), RingLayout<true>::bytes, s>>>(p);
-        }
-    } else {
-        cudaFuncSetAttribute(conv32_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kConvSmem);
-        __nv_bfloat16 *outs[2] = {w.a2, w.a3};  // inference: a3 reuses a1's buffer
-        for (int l = 0; l < 2; ++l) {
-            ConvTc p;
-            p.a_in = ins[l];
-            p.a_out = outs[l];
-            p.z_out = zs[l];
-            p.params = params;
-            p.w_off = off[l][0];
-            p.b_off = off[l][1];
-            p.bd = bd[l + 1];
-            p.tiles = C * (int64_t)bd[l + 1].rows * L / kTileM;
-            const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>(p.tiles, info.sm_count));
-            conv32_tc_kernel<<<grid, kConvThreads, kConvSmem, s>>>(p);
-        }
-        l4_project_kernel<<<grid1d(C * (int64_t)bd[2].rows * L, kThreads), kThreads, 0, s>>>(bd[2], params, w.a3,
-                                                                                             w.P);
+    // the second conv also projects onto layer 4's taps
+    __nv_bfloat16 *outs[2] = {w.a2, train ? w.a3 : nullptr};
+    for (int l = 0; l < 2; ++l) {
+        RingConv p{};
+        const bool fused = l == 0 && !train;
+        if (!fused && !encode_rows(p.tmap, ins[l], L, C)) return nfail(ISING_ECUDA, "cuTensorMapEncodeTiled failed");
+        p.ch = ch;
+        p.flip = flip;
+        p.ta = w.ta;
+        p.a_in = ins[l];
+        p.a_out = outs[l];
+        p.z_out = zs[l];
+        p.P = w.P;
+        p.params = params;
+        p.w_off = off[l][0];
+        p.b_off = off[l][1];
+        p.bd = bd[l + 1];
+        p.segs = seg_count(L);
+        p.tw = seg_width(L);
+        p.units_per_col = (bd[l + 1].rows + kUnitRows - 1) / kUnitRows;
+        p.units = C * p.segs * p.units_per_col;
+        p.withhold = withhold && l == 0;
+        const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>(p.units, 2 * info.sm_count));
+        if (fused)
+            launch_ring<false, false, true>(p, grid, s);
+        else if (l == 0)
+            launch_ring<false, false, false>(p, grid, s);
+        else
+            launch_ring<true, false, false>(p, grid, s);
     }
     const int brows = band ? kBandRows[3] : L / kBlk;
-    if (L % kTileM == 0) {
-        // the projecting ring kernel left row partials of z4 in w.P
-        pool_rows_kernel<<<grid1d(C * brows * (L / kBlk), kThreads), kThreads, 0, s>>>(
-            L, C, brows, band ? flip : nullptr, params, w.P, logits);
-    } else {
-        const int64_t warps = C * brows * (L / kBlk / 4);
-        pool_kernel<<<grid1d(warps * 32, kThreads), kThreads, 0, s>>>(L, C, brows, band ? flip : nullptr, params, w.P,
-                                                                      logits);
-    }
+    // the projecting ring kernel left row partials of z4 in w.P
+    pool_rows_kernel<<<grid1d(C * brows * (L / kBlk), kThreads), kThreads, 0, s>>>(L, C, brows, band ? flip : nullptr,
+                                                                                  params, w.P, logits);
     cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? ISING_OK : nfail(ISING_ECUDA, cudaGetErrorString(e));
 }
@@ -2640,7 +2246,6 @@ ISING_API int ising_net_forward_flipped(int64_t L, int64_t C, const void *black_
     if (logits_x_dev == logits_dev) return nfail(ISING_EINVAL, "logits_x and logits must differ");
     cudaStream_t s = (cudaStream_t)stream;
     Chains ch{(const uint64_t *)black_dev, (const uint64_t *)white_dev, (int)L, (int)(L / 32)};
-    if (!band_supported(L)) return launch_forward(ch, C, flip_block_dev, false, params_dev, logits_dev, w, 0, s);
     cudaError_t e = cudaMemcpyAsync(logits_dev, logits_x_dev, lbytes, cudaMemcpyDeviceToDevice, s);
     if (e != cudaSuccess) return nfail(ISING_ECUDA, cudaGetErrorString(e));
     return launch_forward(ch, C, flip_block_dev, true, params_dev, logits_dev, w, 0, s);
@@ -2695,12 +2300,6 @@ ISING_API int ising_net_backward(int64_t L, int64_t C, const void *black_dev, co
     cudaStream_t s = (cudaStream_t)stream;
     Chains ch{(const uint64_t *)black_dev, (const uint64_t *)white_dev, (int)L, (int)(L / 32)};
     const int64_t npix = C * L * L;
-    const unsigned g = grid1d(npix, kThreads);
-    const size_t smem = (size_t)kN2 * sizeof(float);
-    const unsigned gw = (unsigned)w.n_cta;
-    cudaFuncSetAttribute(conv32_bwd_data_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    const size_t sm32 = (size_t)((kTy + 2) * (kTx + 2) * kCh + kTy * kTx * kCh) * sizeof(float);
-    cudaFuncSetAttribute(wgrad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm32);
     auto reduce = [&](int ne, int nw, int w_off, int b_off, int64_t n_cta) {
         reduce_partials_kernel<<<(unsigned)((ne + 31) / 32), 32 * kReduceWarps, 0, s>>>(w.partial, n_cta, ne, nw,
                                                                                        grad_dev, w_off, b_off);
@@ -2712,38 +2311,24 @@ ISING_API int ising_net_backward(int64_t L, int64_t C, const void *black_dev, co
     const int64_t n_thin = std::min<int64_t>(w.n_cta, 2 * (int64_t)info.sm_count);
     wgrad_thin_kernel<true><<<(unsigned)n_thin, 32 * kThinWarps, 0, s>>>(ch, C, nullptr, w.a3, dlogits_dev, w.partial);
     reduce(kN1 + 1, kN1, kOffW4, kOffB4, n_thin);
-    // for L a multiple of 128 the data and weight gradients of the 32 -> 32
-    // layers run on the tensor cores; their gradients are then also kept as
-    // bfloat16 parts (gb: the rounding, gr: the rounding of the remainder)
-    const bool ring = L % kTileM == 0;
-    l4_bwd_data_kernel<<<grid1d(4 * npix, kThreads), kThreads, 0, s>>>((int)L, C, params_dev, dlogits_dev, w.z3,
-                                                                     w.da, ring ? w.gb1 : nullptr,
-                                                                     ring ? w.gr1 : nullptr);  // dz3
+    // the data and weight gradients of the 32 -> 32 layers run on the tensor
+    // cores; their gradients are then also kept as bfloat16 parts (gb: the
+    // rounding, gr: the rounding of the remainder)
+    l4_bwd_data_kernel<<<grid1d(4 * npix, kThreads), kThreads, 0, s>>>((int)L, C, params_dev, dlogits_dev, w.z3, w.da,
+                                                                     w.gb1, w.gr1);  // dz3
     // layer 3
     int64_t n_tc = 0;
-    if (ring) {
-        rc = launch_wgrad_tc((int)L, C, w.a2, w.gb1, w.gr1, w.partial, w.n_cta, s, &n_tc);
-        if (rc) return rc;
-        reduce(kN2 + kCh, kN2, kOffW3, kOffB3, n_tc);
-        rc = launch_ring_bwd((int)L, C, params_dev, kOffW3, w.gb1, w.z2, w.db, w.gb2, w.gr2, s);  // dz2
-        if (rc) return rc;
-    } else {
-        wgrad_kernel<<<gw, 256, sm32, s>>>(ch, C, w.a2, w.da, w.partial);
-        reduce(kN2 + kCh, kN2, kOffW3, kOffB3, w.n_cta);
-        conv32_bwd_data_kernel<<<g, kThreads, smem, s>>>((int)L, C, params_dev, kOffW3, w.da, w.z2, w.db);  // dz2
-    }
+    rc = launch_wgrad_tc((int)L, C, w.a2, w.gb1, w.gr1, w.partial, w.n_cta, s, &n_tc);
+    if (rc) return rc;
+    reduce(kN2 + kCh, kN2, kOffW3, kOffB3, n_tc);
+    rc = launch_ring_bwd((int)L, C, params_dev, kOffW3, w.gb1, w.z2, w.db, w.gb2, w.gr2, s);  // dz2
+    if (rc) return rc;
     // layer 2
-    if (ring) {
-        rc = launch_wgrad_tc((int)L, C, w.a1, w.gb2, w.gr2, w.partial, w.n_cta, s, &n_tc);
-        if (rc) return rc;
-        reduce(kN2 + kCh, kN2, kOffW2, kOffB2, n_tc);
-        rc = launch_ring_bwd((int)L, C, params_dev, kOffW2, w.gb2, w.z1, w.da, nullptr, nullptr, s);  // dz1
-        if (rc) return rc;
-    } else {
-        wgrad_kernel<<<gw, 256, sm32, s>>>(ch, C, w.a1, w.db, w.partial);
-        reduce(kN2 + kCh, kN2, kOffW2, kOffB2, w.n_cta);
-        conv32_bwd_data_kernel<<<g, kThreads, smem, s>>>((int)L, C, params_dev, kOffW2, w.db, w.z1, w.da);  // dz1
-    }
+    rc = launch_wgrad_tc((int)L, C, w.a1, w.gb2, w.gr2, w.partial, w.n_cta, s, &n_tc);
+    if (rc) return rc;
+    reduce(kN2 + kCh, kN2, kOffW2, kOffB2, n_tc);
+    rc = launch_ring_bwd((int)L, C, params_dev, kOffW2, w.gb2, w.z1, w.da, nullptr, nullptr, s);  // dz1
+    if (rc) return rc;
     // layer 1
     wgrad_thin_kernel<false><<<(unsigned)n_thin, 32 * kThinWarps, 0, s>>>(ch, C, w.da, nullptr, nullptr, w.partial);
     reduce(kN1 + kCh, kN1, kOffW1, kOffB1, n_thin);
