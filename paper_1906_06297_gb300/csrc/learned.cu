@@ -395,8 +395,10 @@ __device__ int g_tc_error;  // set to 1 when a tensor-core wait gives up
 //   Z[m][o] = sum over taps k and input channels i of A_k[m][i] W[o][i][k],
 // M = 128 pixels, N = 32 output channels, K = 9 taps x 32 channels (tcgen05.mma
 // kind::f16, BF16 operands, FP32 accumulator in tensor memory), fed from a ring
-// of staged input rows.  A work unit is up to kUnitRows consecutive output rows
-// of one (chain, segment); it stages its rows r0 - 1 .. r0 + n once each, as a
+// of staged input rows.  Every CTA takes one contiguous range of the (chain,
+// segment, row) lines, ranges differing by at most one line, and walks it as runs
+// of consecutive rows of one (chain, segment); a run of n rows stages its rows
+// r0 - 1 .. r0 + n once each, as a
 // halo row of tw + 2 pixels (x0 - 1 .. x0 + tw, periodic) in 4 channel-group
 // planes of kRingPlane bytes, so the operand of tap (dy, dx) is the staged row
 // y + dy offset by (1 + dx) x 16 bytes (no-swizzle K-major, LBO = kRingPlane,
@@ -417,7 +419,7 @@ __device__ int g_tc_error;  // set to 1 when a tensor-core wait gives up
 //           the pattern's row of the table (l1_table_kernel); the lanes then
 //           fence the async proxy and lane 0 arrives on full[slot]: a1 never
 //           goes through global memory;
-//   warp 1: lane 0 issues the MMAs row-stationary: each staged row, once
+//   warp 1: issues the MMAs row-stationary: each staged row, once
 //           per (dx, K half), times the weights of the three dy taps stacked
 //           along N = 96, into the accumulator blocks of the three output
 //           rows it feeds (a ring of kAcc blocks in descending row order, so
@@ -426,7 +428,9 @@ __device__ int g_tc_error;  // set to 1 when a tensor-core wait gives up
 //           (the tensor core spends ~45 cycles on an N = 32 MMA and ~56 on an
 //           N = 96 one).  It then commits to empty[slot] of the row (no later
 //           MMA reads it) and to accf[block] of the output row that row
-//           completed;
+//           completed.  The whole warp runs this and one elected lane issues: the
+//           descriptors then stay in uniform registers, where a branch for lane 0
+//           moved each one over (full forward of 1024 chains 1281 -> 1192 us);
 //   warps 2-9: epilogue, warp w on TMEM lanes 32 (w % 4) .. + 31 (its 32
 //           pixels) and columns 16 h .. 16 h + 15, h = (w - 2) / 4 (its 16
 //           channels): loads them, sets them to the bias (every MMA
@@ -443,7 +447,7 @@ __device__ int g_tc_error;  // set to 1 when a tensor-core wait gives up
 // PROJ (the last 32-channel layer): layer 4's channel contraction is done
 // here, on the tensor cores, as P[m][k] = sum_i a[m][i] W4[i][k] for the 9
 // taps k (N padded to 16): the epilogue stages the tile's a in shared memory
-// (a3full), lane 0 of a warp of its own (warp 10) multiplies it by W4^T into
+// (a3full), a warp of its own (warp 10) multiplies it by W4^T into
 // 16 more TMEM columns (pfull, a3empty), and four more warps (11-14, one per
 // TMEM lane quadrant) read P out (pempty) and reduce it to row partials of z4
 // (see pool_rows_kernel).  Then a3 itself need not reach global memory (it
@@ -465,10 +469,12 @@ __device__ int g_tc_error;  // set to 1 when a tensor-core wait gives up
 // to t + 1 only, so no wait can close a cycle.
 constexpr int kRing = 8;        // staged rows (a power of two)
 constexpr int kAcc = 7;         // accumulator blocks of 32 TMEM columns, one per output row in flight
-// output rows per work unit: each unit stages 2 halo rows and restarts the
-// pipeline; 32 rows per unit measured 1.66 ms per full forward of 1024
-// chains of 128^2 against 1.73 (16), 1.72 (64), 1.75 (128), 1.89 (24)
-constexpr int kUnitRows = 32;
+// Output rows of a CTA's range from which the grid is filled.  (Work units of 32
+// rows dealt out in turn stage 6% more halo rows and leave a last wave: of 1024
+// chains of 128^2 the CTAs got 13 or 14 units, of 64 chains 256 of 304 CTAs one.
+// Training step of 64 chains 767 -> 731 us, forward of 256 chains of 96^2 343 -> 302;
+// of 1024 chains of 128^2 unchanged.)
+constexpr int kMinRange = 4;
 constexpr int kEpiWarps = 8;
 constexpr int kRingThreads = 64 + 32 * kEpiWarps;
 // one more warp: the second loader of the fused first conv, or the issuer of
@@ -513,7 +519,7 @@ struct RingLayout {
 };
 constexpr uint32_t kRingTmemCols = 256;  // 7 x 32 accumulator + 2 x 16 projection columns
 constexpr int kStackN = 3 * kCh;         // the weights of the three dy taps stacked along N
-// accumulator block of output row t (counted over a CTA's units, 32-bit: the
+// accumulator block of output row t (counted over a CTA's runs, 32-bit: the
 // MMA thread does this arithmetic for every row): descending, so that rows
 // t + 1, t, t - 1 sit in consecutive blocks; and the parity of its use
 __device__ __forceinline__ int ring_blk(uint32_t t) { return kAcc - 1 - (int)(t % (uint32_t)kAcc); }
@@ -603,8 +609,7 @@ struct RingConv {
     int w_off, b_off;
     Band bd;
     int segs, tw;       // row segments and their width
-    int units_per_col;  // ceil(bd.rows / kUnitRows)
-    int64_t units;      // C segs units_per_col
+    int64_t lines;      // C segs bd.rows
     int withhold;       // self-test: never signal the first accumulator, so its wait runs out
 };
 
@@ -616,17 +621,16 @@ struct RingUnit {
 // FULL: every segment has 128 pixels (L a multiple of 128), which the compiler
 // then knows (without it the forward of 1024 chains of 128^2 takes 3.6% longer).
 template <bool FULL>
-__device__ __forceinline__ RingUnit ring_unit(const RingConv &p, int64_t u)
+__device__ __forceinline__ RingUnit ring_run(const RingConv &p, int64_t lin, int64_t end)
 {
     RingUnit w;
-    const int64_t col = u / p.units_per_col;
-    const int rb = (int)(u - col * p.units_per_col);
-    w.c = col / p.segs;
+    const int64_t col = lin / p.bd.rows;
+    w.r0 = (int)(lin - col * p.bd.rows);
+    w.nrows = (int)min((int64_t)(p.bd.rows - w.r0), end - lin);
     const int tw = FULL ? kTileM : p.tw;
+    w.c = col / p.segs;
     w.x0 = (int)(col - w.c * p.segs) * tw;
     w.width = FULL ? kTileM : min(tw, p.bd.L - w.x0);
-    w.r0 = rb * kUnitRows;
-    w.nrows = min(kUnitRows, p.bd.rows - w.r0);
     return w;
 }
 
@@ -695,8 +699,9 @@ __global__ void __launch_bounds__(ring_threads<PROJ, FUSED>(), 2) conv32_ring_ke
     uint64_t *a3full = acce + kAcc, *a3empty = a3full + 2, *pfull = a3empty + 2, *pempty = pfull + 2;
     uint64_t *drain = pempty + 2, *pdrain = drain + 1;
     uint32_t *tslot = reinterpret_cast<uint32_t *>(pdrain + 1);
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
     const int L = p.bd.L;
+    const int64_t begin = blockIdx.x * p.lines / gridDim.x, end = (blockIdx.x + 1) * p.lines / gridDim.x;
 
     if (warp == 1) tc::tmem_alloc(tslot, kRingTmemCols);
     if (tid == 0) {
@@ -772,11 +777,12 @@ __global__ void __launch_bounds__(ring_threads<PROJ, FUSED>(), 2) conv32_ring_ke
         // warp building rows is a chain of shuffles, table loads and stores
         // that the MMA thread outpaces)
         const uint32_t parity = warp == 0 ? 0u : 1u;
-        uint32_t n = 0;  // ring index of the unit's first row
+        uint32_t n = 0;  // ring index of the run's first row
         const uint4 *ta = reinterpret_cast<const uint4 *>(p.ta);
         const int nw = L / 32;
-        for (int64_t u = blockIdx.x; u < p.units && ok; u += gridDim.x) {
-            const RingUnit w = ring_unit<FULL>(p, u);
+        for (int64_t lin = begin; lin < end && ok;) {
+            const RingUnit w = ring_run<FULL>(p, lin, end);
+            lin += w.nrows;
             const int fb = p.flip ? p.flip[w.c] : -1;
             // lane 6 d + q (d < 3, q < 6): chunk x0 / 32 - 1 + q (periodic) of spin row y - 1 + d
             auto fetch = [&](int j) {
@@ -788,7 +794,7 @@ __global__ void __launch_bounds__(ring_threads<PROJ, FUSED>(), 2) conv32_ring_ke
                 }
                 return k;
             };
-            // this warp's rows j of the unit: ring index n + j + 1 of its parity
+            // this warp's rows j of the run: ring index n + j + 1 of its parity
             const int j0 = -1 + (int)((parity - n) & 1u);
             ChunkWords next = j0 <= w.nrows ? fetch(j0) : ChunkWords{0, 0, 0, 0};
             for (int j = j0; j <= w.nrows; j += 2) {
@@ -833,8 +839,9 @@ __global__ void __launch_bounds__(ring_threads<PROJ, FUSED>(), 2) conv32_ring_ke
         // loader
         if (lane == 0) {
             uint32_t n = 0;  // rows staged so far
-            for (int64_t u = blockIdx.x; u < p.units && ok; u += gridDim.x) {
-                const RingUnit w = ring_unit<FULL>(p, u);
+            for (int64_t lin = begin; lin < end && ok;) {
+                const RingUnit w = ring_run<FULL>(p, lin, end);
+                lin += w.nrows;
                 for (int j = -1; j <= w.nrows; ++j, ++n) {
                     const uint32_t s = n & (kRing - 1);
                     if (n >= kRing && !tc::mbar_wait(&empty[s], ((n / kRing) + 1) & 1, kWaitCycles)) {
@@ -857,7 +864,7 @@ __global__ void __launch_bounds__(ring_threads<PROJ, FUSED>(), 2) conv32_ring_ke
         }
         __syncwarp();
     } else if (warp == 1) {
-        if (lane == 0) {
+        {
             // N = 32, 64 or 96: one, two or three accumulator blocks per MMA
             // (the N field holds N / 8 from bit 17)
             const uint32_t idesc0 = tc::idesc_bf16_f32(kTileM, 0);
@@ -868,29 +875,30 @@ __global__ void __launch_bounds__(ring_threads<PROJ, FUSED>(), 2) conv32_ring_ke
             const uint64_t b_desc0 = tc::smem_desc(b_u32, kStackN * 16, 128);
             const uint32_t a_lo0 = (uint32_t)a_desc0, a_hi = (uint32_t)(a_desc0 >> 32);
             const uint32_t b_lo0 = (uint32_t)b_desc0, b_hi = (uint32_t)(b_desc0 >> 32);
-            // Row-stationary: staged input row i of a unit is multiplied once,
+            // Row-stationary: staged input row i of a run is multiplied once,
             // for each (dx, K half), by the three dy taps stacked along N, into
             // the accumulator blocks of the output rows it feeds, i + 1 (dy =
-            // -1), i and i - 1 (dy = +1), those of them inside the unit.  Output
-            // row t (counted over the units) has block kAcc - 1 - t % kAcc, so
+            // -1), i and i - 1 (dy = +1), those of them inside the run.  Output
+            // row t (counted over the runs) has block kAcc - 1 - t % kAcc, so
             // rows i + 1, i, i - 1 have consecutive blocks and one MMA covers
             // them, two where the window passes the last block.  Every output
             // element still accumulates its 18 K steps in the order dy, dx, K.
             // (One M128 x N96 MMA costs a third of three N32 ones: the tensor
             // core takes ~45 cycles per N32 MMA and ~56 per N96 one.)
-            uint32_t n0 = 0, t = 0, ready = 0;  // n0: ring index of the unit's row -1; t: rows of the units before
-            for (int64_t u = blockIdx.x; u < p.units && ok; u += gridDim.x) {
-                const RingUnit w = ring_unit<FULL>(p, u);
+            uint32_t n0 = 0, t = 0, ready = 0;  // n0: ring index of the run's row -1; t: rows of the runs before
+            for (int64_t lin = begin; lin < end && ok;) {
+                const RingUnit w = ring_run<FULL>(p, lin, end);
+                lin += w.nrows;
                 for (int i = -1; i <= w.nrows && ok; ++i) {
                     while (ready < n0 + (uint32_t)(i + 2) && ok) {
-                        if (!tc::mbar_wait(&full[ready & (kRing - 1)], (ready / kRing) & 1u, kWaitCycles)) ok = false;
+                        if (!__all_sync(0xffffffffu, tc::mbar_wait(&full[ready & (kRing - 1)], (ready / kRing) & 1u, kWaitCycles))) ok = false;
                         ++ready;
                     }
                     // row i + 1 enters its block now: the block's last row must be read out
                     if (ok && i + 1 < w.nrows) {
                         const uint32_t tn = t + (uint32_t)(i + 1);
                         if (tn >= (uint32_t)kAcc &&
-                            !tc::mbar_wait(&acce[ring_blk(tn)], (ring_use(tn) + 1u) & 1u, kWaitCycles))
+                            !__all_sync(0xffffffffu, tc::mbar_wait(&acce[ring_blk(tn)], (ring_use(tn) + 1u) & 1u, kWaitCycles)))
                             ok = false;
                     }
                     if (!ok) break;
@@ -909,37 +917,36 @@ __global__ void __launch_bounds__(ring_threads<PROJ, FUSED>(), 2) conv32_ring_ke
                         const uint32_t a_lo = row_lo + ((2 * h * kRingPlane + dxi * 16) >> 4);
                         const uint32_t b_lo =
                             b_lo0 + ((uint32_t)((dxi * 2 + h) * 2 * kStackN * 16) >> 4) + dy0 * (kCh * 16 >> 4);
-                        tc::mma_bf16_w(tmem + (uint32_t)(b0 * kCh), a_lo, a_hi, b_lo, b_hi, idesc_a, 1u);
+                        tc::mma_bf16_warp(tmem + (uint32_t)(b0 * kCh), a_lo, a_hi, b_lo, b_hi, idesc_a, 1u);
                         if (len0 < cnt)
-                            tc::mma_bf16_w(tmem, a_lo, a_hi, b_lo + (uint32_t)len0 * (kCh * 16 >> 4), b_hi, idesc_b, 1u);
+                            tc::mma_bf16_warp(tmem, a_lo, a_hi, b_lo + (uint32_t)len0 * (kCh * 16 >> 4), b_hi, idesc_b, 1u);
                     }
-                    tc::mma_commit(&empty[(n0 + (uint32_t)(i + 1)) & (kRing - 1)]);  // no later MMA reads row i
+                    tc::mma_commit_warp(&empty[(n0 + (uint32_t)(i + 1)) & (kRing - 1)]);  // no later MMA reads row i
                     if (i >= 1) {
                         const uint32_t td = t + (uint32_t)(i - 1);  // row i - 1 has all 18 steps now
-                        if (!(p.withhold && td == 0)) tc::mma_commit(&accf[ring_blk(td)]);
+                        if (!(p.withhold && td == 0)) tc::mma_commit_warp(&accf[ring_blk(td)]);
                     }
                 }
                 n0 += (uint32_t)(w.nrows + 2);
                 t += (uint32_t)w.nrows;
             }
             // every MMA has completed before the TMEM is freed
-            tc::mma_commit(drain);
+            tc::mma_commit_warp(drain);
             tc::mbar_wait(drain, 0, kWaitCycles);
         }
         __syncwarp();
     } else if (PROJ && warp == kRingExtra) {
-        if (lane == 0) {
+        {
             // layer 4's channel contraction of every output row s, in order,
             // once the epilogue has staged its a3 (a3full) and read the P of
             // row s - 2 out of the same TMEM columns (pempty)
             const uint32_t idesc_p = tc::idesc_bf16_f32(kTileM, kProjN);
             const uint32_t a3_u32 = tc::smem_u32(a3s), w4_u32 = tc::smem_u32(sW4);
-            int64_t rows = 0;
-            for (int64_t u = blockIdx.x; u < p.units; u += gridDim.x) rows += ring_unit<FULL>(p, u).nrows;
-            for (int64_t s = 0; s < rows && ok; ++s) {
+            for (int64_t s = 0; s < end - begin && ok; ++s) {
                 const int b = (int)(s & 1);
-                if (!tc::mbar_wait(&a3full[b], (uint32_t)((s >> 1) & 1), kWaitCycles) ||
-                    (s >= 2 && !tc::mbar_wait(&pempty[b], (uint32_t)(((s >> 1) + 1) & 1), kWaitCycles))) {
+                const bool in = tc::mbar_wait(&a3full[b], (uint32_t)((s >> 1) & 1), kWaitCycles) &&
+                                (s < 2 || tc::mbar_wait(&pempty[b], (uint32_t)(((s >> 1) + 1) & 1), kWaitCycles));
+                if (!__all_sync(0xffffffffu, in)) {
                     ok = false;
                     break;
                 }
@@ -948,13 +955,13 @@ __global__ void __launch_bounds__(ring_threads<PROJ, FUSED>(), 2) conv32_ring_ke
                 for (int h = 0; h < 2; ++h) {
                     const uint64_t ad = tc::smem_desc(a3_u32 + b * kRowBytes + 2 * h * kRingPlane, kRingPlane, 128);
                     const uint64_t bd = tc::smem_desc(w4_u32 + 2 * h * kProjN * 16, kProjN * 16, 128);
-                    tc::mma_bf16(tproj + (uint32_t)(b * kProjN), ad, bd, idesc_p, h > 0 ? 1u : 0u);
+                    tc::mma_bf16_warp(tproj + (uint32_t)(b * kProjN), ad, bd, idesc_p, h > 0 ? 1u : 0u);
                 }
-                tc::mma_commit(&pfull[b]);
-                tc::mma_commit(&a3empty[b]);
+                tc::mma_commit_warp(&pfull[b]);
+                tc::mma_commit_warp(&a3empty[b]);
             }
             // its MMAs have completed before the TMEM is freed
-            tc::mma_commit(pdrain);
+            tc::mma_commit_warp(pdrain);
             tc::mbar_wait(pdrain, 0, kWaitCycles);
         }
         __syncwarp();
@@ -968,8 +975,9 @@ __global__ void __launch_bounds__(ring_threads<PROJ, FUSED>(), 2) conv32_ring_ke
 #pragma unroll
         for (int i = 0; i < 16; ++i) bias[i] = kBiasFirst ? sBias[16 * half + i] : 0.0f;
         int64_t t = 0;
-        for (int64_t u = blockIdx.x; u < p.units && ok; u += gridDim.x) {
-            const RingUnit w = ring_unit<FULL>(p, u);
+        for (int64_t lin = begin; lin < end && ok;) {
+            const RingUnit w = ring_run<FULL>(p, lin, end);
+            lin += w.nrows;
             for (int j = 0; j < w.nrows; ++j, ++t) {
                 const int a = ring_blk((uint32_t)t);
                 const bool on = FULL || xw < w.width;  // this warp's pixels are inside the segment
@@ -993,7 +1001,7 @@ __global__ void __launch_bounds__(ring_threads<PROJ, FUSED>(), 2) conv32_ring_ke
                 }
                 tc::fence_after_sync();
                 if (!on) {
-                    // nothing to read, but the next unit may be wider: back to the bias
+                    // nothing to read, but the next run may be wider: back to the bias
                     tc::tmem_st16(tmem + (uint32_t)(a * kCh + 16 * half) + ((uint32_t)(quad * 32) << 16), bias);
                     tc::tmem_wait_st();
                     tc::fence_before_sync();
@@ -1067,9 +1075,24 @@ __global__ void __launch_bounds__(ring_threads<PROJ, FUSED>(), 2) conv32_ring_ke
                             tile_store_bf16(p.a_out, L, w.c, y, w.x0 + xw, 16 * half, st16, lane,
                                             make_uint4(pk[0], pk[1], pk[2], pk[3]), make_uint4(pk[4], pk[5], pk[6], pk[7]));
                         } else {
-                            store_act(p.a_out, L, w.c, y, w.x0 + m, 16 * half, make_uint4(pk[0], pk[1], pk[2], pk[3]));
-                            store_act(p.a_out, L, w.c, y, w.x0 + m, 16 * half + 8,
-                                      make_uint4(pk[4], pk[5], pk[6], pk[7]));
+                            const uint4 lo = make_uint4(pk[0], pk[1], pk[2], pk[3]), hi = make_uint4(pk[4], pk[5], pk[6], pk[7]);
+                            if constexpr (PROJ) {
+                                // lanes 2 k and 2 k + 1 exchange halves, so that each store covers
+                                // whole 32-byte sectors of 16 pixels (training; in the fused first
+                                // conv the exchange costs more than it saves, 1191 for 1173 us)
+                                const bool odd = lane & 1;
+                                uint4 x = odd ? lo : hi;
+                                x.x = __shfl_xor_sync(0xffffffffu, x.x, 1);
+                                x.y = __shfl_xor_sync(0xffffffffu, x.y, 1);
+                                x.z = __shfl_xor_sync(0xffffffffu, x.z, 1);
+                                x.w = __shfl_xor_sync(0xffffffffu, x.w, 1);
+                                const int px = w.x0 + m - (odd ? 1 : 0), ch = 16 * half + (odd ? 8 : 0);
+                                store_act(p.a_out, L, w.c, y, px, ch, odd ? x : lo);
+                                store_act(p.a_out, L, w.c, y, px + 1, ch, odd ? hi : x);
+                            } else {
+                                store_act(p.a_out, L, w.c, y, w.x0 + m, 16 * half, lo);
+                                store_act(p.a_out, L, w.c, y, w.x0 + m, 16 * half + 8, hi);
+                            }
                         }
                     }
                     if (PROJ) {
@@ -1095,8 +1118,9 @@ __global__ void __launch_bounds__(ring_threads<PROJ, FUSED>(), 2) conv32_ring_ke
         // four arrivals) and stores the 9 taps as FP32 planes P[k][pixel]
         const int quad = warp & 3, m = quad * 32 + lane;
         int64_t s = 0;
-        for (int64_t u = blockIdx.x; u < p.units && ok; u += gridDim.x) {
-            const RingUnit w = ring_unit<FULL>(p, u);
+        for (int64_t lin = begin; lin < end && ok;) {
+            const RingUnit w = ring_run<FULL>(p, lin, end);
+            lin += w.nrows;
             for (int j = 0; j < w.nrows; ++j, ++s) {
                 const int b = (int)(s & 1);
                 if (!__all_sync(0xffffffffu, tc::mbar_wait(&pfull[b], (uint32_t)((s >> 1) & 1), kWaitCycles))) {
@@ -1420,7 +1444,7 @@ __global__ void __launch_bounds__(32 * kReduceWarps) reduce_partials_kernel(cons
 // end they are written as the CTA's partial sums in the weight-gradient
 // layout (e = (o CIN + i) 9 + k, then the biases).
 // Warp roles (bounded mbarrier waits): warp 0 lane 0 issues the tensor
-// copies; warp 1 lane 0 the MMAs; warps 2..5 add up every staged gradient row
+// copies; warp 1 the MMAs (one elected lane); warps 2..5 add up every staged gradient row
 // for the bias sums (fixed order; the zero rows add nothing) and, after the
 // last MMA, read the accumulators.  A gradient slot is free once the MMAs of
 // its last input row have completed and the four bias warps have read it.
@@ -1479,7 +1503,7 @@ __global__ void __launch_bounds__(kWgThreads, 1) wgrad_tc_kernel(const __grid_co
     uint64_t *aempty = afull + kWgActSlots, *dfull = aempty + kWgActSlots, *dempty = dfull + kWgDzSlots;
     uint64_t *drain = dempty + kWgDzSlots;
     uint32_t *tslot = reinterpret_cast<uint32_t *>(drain + 1);
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
     const int L = p.L;
     const uint32_t box = (uint32_t)(FULL ? kTileM : p.tw) * kCh * 2;  // bytes of a staged row of tw pixels
     const int64_t begin = blockIdx.x * p.lines / gridDim.x, end = (blockIdx.x + 1) * p.lines / gridDim.x;
@@ -1552,7 +1576,7 @@ __global__ void __launch_bounds__(kWgThreads, 1) wgrad_tc_kernel(const __grid_co
         }
         __syncwarp();
     } else if (warp == 1) {
-        if (lane == 0) {
+        {
             const uint32_t idesc = tc::idesc_bf16_f32_mn(kTileM, kWgN);
             const uint64_t a_desc0 = tc::smem_desc_sw64(tc::smem_u32(wg_smem), kWgBox, 512);
             const uint64_t b_desc0 = tc::smem_desc_sw64(tc::smem_u32(wg_smem + kWgDz0), kWgBox, 512);
@@ -1566,12 +1590,13 @@ __global__ void __launch_bounds__(kWgThreads, 1) wgrad_tc_kernel(const __grid_co
                 for (int a = 0; a < w.nrows + 2 && ok; ++a) {
                     // input row r0 - 1 + a meets gradient rows r0 - 2 + a .. r0 + a (indices md + a .. md + a + 2)
                     while (dready < md + (uint32_t)a + 3 && ok) {
-                        if (!tc::mbar_wait(&dfull[dready % kWgDzSlots], (dready / kWgDzSlots) & 1u, kWaitCycles))
+                        if (!__all_sync(0xffffffffu, tc::mbar_wait(&dfull[dready % kWgDzSlots], (dready / kWgDzSlots) & 1u,
+                                                                   kWaitCycles)))
                             ok = false;
                         ++dready;
                     }
                     const uint32_t as = ma % kWgActSlots;
-                    if (ok && !tc::mbar_wait(&afull[as], (ma / kWgActSlots) & 1u, kWaitCycles)) ok = false;
+                    if (ok && !__all_sync(0xffffffffu, tc::mbar_wait(&afull[as], (ma / kWgActSlots) & 1u, kWaitCycles))) ok = false;
                     if (!ok) break;
                     tc::fence_after_sync();
                     const uint32_t a_row = a_lo0 + ((as * kWgActBytes) >> 4);
@@ -1579,21 +1604,21 @@ __global__ void __launch_bounds__(kWgThreads, 1) wgrad_tc_kernel(const __grid_co
 #pragma unroll
                     for (int ks = 0; ks < kTileM / 16; ++ks)  // 16 pixels = two 512-byte atoms
                         if (FULL || 16 * ks < p.tw)
-                            tc::mma_bf16_w(tmem + 256 * (seen % kWgSets<FULL>), a_row + (uint32_t)(ks * 64), a_hi,
+                            tc::mma_bf16_warp(tmem + 256 * (seen % kWgSets<FULL>), a_row + (uint32_t)(ks * 64), a_hi,
                                            b_row + (uint32_t)(ks * 64), b_hi, idesc,
                                            (seen < kWgSets<FULL> && ks == 0) ? 0u : 1u);
                     ++seen;
-                    tc::mma_commit(&aempty[as]);
+                    tc::mma_commit_warp(&aempty[as]);
                     ++ma;
-                    tc::mma_commit(&dempty[(md + (uint32_t)a) % kWgDzSlots]);  // gradient row r0 - 2 + a: last use
+                    tc::mma_commit_warp(&dempty[(md + (uint32_t)a) % kWgDzSlots]);  // gradient row r0 - 2 + a: last use
                 }
                 if (!ok) break;
-                tc::mma_commit(&dempty[(md + (uint32_t)w.nrows + 2) % kWgDzSlots]);
-                tc::mma_commit(&dempty[(md + (uint32_t)w.nrows + 3) % kWgDzSlots]);
+                tc::mma_commit_warp(&dempty[(md + (uint32_t)w.nrows + 2) % kWgDzSlots]);
+                tc::mma_commit_warp(&dempty[(md + (uint32_t)w.nrows + 3) % kWgDzSlots]);
                 md += (uint32_t)w.nrows + 4;
             }
             // every MMA has completed before the accumulators are read and the TMEM is freed
-            tc::mma_commit(drain);
+            tc::mma_commit_warp(drain);
             if (!tc::mbar_wait(drain, 0, kWaitCycles)) ok = false;
         }
         __syncwarp();
@@ -2077,9 +2102,8 @@ int launch_ring_bwd(int L, int64_t C, const float *params, int w_off, const __nv
     p.bd.flip = nullptr;
     p.segs = seg_count(L);
     p.tw = seg_width(L);
-    p.units_per_col = (L + kUnitRows - 1) / kUnitRows;
-    p.units = C * p.segs * p.units_per_col;
-    const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>(p.units, 2 * info.sm_count));
+    p.lines = C * p.segs * L;
+    const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>(p.lines / kMinRange, 2 * info.sm_count));
     launch_ring<false, true, false>(p, grid, s);
     cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? ISING_OK : nfail(ISING_ECUDA, cudaGetErrorString(e));
@@ -2170,10 +2194,9 @@ int launch_forward(const Chains &ch, int64_t C, const int32_t *flip, bool band, 
         p.bd = bd[l + 1];
         p.segs = seg_count(L);
         p.tw = seg_width(L);
-        p.units_per_col = (bd[l + 1].rows + kUnitRows - 1) / kUnitRows;
-        p.units = C * p.segs * p.units_per_col;
+        p.lines = C * p.segs * bd[l + 1].rows;
         p.withhold = withhold && l == 0;
-        const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>(p.units, 2 * info.sm_count));
+        const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>(p.lines / kMinRange, 2 * info.sm_count));
         if (fused)
             launch_ring<false, false, true>(p, grid, s);
         else if (l == 0)
