@@ -43,8 +43,8 @@
 // the chain's stream) or uniformly; x' = x with block b flipped; the flip is
 // accepted iff the purpose-3 draw of site 1 is below
 // floor(2^32 min(1, exp(-beta dE + log q_x'(b) - log q_x(b)))), dE the exact
-// integer energy change (twice the boundary bond sum).  Softmax sums run in
-// block order in FP64.
+// integer energy change (twice the boundary bond sum).  Softmax sums are FP64, in
+// a fixed order.
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -1799,40 +1799,57 @@ __device__ __forceinline__ uint32_t move_draw(const RoundKeys &rk, uint32_t stre
     return w == 0 ? u.x : w == 1 ? u.y : w == 2 ? u.z : u.w;
 }
 
-// The move kernels run one warp per chain.  FP64 arithmetic is slow on this
-// GPU, so the lanes compute the exponentials of a chunk of 256 blocks in
-// parallel into shared memory and lane 0 adds them up in block order: every
-// FP64 operation, and so every decision, is the one of a sequential loop.
+// The move kernels run one warp per chain and are bound by FP64, which is slow on
+// this GPU: by its latency where one lane adds up a chain's 256 weights in turn
+// (76 us to propose for 1024 chains of 128^2 and 74 to accept), so a lane adds up 8
+// consecutive blocks and a warp scan does the rest, in a fixed order (18 and 35
+// us); each weight is computed once, except where a chain has more than one chunk
+// of 256 blocks and the chosen one is walked again.
 constexpr int kMoveWarps = 4;   // chains per 128-thread CTA
 constexpr int kChunk = 256;     // blocks per chunk
+constexpr int kPerLane = kChunk / 32;
+constexpr int kMaxChunks = (4096 / kBlk) * (4096 / kBlk) / kChunk;
 
-__device__ __forceinline__ double warp_max_logit(const float *l, int nb)
+__device__ __forceinline__ float warp_max_logit(const float *l, int nb)
 {
-    double m = -INFINITY;
-    for (int b = (threadIdx.x & 31); b < nb; b += 32) m = fmax(m, (double)l[b]);
+    float m = -INFINITY;
+    for (int b = (threadIdx.x & 31); b < nb; b += 32) m = fmaxf(m, l[b]);
 #pragma unroll
-    for (int off = 16; off > 0; off >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, off));
+    for (int off = 16; off > 0; off >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, off));
     return m;
 }
 
-// exp(l[b] - m) of the blocks base .. base + n - 1 into e[0 .. n-1]
-__device__ __forceinline__ void chunk_exp(const float *l, double m, int base, int n, double *e)
+// The weights exp(l[b] - m) of this lane's blocks base + 8 lane .. + 7 (0 past the
+// last one), and their sum in order.
+__device__ __forceinline__ double lane_weights(const float *l, float m, int base, int nb, double (&e)[kPerLane])
 {
-    for (int j = (threadIdx.x & 31); j < n; j += 32) e[j] = exp((double)l[base + j] - m);
-    __syncwarp();
+    const int b0 = base + kPerLane * (threadIdx.x & 31);
+    double sum = 0.0;
+#pragma unroll
+    for (int k = 0; k < kPerLane; ++k) {
+        e[k] = b0 + k < nb ? exp((double)l[b0 + k] - (double)m) : 0.0;
+        sum += e[k];
+    }
+    return sum;
 }
 
-// sum over b of exp(l[b] - m) in block order (the value is lane 0's)
-__device__ double warp_exp_sum(const float *l, int nb, double m, double *e)
+// Inclusive sums over the lanes.
+__device__ __forceinline__ double warp_scan(double v)
 {
-    double total = 0.0;
-    for (int base = 0; base < nb; base += kChunk) {
-        const int n = min(kChunk, nb - base);
-        chunk_exp(l, m, base, n, e);
-        if ((threadIdx.x & 31) == 0)
-            for (int j = 0; j < n; ++j) total += e[j];
-        __syncwarp();
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+        const double u = __shfl_up_sync(0xffffffffu, v, off);
+        if ((int)(threadIdx.x & 31) >= off) v += u;
     }
+    return v;
+}
+
+// Sum over all blocks of exp(l[b] - m).
+__device__ double warp_exp_sum(const float *l, int nb, float m)
+{
+    double total = 0.0, e[kPerLane];
+    for (int base = 0; base < nb; base += kChunk)
+        total += __shfl_sync(0xffffffffu, warp_scan(lane_weights(l, m, base, nb, e)), 31);
     return total;
 }
 
@@ -1840,9 +1857,10 @@ __global__ void __launch_bounds__(32 * kMoveWarps) propose_kernel(int64_t C, int
                                                                    const __grid_constant__ RoundKeys rk, uint64_t t,
                                                                    int32_t *block)
 {
-    __shared__ double ebuf[kMoveWarps][kChunk];
+    extern __shared__ double before[];  // per warp: the weight before each chunk
     const int lane = threadIdx.x & 31, wl = threadIdx.x >> 5;
-    double *e = ebuf[wl];
+    const int chunks = (nb + kChunk - 1) / kChunk;
+    double *pre = before + wl * chunks;
     const int64_t nwarps = (int64_t)gridDim.x * kMoveWarps;
     for (int64_t c = (int64_t)blockIdx.x * kMoveWarps + wl; c < C; c += nwarps) {
         const uint32_t u = move_draw(rk, (uint32_t)c, 0, t);
@@ -1852,24 +1870,37 @@ __global__ void __launch_bounds__(32 * kMoveWarps) propose_kernel(int64_t C, int
         } else {
             // inverse CDF: the first block whose cumulative weight exceeds u / 2^32 of the total
             const float *l = logits + c * nb;
-            const double m = warp_max_logit(l, nb);
-            const double target = ((double)u / 4294967296.0) * warp_exp_sum(l, nb, m, e);
-            double acc = 0.0;
-            int found = -1;
-            for (int base = 0; base < nb && found < 0; base += kChunk) {
-                const int n = min(kChunk, nb - base);
-                chunk_exp(l, m, base, n, e);
-                if (lane == 0)
-                    for (int j = 0; j < n; ++j) {
-                        acc += e[j];
-                        if (acc > target) {
-                            found = base + j;
-                            break;
-                        }
-                    }
-                found = __shfl_sync(0xffffffffu, found, 0);
+            const float m = warp_max_logit(l, nb);
+            double e[kPerLane], total = 0.0, upto = 0.0;
+            for (int k = 0; k < chunks; ++k) {
+                upto = warp_scan(lane_weights(l, m, k * kChunk, nb, e));
+                if (lane == 0) pre[k] = total;
+                total += __shfl_sync(0xffffffffu, upto, 31);
             }
-            if (found >= 0) b = found;
+            __syncwarp();
+            const double target = ((double)u / 4294967296.0) * total;
+            // the last chunk that starts at or below the target (the first, if rounding leaves none)
+            int k = 0;
+            for (int q = lane; q < chunks; q += 32)
+                if (pre[q] <= target) k = q;
+#pragma unroll
+            for (int off = 16; off > 0; off >>= 1) k = max(k, __shfl_xor_sync(0xffffffffu, k, off));
+            if (k != chunks - 1) upto = warp_scan(lane_weights(l, m, k * kChunk, nb, e));
+            upto = __shfl_up_sync(0xffffffffu, upto, 1);  // the chunk's weight before this lane's blocks
+            double acc = lane == 0 ? pre[k] : pre[k] + upto;
+            int found = nb;
+#pragma unroll
+            for (int q = 0; q < kPerLane; ++q) {
+                acc += e[q];
+                const int at = k * kChunk + kPerLane * lane + q;
+                if (found == nb && at < nb && acc > target) found = at;
+            }
+#pragma unroll
+            for (int off = 16; off > 0; off >>= 1) found = min(found, __shfl_xor_sync(0xffffffffu, found, off));
+            // none: the next chunk's first block (the sums round differently), or the
+            // last block of all (no target: the logits are not finite)
+            b = found < nb ? found : target == target ? min((k + 1) * kChunk, nb - 1) : nb - 1;
+            __syncwarp();
         }
         if (lane == 0) block[c] = b;
     }
@@ -1881,10 +1912,8 @@ __global__ void __launch_bounds__(32 * kMoveWarps) accept_kernel(Chains ch, uint
                                                                   const __grid_constant__ RoundKeys rk, uint64_t t,
                                                                   int32_t *accepted, int64_t *dE_out)
 {
-    __shared__ double ebuf[kMoveWarps][kChunk];
     const int L = ch.L, nb1 = L / kBlk, nb = nb1 * nb1;
     const int lane = threadIdx.x & 31, wl = threadIdx.x >> 5;
-    double *e = ebuf[wl];
     const int64_t nwarps = (int64_t)gridDim.x * kMoveWarps;
     for (int64_t c = (int64_t)blockIdx.x * kMoveWarps + wl; c < C; c += nwarps) {
         const int b = block[c];
@@ -1902,14 +1931,12 @@ __global__ void __launch_bounds__(32 * kMoveWarps) accept_kernel(Chains ch, uint
         const int dE = 2 * d;
         double x = -beta * (double)dE;
         if (lx != nullptr) {
-            // log q(b) = l_b - (max + log sum exp(l - max)), sums in block order
+            // log q(b) = l_b - (max + log sum exp(l - max))
             const float *lr = lxp + c * nb, *lf = lx + c * nb;
-            const double mr = warp_max_logit(lr, nb);
-            const double sr = warp_exp_sum(lr, nb, mr, e);
-            const double mf = warp_max_logit(lf, nb);
-            const double sf = warp_exp_sum(lf, nb, mf, e);
-            const double logp_rev = (double)lr[b] - (mr + log(sr));
-            const double logp_fwd = (double)lf[b] - (mf + log(sf));
+            const float mr = warp_max_logit(lr, nb), mf = warp_max_logit(lf, nb);
+            const double sr = warp_exp_sum(lr, nb, mr), sf = warp_exp_sum(lf, nb, mf);
+            const double logp_rev = (double)lr[b] - ((double)mr + log(sr));
+            const double logp_fwd = (double)lf[b] - ((double)mf + log(sf));
             x = (x + logp_rev) - logp_fwd;
         }
         if (lane == 0) {
@@ -2396,7 +2423,9 @@ ISING_API int ising_block_propose(int64_t L, int64_t C, const float *logits_dev,
     if (rc) return rc;
     if (check_device_range(block_dev, (size_t)C * 4, "block")) return nfail(ISING_EINVAL, "block must be device memory");
     const int nb = (int)((L / 8) * (L / 8));
-    propose_kernel<<<grid1d(C * 32, 32 * kMoveWarps), 32 * kMoveWarps, 0, (cudaStream_t)stream>>>(
+    const size_t smem = kMoveWarps * (size_t)((nb + kChunk - 1) / kChunk) * sizeof(double);  // 32 KB at most
+    static_assert(kMoveWarps * kMaxChunks * sizeof(double) <= 48 * 1024, "within the default limit");
+    propose_kernel<<<grid1d(C * 32, 32 * kMoveWarps), 32 * kMoveWarps, smem, (cudaStream_t)stream>>>(
         C, nb, logits_dev, make_round_keys(seed), t, block_dev);
     cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? ISING_OK : nfail(ISING_ECUDA, cudaGetErrorString(e));
