@@ -20,7 +20,7 @@
 // pixels: column 0 repeats pixel L - 1 and column L + 1 pixel 0 (the periodic
 // halo, written by the producer), so that one rectangular copy fetches a row
 // segment with both neighbours.  The pre-activations z kept for training and
-// the gradients are NHWC FP32 without halo.
+// the gradients that go on in FP32 are NHWC without halo.
 //
 // Forward kernels: layer 1 by table lookup (l1_table_kernel, l1_kernel); the
 // two 32 -> 32 layers on the tensor cores (tcgen05; conv32_ring_kernel), the
@@ -302,14 +302,18 @@ __device__ __forceinline__ void store_act(__nv_bfloat16 *a, int L, int64_t c, in
 
 // Layer 1 (1 -> 32 channels) sees only the 3 x 3 spins around a pixel, so its
 // output is a function of a 9-bit pattern (bit k set when the spin at tap k =
-// 3 (dy + 1) + (dx + 1) is +1).  l1_table_kernel evaluates z1 and
-// bf16(gelu(z1)) for all 512 patterns, with the arithmetic a direct evaluation
-// would use (bias first, then the taps in order by fmaf); l1_kernel then reads
-// each pixel's pattern and copies its row of the table.
+// 3 (dy + 1) + (dx + 1) is +1).  l1_table_kernel evaluates bf16(gelu(z1)) and
+// gelu'(z1) for all 512 patterns, with the arithmetic a direct evaluation would
+// use (bias first, then the taps in order by fmaf); l1_kernel then reads each
+// pixel's pattern and copies its row of the first table.  A training pass keeps
+// the patterns, 2 bytes per pixel, from which the backward pass gets its factor
+// gelu'(z1) (instead of z1, 128 bytes per pixel written, read and put through
+// gelu' again; with the FP32 dz3 and dz2 that nothing read any more, 722 us per
+// training step of 64 chains of 128^2, without them 672).
 constexpr int kPatterns = 512;
 constexpr int kL1Threads = 128;
 
-__global__ void l1_table_kernel(const float *params, float *tz, __nv_bfloat16 *ta)
+__global__ void l1_table_kernel(const float *params, float *tg, __nv_bfloat16 *ta)
 {
     const int e = blockIdx.x * blockDim.x + threadIdx.x;  // pattern * 32 + output channel
     if (e >= kPatterns * kCh) return;
@@ -317,7 +321,7 @@ __global__ void l1_table_kernel(const float *params, float *tz, __nv_bfloat16 *t
     float v = bf16r(params[kOffB1 + o]);
 #pragma unroll
     for (int k = 0; k < 9; ++k) v = fmaf(bf16r(params[kOffW1 + o * 9 + k]), ((pat >> k) & 1) ? 1.0f : -1.0f, v);
-    tz[e] = v;
+    tg[e] = gelu_grad(v);
     ta[e] = __float2bfloat16_rn(gelu(v));
 }
 
@@ -338,10 +342,10 @@ __device__ __forceinline__ uint32_t spin_up(const Chains &ch, int64_t c, int y, 
 
 // Thread per pixel of the band; blockIdx.y walks the chains and blockIdx.x
 // the 128-pixel tiles of a chain's band, so all index arithmetic is 32-bit.
-// Writes a1 (bfloat16, from the table in shared memory) and, when z_out !=
-// nullptr, z1 (FP32), each store instruction covering whole pixels.
+// Writes a1 (bfloat16, from the table in shared memory), each store instruction
+// covering whole pixels, and the patterns.
 __global__ void __launch_bounds__(kL1Threads) l1_kernel(Chains ch, Band bd, const int32_t *flip,
-                                                        const __nv_bfloat16 *ta, const float *tz, float *z_out,
+                                                        const __nv_bfloat16 *ta, uint16_t *pat_out,
                                                         __nv_bfloat16 *a_out)
 {
     __shared__ uint4 T[kPatterns * kCh * 2 / 16];  // ta, 32 KiB
@@ -369,15 +373,7 @@ __global__ void __launch_bounds__(kL1Threads) l1_kernel(Chains ch, Band bd, cons
                 const uint32_t pt = __shfl_sync(0xffffffffu, pat, pp);
                 store_act(a_out, L, c, y, x_first + pp, 8 * g, T[pt * 4 + g]);
             }
-            if (z_out) {
-#pragma unroll
-                for (int j = 0; j < 8; ++j) {
-                    const int pp = 4 * j + (lane >> 3), g = lane & 7;
-                    const uint32_t pt = __shfl_sync(0xffffffffu, pat, pp);
-                    reinterpret_cast<float4 *>(z_out + ((c * L + y) * (int64_t)L + x_first + pp) * kCh)[g] =
-                        __ldg(reinterpret_cast<const float4 *>(tz + pt * kCh) + g);
-                }
-            }
+            pat_out[(c * L + y) * (int64_t)L + x] = (uint16_t)pat;
         }
     }
 }
@@ -462,8 +458,8 @@ __device__ int g_tc_error;  // set to 1 when a tensor-core wait gives up
 // as the staged rows and the weights transposed and tap-flipped, B_k[i][o] =
 // W[o][i][8 - k], since dz_prev(p)[i] = gelu'(z_prev(p)[i]) sum_k sum_o
 // W[o][i][k] dz(p - off_k)[o] and -off_k = off_{8-k}; the epilogue multiplies
-// by gelu'(z_prev) and writes dz_prev in FP32 (and in bfloat16 with halo
-// columns when a_out is set, for the next data gradient).
+// by gelu'(z_prev) and writes dz_prev in FP32 (layer 1's, for its weight gradient)
+// or as two bfloat16 parts with halo columns, for what takes it from there.
 // Dependencies: the MMAs of staged row i wait on the epilogue of output rows
 // up to i + 1 - kAcc only, the epilogue of row t on the MMAs of staged rows up
 // to t + 1 only, so no wait can close a cycle.
@@ -561,6 +557,29 @@ __device__ __forceinline__ void tile_load_f32(const float *g, float4 *stg, int l
     }
 }
 
+// v[16] = 16 FP32 channels of row `pat` (this lane's) of a table of 32 per row.
+__device__ __forceinline__ void tile_gather_f32(const float *tab, uint32_t pat, float4 *stg, int lane, float (&v)[16])
+{
+    __syncwarp();
+    float4 t[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const uint32_t row = __shfl_sync(0xffffffffu, pat, 8 * k + (lane >> 2));
+        t[k] = __ldg(reinterpret_cast<const float4 *>(tab + row * kCh + 4 * (lane & 3)));
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) stg[stage_slot32(8 * k + (lane >> 2), lane & 3)] = t[k];
+    __syncwarp();
+#pragma unroll
+    for (int cc = 0; cc < 4; ++cc) {
+        const float4 x = stg[stage_slot32(lane, cc)];
+        v[4 * cc] = x.x;
+        v[4 * cc + 1] = x.y;
+        v[4 * cc + 2] = x.z;
+        v[4 * cc + 3] = x.w;
+    }
+}
+
 // The tile at g = this lane's 16 FP32 channels v[16] (pixel pp at g + pp kCh).
 __device__ __forceinline__ void tile_store_f32(float *g, float4 *stg, int lane, const float (&v)[16])
 {
@@ -600,8 +619,10 @@ struct RingConv {
     __nv_bfloat16 *a_lo;   // BWD, nullable: bf16(dz_prev - bf16(dz_prev)) beside a_out (for the weight gradient)
     float *z_out;          // nullable
     float *P;              // PROJ: 9 planes of C L^2
-    const float *zg;       // BWD: z of the layer below (FP32, NHWC) for gelu'
-    float *d_out;          // BWD: dz of the layer below (FP32, NHWC)
+    const float *zg;       // BWD: z of the layer below (FP32, NHWC) for gelu', or, where that is layer 1,
+    const uint16_t *pat;   // the pixels' patterns and
+    const float *tg;       // the table of gelu'(z1)
+    float *d_out;          // BWD: dz of the layer below (FP32, NHWC), nullable
     Chains ch;             // FUSED: the spins (flip[c], or -1, negated)
     const int32_t *flip;
     const __nv_bfloat16 *ta;  // FUSED: layer 1's table, 512 patterns x 32 channels
@@ -989,7 +1010,9 @@ __global__ void __launch_bounds__(ring_threads<PROJ, FUSED>(), 2) conv32_ring_ke
                 const int64_t q0 = q - lane;
                 float gz[16];
                 if constexpr (BWD) {
-                    if (on) {
+                    if (on && p.pat) {
+                        tile_gather_f32(p.tg + 16 * half, p.pat[q], stg, lane, gz);
+                    } else if (on) {
                         tile_load_f32(p.zg + q0 * kCh + 16 * half, stg, lane, gz);
 #pragma unroll
                         for (int i = 0; i < 16; i += 2) gelu_grad2(gz[i], gz[i + 1]);
@@ -1034,7 +1057,7 @@ __global__ void __launch_bounds__(ring_threads<PROJ, FUSED>(), 2) conv32_ring_ke
                 if constexpr (BWD) {
 #pragma unroll
                     for (int i = 0; i < 16; ++i) v[i] *= gz[i];
-                    tile_store_f32(p.d_out + q0 * kCh + 16 * half, stg, lane, v);
+                    if (p.d_out) tile_store_f32(p.d_out + q0 * kCh + 16 * half, stg, lane, v);
                     if (p.a_out) {
                         uint32_t hb[2][4], rb[2][4];
 #pragma unroll
@@ -1208,11 +1231,11 @@ __global__ void __launch_bounds__(kThreads) pool_rows_kernel(int L, int64_t C, i
 }
 
 // ---------------------------------------------------------------------------
-// Backward (uses z1..z3, a1..a3 stored by a training forward)
+// Backward (uses what a training forward stored)
 // ---------------------------------------------------------------------------
 // dz3 = gelu'(z3) * sum_k W4[i][k] * d4(p - off_k),  d4(p) = dlogit(block of p) / 64.
 __global__ void __launch_bounds__(kThreads) l4_bwd_data_kernel(int L, int64_t C, const float *params,
-                                                               const float *dlogits, const float *z3, float *dz3,
+                                                               const float *dlogits, const float *z3,
                                                                __nv_bfloat16 *dz3b, __nv_bfloat16 *dz3r)
 {
     __shared__ float W[kN1];
@@ -1220,8 +1243,8 @@ __global__ void __launch_bounds__(kThreads) l4_bwd_data_kernel(int L, int64_t C,
     __syncthreads();
     const int nb1 = L / kBlk;
     const int64_t npix = C * (int64_t)L * L;
-    // four threads per pixel, 8 channels each: a warp reads and writes 8
-    // pixels' 1 KB of z3 / dz3 contiguously
+    // four threads per pixel, 8 channels each: a warp reads 8 pixels' 1 KB of z3
+    // contiguously
     for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < 4 * npix;
          e += (int64_t)gridDim.x * blockDim.x) {
         const int64_t p = e >> 2;
@@ -1253,17 +1276,12 @@ __global__ void __launch_bounds__(kThreads) l4_bwd_data_kernel(int L, int64_t C,
             for (int k = 0; k < 9; ++k) g = fmaf(W[(i8 + i) * 9 + k], d[k], g);
             v[i] = g * gz[i];
         }
-        float4 *out = reinterpret_cast<float4 *>(dz3 + p * kCh + i8);
-        out[0] = make_float4(v[0], v[1], v[2], v[3]);
-        out[1] = make_float4(v[4], v[5], v[6], v[7]);
-        // bfloat16 copy with halo columns: the operand of the next data gradient on the tensor cores
-        // (and, with the rounding of its remainder, of the weight gradient)
-        if (dz3b) {
-            uint32_t hb[4], rb[4];
-            split_bf16(v, hb, rb);
-            store_act(dz3b, L, c, y, x, i8, make_uint4(hb[0], hb[1], hb[2], hb[3]));
-            if (dz3r) store_act(dz3r, L, c, y, x, i8, make_uint4(rb[0], rb[1], rb[2], rb[3]));
-        }
+        // as bfloat16 with halo columns, the operand of the next data gradient on the
+        // tensor cores, and the rounding of its remainder, for the weight gradient
+        uint32_t hb[4], rb[4];
+        split_bf16(v, hb, rb);
+        store_act(dz3b, L, c, y, x, i8, make_uint4(hb[0], hb[1], hb[2], hb[3]));
+        store_act(dz3r, L, c, y, x, i8, make_uint4(rb[0], rb[1], rb[2], rb[3]));
     }
 }
 
@@ -1982,12 +2000,13 @@ int check_chains(int64_t L, int64_t C)
     return ISING_OK;
 }
 
-// Work layout: training keeps z1 z2 z3 (FP32), a1 a2 a3 (bfloat16) and two
-// FP32 gradient buffers, then the weight-gradient partials; inference keeps a2
+// Work layout: training keeps layer 1's patterns, z2 z3 (FP32), a1 a2 a3
+// (bfloat16), dz1 (FP32) and dz2, dz3 (as two bfloat16 parts), then the weight-gradient partials; inference keeps a2
 // alone (bfloat16).  Both end with the row partials of z4, 9 values per row and
 // 8-pixel block column.
 struct NetWork {
-    float *z1, *z2, *z3, *da, *db, *partial, *P, *tz;
+    float *z2, *z3, *da, *partial, *P, *tg;
+    uint16_t *pat;
     __nv_bfloat16 *a1, *a2, *a3, *ta, *gb1, *gb2;  // gb: bfloat16 gradients with halo columns (training)
     __nv_bfloat16 *gr1, *gr2;                      // the bfloat16 roundings of their remainders
     int64_t n_cta;
@@ -2009,10 +2028,11 @@ NetWork net_layout(int64_t L, int64_t C, int train, char *base)
         return (void *)p;
     };
     if (train) {
-        w.z1 = (float *)take(pix * 4); w.z2 = (float *)take(pix * 4); w.z3 = (float *)take(pix * 4);
+        w.z2 = (float *)take(pix * 4); w.z3 = (float *)take(pix * 4);
+        w.pat = (uint16_t *)take(pix / kCh * 2);
         w.a1 = (__nv_bfloat16 *)take(apx * 2); w.a2 = (__nv_bfloat16 *)take(apx * 2);
         w.a3 = (__nv_bfloat16 *)take(apx * 2);
-        w.da = (float *)take(pix * 4); w.db = (float *)take(pix * 4);
+        w.da = (float *)take(pix * 4);
         w.gb1 = (__nv_bfloat16 *)take(apx * 2); w.gb2 = (__nv_bfloat16 *)take(apx * 2);
         w.gr1 = (__nv_bfloat16 *)take(apx * 2); w.gr2 = (__nv_bfloat16 *)take(apx * 2);
         DeviceInfo info{152};
@@ -2023,7 +2043,7 @@ NetWork net_layout(int64_t L, int64_t C, int train, char *base)
         w.a2 = (__nv_bfloat16 *)take(apx * 2);
     }
     w.P = (float *)take((size_t)C * L * (L / kBlk) * 9 * sizeof(float));
-    w.tz = (float *)take((size_t)kPatterns * kCh * sizeof(float));
+    w.tg = (float *)take((size_t)kPatterns * kCh * sizeof(float));
     w.ta = (__nv_bfloat16 *)take((size_t)kPatterns * kCh * 2);
     w.bytes = o;
     return w;
@@ -2104,11 +2124,12 @@ void launch_ring(const RingConv &p, unsigned grid, cudaStream_t s)
 }
 
 // The data gradient of a 32 -> 32 layer (weights at w_off) on the tensor
-// cores: dz_prev = gelu'(zg) * conv^T(in), in the bfloat16 gradient with halo
-// columns; writes d_out (FP32) and, if given, a_out (bfloat16, halo columns)
-// and a_lo (the bfloat16 rounding of d_out - a_out).
+// cores: dz_prev = gelu'(z_prev) * conv^T(in), in the bfloat16 gradient with halo
+// columns, gelu'(z_prev) from zg = z_prev or from the patterns and their table;
+// writes what is given of d_out (FP32), a_out (bfloat16, halo columns) and a_lo
+// (the bfloat16 rounding of the remainder).
 int launch_ring_bwd(int L, int64_t C, const float *params, int w_off, const __nv_bfloat16 *in, const float *zg,
-                    float *d_out, __nv_bfloat16 *a_out, __nv_bfloat16 *a_lo, cudaStream_t s)
+                    const uint16_t *pat, const float *tg, float *d_out, __nv_bfloat16 *a_out, __nv_bfloat16 *a_lo, cudaStream_t s)
 {
     DeviceInfo info{152};
     device_info(&info);
@@ -2118,6 +2139,8 @@ int launch_ring_bwd(int L, int64_t C, const float *params, int w_off, const __nv
     p.a_out = a_out;
     p.a_lo = a_lo;
     p.zg = zg;
+    p.pat = pat;
+    p.tg = tg;
     p.d_out = d_out;
     p.params = params;
     p.w_off = w_off;
@@ -2195,9 +2218,9 @@ int launch_forward(const Chains &ch, int64_t C, const int32_t *flip, bool band, 
         const int64_t want = (int64_t)info.sm_count * 16;
         const unsigned gx = (unsigned)std::max<int64_t>(1, std::min<int64_t>(tiles, want));
         const unsigned gy = (unsigned)std::max<int64_t>(1, std::min<int64_t>({C, 65535, (want + gx - 1) / gx}));
-        l1_table_kernel<<<kPatterns * kCh / 256, 256, 0, s>>>(params, w.tz, w.ta);
+        l1_table_kernel<<<kPatterns * kCh / 256, 256, 0, s>>>(params, w.tg, w.ta);
         // an inference pass forms layer 1 inside the first conv
-        if (train) l1_kernel<<<dim3(gx, gy), kL1Threads, 0, s>>>(ch, bd[0], flip, w.ta, w.tz, w.z1, w.a1);
+        if (train) l1_kernel<<<dim3(gx, gy), kL1Threads, 0, s>>>(ch, bd[0], flip, w.ta, w.pat, w.a1);
     }
     const int off[2][2] = {{kOffW2, kOffB2}, {kOffW3, kOffB3}};
     const __nv_bfloat16 *ins[2] = {w.a1, w.a2};
@@ -2364,20 +2387,20 @@ ISING_API int ising_net_backward(int64_t L, int64_t C, const void *black_dev, co
     // the data and weight gradients of the 32 -> 32 layers run on the tensor
     // cores; their gradients are then also kept as bfloat16 parts (gb: the
     // rounding, gr: the rounding of the remainder)
-    l4_bwd_data_kernel<<<grid1d(4 * npix, kThreads), kThreads, 0, s>>>((int)L, C, params_dev, dlogits_dev, w.z3, w.da,
-                                                                     w.gb1, w.gr1);  // dz3
+    l4_bwd_data_kernel<<<grid1d(4 * npix, kThreads), kThreads, 0, s>>>((int)L, C, params_dev, dlogits_dev, w.z3, w.gb1,
+                                                                     w.gr1);  // dz3
     // layer 3
     int64_t n_tc = 0;
     rc = launch_wgrad_tc((int)L, C, w.a2, w.gb1, w.gr1, w.partial, w.n_cta, s, &n_tc);
     if (rc) return rc;
     reduce(kN2 + kCh, kN2, kOffW3, kOffB3, n_tc);
-    rc = launch_ring_bwd((int)L, C, params_dev, kOffW3, w.gb1, w.z2, w.db, w.gb2, w.gr2, s);  // dz2
+    rc = launch_ring_bwd((int)L, C, params_dev, kOffW3, w.gb1, w.z2, nullptr, nullptr, nullptr, w.gb2, w.gr2, s);  // dz2
     if (rc) return rc;
     // layer 2
     rc = launch_wgrad_tc((int)L, C, w.a1, w.gb2, w.gr2, w.partial, w.n_cta, s, &n_tc);
     if (rc) return rc;
     reduce(kN2 + kCh, kN2, kOffW2, kOffB2, n_tc);
-    rc = launch_ring_bwd((int)L, C, params_dev, kOffW2, w.gb2, w.z1, w.da, nullptr, nullptr, s);  // dz1
+    rc = launch_ring_bwd((int)L, C, params_dev, kOffW2, w.gb2, nullptr, w.pat, w.tg, w.da, nullptr, nullptr, s);  // dz1
     if (rc) return rc;
     // layer 1
     wgrad_thin_kernel<false><<<(unsigned)n_thin, 32 * kThinWarps, 0, s>>>(ch, C, w.da, nullptr, nullptr, w.partial);
