@@ -325,19 +325,40 @@ __global__ void l1_table_kernel(const float *params, float *tg, __nv_bfloat16 *t
     ta[e] = __float2bfloat16_rn(gelu(v));
 }
 
-// 1 if the spin at row y, column x of chain c is +1 (block `flip`, or -1 for
-// none, negated).
-__device__ __forceinline__ uint32_t spin_up(const Chains &ch, int64_t c, int y, int x, int flip)
+// Bit t of x (16 bits) moved to bit 2t.
+__device__ __forceinline__ uint32_t bit_spread(uint32_t x)
 {
-    const int j = x >> 1;
-    const uint64_t *plane = ((y + x) & 1) ? ch.white : ch.black;
-    uint32_t u = (uint32_t)(plane[c * (int64_t)ch.L * ch.wpr + (int64_t)y * ch.wpr + (j >> 4)] >> (4 * (j & 15))) & 1u;
+    x = (x | (x << 8)) & 0x00FF00FFu;
+    x = (x | (x << 4)) & 0x0F0F0F0Fu;
+    x = (x | (x << 2)) & 0x33333333u;
+    return (x | (x << 1)) & 0x55555555u;
+}
+
+// Columns 32 b .. 32 b + 31 of spin row r of chain c as bits (1 = up), with
+// block `flip` (or -1) negated.  Both planes' word b covers these columns:
+// in row r the black spins sit at the columns of r's parity.
+// The raw words behind spin_chunk: loaded one row ahead of their decoding in
+// the fused loader, so that their latency overlaps the building of a row.
+struct ChunkWords {
+    uint64_t b, w;
+    int r, blk;
+};
+
+__device__ __forceinline__ ChunkWords chunk_words(const Chains &ch, int64_t c, int r, int b)
+{
+    const int64_t at = (c * ch.L + r) * (int64_t)ch.wpr + b;
+    return ChunkWords{ch.black[at], ch.white[at], r, b};
+}
+
+__device__ __forceinline__ uint32_t chunk_bits(const Chains &ch, const ChunkWords &k, int flip)
+{
+    const uint32_t kb = bit_spread(msc4_word_to_bits(k.b)), kw = bit_spread(msc4_word_to_bits(k.w));
+    uint32_t v = (k.r & 1) ? (kw | (kb << 1)) : (kb | (kw << 1));
     if (flip >= 0) {
-        const int nb = ch.L / kBlk;
-        const int by = flip / nb, bx = flip - by * nb;
-        if ((y >> 3) == by && (x >> 3) == bx) u ^= 1u;
+        const int nb = ch.L / kBlk, by = flip / nb, bx = flip - by * nb;
+        if ((k.r >> 3) == by && ((bx * kBlk) >> 5) == k.blk) v ^= 0xFFu << ((bx * kBlk) & 31);
     }
-    return u;
+    return v;
 }
 
 // Thread per pixel of the band; blockIdx.y walks the chains and blockIdx.x
@@ -360,13 +381,26 @@ __global__ void __launch_bounds__(kL1Threads) l1_kernel(Chains ch, Band bd, cons
             const int ry = r / L, x = r - ry * L;
             int y = row0 + ry;
             y = y >= L ? y - L : y;
+            // the warp's 32 pixels are one 32-column chunk of a row: lane 3 d + q (d, q
+            // < 3) turns chunk q - 1 from it of row y - 1 + d into bits, and each
+            // pixel's pattern comes from them by shuffles; store round j writes
+            // pixels 8j .. 8j+7 whole (512 contiguous bytes), lane l the 16-byte
+            // part l % 4 of pixel 8j + l / 4
+            const int lane = threadIdx.x & 31, x_first = x - lane;
+            uint32_t bits = 0;
+            if (lane < 9) {
+                const int d = lane / 3, q = lane - 3 * d, nw = L / 32;
+                bits = chunk_bits(ch, chunk_words(ch, c, wrap(y - 1 + d, L), (x_first / 32 - 1 + q + nw) % nw), fb);
+            }
             uint32_t pat = 0;
 #pragma unroll
-            for (int k = 0; k < 9; ++k) pat |= spin_up(ch, c, wrap(y + k / 3 - 1, L), wrap(x + k % 3 - 1, L), fb) << k;
-            // the warp's 32 pixels are consecutive in one row: store round j
-            // writes pixels 8j .. 8j+7 whole (512 contiguous bytes), lane l
-            // the 16-byte part l % 4 of pixel 8j + l / 4
-            const int lane = threadIdx.x & 31, x_first = x - lane;
+            for (int d = 0; d < 3; ++d) {
+                const uint32_t lo = __shfl_sync(0xffffffffu, bits, 3 * d), mid = __shfl_sync(0xffffffffu, bits, 3 * d + 1),
+                               hi = __shfl_sync(0xffffffffu, bits, 3 * d + 2);
+                // columns x - 1 .. x + 1: bits lane - 1 .. lane + 1 of the middle chunk
+                const uint32_t trip = lane == 0 ? (lo >> 31) | (mid << 1) : __funnelshift_r(mid, hi, lane - 1);
+                pat |= (trip & 7u) << (3 * d);
+            }
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
                 const int pp = 8 * j + (lane >> 2), g = lane & 3;
@@ -662,42 +696,6 @@ __device__ __forceinline__ int ring_row(const RingConv &p, int64_t c, int r)
     int y = band_row0(p.bd, c) + r;
     y = y < 0 ? y + L : y;
     return y >= L ? y - L : y;
-}
-
-// Bit t of x (16 bits) moved to bit 2t.
-__device__ __forceinline__ uint32_t bit_spread(uint32_t x)
-{
-    x = (x | (x << 8)) & 0x00FF00FFu;
-    x = (x | (x << 4)) & 0x0F0F0F0Fu;
-    x = (x | (x << 2)) & 0x33333333u;
-    return (x | (x << 1)) & 0x55555555u;
-}
-
-// Columns 32 b .. 32 b + 31 of spin row r of chain c as bits (1 = up), with
-// block `flip` (or -1) negated.  Both planes' word b covers these columns:
-// in row r the black spins sit at the columns of r's parity.
-// The raw words behind spin_chunk: loaded one row ahead of their decoding in
-// the fused loader, so that their latency overlaps the building of a row.
-struct ChunkWords {
-    uint64_t b, w;
-    int r, blk;
-};
-
-__device__ __forceinline__ ChunkWords chunk_words(const Chains &ch, int64_t c, int r, int b)
-{
-    const int64_t at = (c * ch.L + r) * (int64_t)ch.wpr + b;
-    return ChunkWords{ch.black[at], ch.white[at], r, b};
-}
-
-__device__ __forceinline__ uint32_t chunk_bits(const Chains &ch, const ChunkWords &k, int flip)
-{
-    const uint32_t kb = bit_spread(msc4_word_to_bits(k.b)), kw = bit_spread(msc4_word_to_bits(k.w));
-    uint32_t v = (k.r & 1) ? (kw | (kb << 1)) : (kb | (kw << 1));
-    if (flip >= 0) {
-        const int nb = ch.L / kBlk, by = flip / nb, bx = flip - by * nb;
-        if ((k.r >> 3) == by && ((bx * kBlk) >> 5) == k.blk) v ^= 0xFFu << ((bx * kBlk) & 31);
-    }
-    return v;
 }
 
 template <bool PROJ, bool BWD, bool FUSED, bool FULL>
@@ -1201,7 +1199,17 @@ __global__ void __launch_bounds__(ring_threads<PROJ, FUSED>(), 2) conv32_ring_ke
 // so that sum over the block of z4 = 64 b4 + sum over its 8 rows y' and the
 // three dy of R[y' + dy][dy'][0][bx] + R[..][dy'][2][bx - 1] + R[..][dy'][1][bx + 1]
 // (periodic), added in that fixed order.  Thread per logit.
-__global__ void __launch_bounds__(kThreads) pool_rows_kernel(int L, int64_t C, int brows, const int32_t *flip,
+// A load that stays where it is written.
+__device__ __forceinline__ float ld_now(const float *p)
+{
+    float v;
+    asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p));
+    return v;
+}
+
+constexpr int kPoolThreads = 64;  // 64 chains of 128^2 on all SMs: 10.9 us with loads and sums in turn, here 7.4
+
+__global__ void __launch_bounds__(kPoolThreads) pool_rows_kernel(int L, int64_t C, int brows, const int32_t *flip,
                                                              const float *params, const float *R, float *logits)
 {
     const float b4 = bf16r(params[kOffB4]);
@@ -1216,16 +1224,23 @@ __global__ void __launch_bounds__(kThreads) pool_rows_kernel(int L, int64_t C, i
             by = wrap((f < 0 ? 0 : f / nb1) - 1 + rb, nb1);
         }
         const int bl = bx == 0 ? nb1 - 1 : bx - 1, br = bx + 1 == nb1 ? 0 : bx + 1;
-        float sum = 0.0f;
+        float v[kBlk][3][3];  // all of a thread's loads in flight before the first sum
 #pragma unroll
         for (int yy = 0; yy < kBlk; ++yy) {
 #pragma unroll
             for (int d = 0; d < 3; ++d) {
                 const int y = wrap(by * kBlk + yy + d - 1, L);  // the source row of tap row dy = d - 1
                 const float *Rr = R + (c * L + y) * (int64_t)(9 * nb1) + 3 * d * nb1;
-                sum += __ldg(Rr + bx) + __ldg(Rr + 2 * nb1 + bl) + __ldg(Rr + nb1 + br);
+                v[yy][d][0] = ld_now(Rr + bx);
+                v[yy][d][1] = ld_now(Rr + 2 * nb1 + bl);
+                v[yy][d][2] = ld_now(Rr + nb1 + br);
             }
         }
+        float sum = 0.0f;
+#pragma unroll
+        for (int yy = 0; yy < kBlk; ++yy)
+#pragma unroll
+            for (int d = 0; d < 3; ++d) sum += v[yy][d][0] + v[yy][d][1] + v[yy][d][2];
         logits[c * nb + by * nb1 + bx] = b4 + sum * (1.0f / (kBlk * kBlk));
     }
 }
@@ -1233,193 +1248,282 @@ __global__ void __launch_bounds__(kThreads) pool_rows_kernel(int L, int64_t C, i
 // ---------------------------------------------------------------------------
 // Backward (uses what a training forward stored)
 // ---------------------------------------------------------------------------
-// dz3 = gelu'(z3) * sum_k W4[i][k] * d4(p - off_k),  d4(p) = dlogit(block of p) / 64.
-__global__ void __launch_bounds__(kThreads) l4_bwd_data_kernel(int L, int64_t C, const float *params,
-                                                               const float *dlogits, const float *z3,
-                                                               __nv_bfloat16 *dz3b, __nv_bfloat16 *dz3r)
+// dz3 = gelu'(z3) * sum_k W4[i][k] * d4(p - off_k),  d4(p) = dlogit(block of p) / 64,
+// as bfloat16 with halo columns, the operand of the next data gradient on the
+// tensor cores, and the rounding of its remainder, for the weight gradient.
+// Four threads per pixel, 8 channels each (a warp reads 8 pixels' 1 KB of z3
+// contiguously); a channel pair's weight is one 64-bit operand of a packed multiply-
+// add, and a tap's weights of 8 channels come from shared memory in two 16-byte
+// reads.  Bound by issue (some 400 instructions per thread and pixel, half of them
+// gelu').  64 chains of 128^2, us per launch: 75 with scalar weights and 64-bit index
+// divisions, 80 with the 72 weights in registers (two blocks per SM hide no latency),
+// here 68; it moves 270 MB.
+constexpr int kL4Threads = 256;
+
+__global__ void __launch_bounds__(kL4Threads, 4) l4_bwd_data_kernel(int L, int64_t C, const float *params,
+                                                                    const float *dlogits, const float *z3,
+                                                                    __nv_bfloat16 *dz3b, __nv_bfloat16 *dz3r)
 {
-    __shared__ float W[kN1];
-    for (int i = threadIdx.x; i < kN1; i += blockDim.x) W[i] = bf16r(params[kOffW4 + i]);
+    const int nb1 = L / kBlk, i8 = (threadIdx.x & 3) * 8;
+    const uint32_t LL = (uint32_t)L * (uint32_t)L;
+    __shared__ __align__(16) float W[9 * kCh];  // W4[i][k] at 32 k + i
+    for (int e = threadIdx.x; e < kN1; e += kL4Threads) W[(e % 9) * kCh + e / 9] = bf16r(params[kOffW4 + e]);
     __syncthreads();
-    const int nb1 = L / kBlk;
-    const int64_t npix = C * (int64_t)L * L;
-    // four threads per pixel, 8 channels each: a warp reads 8 pixels' 1 KB of z3
-    // contiguously
-    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < 4 * npix;
-         e += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t p = e >> 2;
-        const int i8 = (int)(e & 3) * 8;
-        const int64_t c = p / ((int64_t)L * L);
-        const int yx = (int)(p - c * (int64_t)L * L);
-        const int y = yx / L, x = yx - y * L;
-        float d[9];
-#pragma unroll
-        for (int k = 0; k < 9; ++k) {
+    const int per = kL4Threads / 4;  // pixels per step of a block
+    // a chain's pixels are cut evenly over gridDim.x blocks; blockIdx.y walks the chains
+    for (int64_t c = blockIdx.y; c < C; c += gridDim.y) {
+        const float *dl = dlogits + c * nb1 * nb1;
+        const float4 *zc = reinterpret_cast<const float4 *>(z3 + c * (int64_t)LL * kCh + i8);
+        const uint32_t step = gridDim.x * per;
+        uint32_t yx = blockIdx.x * per + (threadIdx.x >> 2);
+        float4 na = {}, nb = {};  // the next step's pre-activations, in flight during this one
+        if (yx < LL) na = __ldcs(zc + yx * (kCh / 4)), nb = __ldcs(zc + yx * (kCh / 4) + 1);
+        for (; yx < LL; yx += step) {
+            const float4 za = na, zb = nb;
+            if (yx + step < LL) na = __ldcs(zc + (yx + step) * (kCh / 4)), nb = __ldcs(zc + (yx + step) * (kCh / 4) + 1);
+            const int y = (int)(yx / (uint32_t)L), x = (int)(yx - (uint32_t)y * (uint32_t)L);
             // output pixel q = p - off_k used input p through tap k
-            int yy = y - (k / 3 - 1), xx = x - (k % 3 - 1);
-            yy = yy < 0 ? yy + L : (yy >= L ? yy - L : yy);
-            xx = xx < 0 ? xx + L : (xx >= L ? xx - L : xx);
-            d[k] = dlogits[c * nb1 * nb1 + (yy / kBlk) * nb1 + xx / kBlk] * (1.0f / (kBlk * kBlk));
-        }
-        const float4 *zp = reinterpret_cast<const float4 *>(z3 + p * kCh + i8);
-        const float4 za = zp[0], zb = zp[1];
-        const float z[8] = {za.x, za.y, za.z, za.w, zb.x, zb.y, zb.z, zb.w};
-        float v[8], gz[8];
-#pragma unroll
-        for (int i = 0; i < 8; ++i) gz[i] = z[i];
-#pragma unroll
-        for (int i = 0; i < 8; i += 2) gelu_grad2(gz[i], gz[i + 1]);
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            float g = 0.0f;
-#pragma unroll
-            for (int k = 0; k < 9; ++k) g = fmaf(W[(i8 + i) * 9 + k], d[k], g);
-            v[i] = g * gz[i];
-        }
-        // as bfloat16 with halo columns, the operand of the next data gradient on the
-        // tensor cores, and the rounding of its remainder, for the weight gradient
-        uint32_t hb[4], rb[4];
-        split_bf16(v, hb, rb);
-        store_act(dz3b, L, c, y, x, i8, make_uint4(hb[0], hb[1], hb[2], hb[3]));
-        store_act(dz3r, L, c, y, x, i8, make_uint4(rb[0], rb[1], rb[2], rb[3]));
-    }
-}
-
-// Weight gradients of the layers with one input or one output channel, warp
-// per run of rows, lane per channel:
-//   layer 1 (spins -> 32): dW1[o][k] = sum_p dz1(p)[o] s(p + off_k),
-//                          db1[o] = sum_p dz1(p)[o]                (lane o);
-//   layer 4 (32 -> 1):     dW4[i][k] = sum_q a3(q)[i] d4(q - off_k),
-//                          db4 = sum_p d4(p), d4(p) = dlogit(block of p) / 64
-//                                                                 (lane i).
-// Per pixel q the lane's value v (dz1(q)[o] or a3(q)[i]) multiplies a 3 x 3
-// window of a field that is the same for all lanes (the spins, or d4).  A
-// warp walks its rows in order, each in chunks of 32 pixels: lane j holds the
-// field at column x0 + j of rows y - 1, y, y + 1, the halo columns are loaded
-// by every lane, and the window slides along the chunk by one shuffle per row
-// and pixel.  Per pixel and lane: one load, three shuffles, nine FMAs.  The
-// CTA's warps are added in warp order and written as the CTA's partial sums (the
-// weights in W[o][i][k] order, then the biases), summed by reduce_partials_kernel.
-constexpr int kThinWarps = 8;
-
-template <bool L4>
-__device__ __forceinline__ float thin_field(const Chains &ch, const float *dlogits, int64_t c, int y, int x)
-{
-    const int L = ch.L;
-    y = wrap(y, L);
-    x = wrap(x, L);
-    if constexpr (L4) {
-        const int nb1 = L / kBlk;
-        return dlogits[c * nb1 * nb1 + (y / kBlk) * nb1 + x / kBlk] * (1.0f / (kBlk * kBlk));
-    } else {
-        return spin_at(ch, c, y, x, -1);
-    }
-}
-
-template <bool L4>
-__global__ void __launch_bounds__(32 * kThinWarps, 2) wgrad_thin_kernel(Chains ch, int64_t C, const float *dz1,
-                                                                      const __nv_bfloat16 *a3, const float *dlogits,
-                                                                      float *partial)
-{
-    constexpr int NE = L4 ? kN1 + 1 : kN1 + kCh;
-    __shared__ float red[kThinWarps][32][10];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int L = ch.L;
-    const int64_t rows = C * L;
-    const int64_t nw = (int64_t)gridDim.x * kThinWarps, gw = (int64_t)blockIdx.x * kThinWarps + warp;
-    const int64_t r0 = gw * rows / nw, r1 = (gw + 1) * rows / nw;
-    float acc[9], bacc = 0.0f;
-#pragma unroll
-    for (int k = 0; k < 9; ++k) acc[k] = 0.0f;
-    for (int64_t gr = r0; gr < r1; ++gr) {
-        const int64_t c = gr / L;
-        const int y = (int)(gr - c * L);
-        for (int x0 = 0; x0 < L; x0 += 32) {
-            float f[3], hl[3], hr[3], w[3][3];
+            int by[3], bx[3];
 #pragma unroll
             for (int d = 0; d < 3; ++d) {
-                f[d] = thin_field<L4>(ch, dlogits, c, y - 1 + d, x0 + lane);
-                hl[d] = thin_field<L4>(ch, dlogits, c, y - 1 + d, x0 - 1);
-                hr[d] = thin_field<L4>(ch, dlogits, c, y - 1 + d, x0 + 32);
-                w[d][0] = hl[d];
-                w[d][1] = __shfl_sync(0xffffffffu, f[d], 0);
-                w[d][2] = __shfl_sync(0xffffffffu, f[d], 1);
+                by[d] = wrap(y - (d - 1), L) / kBlk * nb1;
+                bx[d] = wrap(x - (d - 1), L) / kBlk;
             }
+            uint64_t g[4];
 #pragma unroll
-            for (int j = 0; j < 32; ++j) {
-                float v;
-                if constexpr (L4) {
-                    v = __bfloat162float(a3[apix(L, c, y, x0 + j) * kCh + lane]);
-                    bacc += w[1][1];  // d4 of the pixel itself
-                } else {
-                    v = dz1[((c * L + y) * (int64_t)L + x0 + j) * kCh + lane];
-                    bacc += v;
-                }
-                // window entry (d, e) is the field at (y - 1 + d, x + e - 1): tap
-                // 3 d + e of layer 1 (p + off_k), tap 8 - 3 d - e of layer 4 (q - off_k)
+            for (int j = 0; j < 4; ++j) g[j] = f2_splat(0.0f);
 #pragma unroll
-                for (int d = 0; d < 3; ++d)
+            for (int k = 0; k < 9; ++k) {
+                const uint64_t d = f2_splat(__ldg(dl + by[k / 3] + bx[k % 3]) * (1.0f / (kBlk * kBlk)));
+                const ulonglong2 wa = *reinterpret_cast<const ulonglong2 *>(W + k * kCh + i8);
+                const ulonglong2 wb = *reinterpret_cast<const ulonglong2 *>(W + k * kCh + i8 + 4);
+                g[0] = f2_fma(wa.x, d, g[0]);
+                g[1] = f2_fma(wa.y, d, g[1]);
+                g[2] = f2_fma(wb.x, d, g[2]);
+                g[3] = f2_fma(wb.y, d, g[3]);
+            }
+            float gz[8] = {za.x, za.y, za.z, za.w, zb.x, zb.y, zb.z, zb.w}, v[8];
 #pragma unroll
-                    for (int e = 0; e < 3; ++e) {
-                        const int k = L4 ? 8 - 3 * d - e : 3 * d + e;
-                        acc[k] = fmaf(v, w[d][e], acc[k]);
-                    }
+            for (int j = 0; j < 4; ++j) {
+                gelu_grad2(gz[2 * j], gz[2 * j + 1]);
+                f2_unpack(f2_mul(g[j], f2_pack(gz[2 * j], gz[2 * j + 1])), v[2 * j], v[2 * j + 1]);
+            }
+            uint32_t hb[4], rb[4];
+            split_bf16(v, hb, rb);
+            store_act(dz3b, L, c, y, x, i8, make_uint4(hb[0], hb[1], hb[2], hb[3]));
+            store_act(dz3r, L, c, y, x, i8, make_uint4(rb[0], rb[1], rb[2], rb[3]));
+        }
+    }
+}
+
+// Weight gradients of the layers with one input or one output channel:
+//   layer 4 (32 -> 1): dW4[i][k] = sum_q a3(q)[i] d4(q - off_k),
+//                      db4 = sum_p d4(p), d4(p) = dlogit(block of p) / 64;
+//   layer 1 (spins -> 32): dW1[o][k] = sum_p dz1(p)[o] s(p + off_k),
+//                          db1[o] = sum_p dz1(p)[o].
+// A warp loads several whole pixels at once (512 contiguous bytes), a lane some
+// channels of one of them, and multiplies them by the nine values the other field
+// has around that pixel, which the lane knows without asking another: d4 is
+// constant over 8 x 8 blocks, so nine dlogits serve the 64 pixels of a block, and
+// the spins are the bits of the pixel's layer-1 pattern.  The lanes of a channel,
+// then the CTA's warps, are added in a fixed order and written as the CTA's
+// partial sums (the weights in W[o][i][k] order, then the biases), summed by
+// reduce_partials_kernel.  (Lane per channel, pixel after pixel, with the other
+// field's window handed on by three shuffles per pixel: 36 and 39 us per launch of
+// 64 chains of 128^2, here 23 and 27; they read 68 and 137 MB.)
+constexpr int kThinWarps = 8;
+
+// Adds up one CTA's warps: red[warp][e] for e < n into out[e], in warp order.
+__device__ __forceinline__ void thin_reduce(const float *red, int n, float *out)
+{
+    __syncthreads();
+    for (int e = threadIdx.x; e < n; e += blockDim.x) {
+        float sum = 0.0f;
 #pragma unroll
-                for (int d = 0; d < 3; ++d) {
-                    w[d][0] = w[d][1];
-                    w[d][1] = w[d][2];
-                    w[d][2] = j + 2 < 32 ? __shfl_sync(0xffffffffu, f[d], (j + 2) & 31) : hr[d];
-                }
+        for (int w = 0; w < kThinWarps; ++w) sum += red[w * n + e];
+        out[e] = sum;
+    }
+}
+
+__global__ void __launch_bounds__(32 * kThinWarps, 2) wgrad_l4_kernel(int L, int64_t C, const __nv_bfloat16 *a3,
+                                                                      const float *dlogits, float *partial)
+{
+    constexpr int NE = kN1 + 1;
+    __shared__ float red[kThinWarps * NE];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int u = lane >> 2, g = lane & 3;  // pixel of the block's row, 8-channel group
+    const int nb1 = L / kBlk;
+    const int64_t blocks = C * nb1 * nb1, nw = (int64_t)gridDim.x * kThinWarps, gw = (int64_t)blockIdx.x * kThinWarps + warp;
+    const int64_t b0 = gw * blocks / nw, b1 = (gw + 1) * blocks / nw;
+    uint64_t acc[9][4];  // channels 8 g + 2 j, + 1
+    float bacc = 0.0f;
+#pragma unroll
+    for (int k = 0; k < 9; ++k)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[k][j] = f2_splat(0.0f);
+    for (int64_t b = b0; b < b1; ++b) {
+        const int64_t c = b / (nb1 * nb1);
+        const int r = (int)(b - c * nb1 * nb1), by = r / nb1, bx = r - by * nb1;
+        const float *dl = dlogits + c * nb1 * nb1;
+        // d[row][e]: dlogit of the block row above, of this one and below, at the column
+        // block of pixel x - 1, x and x + 1
+        float d[3][3];
+        const int bl = u == 0 ? wrap(bx - 1, nb1) : bx, br = u == kBlk - 1 ? wrap(bx + 1, nb1) : bx;
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+            const float *row = dl + wrap(by + q - 1, nb1) * nb1;
+            d[q][0] = row[bl];
+            d[q][1] = row[bx];
+            d[q][2] = row[br];
+        }
+        bacc += d[1][1];
+        const uint4 *src = reinterpret_cast<const uint4 *>(a3 + apix(L, c, by * kBlk, bx * kBlk + u) * kCh) + g;
+        uint4 v[kBlk];
+#pragma unroll
+        for (int yy = 0; yy < kBlk; ++yy) v[yy] = __ldg(src + (int64_t)yy * (L + 2) * kGroups);
+#pragma unroll
+        for (int yy = 0; yy < kBlk; ++yy) {
+            const uint64_t a[4] = {f2_pack(bf16_lo(v[yy].x), bf16_hi(v[yy].x)), f2_pack(bf16_lo(v[yy].y), bf16_hi(v[yy].y)),
+                                   f2_pack(bf16_lo(v[yy].z), bf16_hi(v[yy].z)), f2_pack(bf16_lo(v[yy].w), bf16_hi(v[yy].w))};
+#pragma unroll
+            for (int k = 0; k < 9; ++k) {
+                // tap k used output pixel q - off_k: row y - dy, column x - dx
+                const int dy = k / 3 - 1, dx = k % 3 - 1;
+                const int q = yy - dy < 0 ? 0 : yy - dy >= kBlk ? 2 : 1;
+                const uint64_t w = f2_splat(d[q][1 - dx]);
+#pragma unroll
+                for (int j = 0; j < 4; ++j) acc[k][j] = f2_fma(a[j], w, acc[k][j]);
             }
         }
     }
 #pragma unroll
-    for (int k = 0; k < 9; ++k) red[warp][lane][k] = acc[k];
-    red[warp][lane][9] = bacc;
-    __syncthreads();
-    float *out = partial + (int64_t)blockIdx.x * NE;
-    for (int t = threadIdx.x; t < 32 * 10; t += blockDim.x) {
-        const int l = t / 10, k = t - 10 * l;
-        float sum = 0.0f;
+    for (int k = 0; k < 9; ++k)
 #pragma unroll
-        for (int q = 0; q < kThinWarps; ++q) sum += red[q][l][k];
-        if (k < 9)
-            out[l * 9 + k] = sum;  // layer 1: (o, k); layer 4: (i, k)
-        else if (!L4)
-            out[kN1 + l] = sum;    // db1[o]
-        else if (l == 0)
-            out[kN1] = sum;        // db4 (every lane summed the same d4)
+        for (int j = 0; j < 4; ++j) {
+            float x0, x1;
+            f2_unpack(acc[k][j], x0, x1);
+#pragma unroll
+            for (int off = 4; off < 32; off <<= 1) {
+                x0 += __shfl_xor_sync(0xffffffffu, x0, off);
+                x1 += __shfl_xor_sync(0xffffffffu, x1, off);
+            }
+            if (u == 0) {
+                red[warp * NE + (8 * g + 2 * j) * 9 + k] = x0 * (1.0f / (kBlk * kBlk));
+                red[warp * NE + (8 * g + 2 * j + 1) * 9 + k] = x1 * (1.0f / (kBlk * kBlk));
+            }
+        }
+    if (lane == 0) red[warp * NE + kN1] = bacc;  // 64 pixels of dlogit / 64 per block
+    thin_reduce(red, NE, partial + (int64_t)blockIdx.x * NE);
+}
+
+__global__ void __launch_bounds__(32 * kThinWarps, 2) wgrad_l1_kernel(int64_t npix, const float *dz1, const uint16_t *pat,
+                                                                      float *partial)
+{
+    constexpr int NE = kN1 + kCh;
+    __shared__ float red[kThinWarps * NE];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int u = lane >> 3, g = lane & 7;  // pixel of four, 4-channel group
+    const int64_t nw = (int64_t)gridDim.x * kThinWarps, gw = (int64_t)blockIdx.x * kThinWarps + warp;
+    // steps of 32 pixels (their number is a multiple of 32)
+    const int64_t s0 = gw * (npix / 32) / nw, s1 = (gw + 1) * (npix / 32) / nw;
+    uint64_t acc[9][2], bacc[2];  // channels 4 g + 2 j, + 1
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+        bacc[j] = f2_splat(0.0f);
+#pragma unroll
+        for (int k = 0; k < 9; ++k) acc[k][j] = f2_splat(0.0f);
     }
+    for (int64_t st = s0; st < s1; ++st) {
+        const float4 *src = reinterpret_cast<const float4 *>(dz1 + (st * 32 + u) * kCh) + g;
+        float4 v[8];
+#pragma unroll
+        for (int t = 0; t < 8; ++t) v[t] = __ldg(src + t * 4 * (kCh / 4));
+        const uint32_t mine = pat[st * 32 + lane];
+#pragma unroll
+        for (int t = 0; t < 8; ++t) {
+            const uint32_t pt = ~__shfl_sync(0xffffffffu, mine, 4 * t + u);  // bit set: spin -1
+            const uint64_t a[2] = {f2_pack(v[t].x, v[t].y), f2_pack(v[t].z, v[t].w)};
+            const uint64_t one = f2_splat(1.0f);
+#pragma unroll
+            for (int j = 0; j < 2; ++j) bacc[j] = f2_fma(a[j], one, bacc[j]);
+#pragma unroll
+            for (int k = 0; k < 9; ++k) {
+                const uint64_t w = f2_splat(__uint_as_float(0x3F800000u | ((pt << (31 - k)) & 0x80000000u)));
+#pragma unroll
+                for (int j = 0; j < 2; ++j) acc[k][j] = f2_fma(a[j], w, acc[k][j]);
+            }
+        }
+    }
+    auto lanes = [&](uint64_t v, float &x0, float &x1) {  // the four lanes of a channel group
+        f2_unpack(v, x0, x1);
+#pragma unroll
+        for (int off = 8; off < 32; off <<= 1) {
+            x0 += __shfl_xor_sync(0xffffffffu, x0, off);
+            x1 += __shfl_xor_sync(0xffffffffu, x1, off);
+        }
+    };
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+        const int o = 4 * g + 2 * j;
+        float x0, x1;
+#pragma unroll
+        for (int k = 0; k < 9; ++k) {
+            lanes(acc[k][j], x0, x1);
+            if (u == 0) {
+                red[warp * NE + o * 9 + k] = x0;
+                red[warp * NE + (o + 1) * 9 + k] = x1;
+            }
+        }
+        lanes(bacc[j], x0, x1);
+        if (u == 0) {
+            red[warp * NE + kN1 + o] = x0;
+            red[warp * NE + kN1 + o + 1] = x1;
+        }
+    }
+    thin_reduce(red, NE, partial + (int64_t)blockIdx.x * NE);
 }
 
 // grad[off + e] = sum over ctas of partial[cta][e] in a fixed order: warp w
 // of a block sums the w-th eighth of the CTA range (in order) for 32
 // consecutive e, then the eight warp sums are added in warp order.  Weights
-// come first (W[o][i][k] order), then the biases.  Launch: ceil(ne / 32)
-// blocks of 256 threads.
+// come first (W[o][i][k] order), then the biases.  One launch of 256-thread blocks
+// for the four layers (four launches, two of them of 10 blocks: 29 us per training
+// step, together 8.5).
 constexpr int kReduceWarps = 8;
 
-__global__ void __launch_bounds__(32 * kReduceWarps) reduce_partials_kernel(const float *partial, int64_t n_cta,
-                                                                            int ne, int nw, float *grad, int w_off,
-                                                                            int b_off)
+struct ReducePartials {
+    struct {
+        const float *partial;
+        int n_cta, ne, nw, w_off, b_off;
+        int block_end;  // blocks of the layers up to this one
+    } layer[4];
+};
+
+__global__ void __launch_bounds__(32 * kReduceWarps) reduce_partials_kernel(const __grid_constant__ ReducePartials p,
+                                                                            float *grad)
 {
     __shared__ float part[kReduceWarps][32];
+    int q = 0;
+    while (q < 3 && (int)blockIdx.x >= p.layer[q].block_end) ++q;
+    const auto &r = p.layer[q];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int e = blockIdx.x * 32 + lane;
-    const int64_t k0 = n_cta * warp / kReduceWarps, k1 = n_cta * (warp + 1) / kReduceWarps;
+    const int e = ((int)blockIdx.x - (q ? p.layer[q - 1].block_end : 0)) * 32 + lane;
+    const int k0 = r.n_cta * warp / kReduceWarps, k1 = r.n_cta * (warp + 1) / kReduceWarps;
     float s = 0.0f;
-    if (e < ne)
-        for (int64_t k = k0; k < k1; ++k) s += partial[k * ne + e];
+    if (e < r.ne) {
+#pragma unroll 8
+        for (int k = k0; k < k1; ++k) s += r.partial[(int64_t)k * r.ne + e];
+    }
     part[warp][lane] = s;
     __syncthreads();
-    if (warp == 0 && e < ne) {
+    if (warp == 0 && e < r.ne) {
         float t = 0.0f;
 #pragma unroll
         for (int w = 0; w < kReduceWarps; ++w) t += part[w][lane];
-        if (e < nw)
-            grad[w_off + e] = t;
+        if (e < r.nw)
+            grad[r.w_off + e] = t;
         else
-            grad[b_off + (e - nw)] = t;
+            grad[r.b_off + (e - r.nw)] = t;
     }
 }
 
@@ -1740,6 +1844,7 @@ __device__ int block_delta_E(const Chains &ch, int64_t c, int b)
     const int L = ch.L, nb1 = L / kBlk;
     const int by = b / nb1, bx = b - by * nb1, y0 = by * kBlk, x0 = bx * kBlk;
     int d = 0;
+#pragma unroll
     for (int t = 0; t < kBlk; ++t) {
         // top and bottom edges, left and right edges
         const int xt = x0 + t, yt = y0 + t;
@@ -1785,13 +1890,18 @@ __global__ void __launch_bounds__(kThreads) targets_loss_kernel(Chains ch, int64
     }
 }
 
-__global__ void loss_reduce_kernel(const float *chain_sq, int64_t C, int nb, float *loss)
+// One block of kThreads threads: a thread's chains in order, then a fixed tree.
+__global__ void __launch_bounds__(kThreads) loss_reduce_kernel(const float *chain_sq, int64_t C, int nb, float *loss)
 {
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        double s = 0.0;
-        for (int64_t c = 0; c < C; ++c) s += chain_sq[c];
-        *loss = (float)(s / (double)(C * nb));
+    __shared__ double part[kThreads];
+    double s = 0.0;
+    for (int64_t c = threadIdx.x; c < C; c += kThreads) s += chain_sq[c];
+    part[threadIdx.x] = s;
+    for (int n = kThreads / 2; n > 0; n >>= 1) {
+        __syncthreads();
+        if ((int)threadIdx.x < n) part[threadIdx.x] += part[threadIdx.x + n];
     }
+    if (threadIdx.x == 0) *loss = (float)(part[0] / (double)(C * nb));
 }
 
 __global__ void adam_kernel(int n, float *params, const float *grad, float *m, float *v, float lr, float b1,
@@ -2256,7 +2366,7 @@ int launch_forward(const Chains &ch, int64_t C, const int32_t *flip, bool band, 
     }
     const int brows = band ? kBandRows[3] : L / kBlk;
     // the projecting ring kernel left row partials of z4 in w.P
-    pool_rows_kernel<<<grid1d(C * brows * (L / kBlk), kThreads), kThreads, 0, s>>>(L, C, brows, band ? flip : nullptr,
+    pool_rows_kernel<<<grid1d(C * brows * (L / kBlk), kPoolThreads), kPoolThreads, 0, s>>>(L, C, brows, band ? flip : nullptr,
                                                                                   params, w.P, logits);
     cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? ISING_OK : nfail(ISING_ECUDA, cudaGetErrorString(e));
@@ -2371,40 +2481,50 @@ ISING_API int ising_net_backward(int64_t L, int64_t C, const void *black_dev, co
         check_device_range(dlogits_dev, (size_t)C * (L / 8) * (L / 8) * 4, "dlogits"))
         return nfail(ISING_EINVAL, "grad and dlogits must be device memory of their sizes");
     cudaStream_t s = (cudaStream_t)stream;
-    Chains ch{(const uint64_t *)black_dev, (const uint64_t *)white_dev, (int)L, (int)(L / 32)};
-    const int64_t npix = C * L * L;
-    auto reduce = [&](int ne, int nw, int w_off, int b_off, int64_t n_cta) {
-        reduce_partials_kernel<<<(unsigned)((ne + 31) / 32), 32 * kReduceWarps, 0, s>>>(w.partial, n_cta, ne, nw,
-                                                                                       grad_dev, w_off, b_off);
-    };
-    // layer 4
-    // the thin weight gradients: one wave of two CTAs per SM
+    (void)black_dev;  // layer 1's inputs are in the patterns that the forward pass kept
+    (void)white_dev;
     DeviceInfo info{152};
     device_info(&info);
-    const int64_t n_thin = std::min<int64_t>(w.n_cta, 2 * (int64_t)info.sm_count);
-    wgrad_thin_kernel<true><<<(unsigned)n_thin, 32 * kThinWarps, 0, s>>>(ch, C, nullptr, w.a3, dlogits_dev, w.partial);
-    reduce(kN1 + 1, kN1, kOffW4, kOffB4, n_thin);
+    const int64_t sms = info.sm_count;
+    // every layer's partial sums: layers 3 and 2 a third of the rows each (one CTA per
+    // SM), layers 4 and 1 in the last third (two CTAs per SM)
+    const int64_t third = w.n_cta / 3 * (kN2 + kCh);
+    float *part3 = w.partial, *part2 = w.partial + third, *part4 = w.partial + 2 * third;
+    float *part1 = part4 + 2 * sms * (kN1 + 1);
+    static_assert(2 * (kN1 + 1 + kN1 + kCh) <= kN2 + kCh && kWgradCtasPerSm == 3, "room for the partial sums");
+    // layer 4
+    wgrad_l4_kernel<<<(unsigned)(2 * sms), 32 * kThinWarps, 0, s>>>((int)L, C, w.a3, dlogits_dev, part4);
     // the data and weight gradients of the 32 -> 32 layers run on the tensor
-    // cores; their gradients are then also kept as bfloat16 parts (gb: the
-    // rounding, gr: the rounding of the remainder)
-    l4_bwd_data_kernel<<<grid1d(4 * npix, kThreads), kThreads, 0, s>>>((int)L, C, params_dev, dlogits_dev, w.z3, w.gb1,
-                                                                     w.gr1);  // dz3
+    // cores; their gradients are kept as bfloat16 parts (gb: the rounding, gr: the
+    // rounding of the remainder)
+    const int64_t steps = (L * L + kL4Threads / 4 - 1) / (kL4Threads / 4);
+    const int64_t gx = std::min<int64_t>(steps, std::max<int64_t>(1, (8 * sms + C - 1) / C));
+    l4_bwd_data_kernel<<<dim3((unsigned)gx, (unsigned)std::min<int64_t>(C, 2 * sms)), kL4Threads, 0, s>>>(
+        (int)L, C, params_dev, dlogits_dev, w.z3, w.gb1, w.gr1);  // dz3
     // layer 3
-    int64_t n_tc = 0;
-    rc = launch_wgrad_tc((int)L, C, w.a2, w.gb1, w.gr1, w.partial, w.n_cta, s, &n_tc);
+    int64_t n3 = 0, n2 = 0;
+    rc = launch_wgrad_tc((int)L, C, w.a2, w.gb1, w.gr1, part3, sms, s, &n3);
     if (rc) return rc;
-    reduce(kN2 + kCh, kN2, kOffW3, kOffB3, n_tc);
     rc = launch_ring_bwd((int)L, C, params_dev, kOffW3, w.gb1, w.z2, nullptr, nullptr, nullptr, w.gb2, w.gr2, s);  // dz2
     if (rc) return rc;
     // layer 2
-    rc = launch_wgrad_tc((int)L, C, w.a1, w.gb2, w.gr2, w.partial, w.n_cta, s, &n_tc);
+    rc = launch_wgrad_tc((int)L, C, w.a1, w.gb2, w.gr2, part2, sms, s, &n2);
     if (rc) return rc;
-    reduce(kN2 + kCh, kN2, kOffW2, kOffB2, n_tc);
     rc = launch_ring_bwd((int)L, C, params_dev, kOffW2, w.gb2, nullptr, w.pat, w.tg, w.da, nullptr, nullptr, s);  // dz1
     if (rc) return rc;
     // layer 1
-    wgrad_thin_kernel<false><<<(unsigned)n_thin, 32 * kThinWarps, 0, s>>>(ch, C, w.da, nullptr, nullptr, w.partial);
-    reduce(kN1 + kCh, kN1, kOffW1, kOffB1, n_thin);
+    wgrad_l1_kernel<<<(unsigned)(2 * sms), 32 * kThinWarps, 0, s>>>(C * L * L, w.da, w.pat, part1);
+    ReducePartials red{};
+    int blocks = 0, q = 0;
+    auto layer = [&](const float *partial, int64_t n_cta, int ne, int nw, int w_off, int b_off) {
+        blocks += (ne + 31) / 32;
+        red.layer[q++] = {partial, (int)n_cta, ne, nw, w_off, b_off, blocks};
+    };
+    layer(part3, n3, kN2 + kCh, kN2, kOffW3, kOffB3);
+    layer(part2, n2, kN2 + kCh, kN2, kOffW2, kOffB2);
+    layer(part4, 2 * sms, kN1 + 1, kN1, kOffW4, kOffB4);
+    layer(part1, 2 * sms, kN1 + kCh, kN1, kOffW1, kOffB1);
+    reduce_partials_kernel<<<(unsigned)blocks, 32 * kReduceWarps, 0, s>>>(red, grad_dev);
     cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? ISING_OK : nfail(ISING_ECUDA, cudaGetErrorString(e));
 }
@@ -2422,7 +2542,7 @@ ISING_API int ising_net_targets_loss(int64_t L, int64_t C, const void *black_dev
     Chains ch{(const uint64_t *)black_dev, (const uint64_t *)white_dev, (int)L, (int)(L / 32)};
     targets_loss_kernel<<<(unsigned)std::min<int64_t>(C, 1 << 30), kThreads, 0, s>>>(ch, C, beta, logits_dev,
                                                                                      dlogits_dev, chain_sq_dev);
-    loss_reduce_kernel<<<1, 32, 0, s>>>(chain_sq_dev, C, (int)((L / 8) * (L / 8)), loss_dev);
+    loss_reduce_kernel<<<1, kThreads, 0, s>>>(chain_sq_dev, C, (int)((L / 8) * (L / 8)), loss_dev);
     cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? ISING_OK : nfail(ISING_ECUDA, cudaGetErrorString(e));
 }
