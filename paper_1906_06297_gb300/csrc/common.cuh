@@ -190,33 +190,28 @@ __device__ __forceinline__ void block_reduce_add2(long long a, long long b, long
     }
 }
 
-// The same for any block size of up to 1024 threads.
-__device__ __forceinline__ void block_reduce_add2_any(long long a, long long b, long long *out)
+// The same from two 32-bit counts per thread (their sums over the block fit 32
+// bits) for blocks of up to 1024 threads: adds mul_a sum(a) + add_a and mul_b sum(b) +
+// add_b, the add terms once per block.  Two warp reductions instead of ten 64-bit
+// shuffles, which sit between a small kernel's last store and its end.
+__device__ __forceinline__ void block_count_add2(uint32_t a, uint32_t b, int mul_a, long long add_a, int mul_b,
+                                                 long long add_b, long long *out)
 {
-    __shared__ long long sa[32], sb[32];  // any block size
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-        a += __shfl_xor_sync(0xffffffffu, a, off);
-        b += __shfl_xor_sync(0xffffffffu, b, off);
-    }
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    __shared__ uint32_t sa[32], sb[32];
+    a = __reduce_add_sync(0xffffffffu, a);
+    b = __reduce_add_sync(0xffffffffu, b);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = (blockDim.x + 31) >> 5;
     if (lane == 0) {
         sa[warp] = a;
         sb[warp] = b;
     }
     __syncthreads();
     if (warp == 0) {
-        const int warps = (blockDim.x + 31) >> 5;
-        a = lane < warps ? sa[lane] : 0;
-        b = lane < warps ? sb[lane] : 0;
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) {
-            a += __shfl_xor_sync(0xffffffffu, a, off);
-            b += __shfl_xor_sync(0xffffffffu, b, off);
-        }
-        if (lane == 0) {
-            atomicAdd(reinterpret_cast<unsigned long long *>(out), (unsigned long long)a);
-            atomicAdd(reinterpret_cast<unsigned long long *>(out + 1), (unsigned long long)b);
+        a = __reduce_add_sync(0xffffffffu, lane < warps ? sa[lane] : 0u);
+        b = __reduce_add_sync(0xffffffffu, lane < warps ? sb[lane] : 0u);
+        if (lane < 2) {
+            const long long v = lane == 0 ? mul_a * (long long)a + add_a : mul_b * (long long)b + add_b;
+            atomicAdd(reinterpret_cast<unsigned long long *>(out + lane), (unsigned long long)v);
         }
     }
 }

@@ -252,9 +252,12 @@ __global__ void __launch_bounds__(kThreads, ISING_MSC4_MIN_BLOCKS)
 // kernel gather on the SMs that finish first, 17.7 instead of 5.4 us per sweep
 // of 2048^2.)  From four steps per block on, where hiding a step's loads counts
 // more than the overlap, two blocks per SM: 4096^2 16.0 -> 15.2 us, 6400^2 35.3
-// -> 33.2 (2 to 3 steps: 3200^2 10.6 -> 13.9).  Measured, us per sweep with the trace, marching kernel (at least
-// 16 rows per warp) / this one: 256^2 66 / 3.6 (the host's launch rate), 2112^2
-// 66.7 / 5.6, 4096^2 67.7 / 15.2, 8192^2 68.0 / 52.5.
+// -> 33.2 (2 to 3 steps: 3200^2 10.6 -> 13.9).  The block's observables are 32-bit
+// counts, two warp reductions each: ten 64-bit shuffles after the last store
+// cost 0.6 us of 5.55 at 2112^2 and 1.2 of 15.25 at 4096^2.  Measured, us per
+// sweep with the trace, marching kernel (at least 16 rows per warp) / this one:
+// 256^2 66 / 3.6 (the host's launch rate), 2112^2 66.7 / 4.9, 4096^2 67.7 / 14.0,
+// 8192^2 68.0 / 51.7.
 // ---------------------------------------------------------------------------
 constexpr int kFlatThreads = 512;
 
@@ -297,7 +300,7 @@ __global__ void __launch_bounds__(kFlatThreads, 2)
     const uint32_t end = min(f.items, (blockIdx.x + 1) * f.per);
     const DrawCtx dc{p.c2, p.c3, p.acc.T3, p.acc.T4, p.acc.zero};
     const int64_t stride = 2 * p.stride;  // in half words
-    uint32_t ones = 0, dsum = 0, n = 0;
+    uint32_t ones = 0, dsum = 0;
     bool waited = false;
     for (uint32_t e = blockIdx.x * f.per + threadIdx.x; e < end; e += blockDim.x) {
         const uint32_t row = e / f.upr, u = e - row * f.upr;
@@ -336,16 +339,14 @@ __global__ void __launch_bounds__(kFlatThreads, 2)
             const uint32_t sb = (n8 & 0x0F0F0F0Fu) + ((n8 >> 4) & 0x0F0F0F0Fu);
             ones += (sb * 0x01010101u) >> 24;
             dsum += (dacc * 0x01010101u) >> 24;
-            n += HALVES;
         }
     }
     // the kernel after this one relies on this one's wait, so every thread waits
     if (!waited) asm volatile("griddepcontrol.wait;" ::: "memory");
     if (OBS) {
         // 8 white and 8 black spins and 32 bonds per half word
-        const long long sum_s = 2 * (long long)ones - 16 * (long long)n;
-        const long long sum_b = 32 * (long long)n - 2 * (long long)dsum;
-        block_reduce_add2_any(sum_s, sum_b, p.obs);
+        const long long n = (long long)HALVES * (end - blockIdx.x * f.per);
+        block_count_add2(ones, dsum, 2, -16 * n, -2, 32 * n, p.obs);
     }
 }
 
