@@ -105,7 +105,7 @@ ISING_API int ising_half_sweep(const ising_lattice_t *lat, double beta, int32_t 
                                uint64_t t, int64_t *obs_dev, ising_stream_t stream);
 
 /* n_sweeps sweeps with sweep indices sweep_offset .. sweep_offset+n_sweeps-1
- * (Sec. 3.3: two launches per step, black then white).  trace_dev, if not
+ * (Sec. 3.3: a step updates black, then white).  trace_dev, if not
  * NULL, receives n_sweeps x 2 int64 {sum of spins, sum over bonds} after each
  * sweep (the call zeroes it first).  Running a sweeps and then b sweeps with
  * offset a gives the same lattice as a + b sweeps in one call. */
@@ -118,8 +118,8 @@ ISING_API int ising_sweep(const ising_lattice_t *lat, double beta, int64_t n_swe
  * the trace (if trace_host is not NULL; trace_dev is then required as device
  * staging of n_sweeps x 2 int64) back.  Pinned host memory makes the copies
  * asynchronous; the call does not synchronise the stream.  One sweep of an
- * MSC4 lattice runs in row bands (about 16 MiB of host plane each, smaller
- * first and last bands) on streams of the library's own: plane bands are
+ * MSC4 lattice of a few MB or more runs in row bands (3 to 32 with the size,
+ * smaller first and last bands) on streams of the library's own: plane bands are
  * copied in in the order the half-sweeps need them and each is copied out as
  * soon as it is final, so that both directions of the host link are busy
  * while the bands are swept.  The schedule is captured and replayed on
@@ -152,10 +152,10 @@ ISING_API int ising_bits_to_msc4(const void *black_bits, const void *white_bits,
  * format: black_host / white_host are bit planes (4-byte aligned; pinned for
  * asynchronous copies), `dev` an MSC4 device lattice of the same L that holds
  * the state during the call, stage_dev caller-owned device scratch of
- * 2 x ising_bits_bytes (16-byte aligned).  One sweep runs in row bands as in
- * ising_sweep_host, each band converted on the device after its copy in and
- * before its copy out; n_sweeps != 1 copies and converts whole planes.  The
- * result equals ising_sweep on the unpacked lattice, converted back. */
+ * 2 x ising_bits_bytes (16-byte aligned).  One sweep runs as in
+ * ising_sweep_host, on the bit planes in stage_dev, and writes the new spins to
+ * `dev` too; n_sweeps != 1 copies and converts whole planes.  The result equals
+ * ising_sweep on the unpacked lattice, converted back. */
 ISING_API int ising_sweep_host_bits(const ising_lattice_t *dev, void *black_host, void *white_host,
                                     void *stage_dev, double beta, int64_t n_sweeps, uint64_t seed,
                                     uint64_t sweep_offset, int64_t *trace_dev, int64_t *trace_host,

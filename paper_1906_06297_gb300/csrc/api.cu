@@ -596,8 +596,9 @@ ISING_API int ising_slab_sweep(const ising_slab_t *slabs, int32_t n, double beta
 namespace {
 
 // One sweep of an MSC4 lattice held in host memory, in K row bands so that
-// the copies overlap the half-sweeps and each other (the host link, not the
-// sweep, bounds this path).  The compute stream runs black band 0, black 1,
+// the copies overlap the half-sweeps and each other (MSC4 planes are bound by
+// the host link, bit planes by the link and the half-sweeps alike).  With MSC4
+// planes the compute stream runs black band 0, black 1,
 // then black k before white k-1 for k = 2 .. K-1, then white K-1 and white 0:
 // black band k reads the white rows next to it unchanged (white k-1 runs after
 // black k, white 0 last because black K-1 reads white row 0) and white band k
@@ -611,18 +612,35 @@ namespace {
 //
 // Host formats: with stage == nullptr the host planes are MSC4 rows of `hrow`
 // bytes copied straight into the lattice; otherwise they are bit-packed rows
-// of `hrow` = L/16 bytes, copied into `stage` (black's plane, then white's)
-// and converted to and from MSC4 on the compute stream around each band's
-// half-sweeps.
-constexpr int kMaxHostBands = 72;
+// of `hrow` = L/16 bytes, copied into `stage` (black's plane, then white's) and
+// swept there by kernels that write the MSC4 lattice as well.  One launch then
+// sweeps black band k and white band k-2, from k = 3 on, and a last one the
+// white bands K-2, K-1 and 0.
+constexpr int kMaxHostBands = 40;
 
-// Nominal bands of about 16 MiB per host plane: 16 .. 64 bands, and at least
-// 8 rows each.
+// `rows` rows of `row` bytes; dense on both sides in one piece (11584^2 MSC4,
+// rows of 5792 bytes, as 2D copies 1480 us per host sweep, so 683).
+cudaError_t copy_plane(void *dst, size_t dpitch, const void *src, size_t spitch, size_t row, int64_t rows,
+                       cudaMemcpyKind kind, cudaStream_t s)
+{
+    if (dpitch == row && spitch == row) return cudaMemcpyAsync(dst, src, row * (size_t)rows, kind, s);
+    return cudaMemcpy2DAsync(dst, dpitch, src, spitch, row, (size_t)rows, kind, s);
+}
+
+// Nominal bands of a plane of L rows of hrow bytes: more of them shorten the wait
+// for the first copy in and the last one out (time / bands), each costs two
+// copies each way and a launch or two (about 10 us of the streams), so their
+// number goes with the root of the plane's size: 1.5 per root megabyte, at most
+// 32, measured best within 3% from 4 MB to 1 GB in either format.  us per
+// sweep of bit planes with 3 / 8 / 12 / 16 / 32 bands: 8192^2 143 / 166 / 188 / 231 /
+// -, 16384^2 439 / 376 / 396 / 410 / 490, 32768^2 1592 / 1178 / 1140 / 1155 / 1215;
+// MSC4 planes of 65536^2 18831 / 15166 / 14424 / 14101 / 13837.  Below 3 the sweep
+// runs on whole planes without bands: 4096^2 58 against 67 with 3 (bit planes),
+// 2048^2 45 against 60 (MSC4), 256^2 25 against 45.
 int host_band_count(int64_t L, size_t hrow)
 {
-    const int64_t by_bytes = (int64_t)(((size_t)L * hrow) >> 24);
-    const int64_t k = std::min<int64_t>(std::max<int64_t>(by_bytes, 16), 64);
-    return (int)std::min<int64_t>(k, L / 8);
+    const double mb = 1e-6 * (double)L * (double)hrow;
+    return (int)std::min<int64_t>((int64_t)(1.5 * std::sqrt(std::min(mb, 455.0))), L / 8);
 }
 
 // Band starts and sizes (rows): nominal bands, except that where the lattice
@@ -677,6 +695,26 @@ int host_events(int dev, cudaEvent_t **ev)
     return ISING_OK;
 }
 
+// The half-sweeps of sweep t of a bit-packed lattice staged in `stage` (black's
+// plane, then white's).
+BitsSweepParams bits_params(const ising_lattice_t *dev, void *stage, size_t hrow, const Accept &acc, const RoundKeys &rk,
+                            uint64_t t, int64_t *trace_dev)
+{
+    BitsSweepParams p = {};
+    p.bits[0] = (uint32_t *)stage;
+    p.bits[1] = (uint32_t *)((char *)stage + (size_t)dev->L * hrow);
+    p.msc4[0] = (uint64_t *)dev->black;
+    p.msc4[1] = (uint64_t *)dev->white;
+    p.L = dev->L;
+    p.stride_words = dev->row_stride_bytes / 8;
+    p.c2 = (uint32_t)t;
+    p.c3 = counter_word3(0, kPurposeMetropolis, t);
+    p.acc = acc;
+    p.rk = rk;
+    p.obs = (long long *)trace_dev;
+    return p;
+}
+
 // Queues one banded host sweep: stream `s` starts and ends it (it may be a
 // stream in capture), `cmp` and `out` are the compute and copy-out streams,
 // `ev` the event pool (caller holds g_dev.host_mu).
@@ -694,22 +732,17 @@ int enqueue_banded(const ising_lattice_t *dev, char *host[2], char *stage, size_
     char *devp[2] = {(char *)dev->black, (char *)dev->white};
     char *stg[2] = {stage, bits ? stage + (size_t)L * hrow : nullptr};
     const size_t pitch = (size_t)dev->row_stride_bytes;
-    const int64_t stride_words = dev->row_stride_bytes / 8;
-    auto copy = [&](int c, int k, bool in, cudaStream_t st) {
-        char *d = devp[c] + b0[k] * pitch, *h = host[c] + b0[k] * hrow;
+    auto copy_rows = [&](int c, int64_t row0, int64_t rows, bool in, cudaStream_t st) {
+        char *d = devp[c] + row0 * pitch, *h = host[c] + row0 * hrow;
         if (bits) {
-            char *g = stg[c] + b0[k] * hrow;
-            return in ? cudaMemcpyAsync(g, h, (size_t)br[k] * hrow, cudaMemcpyHostToDevice, st)
-                      : cudaMemcpyAsync(h, g, (size_t)br[k] * hrow, cudaMemcpyDeviceToHost, st);
+            char *g = stg[c] + row0 * hrow;
+            return in ? cudaMemcpyAsync(g, h, (size_t)rows * hrow, cudaMemcpyHostToDevice, st)
+                      : cudaMemcpyAsync(h, g, (size_t)rows * hrow, cudaMemcpyDeviceToHost, st);
         }
-        return in ? cudaMemcpy2DAsync(d, pitch, h, hrow, hrow, (size_t)br[k], cudaMemcpyHostToDevice, st)
-                  : cudaMemcpy2DAsync(h, hrow, d, pitch, hrow, (size_t)br[k], cudaMemcpyDeviceToHost, st);
+        return in ? copy_plane(d, pitch, h, hrow, hrow, rows, cudaMemcpyHostToDevice, st)
+                  : copy_plane(h, hrow, d, pitch, hrow, rows, cudaMemcpyDeviceToHost, st);
     };
-    // bits mode: staged band -> MSC4 band (after its copy in) and back (before its copy out)
-    // bits mode: staged plane band -> MSC4 band (as a conversion job)
-    auto unpack_job = [&](int c, int k) {
-        return ConvJob{stg[c] + b0[k] * hrow, devp[c] + b0[k] * pitch, br[k]};
-    };
+    auto copy = [&](int c, int k, bool in, cudaStream_t st) { return copy_rows(c, b0[k], br[k], in, st); };
     e = cudaEventRecord(start, s);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(cmp, start, 0);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(out, start, 0);
@@ -731,67 +764,55 @@ int enqueue_banded(const ising_lattice_t *dev, char *host[2], char *stage, size_
     if (e == cudaSuccess) e = in_black(K - 1);
     if (e == cudaSuccess && trace_dev) e = cudaMemsetAsync(trace_dev, 0, 2 * sizeof(int64_t), cmp);
     if (e != cudaSuccess) return cuda_fail(e, "host sweep: copy in");
-    // compute.  Plane bands that are final wait in `pend` and are flushed to
-    // the copy-out stream behind one event: in MSC4 mode after every
-    // half-sweep; in bits mode after every white half-sweep, packed by one
-    // conversion launch for all of them (black k and white k-1).  In bits mode
-    // black k first unpacks, in one launch, its own band and the white bands
-    // it is the first to need, in their copy-in order (K-1, 0, 1, .., K-2):
-    // the first min(k + 3, K) of that order.  Fewer, larger launches: each
-    // launch leaves the SMs partly idle at its start and end.
-    int unpacked = 0, n_flush = 0, npend = 0;
-    int pend_c[kMaxConvJobs], pend_k[kMaxConvJobs];
-    auto flush = [&]() -> int {
-        if (npend == 0) return ISING_OK;
-        cudaError_t r = cudaSuccess;
-        if (bits) {
-            ConvJob jobs[kMaxConvJobs];
-            for (int i = 0; i < npend; ++i) {
-                const int c = pend_c[i], k = pend_k[i];
-                jobs[i] = ConvJob{devp[c] + b0[k] * pitch, stg[c] + b0[k] * hrow, br[k]};
-            }
-            r = msc4_to_bits_multi(jobs, npend, stride_words, L, cmp);
-        }
+    // compute; each plane band goes to the copy-out stream as soon as it is final
+    int n_flush = 0;
+    auto flush = [&](const BitsBand *band, int n) -> cudaError_t {
         cudaEvent_t f = ev_flush[n_flush++];
-        if (r == cudaSuccess) r = cudaEventRecord(f, cmp);
+        cudaError_t r = cudaEventRecord(f, cmp);
         if (r == cudaSuccess) r = cudaStreamWaitEvent(out, f, 0);
-        for (int i = 0; i < npend && r == cudaSuccess; ++i) r = copy(pend_c[i], pend_k[i], false, out);
-        npend = 0;
-        return r == cudaSuccess ? ISING_OK : cuda_fail(r, "host sweep: copy out");
+        for (int i = 0; i < n && r == cudaSuccess; ++i) r = copy_rows(band[i].colour, band[i].row0, band[i].rows, false, out);
+        return r;
     };
-    auto black = [&](int k) -> int {
-        cudaError_t r = cudaStreamWaitEvent(cmp, ev_in[k], 0);
-        if (r == cudaSuccess && bits) {
-            ConvJob jobs[kMaxConvJobs];
-            int n = 0;
-            for (; unpacked < std::min(k + 3, K); ++unpacked)
-                jobs[n++] = unpack_job(1, unpacked == 0 ? K - 1 : unpacked - 1);
-            jobs[n++] = unpack_job(0, k);
-            r = bits_to_msc4_multi(jobs, n, stride_words, L, cmp);
+    auto band = [&](int c, int k) { return BitsBand{c, b0[k], br[k]}; };
+    if (bits) {
+        // black band k and white band k - 2 in one launch (neither reads what the
+        // other writes), at the end the last two white bands and band 0
+        BitsSweepParams p = bits_params(dev, stage, hrow, acc, rk, t, trace_dev);
+        for (int k = 0; k <= K && e == cudaSuccess; ++k) {
+            p.n = 0;
+            if (k < K) {
+                p.band[p.n++] = band(0, k);
+                if (k >= 3) p.band[p.n++] = band(1, k - 2);
+                e = cudaStreamWaitEvent(cmp, ev_in[k], 0);
+            } else {
+                p.band[p.n++] = band(1, K - 2);
+                p.band[p.n++] = band(1, K - 1);
+                p.band[p.n++] = band(1, 0);
+            }
+            if (e == cudaSuccess) e = bits_half_sweeps(p, cmp);
+            if (e == cudaSuccess) e = flush(p.band, p.n);
         }
-        if (r != cudaSuccess) return cuda_fail(r, "host sweep: unpack");
-        int x = band_half_sweep_impl(dev, acc, rk, 0, t, b0[k], br[k], nullptr, cmp);
-        if (x) return x;
-        pend_c[npend] = 0;
-        pend_k[npend++] = k;
-        return bits ? ISING_OK : flush();
-    };
-    auto white = [&](int k) -> int {
-        int x = band_half_sweep_impl(dev, acc, rk, 1, t, b0[k], br[k], trace_dev, cmp);
-        if (x) return x;
-        pend_c[npend] = 1;
-        pend_k[npend++] = k;
-        return flush();
-    };
-    rc = black(0);
-    if (!rc) rc = black(1);
-    for (int k = 2; k < K && !rc; ++k) {
-        rc = black(k);
-        if (!rc) rc = white(k - 1);
+    } else {
+        auto half = [&](int c, int k) -> int {
+            cudaError_t r = c == 0 ? cudaStreamWaitEvent(cmp, ev_in[k], 0) : cudaSuccess;
+            if (r != cudaSuccess) return cuda_fail(r, "host sweep: wait for copy in");
+            const int x = band_half_sweep_impl(dev, acc, rk, c, t, b0[k], br[k], c ? trace_dev : nullptr, cmp);
+            if (x) return x;
+            const BitsBand b = band(c, k);
+            r = flush(&b, 1);
+            return r == cudaSuccess ? ISING_OK : cuda_fail(r, "host sweep: copy out");
+        };
+        rc = half(0, 0);
+        if (!rc) rc = half(0, 1);
+        for (int k = 2; k < K && !rc; ++k) {
+            rc = half(0, k);
+            if (!rc) rc = half(1, k - 1);
+        }
+        if (!rc) rc = half(1, K - 1);
+        if (!rc) rc = half(1, 0);
+        if (rc) return rc;
     }
-    if (!rc) rc = white(K - 1);
-    if (!rc) rc = white(0);
-    if (rc) return rc;
+    if (e != cudaSuccess) return cuda_fail(e, "host sweep");
     if (trace_host != nullptr)
         e = cudaMemcpyAsync(trace_host, trace_dev, 2 * sizeof(int64_t), cudaMemcpyDeviceToHost, out);
     if (e == cudaSuccess) e = cudaEventRecord(end, out);
@@ -799,7 +820,7 @@ int enqueue_banded(const ising_lattice_t *dev, char *host[2], char *stage, size_
     return e == cudaSuccess ? ISING_OK : cuda_fail(e, "host sweep: copy out");
 }
 
-// One banded host sweep.  The schedule (about 4 launches and 4 copies per
+// One banded host sweep.  The schedule (one or two launches and 4 copies per
 // band, with cross-stream events) is captured on the library's capture stream
 // and replayed as a CUDA graph on `s`: the executable graph of the previous
 // call is updated in place (new sweep index, keys, buffers) where the
@@ -876,21 +897,22 @@ ISING_API int ising_sweep_host(const ising_lattice_t *dev, void *black_host, voi
             if (rc) return rc;
         }
         char *host[2] = {(char *)black_host, (char *)white_host};
-        return sweep_host_banded(dev, host, nullptr, row, acc, make_round_keys(seed), sweep_offset, trace_dev,
-                                 trace_host, s);
+        if (host_band_count(dev->L, row) >= 3)
+            return sweep_host_banded(dev, host, nullptr, row, acc, make_round_keys(seed), sweep_offset, trace_dev,
+                                     trace_host, s);
     }
     void *host[2] = {black_host, white_host};
     void *devp[2] = {dev->black, dev->white};
     for (int c = 0; c < 2; ++c) {
-        cudaError_t e = cudaMemcpy2DAsync(devp[c], (size_t)dev->row_stride_bytes, host[c], row, row, (size_t)dev->L,
-                                          cudaMemcpyHostToDevice, s);
+        cudaError_t e = copy_plane(devp[c], (size_t)dev->row_stride_bytes, host[c], row, row, dev->L,
+                                   cudaMemcpyHostToDevice, s);
         if (e != cudaSuccess) return cuda_fail(e, "host-to-device copy");
     }
     rc = ising_sweep(dev, beta, n_sweeps, seed, sweep_offset, trace_dev, stream);
     if (rc) return rc;
     for (int c = 0; c < 2; ++c) {
-        cudaError_t e = cudaMemcpy2DAsync(host[c], row, devp[c], (size_t)dev->row_stride_bytes, row, (size_t)dev->L,
-                                          cudaMemcpyDeviceToHost, s);
+        cudaError_t e = copy_plane(host[c], row, devp[c], (size_t)dev->row_stride_bytes, row, dev->L,
+                                   cudaMemcpyDeviceToHost, s);
         if (e != cudaSuccess) return cuda_fail(e, "device-to-host copy");
     }
     if (trace_host != nullptr && n_sweeps > 0) {
@@ -990,17 +1012,28 @@ ISING_API int ising_sweep_host_bits(const ising_lattice_t *dev, void *black_host
     cudaStream_t s = (cudaStream_t)stream;
     char *host[2] = {(char *)black_host, (char *)white_host};
     char *stg[2] = {(char *)stage_dev, (char *)stage_dev + nb};
-    if (n_sweeps == 1)
+    if (n_sweeps == 1 && host_band_count(dev->L, hrow) >= 3)
         return sweep_host_banded(dev, host, (char *)stage_dev, hrow, acc, make_round_keys(seed), sweep_offset,
                                  trace_dev, trace_host, s);
     for (int c = 0; c < 2; ++c) {
         cudaError_t e = cudaMemcpyAsync(stg[c], host[c], nb, cudaMemcpyHostToDevice, s);
         if (e != cudaSuccess) return cuda_fail(e, "host-to-device copy");
     }
-    rc = ising_bits_to_msc4(stg[0], stg[1], dev, stream);
-    if (!rc) rc = ising_sweep(dev, beta, n_sweeps, seed, sweep_offset, trace_dev, stream);
-    if (!rc) rc = ising_msc4_to_bits(dev, stg[0], stg[1], stream);
-    if (rc) return rc;
+    if (n_sweeps == 1) {
+        cudaError_t e = trace_dev ? cudaMemsetAsync(trace_dev, 0, 2 * sizeof(int64_t), s) : cudaSuccess;
+        BitsSweepParams p = bits_params(dev, stage_dev, hrow, acc, make_round_keys(seed), sweep_offset, trace_dev);
+        p.n = 1;
+        for (int c = 0; c < 2 && e == cudaSuccess; ++c) {
+            p.band[0] = BitsBand{c, 0, dev->L};
+            e = bits_half_sweeps(p, s);
+        }
+        if (e != cudaSuccess) return cuda_fail(e, "half-sweep launch");
+    } else {
+        rc = ising_bits_to_msc4(stg[0], stg[1], dev, stream);
+        if (!rc) rc = ising_sweep(dev, beta, n_sweeps, seed, sweep_offset, trace_dev, stream);
+        if (!rc) rc = ising_msc4_to_bits(dev, stg[0], stg[1], stream);
+        if (rc) return rc;
+    }
     for (int c = 0; c < 2; ++c) {
         cudaError_t e = cudaMemcpyAsync(host[c], stg[c], nb, cudaMemcpyDeviceToHost, s);
         if (e != cudaSuccess) return cuda_fail(e, "device-to-host copy");

@@ -119,6 +119,26 @@ struct Int8SweepParams {
     long long *obs;
 };
 
+// Half-sweeps of row bands of a periodic lattice held bit-packed (bits.cu): black
+// bands before white ones, and no band reads what another one writes.
+constexpr int kMaxBitsBands = 3;
+struct BitsBand {
+    int32_t colour;
+    int64_t row0, rows;
+};
+struct BitsSweepParams {
+    uint32_t *bits[2];     // black, white: L rows of L / 64 words, dense
+    uint64_t *msc4[2];     // their MSC4 planes, which receive the new spins too
+    int64_t L;
+    int64_t stride_words;  // MSC4 row stride
+    uint32_t c2, c3;       // counter words 2 and 3 of the black half-sweep
+    Accept acc;
+    RoundKeys rk;
+    long long *obs;        // {sum s, sum bonds} accumulators of the white bands or nullptr
+    int32_t n;
+    BitsBand band[kMaxBitsBands];
+};
+
 // A sweep call of a small lattice in one launch (resident.cu).
 struct ResidentSweep {
     void *plane[2];     // black, white
