@@ -283,15 +283,17 @@ __device__ __forceinline__ void march_flush(long long *acc, int64_t lat, unsigne
                                             uint32_t &ones, uint32_t &dsum, uint32_t &nrows)
 {
     if (!OBS) return;
-    long long a = ones, b = dsum, c = nrows;
+    uint32_t a = ones, b = dsum, c = nrows;  // at most 128 per lane and row, a lattice has 2^16 of them
     for (int off = lpr >> 1; off > 0; off >>= 1) {
         a += __shfl_xor_sync(gmask, a, off);
         b += __shfl_xor_sync(gmask, b, off);
         c += __shfl_xor_sync(gmask, c, off);
     }
     if (j == 0 && c > 0) {
-        atomicAdd(reinterpret_cast<unsigned long long *>(acc + 2 * lat), (unsigned long long)(2 * a - 64 * c));
-        atomicAdd(reinterpret_cast<unsigned long long *>(acc + 2 * lat + 1), (unsigned long long)(128 * c - 2 * b));
+        atomicAdd(reinterpret_cast<unsigned long long *>(acc + 2 * lat),
+                  (unsigned long long)(2 * (long long)a - 64 * (long long)c));
+        atomicAdd(reinterpret_cast<unsigned long long *>(acc + 2 * lat + 1),
+                  (unsigned long long)(128 * (long long)c - 2 * (long long)b));
     }
     ones = dsum = nrows = 0;
 }
@@ -359,6 +361,14 @@ __device__ void march_rows(const BatchParams &p, const BatchGroup &G, int64_t c0
         cp16_if(&ring.src[(s + 2) & 3][lane], src2, ahead);
         cp16_if(&ring.tgt[(s + 1) & 1][lane], tgt_r + wpr, ahead);
         cp_commit();
+        // the marks while the row is on its way: what a run's first row costs after a
+        // barrier is then the longer of the two, not their sum (256^2 x 304: 16.7 ->
+        // 16.1 us per sweep, 128^2 x 608 9.9 -> 9.35, the replica-exchange batch 217 -> 213.6)
+        uint4 g;
+        g.x = half_marks(q, stream, dc, p.rk);
+        g.y = half_marks(q | 2, stream, dc, p.rk);
+        g.z = half_marks(q | 4, stream, dc, p.rk);
+        g.w = half_marks(q | 6, stream, dc, p.rk);
         cp_wait_all_but_last();
         const uint4 up = ring.src[(s + 3) & 3][lane];
         const uint4 cur = ring.src[s & 3][lane];
@@ -380,10 +390,10 @@ __device__ void march_rows(const BatchParams &p, const BatchGroup &G, int64_t c0
         }
         uint32_t dacc = 0;
         uint4 ns;
-        ns.x = update_half<OBS, false>(tg.x, up.x + dn.x + cur.x, sd.x, q, stream, dc, p.rk, dacc);
-        ns.y = update_half<OBS, false>(tg.y, up.y + dn.y + cur.y, sd.y, q | 2, stream, dc, p.rk, dacc);
-        ns.z = update_half<OBS, false>(tg.z, up.z + dn.z + cur.z, sd.z, q | 4, stream, dc, p.rk, dacc);
-        ns.w = update_half<OBS, false>(tg.w, up.w + dn.w + cur.w, sd.w, q | 6, stream, dc, p.rk, dacc);
+        ns.x = decide_half<OBS, false>(tg.x, up.x + dn.x + cur.x, sd.x, g.x, dacc);
+        ns.y = decide_half<OBS, false>(tg.y, up.y + dn.y + cur.y, sd.y, g.y, dacc);
+        ns.z = decide_half<OBS, false>(tg.z, up.z + dn.z + cur.z, sd.z, g.z, dacc);
+        ns.w = decide_half<OBS, false>(tg.w, up.w + dn.w + cur.w, sd.w, g.w, dacc);
         *reinterpret_cast<uint4 *>(tgt_r) = ns;
         if (OBS) {
             const uint32_t n8 = ns.x + ns.y + ns.z + ns.w + cur.x + cur.y + cur.z + cur.w;
@@ -431,13 +441,9 @@ __device__ void batch_half(const BatchParams &p, const Split &sp, int64_t cb, in
     uint32_t ones = 0, dsum = 0, nitems = 0;
     auto flush = [&]() {
         if (OBS && cur_lat >= 0) {
-            long long a = ones, b = dsum, c = nitems;
-#pragma unroll
-            for (int off = 16; off > 0; off >>= 1) {
-                a += __shfl_xor_sync(0xffffffffu, a, off);
-                b += __shfl_xor_sync(0xffffffffu, b, off);
-                c += __shfl_xor_sync(0xffffffffu, c, off);
-            }
+            // at most 4 per site; a warp's share of a lattice is far below 2^30 sites
+            const long long a = __reduce_add_sync(0xffffffffu, ones), b = __reduce_add_sync(0xffffffffu, dsum),
+                            c = __reduce_add_sync(0xffffffffu, nitems);
             if (lane == 0) {
                 // c white sites and c black centres were counted, a of them up;
                 // each white site adds 4 - 2d over its 4 bonds
@@ -514,20 +520,24 @@ __device__ void batch_half(const BatchParams &p, const Split &sp, int64_t cb, in
     flush();
 }
 
-// Whether slots k and k + 1 of ladder l, held by lattices a and b, exchange at
-// sweep t.
-__device__ __forceinline__ bool pair_swaps(const BatchParams &p, const long long *acc, int64_t l, int k, int32_t a,
-                                           int32_t b, uint64_t t)
+// The draw of the exchange of slots k and k + 1 of ladder l at sweep t.
+__device__ __forceinline__ uint32_t pair_draw(const BatchParams &p, int64_t l, int k, uint64_t t)
+{
+    const uint32_t site = (uint32_t)k;
+    const uint4 u4 = philox(site >> 2, (uint32_t)l, (uint32_t)t, counter_word3(0, kPurposeExchange, t), p.rk);
+    return (site & 3) == 0 ? u4.x : (site & 3) == 1 ? u4.y : (site & 3) == 2 ? u4.z : u4.w;
+}
+
+// Whether slots k and k + 1, held by lattices a and b, exchange on the draw w;
+// `off` and `len` are the pair's table.
+__device__ __forceinline__ bool pair_swaps(const BatchParams &p, const long long *acc, int32_t a, int32_t b, uint32_t w,
+                                           int64_t off, int64_t len)
 {
     const long long D = acc[2 * a + 1] - acc[2 * b + 1];  // E_b - E_a
     if (D >= 0) return true;
     if ((D & 3) != 0) atomicCAS(p.err, 0, (int)ISING_EINVAL);
     const int64_t m = -D;
-    const uint64_t TS = m < p.swap_len[k] ? p.swap_tab[p.swap_off[k] + m] : 0ull;
-    const uint32_t site = (uint32_t)k;
-    const uint4 u4 = philox(site >> 2, (uint32_t)l, (uint32_t)t, counter_word3(0, kPurposeExchange, t), p.rk);
-    const uint32_t w = (site & 3) == 0 ? u4.x : (site & 3) == 1 ? u4.y : (site & 3) == 2 ? u4.z : u4.w;
-    return (uint64_t)w < TS;
+    return (uint64_t)w < (m < len ? p.swap_tab[off + m] : 0ull);
 }
 
 // The owners' form of record and exchange, without a barrier behind it: a thread
@@ -535,38 +545,67 @@ __device__ __forceinline__ bool pair_swaps(const BatchParams &p, const long long
 // partner's thread comes to the same answer), from the state `at` that event left
 // by the last one; the new state goes to the other buffer, `at_next`.  The sums
 // read here are cleared at the next event, when every thread has read them.
-__device__ void owner_exchange(const BatchParams &p, uint64_t t, const int32_t *at, int32_t *at_next,
-                               const long long *acc, long long *acc_next)
+// Everything but the sums is fetched ahead of the barrier that completes them:
+// one load of the sums, one of the table stand behind it instead of a chain of
+// five (a record of 384 lattices of sides 64 to 256: 5.6 -> 4.6 us).
+struct OwnerPair {
+    int32_t x, k, pk, y;  // the lattice, its slot, its partner's slot (-1: none) and lattice
+    uint32_t w;
+    int64_t off, len;
+};
+
+// Lattice number i of the block's owner (x = -1 behind the last one).
+__device__ __forceinline__ OwnerPair owner_pair(const BatchParams &p, uint64_t t, int64_t i, const int32_t *at)
 {
-    const int o = (int)blockIdx.x / p.cs, rank = (int)blockIdx.x % p.cs;
-    const int64_t e = (int64_t)((t + 1) / (uint64_t)p.record_every) - 1;
-    const uint32_t S = (uint32_t)p.S;
-    for (int g = 0; g < p.n_groups; ++g) {
-        const int64_t first = p.part[g][o], last = p.part[g][o + 1];
-        for (int64_t i = first + rank + (int64_t)p.cs * threadIdx.x; i < last; i += (int64_t)p.cs * blockDim.x) {
-            const int32_t x = (int32_t)(p.g[g].first + i);
-            const uint32_t l = (uint32_t)x / S;
-            int k = p.slot_of[x];
-            if (p.trace != nullptr) {
-                long long *row = p.trace + 2 * ((e - p.event_first) * p.n + (int64_t)l * S + k);
-                row[0] = acc[2 * x];
-                row[1] = acc[2 * x + 1];
-            }
-            if (p.swaps) {
-                const bool lower = ((k ^ (int)e) & 1) == 0;  // x holds the lower slot of its pair
-                const int pk = lower ? k + 1 : k - 1;
-                if (pk >= 0 && pk < (int)S) {
-                    const int32_t y = at[(int64_t)l * S + pk];
-                    if (pair_swaps(p, acc, l, lower ? k : pk, lower ? x : y, lower ? y : x, t)) {
-                        k = pk;
-                        p.slot_of[x] = k;
-                    }
-                }
-            }
-            at_next[(int64_t)l * S + k] = x;
-            acc_next[2 * x] = 0;
-            acc_next[2 * x + 1] = 0;
+    OwnerPair r = {-1, 0, -1, 0, 0u, 0, 0};
+    const int o = (int)blockIdx.x / p.cs;
+    for (int g = 0; g < p.n_groups && r.x < 0; ++g) {
+        const int64_t first = p.part[g][o], count = p.part[g][o + 1] - first;
+        if (i < count) r.x = (int32_t)(p.g[g].first + first + i);
+        i -= count;
+    }
+    if (r.x < 0) return r;
+    const int64_t l = r.x / p.S;
+    r.k = p.slot_of[r.x];
+    if (p.swaps) {
+        const int e = (int)((t + 1) / (uint64_t)p.record_every) - 1;
+        const bool lower = ((r.k ^ e) & 1) == 0;  // x holds the lower slot of its pair
+        const int pk = lower ? r.k + 1 : r.k - 1, k = lower ? r.k : pk;
+        if (pk >= 0 && pk < p.S) {
+            r.pk = pk;
+            r.y = at[l * p.S + pk];
+            r.off = p.swap_off[k];
+            r.len = p.swap_len[k];
+            r.w = pair_draw(p, l, k, t);
         }
+    }
+    return r;
+}
+
+__device__ __forceinline__ void owner_exchange(const BatchParams &p, uint64_t t, OwnerPair r, int64_t i,
+                                               const int32_t *at, int32_t *at_next, const long long *acc,
+                                               long long *acc_next)
+{
+    const int64_t e = (int64_t)((t + 1) / (uint64_t)p.record_every) - 1;
+    while (r.x >= 0) {
+        const int64_t l = r.x / p.S;
+        if (p.trace != nullptr) {
+            long long *row = p.trace + 2 * ((e - p.event_first) * p.n + l * p.S + r.k);
+            row[0] = acc[2 * r.x];
+            row[1] = acc[2 * r.x + 1];
+        }
+        if (r.pk >= 0) {
+            const bool lower = r.pk > r.k;
+            if (pair_swaps(p, acc, lower ? r.x : r.y, lower ? r.y : r.x, r.w, r.off, r.len)) {
+                r.k = r.pk;
+                p.slot_of[r.x] = r.k;
+            }
+        }
+        at_next[l * p.S + r.k] = r.x;
+        acc_next[2 * r.x] = 0;
+        acc_next[2 * r.x + 1] = 0;
+        i += (int64_t)p.cs * blockDim.x;
+        r = owner_pair(p, t, i, at);
     }
 }
 
@@ -591,7 +630,8 @@ __device__ void batch_exchange(const BatchParams &p, uint64_t t)
         if (p.swaps) {
             for (int k = (int)(e & 1) + 2 * lane; k + 1 < p.S; k += 64) {
                 const int32_t a = at[k], b = at[k + 1];
-                const bool swap = pair_swaps(p, p.acc, l, k, a, b, t);
+                const bool swap =
+                    pair_swaps(p, p.acc, a, b, pair_draw(p, l, k, t), p.swap_off[k], p.swap_len[k]);
                 if (swap) {
                     at[k] = b;
                     at[k + 1] = a;
@@ -630,10 +670,14 @@ __global__ void __launch_bounds__(512, 1) batch_kernel(const __grid_constant__ B
         if (rec) {
             const bool odd = p.cs > 0 && (events & 1);
             batch_half<true>(p, sp, cb, ce, 1, t, odd ? p.acc2 : p.acc, ring);
+            const int64_t mine = (int)blockIdx.x % max(p.cs, 1) + (int64_t)p.cs * threadIdx.x;
+            const int32_t *at = odd ? p.lattice_at2 : p.lattice_at;
+            OwnerPair pair = {-1};
+            if (p.cs > 0) pair = owner_pair(p, t, mine, at);
             if (!grid_sync(p)) return;
             if (p.cs > 0) {
-                owner_exchange(p, t, odd ? p.lattice_at2 : p.lattice_at, odd ? p.lattice_at : p.lattice_at2,
-                               odd ? p.acc2 : p.acc, odd ? p.acc : p.acc2);
+                owner_exchange(p, t, pair, mine, at, odd ? p.lattice_at : p.lattice_at2, odd ? p.acc2 : p.acc,
+                               odd ? p.acc : p.acc2);
                 ++events;
                 phase_sync(p);
             } else {
