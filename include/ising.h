@@ -108,7 +108,9 @@ ISING_API int ising_half_sweep(const ising_lattice_t *lat, double beta, int32_t 
  * (Sec. 3.3: a step updates black, then white).  trace_dev, if not
  * NULL, receives n_sweeps x 2 int64 {sum of spins, sum over bonds} after each
  * sweep (the call zeroes it first).  Running a sweeps and then b sweeps with
- * offset a gives the same lattice as a + b sweeps in one call. */
+ * offset a gives the same lattice as a + b sweeps in one call.  L <= 512 runs in
+ * one cluster whose CTAs wait for one another, each wait bounded (~2 s): should
+ * one give up, the next such call returns ISING_ETIMEOUT. */
 ISING_API int ising_sweep(const ising_lattice_t *lat, double beta, int64_t n_sweeps, uint64_t seed,
                           uint64_t sweep_offset, int64_t *trace_dev, ising_stream_t stream);
 

@@ -479,7 +479,8 @@ ISING_API int ising_sweep(const ising_lattice_t *lat, double beta, int64_t n_swe
         if (rc) return rc;
     }
     const RoundKeys rk = make_round_keys(seed);
-    if (resident_fits(lat->L)) {
+    if (resident_fits(lat->L, n_sweeps)) {
+        if (resident_timed_out()) return fail(ISING_ETIMEOUT, "a wait of an earlier small-lattice sweep gave up");
         ResidentSweep p{};
         p.plane[0] = lat->black;
         p.plane[1] = lat->white;

@@ -146,6 +146,8 @@ struct ResidentSweep {
     int32_t L;
     int32_t hpr;        // half words (8 spins) per plane row; set by resident_sweep
     int32_t bytes;      // one byte per spin (else MSC4)
+    int32_t wide;       // one-byte rows are 8-byte aligned; set by resident_sweep
+    int32_t deciders;   // threads of a CTA that decide; set by resident_sweep
     int32_t n_sweeps;   // set by resident_sweep
     uint64_t t0;        // index of the first sweep
     Accept acc;

@@ -51,8 +51,10 @@ cudaError_t int8_observables(const int8_t *black, const int8_t *white, int64_t L
 
 // Sweeps of a small lattice, either layout, all of a call's in launches of one
 // cluster (resident_fits: the sides it is for); writes (not adds to) the trace.
-bool resident_fits(int64_t L);
+bool resident_fits(int64_t L, int64_t n_sweeps);
 cudaError_t resident_sweep(ResidentSweep p, int64_t n_sweeps, cudaStream_t s);
+// Whether a wait of an earlier such launch has given up since the last question.
+bool resident_timed_out();
 
 // Throughput probes (probe.cu): the generator alone, shaped like the sweep
 // (n_blocks <= 2^34), and the 32 x 32 -> 64-bit multiply alone (*multiplies

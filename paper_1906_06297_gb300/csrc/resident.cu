@@ -4,41 +4,42 @@
 // A half-sweep of a small lattice is too little work for a launch: at 256^2 the
 // multiplies of its draws take the whole chip 17 ns, while two launches per
 // sweep cost 3.6 us of host time alone.  Here up to 16 CTAs of one cluster hold
-// the lattice in shared memory for all sweeps of the call, a band of rows each,
-// and meet at the cluster's hardware barrier after every half-sweep.  256^2,
-// 1000 recorded sweeps: 8.2 us per sweep with two launches of a thread per Philox
-// block, 3.55 with two overlapped flat launches, 1.15 here.  Of ~860 cycles per
-// half-sweep then ~500 are the marks (a chain of ten Philox rounds that two
-// warps per scheduler do not hide), ~200 the decision and its shared-memory
-// reads, ~100 the rest of the barrier.
+// the lattice in shared memory for all sweeps of the call, a band of rows each.
 //
 // Both layouts are held the same way: 8 spins of a row to a 32-bit half word,
-// one per nibble (0/1), ceil(L/2 / 8) half words per row and colour.  A thread
-// owns up to K half words of each colour for the whole call.  Per half-sweep it
-// forms their draws' marks, then waits for the other CTAs' last half-sweep,
-// then decides; so the barrier's latency passes behind the generator, which is
-// nearly all of the arithmetic.  The first and last row of a band are also
-// copied into the halo rows of the CTAs above and below (distributed shared
-// memory), so every read after the wait is local.  A neighbour's halo row of one
-// colour is only written after that neighbour has passed the barrier behind its
-// last reads of it, one half-sweep of the other colour earlier.
+// one per nibble (0/1), ceil(L/2 / 8) half words per row and colour.  The last
+// warps of a CTA decide, up to K half words of each colour per thread, whose own
+// spins stay in registers; the others form the marks of the next sweep's draws
+// meanwhile, in shared memory, a buffer per parity of the sweep.  The deciding
+// warps meet between the colours, all of them behind each sweep.  What a band's
+// first and last row become goes to the halo rows of the CTAs above and below as
+// asynchronous remote stores that count at a barrier there (one per colour),
+// which only the threads of the edge rows wait for.  Such a word is
+// overwritten, two half-sweeps later, only after the row of the thread that reads
+// it, sent behind that read, has arrived at its writer; so no other order is
+// needed between CTAs.
 //
 // RAGGED: rows of one-byte lattices with L/2 not a multiple of 8.  The last half
 // word of a row holds fewer spins (its other nibbles stay 0) and a half word's
 // draws may start in the middle of a Philox block.
 //
-// One warp of each CTA computes nothing: behind the CTA's own barrier it copies
-// the band's first and last rows into the neighbours and alone makes the
-// cluster-wide release.  (A release by every thread costs each half-sweep ~280
-// cycles of fence on top of the ~100 of the hardware barrier, which the marks,
-// ~500 cycles, then no longer hide.  64-bit shared atomics for the sums cost another
-// 600 per sweep; each warp has a word of its own instead.)
+// Bound at 64^2 to 256^2 by the remote stores' way (~400 cycles per half-sweep)
+// and a decision's chain of loads and logic (~150), beyond by the 16 SMs'
+// multipliers.  us per sweep of 1000 recorded ones, with two launches per sweep /
+// with marks, decisions and a cluster barrier with a release (~500 cycles of fence
+// and remote stores) one after the other / this way: 32^2 3.6 / 0.89 / 0.44, 64^2 3.6 /
+// 0.91 / 0.53, 256^2 3.6 / 1.12 / 0.79, 384^2 3.6 / 1.79 / 1.48, 512^2 3.6 / 2.66 / 2.32.
+// On the way there: the same barrier with drawing warps 1.11 at 256^2, remote
+// stores with branching decisions from addresses worked out in each of them 1.08 to
+// 1.23.  (64-bit shared atomics for the sums cost 600 cycles per sweep; each warp
+// has a word of its own instead.)
 //
 // The observables of each sweep are added up in the CTAs' shared memory and
 // written by the first CTA every kTraceRows sweeps.
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "common.cuh"
 #include "launch.h"
@@ -52,17 +53,18 @@ constexpr int kMaxThreads = 1024;
 constexpr int kMaxCluster = 16;
 constexpr int kTraceRows = 128;
 // Half words per CTA and colour below which the cluster is not doubled: 64^2 takes
-// 0.95 us per sweep with at least 64, 0.99 with 128 and 1.12 with 256.
+// 0.51 us per sweep with at least 64, 0.64 with 128 and 0.71 with 256; 32^2, with at
+// least 32, 0.51 in two CTAs and 0.38 in one.
 constexpr int64_t kItems = 64;
 // Sweeps per launch (some 10 ms): another stream's work is not kept waiting for
 // the whole of a long call.
 constexpr int64_t kMaxSweeps = 16384;
+constexpr long long kWaitCycles = 4000000000LL;  // ~2 s
+
+// Set by a wait that gave up, reported by the next call.
+__device__ __managed__ int g_resident_error;
 
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
-__device__ __forceinline__ void cluster_arrive_relaxed()
-{
-    asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
-}
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 
 __device__ __forceinline__ uint32_t cluster_rank()
@@ -80,9 +82,51 @@ __device__ __forceinline__ uint32_t peer_addr(uint32_t a, uint32_t rank)
     return r;
 }
 
-__device__ __forceinline__ void peer_store(uint32_t a, uint32_t v)
+// Where `on`, writes v to the cluster address `a` and counts its bytes at the
+// barrier `bar` of the same CTA.
+__device__ __forceinline__ void peer_store_if(bool on, uint32_t a, uint32_t v, uint32_t bar)
 {
-    asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
+    asm volatile("{\n\t"
+                 ".reg .pred q;\n\t"
+                 "setp.ne.u32 q, %3, 0;\n\t"
+                 "@q st.async.shared::cluster.mbarrier::complete_tx::bytes.u32 [%0], %1, [%2];\n\t"
+                 "}" ::"r"(a), "r"(v), "r"(bar), "r"((uint32_t)on)
+                 : "memory");
+}
+
+__device__ __forceinline__ void bar_init(uint32_t bar)
+{
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar) : "memory");
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+}
+
+__device__ __forceinline__ void bar_expect(uint32_t bar, uint32_t bytes)
+{
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
+}
+
+// Waits until the barrier's phase of the given parity is over, at most ~2 s.
+__device__ __forceinline__ void bar_wait(uint32_t bar, uint32_t parity, bool &dead)
+{
+    if (dead) return;
+    const long long start = clock64();
+    for (;;) {
+        uint32_t done;
+        asm volatile("{\n\t"
+                     ".reg .pred q;\n\t"
+                     "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 q, [%1], %2;\n\t"
+                     "selp.u32 %0, 1, 0, q;\n\t"
+                     "}"
+                     : "=r"(done)
+                     : "r"(bar), "r"(parity)
+                     : "memory");
+        if (done) return;
+        if (clock64() - start > kWaitCycles) {
+            g_resident_error = 1;
+            dead = true;
+            return;
+        }
+    }
 }
 
 __device__ __forceinline__ unsigned long long peer_load(uint32_t a)
@@ -92,11 +136,17 @@ __device__ __forceinline__ unsigned long long peer_load(uint32_t a)
     return v;
 }
 
-// Half word u of one plane row, and back (one-byte rows: nv spins of it).
+// Half word u of one plane row, and back (one-byte rows: nv spins of it, eight
+// as one access where the rows are 8-byte aligned).
 __device__ __forceinline__ uint32_t load_half(const ResidentSweep &p, int colour, int row, int u, int nv)
 {
     const char *r = static_cast<const char *>(p.plane[colour]) + row * p.stride;
     if (!p.bytes) return reinterpret_cast<const uint32_t *>(r)[u];
+    if (nv == 8 && p.wide) {
+        const uint2 v = reinterpret_cast<const uint2 *>(r)[u];
+        const uint32_t lo = __vcmpgts4(v.x, 0u) & 0x01010101u, hi = __vcmpgts4(v.y, 0u) & 0x01010101u;
+        return __byte_perm(lo, hi, 0x6420) | (__byte_perm(lo, hi, 0x7531) << 4);
+    }
     uint32_t x = 0;
 #pragma unroll
     for (int k = 0; k < 8; ++k)
@@ -109,6 +159,13 @@ __device__ __forceinline__ void store_half(const ResidentSweep &p, int colour, i
     char *r = static_cast<char *>(p.plane[colour]) + row * p.stride;
     if (!p.bytes) {
         reinterpret_cast<uint32_t *>(r)[u] = x;
+        return;
+    }
+    if (nv == 8 && p.wide) {
+        auto bytes = [](uint32_t h, uint32_t sel) {  // four nibbles to +1 (0x01) or -1 (0xFF)
+            return 0xFFFFFFFFu ^ (__byte_perm(h & 0x01010101u, (h >> 4) & 0x01010101u, sel) * 0xFEu);
+        };
+        reinterpret_cast<uint2 *>(r)[u] = make_uint2(bytes(x, 0x5140), bytes(x, 0x7362));
         return;
     }
 #pragma unroll
@@ -135,165 +192,271 @@ __device__ __forceinline__ uint32_t marks8(uint32_t b, uint32_t o, const DrawCtx
     return RAGGED ? __funnelshift_r(lo, m[2], 4 * o) : lo;
 }
 
+// What a CTA of the cluster works on; offsets into its shared memory in words.
+struct Resident {
+    int hpr, half, rows, r0, items;
+    int nc;           // deciding threads, the last ones; the others draw
+    int plane_words;  // per colour: local rows 0 (halo above), 1 .. rows, rows + 1 (halo below)
+    int mark_words;   // per colour and sweep parity
+    int last_nv;      // spins of a row's last half word
+    int tw, plane, marks;
+};
+
+extern __shared__ __align__(16) uint32_t res_smem[];
+
+// The marks of one half-sweep of a CTA's band, half words tid + k nc.
+template <int K, bool RAGGED>
+struct Drawer {
+    uint32_t site[K];
+
+    __device__ __forceinline__ Drawer(const Resident &c, int tid)
+    {
+#pragma unroll
+        for (int k = 0; k < K; ++k) {
+            const int it = min(tid + k * c.nc, c.items - 1), row = it / c.hpr;
+            site[k] = (uint32_t)(c.r0 + row) * (uint32_t)c.half + 8u * (uint32_t)(it - row * c.hpr);
+        }
+    }
+
+    __device__ __forceinline__ void draw(const ResidentSweep &p, const Resident &c, int tid, uint64_t t, int colour, int to)
+    {
+        const DrawCtx dc{(uint32_t)t, counter_word3(colour, kPurposeMetropolis, t), p.acc.T3, p.acc.T4, p.acc.zero};
+#pragma unroll
+        for (int k = 0; k < K; ++k)
+            if (tid + k * c.nc < c.items)
+                res_smem[to + k * c.nc] = marks8<RAGGED>(site[k] >> 2, site[k] & 3u, dc, p.rk);
+    }
+};
+
+// Half words tid + k nc of a CTA's band, their current spins and what deciding
+// them takes.  Everything that can be is worked out before the first sweep and
+// nothing branches: a decision is a chain of loads and logic that one or two
+// warps per scheduler do not hide.
+template <int K, bool RAGGED>
+struct Decider {
+    int at[K];              // index in a plane
+    int up[K], dn[K];       // rows above and below
+    int left[K], right[K];  // the word beside it in its row, periodically
+    uint32_t spins[2][K];
+    uint32_t odd;           // bit k: odd row
+    uint32_t ends;          // RAGGED, bit k: first of its row, bit k + 16: last
+    uint32_t dst[K];        // where the halo copy of an edge row's word goes, as a cluster address; 0: nowhere
+    uint32_t dst_bar[K];
+    bool edge;
+
+    __device__ __forceinline__ Decider(const Resident &c, int tid, bool alone, uint32_t to_above, uint32_t to_below,
+                                       uint32_t bar_above, uint32_t bar_below)
+    {
+        edge = false;
+        odd = ends = 0;
+#pragma unroll
+        for (int k = 0; k < K; ++k) {
+            const bool ok = tid + k * c.nc < c.items;
+            const int it = ok ? tid + k * c.nc : 0, row = it / c.hpr, u = it - row * c.hpr;
+            at[k] = it + c.hpr;
+            up[k] = alone && row == 0 ? at[k] + (c.rows - 1) * c.hpr : at[k] - c.hpr;
+            dn[k] = alone && row == c.rows - 1 ? at[k] - (c.rows - 1) * c.hpr : at[k] + c.hpr;
+            left[k] = at[k] + (u == 0 ? c.hpr - 1 : -1);
+            right[k] = at[k] + (u == c.hpr - 1 ? 1 - c.hpr : 1);
+            odd |= (uint32_t)((c.r0 + row) & 1) << k;
+            ends |= (u == 0 ? 1u << k : 0u) | (u == c.hpr - 1 ? 0x10000u << k : 0u);
+            // a band has two rows at least
+            dst[k] = alone || !ok ? 0u : row == 0 ? to_above + 4u * u : row == c.rows - 1 ? to_below + 4u * u : 0u;
+            dst_bar[k] = row == 0 ? bar_above : bar_below;
+            edge = edge || dst[k] != 0u;
+            for (int b = 0; b < 2; ++b) spins[b][k] = res_smem[c.plane + b * c.plane_words + at[k]];
+        }
+    }
+
+    // Half word k of `colour`; its sums are added to `sums` for white.
+    template <int COLOUR>
+    __device__ __forceinline__ void decide(const Resident &c, int k, bool ok, uint32_t g, bool always, uint32_t &sums)
+    {
+        const int src = c.plane + (1 - COLOUR) * c.plane_words, tgt = c.plane + COLOUR * c.plane_words;
+        const bool on_left = ((odd >> k) & 1u) == (uint32_t)COLOUR;
+        const uint32_t above = res_smem[src + up[k]], below = res_smem[src + dn[k]], cur = spins[1 - COLOUR][k];
+        const uint32_t w = res_smem[src + (on_left ? left[k] : right[k])];
+        uint32_t sl, sr, mask = 0xFFFFFFFFu;
+        if (RAGGED) {
+            const uint32_t n4 = 4u * (uint32_t)c.last_nv;  // 4 .. 32 bits of a row's last half word
+            const bool first = (ends >> k) & 1u, last = (ends >> (k + 16)) & 1u;
+            sl = (cur << 4) | (w >> (first ? n4 - 4 : 28u));
+            sr = (cur >> 4) | (w << (last ? n4 - 4 : 28u));
+            if (last) mask = 0xFFFFFFFFu >> (32u - n4);
+        } else {
+            sl = __funnelshift_l(w, cur, 4);
+            sr = __funnelshift_r(cur, w, 4);
+        }
+        const uint32_t e = above + below + cur + (on_left ? sl : sr);
+        const uint32_t a8 = e + 0x88888888u, b8 = 0xCCCCCCCCu - e, tg = spins[COLOUR][k];
+        uint32_t none = 0;
+        uint32_t nt = always ? tg ^ kNibbleLsb : decide_sums<false, false>(tg, a8, b8, g, none);
+        if (RAGGED) nt &= mask;
+        spins[COLOUR][k] = nt;
+        if (ok) res_smem[tgt + at[k]] = nt;
+        peer_store_if(dst[k] != 0u, dst[k] + 4u * (COLOUR * c.plane_words), nt, dst_bar[k] + 8u * COLOUR);
+        if (COLOUR == 1) {
+            const uint32_t m = nt * 15u;
+            uint32_t d2 = ((a8 & ~m) | (b8 & m)) & 0x77777777u;  // anti-aligned neighbours
+            if (RAGGED) d2 &= mask;
+            const uint32_t by = (d2 & 0x0F0F0F0Fu) + (d2 >> 4 & 0x0F0F0F0Fu);
+            const uint32_t v = ((by * 0x01010101u) >> 24) | ((uint32_t)(__popc(nt) + __popc(cur)) << 16);
+            sums += ok ? v : 0u;
+        }
+    }
+};
+
 template <int K, bool RAGGED>
 __global__ void __launch_bounds__(kMaxThreads, 1) resident_kernel(const __grid_constant__ ResidentSweep p)
 {
-    extern __shared__ __align__(16) uint32_t res_smem[];
-    const int L = p.L, hpr = p.hpr, half = L / 2, tid = threadIdx.x, lane = tid & 31;
-    const int nc = (int)blockDim.x - 32;  // threads that compute; the last warp exchanges the halo rows
-    const bool halo = tid >= nc;
+    __shared__ __align__(8) uint64_t halo_bar[2];  // per colour: the halo rows of its next update have arrived
+    const int L = p.L, tid = threadIdx.x, lane = tid & 31;
     const int cs = (int)gridDim.x, rank = (int)cluster_rank();
-    const int r0 = rank * L / cs, rows = (rank + 1) * L / cs - r0;
-    const int plane_words = ((L + cs - 1) / cs + 2) * hpr;
+    Resident c;
+    c.hpr = p.hpr;
+    c.half = L / 2;
+    c.r0 = rank * L / cs;
+    c.rows = (rank + 1) * L / cs - c.r0;
+    c.items = c.rows * c.hpr;
+    c.nc = p.deciders;
+    const int most_rows = (L + cs - 1) / cs;
+    c.plane_words = (most_rows + 2) * c.hpr;
+    c.mark_words = most_rows * c.hpr;
+    c.last_nv = c.half - 8 * (c.hpr - 1);
     // each traced sweep's sums [kTraceRows] (up spins in the high half, anti-
-    // aligned pairs in the low half), the same per warp (16 bits each), then the
-    // black and the white plane: local rows 0 (halo above), 1 .. rows, rows + 1
-    // (halo below)
-    const int nw = nc >> 5;
+    // aligned pairs in the low half), the same per deciding warp (16 bits each),
+    // the planes, the marks of two sweeps
+    const int nw = c.nc >> 5;
     unsigned long long *tr = reinterpret_cast<unsigned long long *>(res_smem);
-    uint32_t *tw = res_smem + 2 * kTraceRows;
-    uint32_t *pl = tw + kTraceRows * nw;
-    const int last_nv = half - 8 * (hpr - 1);  // spins of a row's last half word
+    c.tw = 2 * kTraceRows;
+    c.plane = c.tw + kTraceRows * nw;
+    c.marks = c.plane + 2 * c.plane_words;
+    const int hpr = c.hpr, rows = c.rows, r0 = c.r0;
+    const uint32_t bar = (uint32_t)__cvta_generic_to_shared(halo_bar), halo_bytes = 8u * (uint32_t)hpr;
 
+    if (tid == 0) {
+        for (int b = 0; b < 2; ++b) bar_init(bar + 8 * b);
+        for (int b = 0; b < 2; ++b) bar_expect(bar + 8 * b, halo_bytes);
+    }
     for (int i = tid; i < (rows + 2) * hpr; i += blockDim.x) {
         const int lr = i / hpr, u = i - lr * hpr;
         int row = r0 - 1 + lr;
         row = row < 0 ? row + L : (row >= L ? row - L : row);
-        const int nv = u == hpr - 1 ? last_nv : 8;
 #pragma unroll
-        for (int c = 0; c < 2; ++c) pl[c * plane_words + i] = load_half(p, c, row, u, nv);
+        for (int b = 0; b < 2; ++b)
+            res_smem[c.plane + b * c.plane_words + i] = load_half(p, b, row, u, u == hpr - 1 ? c.last_nv : 8);
     }
-    // this thread's half words: local index and first draw
-    int at[K], u[K];
-    bool odd[K];  // parity of the lattice row
-    uint32_t blk[K], off[K];
-    const int items = rows * hpr;
-#pragma unroll
-    for (int k = 0; k < K; ++k) {
-        const int it = tid + k * nc;
-        const int row = it / hpr;
-        u[k] = it - row * hpr;
-        at[k] = it < items && !halo ? it + hpr : -1;
-        odd[k] = ((r0 + row) & 1) != 0;
-        const uint32_t site = (uint32_t)(r0 + row) * (uint32_t)half + 8u * (uint32_t)u[k];
-        blk[k] = site >> 2;
-        off[k] = site & 3u;
-    }
-    // where the halo rows of the CTAs above (its row below) and below (its row above) are
-    const uint32_t pl_u32 = (uint32_t)__cvta_generic_to_shared(pl);
-    const int above = rank == 0 ? cs - 1 : rank - 1, below = rank + 1 == cs ? 0 : rank + 1;
-    const int rows_above = (above + 1) * L / cs - above * L / cs;
-    const uint32_t to_above = peer_addr(pl_u32 + 4u * (uint32_t)((rows_above + 1) * hpr), (uint32_t)above);
-    const uint32_t to_below = peer_addr(pl_u32, (uint32_t)below);
-    const uint32_t last_mask = last_nv == 8 ? 0xFFFFFFFFu : (1u << (4 * last_nv)) - 1u;
-    const bool always = p.acc.always != 0;
-    cluster_arrive();
+    const bool always = p.acc.always != 0, trace = p.trace != nullptr, draws = tid < (int)blockDim.x - c.nc;
+    const int me = draws ? tid : tid - ((int)blockDim.x - c.nc);
+    const bool two = (int)blockDim.x == 2 * c.nc;  // a drawing thread serves both colours
+    bool dead = false;  // a wait ran out: no further ones, so that the launch ends
+    int traced = 0;     // sweeps summed in tr
 
-    int traced = 0;  // sweeps summed in tr
-    for (int s = 0; s < p.n_sweeps; ++s) {
-        const uint64_t t = p.t0 + (uint64_t)s;
-#pragma unroll 1
-        for (int colour = 0; colour < 2; ++colour) {
-            const DrawCtx dc{(uint32_t)t, counter_word3(colour, kPurposeMetropolis, t), p.acc.T3, p.acc.T4, p.acc.zero};
-            uint32_t *tgt = pl + colour * plane_words;
-            const uint32_t *src = pl + (1 - colour) * plane_words;
-            if (halo) {
-                cluster_wait();
-                __syncthreads();  // the colour is updated
-                const uint32_t o = 4u * (uint32_t)(colour * plane_words);
-                for (int i = lane; i < hpr; i += 32) {
-                    peer_store(to_above + o + 4u * i, tgt[hpr + i]);
-                    peer_store(to_below + o + 4u * i, tgt[rows * hpr + i]);
-                }
-                cluster_arrive();
-                continue;
+    // Behind the sweeps of a trace's rows, by all threads: every CTA adds up its
+    // warps; behind one more barrier the first CTA adds up the CTAs, and behind
+    // another the sums may be written again.
+    auto sweep_end = [&](int s) {
+        __syncthreads();
+        if (!trace || (++traced < kTraceRows && s + 1 < p.n_sweeps)) return;
+        for (int i = tid; i < traced; i += blockDim.x) {
+            unsigned long long v = 0;
+            for (int w = 0; w < nw; ++w) {
+                const uint32_t x = res_smem[c.tw + i * nw + w];
+                v += ((unsigned long long)(x >> 16) << 32) | (x & 0xFFFFu);
             }
-            uint32_t g[K];
-#pragma unroll
-            for (int k = 0; k < K; ++k) g[k] = at[k] >= 0 && !always ? marks8<RAGGED>(blk[k], off[k], dc, p.rk) : 0u;
+            tr[i] = v;
+        }
+        __syncwarp();
+        cluster_arrive();
+        cluster_wait();
+        if (rank == 0) {
+            const uint32_t tr_u32 = (uint32_t)__cvta_generic_to_shared(tr);
+            const long long area = (long long)L * L;
+            for (int i = tid; i < traced; i += blockDim.x) {
+                long long ones = 0, anti = 0;
+                for (int b = 0; b < cs; ++b) {
+                    const unsigned long long v = peer_load(peer_addr(tr_u32 + 8u * (uint32_t)i, (uint32_t)b));
+                    ones += (long long)(v >> 32);
+                    anti += (long long)(v & 0xFFFFFFFFull);
+                }
+                // L^2 / 2 white spins with 4 bonds each, as many black ones
+                long long *row = p.trace + 2 * (int64_t)(s + 1 - traced + i);
+                row[0] = 2 * ones - area;
+                row[1] = 2 * area - 2 * anti;
+            }
+        }
+        traced = 0;
+        __syncwarp();
+        cluster_arrive();
+        cluster_wait();
+    };
+
+    if (draws) {
+        const int colour = me >= c.nc, mine = me - colour * c.nc;
+        const int to = c.marks + colour * c.mark_words + mine;
+        Drawer<K, RAGGED> drawer(c, mine);
+        if (!always) drawer.draw(p, c, mine, p.t0, colour, to);
+        if (two && !always) drawer.draw(p, c, mine, p.t0, 1, to + c.mark_words);
+        __syncthreads();
+        cluster_arrive();
+        cluster_wait();
+        for (int s = 0; s < p.n_sweeps; ++s) {
+            if (!always && s + 1 < p.n_sweeps) {
+                drawer.draw(p, c, mine, p.t0 + (uint64_t)s + 1, colour, to + 2 * ((s + 1) & 1) * c.mark_words);
+                if (two) drawer.draw(p, c, mine, p.t0 + (uint64_t)s + 1, 1, to + (2 * ((s + 1) & 1) + 1) * c.mark_words);
+            }
+            sweep_end(s);
+        }
+    } else {
+        __syncthreads();
+        // the halo rows of the CTAs above (its row below) and below (its row above), and their barriers
+        const uint32_t plane = (uint32_t)__cvta_generic_to_shared(res_smem + c.plane);
+        const int above = rank == 0 ? cs - 1 : rank - 1, below = rank + 1 == cs ? 0 : rank + 1;
+        const int rows_above = (above + 1) * L / cs - above * L / cs;
+        Decider<K, RAGGED> d(c, me, cs == 1, peer_addr(plane + 4u * (uint32_t)((rows_above + 1) * hpr), (uint32_t)above),
+                             peer_addr(plane, (uint32_t)below), peer_addr(bar, (uint32_t)above),
+                             peer_addr(bar, (uint32_t)below));
+        cluster_arrive();
+        cluster_wait();
+        for (int s = 0; s < p.n_sweeps; ++s) {
             uint32_t sums = 0;
-            cluster_wait();
+            auto half_sweep = [&](auto colour_constant) {
+                constexpr int COLOUR = decltype(colour_constant)::value;
+                uint32_t g[K];
 #pragma unroll
-            for (int k = 0; k < K; ++k) {
-                if (at[k] < 0) continue;
-                const int i = at[k];
-                const uint32_t cur = src[i], tg = tgt[i];
-                const bool left = odd[k] == (colour == 1), last = u[k] == hpr - 1;
-                uint32_t side;
-                if (left) {
-                    uint32_t prev = src[u[k] == 0 ? i + hpr - 1 : i - 1];
-                    if (RAGGED && u[k] == 0) prev <<= 4 * (8 - last_nv);
-                    side = __funnelshift_l(prev, cur, 4);
-                } else {
-                    const uint32_t next = src[last ? i - u[k] : i + 1];
-                    if (RAGGED && last && last_nv < 8)
-                        side = (cur | (next << (4 * last_nv))) >> 4;
-                    else
-                        side = __funnelshift_r(cur, next, 4);
+                for (int k = 0; k < K; ++k)
+                    g[k] = res_smem[c.marks + (2 * (s & 1) + COLOUR) * c.mark_words + min(me + k * c.nc, c.items - 1)];
+                if (d.edge && (s > 0 || COLOUR == 1)) {
+                    // the other colour's halo rows: its update s, or s - 1 before black's
+                    const uint32_t b = bar + 8 * (1 - COLOUR);
+                    bar_wait(b, (uint32_t)(COLOUR == 1 ? s : s - 1) & 1u, dead);
+                    if (me == 0) bar_expect(b, halo_bytes);
                 }
-                const uint32_t e = src[i - hpr] + src[i + hpr] + cur;
-                const uint32_t a8 = e + side + 0x88888888u, b8 = 0xCCCCCCCCu - e - side;
-                uint32_t none = 0;
-                uint32_t nt = always ? tg ^ kNibbleLsb : decide_sums<false, false>(tg, a8, b8, g[k], none);
-                if (RAGGED && last) nt &= last_mask;
-                tgt[i] = nt;
-                if (colour == 1 && p.trace != nullptr) {
-                    const uint32_t m = nt * 15u;
-                    uint32_t d2 = ((a8 & ~m) | (b8 & m)) & 0x77777777u;  // anti-aligned neighbours
-                    if (RAGGED && last) d2 &= last_mask;
-                    const uint32_t by = (d2 & 0x0F0F0F0Fu) + (d2 >> 4 & 0x0F0F0F0Fu);
-                    sums += ((by * 0x01010101u) >> 24) | ((uint32_t)(__popc(nt) + __popc(cur)) << 16);
-                }
-            }
-            __syncthreads();
-            cluster_arrive_relaxed();
-            if (colour == 1 && p.trace != nullptr) {
+#pragma unroll
+                for (int k = 0; k < K; ++k)
+                    d.template decide<COLOUR>(c, k, me + k * c.nc < c.items, g[k], always, sums);
+            };
+            half_sweep(std::integral_constant<int, 0>{});
+            asm volatile("bar.sync 1, %0;" ::"r"(c.nc) : "memory");
+            half_sweep(std::integral_constant<int, 1>{});
+            if (trace) {
                 // at most 32 K of each per lane: both sums of a warp fit 16 bits
                 sums = __reduce_add_sync(0xffffffffu, sums);
-                if (lane == 0) tw[traced * nw + (tid >> 5)] = sums;
+                if (lane == 0) res_smem[c.tw + traced * nw + (me >> 5)] = sums;
             }
+            sweep_end(s);
         }
-        if (p.trace != nullptr && (++traced == kTraceRows || s + 1 == p.n_sweeps)) {
-            // every CTA adds up its warps; behind one more barrier the first CTA
-            // adds up the CTAs, and behind another the sums may be written again
-            cluster_wait();
-            __syncthreads();
-            for (int i = tid; i < traced; i += blockDim.x) {
-                unsigned long long v = 0;
-                for (int w = 0; w < nw; ++w) {
-                    const uint32_t x = tw[i * nw + w];
-                    v += ((unsigned long long)(x >> 16) << 32) | (x & 0xFFFFu);
-                }
-                tr[i] = v;
-            }
-            cluster_arrive();
-            cluster_wait();
-            if (rank == 0) {
-                const uint32_t tr_u32 = (uint32_t)__cvta_generic_to_shared(tr);
-                const long long area = (long long)L * L;
-                for (int i = tid; i < traced; i += blockDim.x) {
-                    long long ones = 0, anti = 0;
-                    for (int c = 0; c < cs; ++c) {
-                        const unsigned long long v = peer_load(peer_addr(tr_u32 + 8u * (uint32_t)i, (uint32_t)c));
-                        ones += (long long)(v >> 32);
-                        anti += (long long)(v & 0xFFFFFFFFull);
-                    }
-                    // L^2 / 2 white spins with 4 bonds each, as many black ones
-                    long long *row = p.trace + 2 * (int64_t)(s + 1 - traced + i);
-                    row[0] = 2 * ones - area;
-                    row[1] = 2 * area - 2 * anti;
-                }
-            }
-            traced = 0;
-            cluster_arrive();
-        }
+        // no CTA leaves while another's halo words are on their way to it
+        if (d.edge) bar_wait(bar + 8, (uint32_t)(p.n_sweeps - 1) & 1u, dead);
+        __syncwarp();
     }
-    cluster_wait();  // no CTA leaves while another may still write its halo rows
-    for (int i = tid; i < items; i += blockDim.x) {
+    cluster_arrive();
+    cluster_wait();
+    for (int i = tid; i < c.items; i += blockDim.x) {
         const int row = i / hpr, uu = i - row * hpr;
 #pragma unroll
-        for (int c = 0; c < 2; ++c)
-            store_half(p, c, r0 + row, uu, uu == hpr - 1 ? last_nv : 8, pl[c * plane_words + hpr + i]);
+        for (int b = 0; b < 2; ++b)
+            store_half(p, b, r0 + row, uu, uu == hpr - 1 ? c.last_nv : 8, res_smem[c.plane + b * c.plane_words + hpr + i]);
     }
 }
 
@@ -302,6 +465,8 @@ cudaError_t launch(const ResidentSweep &p, int cs, int threads, size_t smem, cud
 {
     auto kernel = resident_kernel<K, RAGGED>;
     cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e == cudaSuccess && smem > 48 * 1024)
+        e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)cs);
@@ -318,28 +483,49 @@ cudaError_t launch(const ResidentSweep &p, int cs, int threads, size_t smem, cud
     return cudaLaunchKernelEx(&cfg, kernel, p);
 }
 
+template <bool RAGGED>
+cudaError_t launch_k(const ResidentSweep &p, int k, int cs, int threads, size_t smem, cudaStream_t s)
+{
+    // at most 1024 half words per CTA on this route: one or two per thread
+    return k == 1 ? launch<1, RAGGED>(p, cs, threads, smem, s) : launch<2, RAGGED>(p, cs, threads, smem, s);
+}
+
 }  // namespace
 
 // Where the line lies, us per recorded sweep here / with two launches per sweep
-// (the host's rate): 512^2 2.7 / 3.4, 576^2 3.5 / 3.4 (16 SMs' multipliers bind);
-// ragged rows 258^2 2.0 / 3.6, 510^2 4.2 / 3.5.
-bool resident_fits(int64_t L) { return L <= (L % 16 ? 400 : 512); }
+// (the host's rate): 512^2 2.3 / 3.6, 576^2 3.35 / 3.6 (16 SMs' multipliers bind);
+// ragged rows 430^2 2.7 / 3.6, 510^2 3.4 / 3.6, 530^2 4.9 / 3.6.  A single call of
+// few sweeps of ragged rows is no faster here from about 400^2 on (510^2, us per
+// call of 1 / 3 / 10 sweeps: 14.7 / 22.6 / 45.5 here, 12.5 / 21.3 / 50.5 launched).
+bool resident_fits(int64_t L, int64_t n_sweeps) { return L <= (L % 16 && n_sweeps < 6 ? 400 : 512); }
+
+bool resident_timed_out()
+{
+    const bool out = g_resident_error != 0;
+    g_resident_error = 0;
+    return out;
+}
 
 cudaError_t resident_sweep(ResidentSweep p, int64_t n_sweeps, cudaStream_t s)
 {
     const int half = p.L / 2;
     p.hpr = (half + 7) / 8;
+    p.wide = ((uintptr_t)p.plane[0] | (uintptr_t)p.plane[1] | (uint64_t)p.stride) % 8 == 0;
     int cs = 1;
     while (cs < kMaxCluster && 2 * cs <= p.L && (int64_t)p.L * p.hpr >= kItems * 2 * cs) cs *= 2;
     const int rows = (p.L + cs - 1) / cs, items = rows * p.hpr;
-    const int k = (items + kMaxThreads - 33) / (kMaxThreads - 32);
-    const int threads = ((items + k - 1) / k + 31) / 32 * 32 + 32;
-    const size_t smem = ((2 + (threads - 32) / 32) * kTraceRows + 2 * (size_t)(rows + 2) * p.hpr) * sizeof(uint32_t);
+    const int k = (items + kMaxThreads / 2 - 1) / (kMaxThreads / 2);
+    p.deciders = ((items + k - 1) / k + 31) / 32 * 32;
+    // as many threads draw, or twice as many where drawing takes longest and the
+    // block has room: at two half words per thread (384^2 1.64 -> 1.43 us per sweep)
+    // and with ragged rows, three Philox blocks per half word (100^2 0.89 -> 0.69; but
+    // 256^2, one word each, 0.80 -> 0.84)
+    const int threads = p.deciders * ((k > 1 || half % 8) && 3 * p.deciders <= kMaxThreads ? 3 : 2);
+    const size_t smem =
+        ((2 + p.deciders / 32) * kTraceRows + 2 * (size_t)(rows + 2) * p.hpr + 4 * (size_t)items) * sizeof(uint32_t);
     while (n_sweeps > 0) {
         p.n_sweeps = (int32_t)std::min<int64_t>(n_sweeps, kMaxSweeps);
-        // at most 1024 half words per CTA on this route: one or two per thread
-        cudaError_t e = half % 8 ? (k == 1 ? launch<1, true>(p, cs, threads, smem, s) : launch<2, true>(p, cs, threads, smem, s))
-                                 : (k == 1 ? launch<1, false>(p, cs, threads, smem, s) : launch<2, false>(p, cs, threads, smem, s));
+        cudaError_t e = half % 8 ? launch_k<true>(p, k, cs, threads, smem, s) : launch_k<false>(p, k, cs, threads, smem, s);
         if (e != cudaSuccess) return e;
         n_sweeps -= p.n_sweeps;
         p.t0 += (uint64_t)p.n_sweeps;

@@ -134,3 +134,21 @@ def test_conversions_at_any_row_alignment(L, stride):
     ising.ising_observables(m, obs[1])
     want = [int(s.sum()), int((s.astype(int) * (np.roll(s, -1, 0) + np.roll(s, -1, 1))).sum())]
     assert obs.tolist() == [want, want]
+
+
+# the cluster kernel's halo rows over many sweeps: 2 to 16 CTAs, a draw thread
+# per half word and two, ragged rows of one and two half words per thread, and
+# more sweeps than one launch takes
+@pytest.mark.parametrize("layout,L,n", [
+    ("int8", 48, 2000), ("msc4", 128, 1500), ("int8", 100, 1500), ("int8", 256, 1500), ("msc4", 384, 400),
+    ("int8", 450, 150), ("int8", 498, 130), ("int8", 510, 130), ("int8", 512, 300), ("int8", 32, 16500)])
+def test_cluster_sweeps_stay_in_step(layout, L, n):
+    lat = ising.Lattice(L, layout)
+    ising.ising_init_lattice(lat, ising.ISING_INIT_RANDOM, 8)
+    s = oracle.init(L, oracle.MODE_RANDOM, 8)
+    trace = torch.full((n, 2), 77, dtype=torch.int64, device="cuda")
+    ising.ising_sweep(lat, BETA, n, 8, 1, trace)
+    want = oracle.run(s, BETA, n, 8, 1)
+    unpack = oracle.from_planes_int8 if layout == "int8" else oracle.from_planes_msc4
+    assert np.array_equal(unpack(L, *lat.planes_numpy()), s)
+    assert np.array_equal(trace.cpu().numpy(), want)
