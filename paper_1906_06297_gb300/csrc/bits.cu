@@ -16,80 +16,85 @@ namespace ising {
 
 // ---------------------------------------------------------------------------
 // MSC4 plane rows <-> the bit-packed format (one bit per spin, L/16 bytes per
-// row, dense rows): a thread converts V pairs of words (32 spins each) <-> V
-// uint32, V = 4 on rows of 4 pairs or more, else 1; blockIdx.x covers (row,
-// chunk of the row).  MSC4 -> bits: a thread's pairs are adjacent (one 16-byte
-// store of bits, where the row length and the buffer's alignment allow it);
-// bits -> MSC4: a thread's pairs are 256 apart, so that each warp store is part
-// of 512 contiguous bytes.
+// row, dense rows): a thread converts pairs of words (32 spins each) <-> uint32.
+// MSC4 -> bits: V adjacent pairs, 4 where that makes one aligned 16-byte store of
+// bits, else 1 (16384^2, four planes in turn: 16.5 and 20.6 us per plane; four pairs
+// a block's width apart 22.7); bits -> MSC4: kConvPairs pairs a block's width apart, so
+// that each warp store is contiguous (16.7 us; by rows, with blocks that 256 pairs
+// per row left three quarters idle, 20.5).  HBM-bound: 84 MB, 5.1 TB/s.
 // ---------------------------------------------------------------------------
-template <int V>
-__global__ void __launch_bounds__(256) msc4_to_bits_kernel(const uint64_t *plane, uint32_t *bits, int64_t stride_words,
-                                                           int64_t pairs, unsigned chunks)
+constexpr int kConvThreads = 256, kConvPairs = 4;
+
+template <typename I, int V>
+__global__ void __launch_bounds__(kConvThreads) msc4_to_bits_kernel(const uint64_t *plane, uint32_t *bits,
+                                                                    int64_t stride_words, I pairs, I n)
 {
-    const unsigned r = blockIdx.x / chunks;
-    const int64_t p = ((int64_t)(blockIdx.x - r * chunks) * 256 + threadIdx.x) * V;
-    if (p >= pairs) return;
-    const ulonglong2 *src = reinterpret_cast<const ulonglong2 *>(plane + (int64_t)r * stride_words + 2 * p);
+    const I p = ((I)blockIdx.x * kConvThreads + threadIdx.x) * V;
+    if (p >= n) return;
+    const I r = p / pairs;
+    const ulonglong2 *src =
+        reinterpret_cast<const ulonglong2 *>(plane + (int64_t)r * stride_words) + (int64_t)(p - r * pairs);
     uint32_t out[V];
 #pragma unroll
     for (int v = 0; v < V; ++v) {
         const ulonglong2 w = src[v];
         out[v] = msc4_word_to_bits(w.x) | (msc4_word_to_bits(w.y) << 16);
     }
-    uint32_t *dst = bits + (int64_t)r * pairs + p;
-    if constexpr (V == 4)
-        *reinterpret_cast<uint4 *>(dst) = make_uint4(out[0], out[1], out[2], out[3]);
-    else
-        dst[0] = out[0];
+    if constexpr (V == 4) *reinterpret_cast<uint4 *>(bits + p) = make_uint4(out[0], out[1], out[2], out[3]);
+    else bits[p] = out[0];
 }
 
-template <int V>
-__global__ void __launch_bounds__(256) bits_to_msc4_kernel(const uint32_t *bits, uint64_t *plane, int64_t stride_words,
-                                                           int64_t pairs, unsigned chunks)
+template <typename I>
+__global__ void __launch_bounds__(kConvThreads) bits_to_msc4_kernel(const uint32_t *bits, uint64_t *plane,
+                                                                    int64_t stride_words, I pairs, I n)
 {
-    const unsigned r = blockIdx.x / chunks;
-    const int64_t p0 = (int64_t)(blockIdx.x - r * chunks) * 256 * V + threadIdx.x;
-    const uint32_t *src = bits + (int64_t)r * pairs;
-    ulonglong2 *dst = reinterpret_cast<ulonglong2 *>(plane + (int64_t)r * stride_words);
-    uint32_t b[V];
+    const I base = (I)blockIdx.x * (kConvThreads * kConvPairs) + threadIdx.x;
+    uint32_t b[kConvPairs];
 #pragma unroll
-    for (int v = 0; v < V; ++v) b[v] = p0 + 256 * v < pairs ? src[p0 + 256 * v] : 0u;
+    for (int v = 0; v < kConvPairs; ++v) b[v] = base + kConvThreads * v < n ? bits[base + kConvThreads * v] : 0u;
 #pragma unroll
-    for (int v = 0; v < V; ++v)
-        if (p0 + 256 * v < pairs)
-            dst[p0 + 256 * v] = make_ulonglong2(bits_to_msc4_word(b[v] & 0xFFFFu), bits_to_msc4_word(b[v] >> 16));
+    for (int v = 0; v < kConvPairs; ++v) {
+        const I i = base + kConvThreads * v;
+        if (i < n) {
+            const I r = i / pairs;
+            *reinterpret_cast<ulonglong2 *>(plane + (int64_t)r * stride_words + 2 * (int64_t)(i - r * pairs)) =
+                make_ulonglong2(bits_to_msc4_word(b[v] & 0xFFFFu), bits_to_msc4_word(b[v] >> 16));
+        }
+    }
+}
+
+// Calls go(index, blocks) with an index type wide enough for n pairs, `per` of
+// them per block.
+template <typename Go>
+cudaError_t conv_launch(int64_t n, int per, Go go)
+{
+    const int64_t blocks = (n + per - 1) / per;
+    if (blocks > INT32_MAX) return cudaErrorInvalidConfiguration;
+    if (n < (int64_t(1) << 31)) go(uint32_t{}, (unsigned)blocks);
+    else go(uint64_t{}, (unsigned)blocks);
+    return cudaGetLastError();
 }
 
 cudaError_t msc4_to_bits(const uint64_t *plane, int64_t stride_words, uint32_t *bits, int64_t L, int64_t rows,
                          cudaStream_t s)
 {
-    const int64_t pairs = L / 64;
-    // V = 4 needs a multiple of 4 pairs per row and 16-byte aligned bit rows
-    const int V = pairs % 4 == 0 && (uintptr_t)bits % 16 == 0 ? 4 : 1;
-    const unsigned chunks = (unsigned)((pairs / V + 255) / 256);
-    if (rows * (int64_t)chunks > INT32_MAX) return cudaErrorInvalidConfiguration;
-    const unsigned grid = (unsigned)(rows * chunks);
-    if (V == 4)
-        msc4_to_bits_kernel<4><<<grid, 256, 0, s>>>(plane, bits, stride_words, pairs, chunks);
-    else
-        msc4_to_bits_kernel<1><<<grid, 256, 0, s>>>(plane, bits, stride_words, pairs, chunks);
-    return cudaGetLastError();
+    const int64_t pairs = L / 64, n = rows * pairs;
+    const bool wide = pairs % 4 == 0 && (uintptr_t)bits % 16 == 0;
+    return conv_launch(n, kConvThreads * (wide ? 4 : 1), [&](auto index, unsigned blocks) {
+        using I = decltype(index);
+        if (wide) msc4_to_bits_kernel<I, 4><<<blocks, kConvThreads, 0, s>>>(plane, bits, stride_words, (I)pairs, (I)n);
+        else msc4_to_bits_kernel<I, 1><<<blocks, kConvThreads, 0, s>>>(plane, bits, stride_words, (I)pairs, (I)n);
+    });
 }
 
 cudaError_t bits_to_msc4(const uint32_t *bits, uint64_t *plane, int64_t stride_words, int64_t L, int64_t rows,
                          cudaStream_t s)
 {
-    const int64_t pairs = L / 64;
-    const int V = pairs >= 4 ? 4 : 1;
-    const unsigned chunks = (unsigned)((pairs + 256 * V - 1) / (256 * V));
-    if (rows * (int64_t)chunks > INT32_MAX) return cudaErrorInvalidConfiguration;
-    const unsigned grid = (unsigned)(rows * chunks);
-    if (V == 4)
-        bits_to_msc4_kernel<4><<<grid, 256, 0, s>>>(bits, plane, stride_words, pairs, chunks);
-    else
-        bits_to_msc4_kernel<1><<<grid, 256, 0, s>>>(bits, plane, stride_words, pairs, chunks);
-    return cudaGetLastError();
+    const int64_t pairs = L / 64, n = rows * pairs;
+    return conv_launch(n, kConvThreads * kConvPairs, [&](auto index, unsigned blocks) {
+        using I = decltype(index);
+        bits_to_msc4_kernel<I><<<blocks, kConvThreads, 0, s>>>(bits, plane, stride_words, (I)pairs, (I)n);
+    });
 }
 
 // ---------------------------------------------------------------------------

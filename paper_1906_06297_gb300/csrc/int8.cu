@@ -31,15 +31,14 @@ constexpr int kThreads = 256;
 constexpr int kFlatThreads = 512;
 
 // ---------------------------------------------------------------------------
-// Four spins at once, one per byte of a 32-bit word (+1 = 0x01, -1 = 0xFF).
-// Bit 1 of a byte says "down", so the sum of four words masked to that bit is
-// twice the number of down neighbours, y = 2 kd in 0..8, and no carry leaves a
-// byte.  With d the number of anti-aligned neighbours (kd for an up spin, 4 - kd
-// for a down spin) and G the draw's marks (half_marks), the decision is "flip
-// iff d >= G"; per byte 16 + 2 d - 2 G lies in 12..24, and its bit 4 is the flip.
+// Four spins at once, one per byte of a 32-bit word (+1 = 0x01, -1 = 0xFF): bits 1
+// to 7 of a byte all say "down", so any of them can hold a plane of a bitwise sum.
+// With a = up ^ down ^ centre and m their majority, the number d of neighbours that
+// differ from the spin t is odd where a ^ side, and 2 or more where (m ^ t) |
+// (a ^ t) & (side ^ t).  A spin flips iff d >= 2, or d = 1 and its draw is below T3, or
+// its draw is below T4 (T4 <= T3); the draws' marks have bit 6 of a byte set where
+// u >= T3, bit 7 where u >= T4.
 // ---------------------------------------------------------------------------
-constexpr uint32_t kDown = 0x02020202u;
-
 __device__ __forceinline__ uint32_t byte_signs(uint32_t x)  // 0xFF where the byte's top bit is set
 {
     uint32_t r;
@@ -47,50 +46,59 @@ __device__ __forceinline__ uint32_t byte_signs(uint32_t x)  // 0xFF where the by
     return r;
 }
 
+__device__ __forceinline__ void mark_byte(uint32_t &g, uint32_t u, uint32_t T3, uint32_t T4, uint32_t bit6, uint32_t bit7)
+{
+    asm("{\n\t"
+        ".reg .pred p3, p4;\n\t"
+        "setp.ge.u32 p3, %1, %3;\n\t"
+        "setp.ge.u32 p4, %1, %4;\n\t"
+        "@p3 add.u32 %0, %0, %2;\n\t"
+        "@p4 add.u32 %0, %0, %5;\n\t"
+        "}"
+        : "+r"(g)
+        : "r"(u), "r"(bit6), "r"(T3), "r"(T4), "r"(bit7));
+}
+
 __device__ __forceinline__ uint32_t block_marks(uint32_t q, const DrawCtx &dc, const RoundKeys &rk)
 {
     const uint4 u = philox(q, 0u, dc.c2, dc.c3, rk);
-    uint32_t g = 0, unused = 0;
-    mark_ge(g, unused, u.x, dc.T3, dc.T4, 1u << 1);
-    mark_ge(g, unused, u.y, dc.T3, dc.T4, 1u << 9);
-    mark_ge(g, unused, u.z, dc.T3, dc.T4, 1u << 17);
-    mark_ge(g, unused, u.w, dc.T3, dc.T4, 1u << 25);
+    uint32_t g = 0;
+    mark_byte(g, u.x, dc.T3, dc.T4, 1u << 6, 1u << 7);
+    mark_byte(g, u.y, dc.T3, dc.T4, 1u << 14, 1u << 15);
+    mark_byte(g, u.z, dc.T3, dc.T4, 1u << 22, 1u << 23);
+    mark_byte(g, u.w, dc.T3, dc.T4, 1u << 30, 1u << 31);
     return g;
 }
 
-__device__ __forceinline__ uint32_t neighbour_downs(uint32_t up, uint32_t cur, uint32_t dn, uint32_t side)
+__device__ __forceinline__ uint32_t majority(uint32_t a, uint32_t b, uint32_t c) { return (a & b) | (a & c) | (b & c); }
+
+// Adds the down spins among t and the centres to `down` and t's differing
+// neighbours to `anti`, over the bytes of mask `in`: d is the plane a ^ side plus
+// twice two others, so one count of bits takes them all from bits of their own.
+__device__ __forceinline__ void count_bytes(uint32_t t, uint32_t a, uint32_t m, uint32_t cur, uint32_t side, uint32_t in,
+                                            uint32_t &down, uint32_t &anti)
 {
-    return (up & kDown) + (cur & kDown) + (dn & kDown) + (side & kDown);
+    const uint32_t two = (a ^ t) & (side ^ t);
+    const uint32_t d = ((a ^ side) & 0x02020202u) | ((m ^ t) & 0x0C0C0C0Cu) | (two & 0x30303030u);
+    const uint32_t n = (t & 0x02020202u) | (cur & 0x04040404u);
+    anti += __popc(d & in);
+    down += __popc(n & in);
 }
 
-// Adds twice the down spins among t and the centres, and twice t's anti-aligned
-// counts given y, over the bytes of mask `in`.
-__device__ __forceinline__ void count_bytes(uint32_t t, uint32_t y, uint32_t cur, uint32_t in, uint32_t &down,
-                                            uint32_t &anti)
-{
-    const uint32_t m = byte_signs(t);
-    const uint32_t d2 = ((y & ~m) | ((0x08080808u - y) & m)) & in;  // 2 d in 0..8
-    down += (((t & (kDown & in)) + (cur & (kDown & in))) * 0x01010101u) >> 24;
-    anti += (d2 * 0x01010101u) >> 24;
-}
-
-// New values of the four spins t; with OBS, adds to `down` twice the number of
-// down spins among the new values and the centres and to `anti` twice the
-// anti-aligned counts after the update, both over the bytes of mask `in`.
+// New values of the four spins t; with OBS, counts them over the bytes of mask `in`.
 template <bool OBS, bool ALWAYS>
 __device__ __forceinline__ uint32_t decide_bytes(uint32_t t, uint32_t up, uint32_t cur, uint32_t dn, uint32_t side,
                                                  uint32_t g, uint32_t in, uint32_t &down, uint32_t &anti)
 {
-    const uint32_t y = neighbour_downs(up, cur, dn, side);
+    const uint32_t a = up ^ dn ^ cur, m = majority(up, dn, cur);
     uint32_t nt;
     if (ALWAYS) {
         nt = t ^ 0xFEFEFEFEu;
     } else {
-        const uint32_t m = byte_signs(t);
-        const uint32_t x = (((y + 0x10101010u) & ~m) | ((0x18181818u - y) & m)) - g;
-        nt = t ^ (byte_signs(x << 3) & 0xFEFEFEFEu);
+        const uint32_t two = (m ^ t) | ((a ^ t) & (side ^ t)), one = ((a ^ side) & ~g) << 1;
+        nt = t ^ (byte_signs(two | one | ~g) & 0xFEFEFEFEu);
     }
-    if (OBS) count_bytes(nt, y, cur, in, down, anti);
+    if (OBS) count_bytes(nt, a, m, cur, side, in, down, anti);
     return nt;
 }
 
@@ -106,7 +114,8 @@ struct FlatSplit {
 // its logic instructions per spin.  Launched as msc4_flat_kernel is (one block
 // per SM, marks before the wait for the kernel before it).  2560^2, us per
 // sweep: thread per Philox block with 64-bit site indices and byte accesses
-// 36.9, this kernel 9.0 with the observables and 8.55 without.
+// 36.9, this kernel with sums of two-bit fields and a compare per byte 8.55, with the
+// bitwise planes 8.3 (9.0 with the observables either way).
 template <bool OBS, bool ALWAYS>
 __global__ void __launch_bounds__(kFlatThreads, 2)
     int8_words_kernel(const __grid_constant__ Int8SweepParams p, const __grid_constant__ FlatSplit f)
@@ -155,7 +164,7 @@ __global__ void __launch_bounds__(kFlatThreads, 2)
     if (OBS) {
         // n white and n black spins, 4 n bonds
         const long long n = 16 * (long long)(end - blockIdx.x * f.per);
-        block_count_add2(down, anti, -1, 2 * n, -1, 4 * n, p.obs);
+        block_count_add2(down, anti, -2, 2 * n, -2, 4 * n, p.obs);
     }
 }
 
@@ -257,7 +266,7 @@ __global__ void __launch_bounds__(kFlatThreads, 2)
         // the sites of units [lo, end): whole rows of L / 2 and what is left of the last
         auto sites = [&](uint32_t e) { return (long long)(e / f.upr) * half + min(4u * WORDS * (e % f.upr), half); };
         const long long n = sites(end) - sites(blockIdx.x * f.per);
-        block_count_add2(down, anti, -1, 2 * n, -1, 4 * n, p.obs);
+        block_count_add2(down, anti, -2, 2 * n, -2, 4 * n, p.obs);
     }
 }
 
@@ -414,13 +423,13 @@ __global__ void __launch_bounds__(256) int8_obs_kernel(const int8_t *__restrict_
         for (int h = 0; h < 4; ++h) {
             const uint32_t m = bytes_in(h, nv);
             const uint32_t side = row_side<4>(cur, edge, left, h, nv);
-            count_bytes(t[h], neighbour_downs(up[h], cur[h], dn[h], side), cur[h], m, down, anti);
+            count_bytes(t[h], up[h] ^ dn[h] ^ cur[h], majority(up[h], dn[h], cur[h]), cur[h], side, m, down, anti);
         }
         n += nv;
         down_sum += down;
         anti_sum += anti;
     }
-    block_reduce_add2<256>(2 * n - down_sum, 4 * n - anti_sum, out);
+    block_reduce_add2<256>(2 * n - 2 * down_sum, 4 * n - 2 * anti_sum, out);
 }
 
 unsigned grid_for(int64_t n, int threads, int per_sm)
