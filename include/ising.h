@@ -270,8 +270,9 @@ ISING_API int ising_slab_sweep(const ising_slab_t *slabs, int32_t n, double beta
 /* Batches of lattices with replica exchange.  Not in the paper: the batched */
 /* form of its sweep.  n lattices (sides L[i], multiples of 32 up to 65536,  */
 /* MSC4 planes) are swept together in ONE persistent cooperative launch with */
-/* grid-wide barriers (each wait bounded: a timeout sets ISING_ETIMEOUT,     */
-/* read back by ising_batch_check).  Lattices [l*S, (l+1)*S) form ladder l   */
+/* barriers between half-sweeps and at records (each wait across the grid    */
+/* bounded: a timeout sets ISING_ETIMEOUT, read back by ising_batch_check).  */
+/* Lattices [l*S, (l+1)*S) form ladder l                                     */
 /* over S increasing inverse temperatures beta[0..S-1]; lattice i starts at  */
 /* slot i mod S and is swept at the beta of its current slot.  Lattice i     */
 /* draws in stream i (i added to Philox counter word 1), so lattice 0 follows */

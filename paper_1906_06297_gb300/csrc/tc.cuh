@@ -138,37 +138,11 @@ __device__ __forceinline__ void tma_load_4d(void *smem_dst, const void *tmap, in
         : "memory");
 }
 
-// D[tmem] (+)= A[smem] * B[smem]^T, issued by one thread.
-__device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
-                                         uint32_t accumulate)
-{
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
-        "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
-        : "memory");
-}
-
-// The same MMA with each descriptor given as its two 32-bit words.  Only the
-// low word holds the start address (bits 0-13, in 16-byte units), so moving an
-// operand by a multiple of 16 bytes below the 2^18-byte shared window is one
-// 32-bit add on the low word.
-__device__ __forceinline__ void mma_bf16_w(uint32_t d_tmem, uint32_t a_lo, uint32_t a_hi, uint32_t b_lo, uint32_t b_hi,
-                                           uint32_t idesc, uint32_t accumulate)
-{
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t.reg .b64 a, b;\n\t"
-        "setp.ne.b32 p, %6, 0;\n\t"
-        "mov.b64 a, {%1, %2};\n\t"
-        "mov.b64 b, {%3, %4};\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %5, p;\n\t}" ::"r"(d_tmem),
-        "r"(a_lo), "r"(a_hi), "r"(b_lo), "r"(b_hi), "r"(idesc), "r"(accumulate)
-        : "memory");
-}
-
-// The same and its commit by a whole converged warp, of which one elected lane
-// (the same one each time) issues.
+// D[tmem] (+)= A[smem] * B[smem]^T and its commit by a whole converged warp, of
+// which one elected lane (the same one each time) issues.  Each descriptor is
+// given as its two 32-bit words: only the low word holds the start address (bits
+// 0-13, in 16-byte units), so moving an operand by a multiple of 16 bytes below
+// the 2^18-byte shared window is one 32-bit add on it.
 __device__ __forceinline__ void mma_bf16_warp(uint32_t d_tmem, uint32_t a_lo, uint32_t a_hi, uint32_t b_lo, uint32_t b_hi,
                                               uint32_t idesc, uint32_t accumulate)
 {
@@ -197,14 +171,6 @@ __device__ __forceinline__ void mma_commit_warp(uint64_t *bar)
                  : "memory");
 }
 
-// The mbarrier gets one arrival when every MMA this thread issued before has
-// completed.
-__device__ __forceinline__ void mma_commit(uint64_t *bar)
-{
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
-                 : "memory");
-}
-
 // 16 consecutive 32-bit columns of this warp's 32 TMEM lanes (thread t gets
 // lane base + t); waits for the load before returning.
 __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16])
@@ -228,17 +194,6 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16])
     for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
 }
 
-// Zeros 16 consecutive 32-bit columns of this warp's 32 TMEM lanes; the
-// stores are complete once tmem_wait_st() returns.
-__device__ __forceinline__ void tmem_st16_zero(uint32_t taddr)
-{
-    const uint32_t z = 0u;
-    asm volatile(
-        "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, "
-        "%1};" ::"r"(taddr),
-        "r"(z)
-        : "memory");
-}
 // Stores 16 values into 16 consecutive 32-bit columns of this warp's 32 TMEM
 // lanes (every lane the same 16 values); complete once tmem_wait_st() returns.
 __device__ __forceinline__ void tmem_st16(uint32_t taddr, const float (&v)[16])
