@@ -418,7 +418,8 @@ cudaError_t launch_sweep(const Msc4SweepParams &p, cudaStream_t s)
     return cudaGetLastError();
 }
 
-// Where the lines lie (us per sweep with the trace): one half word per thread
+// Where the lines lie (us per sweep with the trace, observables by 64-bit shuffles,
+// which both sides share): one half word per thread
 // up to 1024 of them per SM, for the shortest chain from a kernel's wait to its
 // stores (1536^2: 4.6 against 5.2 with four), else four (2048^2: 5.4 against
 // 7.0; two are never best); and the marching kernel above 3 million pairs of
