@@ -545,19 +545,23 @@ __device__ __forceinline__ bool pair_swaps(const BatchParams &p, const long long
 // partner's thread comes to the same answer), from the state `at` that event left
 // by the last one; the new state goes to the other buffer, `at_next`.  The sums
 // read here are cleared at the next event, when every thread has read them.
-// Everything but the sums is fetched ahead of the barrier that completes them:
-// one load of the sums, one of the table stand behind it instead of a chain of
-// five (a record of 384 lattices of sides 64 to 256: 5.6 -> 4.6 us).
+// What other owners write is read behind the barrier alone: the sums, and the
+// partner's entry of `at`, which its owner wrote behind the last event's barrier (no
+// barrier of the grid lies between that store and the front of this one, so an
+// early owner would find the state of two events ago there).  The lattice's slot,
+// the draw and the pair's table are the owner's own or constant and are fetched ahead
+// of the barrier (384 lattices of sides 64 to 256 recorded every second sweep: 1329 us
+// per 100 sweeps).
 struct OwnerPair {
-    int32_t x, k, pk, y;  // the lattice, its slot, its partner's slot (-1: none) and lattice
+    int32_t x, k, pk;  // the lattice, its slot, its partner's slot (-1: none)
     uint32_t w;
     int64_t off, len;
 };
 
 // Lattice number i of the block's owner (x = -1 behind the last one).
-__device__ __forceinline__ OwnerPair owner_pair(const BatchParams &p, uint64_t t, int64_t i, const int32_t *at)
+__device__ __forceinline__ OwnerPair owner_pair(const BatchParams &p, uint64_t t, int64_t i)
 {
-    OwnerPair r = {-1, 0, -1, 0, 0u, 0, 0};
+    OwnerPair r = {-1, 0, -1, 0u, 0, 0};
     const int o = (int)blockIdx.x / p.cs;
     for (int g = 0; g < p.n_groups && r.x < 0; ++g) {
         const int64_t first = p.part[g][o], count = p.part[g][o + 1] - first;
@@ -565,7 +569,6 @@ __device__ __forceinline__ OwnerPair owner_pair(const BatchParams &p, uint64_t t
         i -= count;
     }
     if (r.x < 0) return r;
-    const int64_t l = r.x / p.S;
     r.k = p.slot_of[r.x];
     if (p.swaps) {
         const int e = (int)((t + 1) / (uint64_t)p.record_every) - 1;
@@ -573,10 +576,9 @@ __device__ __forceinline__ OwnerPair owner_pair(const BatchParams &p, uint64_t t
         const int pk = lower ? r.k + 1 : r.k - 1, k = lower ? r.k : pk;
         if (pk >= 0 && pk < p.S) {
             r.pk = pk;
-            r.y = at[l * p.S + pk];
             r.off = p.swap_off[k];
             r.len = p.swap_len[k];
-            r.w = pair_draw(p, l, k, t);
+            r.w = pair_draw(p, r.x / p.S, k, t);
         }
     }
     return r;
@@ -589,6 +591,7 @@ __device__ __forceinline__ void owner_exchange(const BatchParams &p, uint64_t t,
     const int64_t e = (int64_t)((t + 1) / (uint64_t)p.record_every) - 1;
     while (r.x >= 0) {
         const int64_t l = r.x / p.S;
+        const int32_t y = r.pk >= 0 ? at[l * p.S + r.pk] : 0;
         if (p.trace != nullptr) {
             long long *row = p.trace + 2 * ((e - p.event_first) * p.n + l * p.S + r.k);
             row[0] = acc[2 * r.x];
@@ -596,7 +599,7 @@ __device__ __forceinline__ void owner_exchange(const BatchParams &p, uint64_t t,
         }
         if (r.pk >= 0) {
             const bool lower = r.pk > r.k;
-            if (pair_swaps(p, acc, lower ? r.x : r.y, lower ? r.y : r.x, r.w, r.off, r.len)) {
+            if (pair_swaps(p, acc, lower ? r.x : y, lower ? y : r.x, r.w, r.off, r.len)) {
                 r.k = r.pk;
                 p.slot_of[r.x] = r.k;
             }
@@ -605,7 +608,7 @@ __device__ __forceinline__ void owner_exchange(const BatchParams &p, uint64_t t,
         acc_next[2 * r.x] = 0;
         acc_next[2 * r.x + 1] = 0;
         i += (int64_t)p.cs * blockDim.x;
-        r = owner_pair(p, t, i, at);
+        r = owner_pair(p, t, i);
     }
 }
 
@@ -673,7 +676,7 @@ __global__ void __launch_bounds__(512, 1) batch_kernel(const __grid_constant__ B
             const int64_t mine = (int)blockIdx.x % max(p.cs, 1) + (int64_t)p.cs * threadIdx.x;
             const int32_t *at = odd ? p.lattice_at2 : p.lattice_at;
             OwnerPair pair = {-1};
-            if (p.cs > 0) pair = owner_pair(p, t, mine, at);
+            if (p.cs > 0) pair = owner_pair(p, t, mine);
             if (!grid_sync(p)) return;
             if (p.cs > 0) {
                 owner_exchange(p, t, pair, mine, at, odd ? p.lattice_at : p.lattice_at2, odd ? p.acc2 : p.acc,
