@@ -8,6 +8,7 @@
 #include <algorithm>
 #include <climits>
 #include <cstdint>
+#include <type_traits>
 
 #include "common.cuh"
 #include "launch.h"
@@ -141,11 +142,13 @@ struct BitsSplit {
     uint32_t end[kMaxBitsBands];  // cumulative rows of the bands
 };
 
-// Q64: the Philox counter q = site / 4 needs 64 bits (L above 185363).
+// Q64: the Philox counter q = site / 4 needs 64 bits (L above 185363), and so do the
+// plane's word indices from L = 524352 on; below, these stay under 2^30.
 template <bool ALWAYS, bool Q64>
 __global__ void __launch_bounds__(kBitsThreads, 2)
     bits_sweep_kernel(const __grid_constant__ BitsSweepParams p, const __grid_constant__ BitsSplit f)
 {
+    using I = typename std::conditional<Q64, uint64_t, uint32_t>::type;
     const uint32_t lo = blockIdx.x * f.per, end = min(f.items, lo + f.per), L = (uint32_t)p.L;
     uint32_t rcat = (lo + threadIdx.x) / f.upr, u = lo + threadIdx.x - rcat * f.upr;
     const uint32_t step_rows = blockDim.x / f.upr, step_u = blockDim.x - step_rows * f.upr;
@@ -159,11 +162,11 @@ __global__ void __launch_bounds__(kBitsThreads, 2)
         const BitsBand &b = p.band[j];
         const uint32_t row = (uint32_t)b.row0 + rcat - (j ? f.end[j - 1] : 0u);
         const uint32_t *src = p.bits[1 - b.colour];
-        const uint32_t at = row * f.upr + u;  // below 2^30
+        const I at = (I)row * f.upr + u;
         uint32_t *tp = p.bits[b.colour] + at;
         const bool left = ((row + (uint32_t)b.colour) & 1) == 0;
-        const uint32_t up = src[(row == 0 ? L - 1 : row - 1) * f.upr + u];
-        const uint32_t dn = src[(row + 1 == L ? 0 : row + 1) * f.upr + u];
+        const uint32_t up = src[(I)(row == 0 ? L - 1 : row - 1) * f.upr + u];
+        const uint32_t dn = src[(I)(row + 1 == L ? 0 : row + 1) * f.upr + u];
         const uint32_t cur = src[at], t = *tp;
         const uint32_t edge = src[left ? (u == 0 ? at + f.upr : at) - 1 : (u + 1 == f.upr ? at + 1 - f.upr : at + 1)];
         uint32_t ns;
@@ -172,7 +175,7 @@ __global__ void __launch_bounds__(kBitsThreads, 2)
         if (ALWAYS) {
             ns = ~t;
         } else {
-            const uint32_t c0 = 8 * at, c1 = Q64 ? at >> 29 : 0u, c3 = p.c3 | (uint32_t)b.colour;
+            const uint32_t c0 = 8 * (uint32_t)at, c1 = Q64 ? (uint32_t)((uint64_t)at >> 29) : 0u, c3 = p.c3 | (uint32_t)b.colour;
             uint32_t g3 = 0, g4 = 0;
 #pragma unroll
             for (int k = 0; k < 8; ++k) {
