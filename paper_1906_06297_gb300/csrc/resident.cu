@@ -416,6 +416,7 @@ __global__ void __launch_bounds__(kMaxThreads, 1) resident_kernel(const __grid_c
         Decider<K, RAGGED> d(c, me, cs == 1, peer_addr(plane + 4u * (uint32_t)((rows_above + 1) * hpr), (uint32_t)above),
                              peer_addr(plane, (uint32_t)below), peer_addr(bar, (uint32_t)above),
                              peer_addr(bar, (uint32_t)below));
+        __syncwarp();
         cluster_arrive();
         cluster_wait();
         for (int s = 0; s < p.n_sweeps; ++s) {
@@ -437,7 +438,9 @@ __global__ void __launch_bounds__(kMaxThreads, 1) resident_kernel(const __grid_c
                     d.template decide<COLOUR>(c, k, me + k * c.nc < c.items, g[k], always, sums);
             };
             half_sweep(std::integral_constant<int, 0>{});
-            asm volatile("bar.sync 1, %0;" ::"r"(c.nc) : "memory");
+            // not bar.sync, which wants whole warps: edge and inner rows may share one, whose
+            // lanes leave the wait above one by one
+            asm volatile("barrier.sync 1, %0;" ::"r"(c.nc) : "memory");
             half_sweep(std::integral_constant<int, 1>{});
             if (trace) {
                 // at most 32 K of each per lane: both sums of a warp fit 16 bits
