@@ -110,9 +110,23 @@ ISING_API int ising_half_sweep(const ising_lattice_t *lat, double beta, int32_t 
  * sweep (the call zeroes it first).  Running a sweeps and then b sweeps with
  * offset a gives the same lattice as a + b sweeps in one call.  L <= 512 runs in
  * one cluster whose CTAs wait for one another, each wait bounded (~2 s): should
- * one give up, the next such call returns ISING_ETIMEOUT. */
+ * one give up, the lattice and the trace are not to be used and ising_sweep_check
+ * says so. */
 ISING_API int ising_sweep(const ising_lattice_t *lat, double beta, int64_t n_sweeps, uint64_t seed,
                           uint64_t sweep_offset, int64_t *trace_dev, ising_stream_t stream);
+
+/* Synchronises `stream`, then reports ISING_ETIMEOUT (and clears the flag, one per
+ * device) if a wait of a small-lattice sweep on the current device, called or
+ * replayed from a graph, gave up since the last check, else ISING_OK.  Refuses no
+ * sweep: calls made before the check run as usual. */
+ISING_API int ising_sweep_check(ising_stream_t stream);
+
+/* Failure-path self-test of those waits: a few sweeps of `lat` (48 <= L <= 512) in
+ * which one CTA sends its neighbours nothing, so that their waits run out after
+ * about 1 ms.  The launch ends, the lattice holds meaningless spins, and the next
+ * ising_sweep_check reports ISING_ETIMEOUT; the device stays usable.  Not part of
+ * the method. */
+ISING_API int ising_sweep_wait_selftest(const ising_lattice_t *lat, ising_stream_t stream);
 
 /* Same as ising_sweep, for a lattice held in host memory: copies the dense
  * host planes (L rows of ising_lattice_bytes' row_bytes each) into the

@@ -82,6 +82,8 @@ def _load():
             "ising_init_lattice": [LP, i32, u64, P],
             "ising_half_sweep": [LP, dbl, i32, u64, u64, P, P],
             "ising_sweep": [LP, dbl, i64, u64, u64, P, P],
+            "ising_sweep_check": [P],
+            "ising_sweep_wait_selftest": [LP, P],
             "ising_sweep_host": [LP, P, P, dbl, i64, u64, u64, P, P, P],
             "ising_bits_bytes": [i64, P],
             "ising_msc4_to_bits": [LP, P, P, P],
@@ -225,6 +227,14 @@ def ising_half_sweep(lat, beta: float, colour: int, seed: int, t: int, obs=None,
 def ising_sweep(lat, beta: float, n_sweeps: int, seed: int, sweep_offset: int = 0, trace=None, stream=None):
     _check(_load().ising_sweep(ctypes.byref(_struct(lat)), float(beta), n_sweeps, seed, sweep_offset, _addr(trace),
                                _stream(stream)), "ising_sweep")
+
+
+def ising_sweep_check(stream=None):
+    _check(_load().ising_sweep_check(_stream(stream)), "ising_sweep_check")
+
+
+def ising_sweep_wait_selftest(lat, stream=None):
+    _check(_load().ising_sweep_wait_selftest(ctypes.byref(_struct(lat)), _stream(stream)), "ising_sweep_wait_selftest")
 
 
 def ising_sweep_host(dev_lat, black_host, white_host, beta: float, n_sweeps: int, seed: int, sweep_offset: int = 0,

@@ -109,6 +109,22 @@ int build_accept(double beta, Accept *acc, uint64_t T[5])
     return ISING_OK;
 }
 
+ResidentSweep resident_params(const ising_lattice_t *lat, const Accept &acc, const RoundKeys &rk, uint64_t t0,
+                              int64_t *trace)
+{
+    ResidentSweep p{};
+    p.plane[0] = lat->black;
+    p.plane[1] = lat->white;
+    p.stride = lat->row_stride_bytes;
+    p.L = (int32_t)lat->L;
+    p.bytes = lat->layout == ISING_INT8;
+    p.t0 = t0;
+    p.acc = acc;
+    p.rk = rk;
+    p.trace = (long long *)trace;
+    return p;
+}
+
 int half_sweep_impl(const ising_lattice_t *lat, const Accept &acc, const RoundKeys &rk, int colour, uint64_t t,
                     int64_t *obs, cudaStream_t s)
 {
@@ -480,18 +496,7 @@ ISING_API int ising_sweep(const ising_lattice_t *lat, double beta, int64_t n_swe
     }
     const RoundKeys rk = make_round_keys(seed);
     if (resident_fits(lat->L, n_sweeps)) {
-        if (resident_timed_out()) return fail(ISING_ETIMEOUT, "a wait of an earlier small-lattice sweep gave up");
-        ResidentSweep p{};
-        p.plane[0] = lat->black;
-        p.plane[1] = lat->white;
-        p.stride = lat->row_stride_bytes;
-        p.L = (int32_t)lat->L;
-        p.bytes = lat->layout == ISING_INT8;
-        p.t0 = sweep_offset;
-        p.acc = acc;
-        p.rk = rk;
-        p.trace = (long long *)trace_dev;
-        cudaError_t e = resident_sweep(p, n_sweeps, s);
+        cudaError_t e = resident_sweep(resident_params(lat, acc, rk, sweep_offset, trace_dev), n_sweeps, s);
         return e == cudaSuccess ? ISING_OK : cuda_fail(e, "resident sweep launch");
     }
     if (traced) {
@@ -506,6 +511,32 @@ ISING_API int ising_sweep(const ising_lattice_t *lat, double beta, int64_t n_swe
         if (rc) return rc;
     }
     return ISING_OK;
+}
+
+ISING_API int ising_sweep_check(ising_stream_t stream)
+{
+    bool gave_up = false;
+    cudaError_t e = resident_check(&gave_up, (cudaStream_t)stream);
+    if (e != cudaSuccess) return cuda_fail(e, "sweep check");
+    return gave_up ? fail(ISING_ETIMEOUT, "a wait of a small-lattice sweep gave up") : ISING_OK;
+}
+
+ISING_API int ising_sweep_wait_selftest(const ising_lattice_t *lat, ising_stream_t stream)
+{
+    int rc = check_lattice(lat);
+    if (rc) return rc;
+    constexpr int64_t kSweeps = 8;
+    if (lat->L < 48 || !resident_fits(lat->L, kSweeps))
+        return fail(ISING_EINVAL, "L = %lld: not a lattice that several CTAs of one cluster sweep", (long long)lat->L);
+    Accept acc;
+    uint64_t T[5];
+    rc = build_accept(0.5, &acc, T);
+    if (rc) return rc;
+    ResidentSweep p = resident_params(lat, acc, make_round_keys(0), 0, nullptr);
+    p.wait_cycles = 2000000;  // ~1 ms
+    p.withhold = 1;
+    cudaError_t e = resident_sweep(p, kSweeps, (cudaStream_t)stream);
+    return e == cudaSuccess ? ISING_OK : cuda_fail(e, "resident sweep launch");
 }
 
 ISING_API int ising_slab_bytes(int64_t L, int64_t rows, int32_t layout, size_t *row_bytes, size_t *plane_bytes)

@@ -153,6 +153,8 @@ struct ResidentSweep {
     Accept acc;
     RoundKeys rk;
     long long *trace;   // {sum s, sum bonds} per sweep or nullptr
+    long long wait_cycles;  // limit of each wait for halo rows
+    int32_t withhold;   // self-test: the first CTA sends no halo rows, so that the others' waits run out
 };
 
 constexpr uint32_t kNibbleLsb = 0x11111111u;

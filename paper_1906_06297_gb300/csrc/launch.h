@@ -53,8 +53,9 @@ cudaError_t int8_observables(const int8_t *black, const int8_t *white, int64_t L
 // cluster (resident_fits: the sides it is for); writes (not adds to) the trace.
 bool resident_fits(int64_t L, int64_t n_sweeps);
 cudaError_t resident_sweep(ResidentSweep p, int64_t n_sweeps, cudaStream_t s);
-// Whether a wait of an earlier such launch has given up since the last question.
-bool resident_timed_out();
+// Synchronises s; whether a wait of such a launch on this device has given up since
+// the last question.
+cudaError_t resident_check(bool *gave_up, cudaStream_t s);
 
 // Throughput probes (probe.cu): the generator alone, shaped like the sweep
 // (n_blocks <= 2^34), and the 32 x 32 -> 64-bit multiply alone (*multiplies

@@ -39,6 +39,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <mutex>
 #include <type_traits>
 
 #include "common.cuh"
@@ -56,13 +57,17 @@ constexpr int kTraceRows = 128;
 // 0.51 us per sweep with at least 64, 0.64 with 128 and 0.71 with 256; 32^2, with at
 // least 32, 0.51 in two CTAs and 0.38 in one.
 constexpr int64_t kItems = 64;
-// Sweeps per launch (some 10 ms): another stream's work is not kept waiting for
-// the whole of a long call.
+// Sweeps per launch (7 ms at 32^2, 38 at 512^2): another stream's work is not kept
+// waiting for the whole of a long call.
 constexpr int64_t kMaxSweeps = 16384;
 constexpr long long kWaitCycles = 4000000000LL;  // ~2 s
+// What a cluster in which a wait gave up lingers at its end: remote stores issued
+// before its last barrier have long landed then.
+constexpr long long kLingerCycles = 200000LL;  // ~0.1 ms
 
-// Set by a wait that gave up, reported by the next call.
-__device__ __managed__ int g_resident_error;
+// Set by a wait that gave up; resident_check reads and clears it.
+__device__ int g_resident_error;
+__device__ int g_resident_seen;  // what resident_check found
 
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
@@ -105,8 +110,9 @@ __device__ __forceinline__ void bar_expect(uint32_t bar, uint32_t bytes)
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
 }
 
-// Waits until the barrier's phase of the given parity is over, at most ~2 s.
-__device__ __forceinline__ void bar_wait(uint32_t bar, uint32_t parity, bool &dead)
+// Waits until the barrier's phase of the given parity is over, at most `limit`
+// cycles; sets `dead` if that was too short.
+__device__ __forceinline__ void bar_wait(uint32_t bar, uint32_t parity, long long limit, bool &dead)
 {
     if (dead) return;
     const long long start = clock64();
@@ -121,8 +127,8 @@ __device__ __forceinline__ void bar_wait(uint32_t bar, uint32_t parity, bool &de
                      : "r"(bar), "r"(parity)
                      : "memory");
         if (done) return;
-        if (clock64() - start > kWaitCycles) {
-            g_resident_error = 1;
+        if (clock64() - start > limit) {
+            atomicExch(&g_resident_error, 1);
             dead = true;
             return;
         }
@@ -244,6 +250,13 @@ struct Decider {
     uint32_t dst_bar[K];
     bool edge;
 
+    // Sends no more halo words.
+    __device__ __forceinline__ void mute()
+    {
+#pragma unroll
+        for (int k = 0; k < K; ++k) dst[k] = 0u;
+    }
+
     __device__ __forceinline__ Decider(const Resident &c, int tid, bool alone, uint32_t to_above, uint32_t to_below,
                                        uint32_t bar_above, uint32_t bar_below)
     {
@@ -349,7 +362,9 @@ __global__ void __launch_bounds__(kMaxThreads, 1) resident_kernel(const __grid_c
     const bool always = p.acc.always != 0, trace = p.trace != nullptr, draws = tid < (int)blockDim.x - c.nc;
     const int me = draws ? tid : tid - ((int)blockDim.x - c.nc);
     const bool two = (int)blockDim.x == 2 * c.nc;  // a drawing thread serves both colours
-    bool dead = false;  // a wait ran out: no further ones, so that the launch ends
+    // a wait ran out: no further ones, so that the launch ends, and nothing more is
+    // sent or expected, so that no barrier counts what it was not told of
+    bool dead = false;
     int traced = 0;     // sweeps summed in tr
 
     // Behind the sweeps of a trace's rows, by all threads: every CTA adds up its
@@ -416,6 +431,7 @@ __global__ void __launch_bounds__(kMaxThreads, 1) resident_kernel(const __grid_c
         Decider<K, RAGGED> d(c, me, cs == 1, peer_addr(plane + 4u * (uint32_t)((rows_above + 1) * hpr), (uint32_t)above),
                              peer_addr(plane, (uint32_t)below), peer_addr(bar, (uint32_t)above),
                              peer_addr(bar, (uint32_t)below));
+        if (p.withhold && rank == 0) d.mute();
         __syncwarp();
         cluster_arrive();
         cluster_wait();
@@ -430,8 +446,9 @@ __global__ void __launch_bounds__(kMaxThreads, 1) resident_kernel(const __grid_c
                 if (d.edge && (s > 0 || COLOUR == 1)) {
                     // the other colour's halo rows: its update s, or s - 1 before black's
                     const uint32_t b = bar + 8 * (1 - COLOUR);
-                    bar_wait(b, (uint32_t)(COLOUR == 1 ? s : s - 1) & 1u, dead);
-                    if (me == 0) bar_expect(b, halo_bytes);
+                    bar_wait(b, (uint32_t)(COLOUR == 1 ? s : s - 1) & 1u, p.wait_cycles, dead);
+                    if (dead) d.mute();
+                    else if (me == 0) bar_expect(b, halo_bytes);
                 }
 #pragma unroll
                 for (int k = 0; k < K; ++k)
@@ -450,18 +467,24 @@ __global__ void __launch_bounds__(kMaxThreads, 1) resident_kernel(const __grid_c
             sweep_end(s);
         }
         // no CTA leaves while another's halo words are on their way to it
-        if (d.edge) bar_wait(bar + 8, (uint32_t)(p.n_sweeps - 1) & 1u, dead);
+        if (d.edge) bar_wait(bar + 8, (uint32_t)(p.n_sweeps - 1) & 1u, p.wait_cycles, dead);
         __syncwarp();
     }
     cluster_arrive();
     cluster_wait();
+    // set by any CTA of this cluster before the barrier (or by an earlier launch)
+    const int gave_up = *(volatile int *)&g_resident_error;
     for (int i = tid; i < c.items; i += blockDim.x) {
         const int row = i / hpr, uu = i - row * hpr;
 #pragma unroll
         for (int b = 0; b < 2; ++b)
             store_half(p, b, r0 + row, uu, uu == hpr - 1 ? c.last_nv : 8, res_smem[c.plane + b * c.plane_words + hpr + i]);
     }
+    if (gave_up)
+        for (const long long start = clock64(); clock64() - start < kLingerCycles;) __nanosleep(1000);
 }
+
+__global__ void resident_flag_kernel() { g_resident_seen = atomicExch(&g_resident_error, 0); }
 
 template <int K, bool RAGGED>
 cudaError_t launch(const ResidentSweep &p, int cs, int threads, size_t smem, cudaStream_t s)
@@ -502,11 +525,17 @@ cudaError_t launch_k(const ResidentSweep &p, int k, int cs, int threads, size_t 
 // call of 1 / 3 / 10 sweeps: 14.7 / 22.6 / 45.5 here, 12.5 / 21.3 / 50.5 launched).
 bool resident_fits(int64_t L, int64_t n_sweeps) { return L <= (L % 16 && n_sweeps < 6 ? 400 : 512); }
 
-bool resident_timed_out()
+cudaError_t resident_check(bool *gave_up, cudaStream_t s)
 {
-    if (g_resident_error == 0) return false;  // no write: one that a kernel makes meanwhile stays
-    g_resident_error = 0;
-    return true;
+    static std::mutex mu;  // g_resident_seen serves one caller at a time
+    std::lock_guard<std::mutex> lock(mu);
+    int seen = 0;
+    resident_flag_kernel<<<1, 1, 0, s>>>();
+    cudaError_t e = cudaGetLastError();
+    if (e == cudaSuccess) e = cudaMemcpyFromSymbolAsync(&seen, g_resident_seen, sizeof(int), 0, cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    *gave_up = seen != 0;
+    return e;
 }
 
 cudaError_t resident_sweep(ResidentSweep p, int64_t n_sweeps, cudaStream_t s)
@@ -514,6 +543,7 @@ cudaError_t resident_sweep(ResidentSweep p, int64_t n_sweeps, cudaStream_t s)
     const int half = p.L / 2;
     p.hpr = (half + 7) / 8;
     p.wide = ((uintptr_t)p.plane[0] | (uintptr_t)p.plane[1] | (uint64_t)p.stride) % 8 == 0;
+    if (p.wait_cycles == 0) p.wait_cycles = kWaitCycles;
     int cs = 1;
     while (cs < kMaxCluster && 2 * cs <= p.L && (int64_t)p.L * p.hpr >= kItems * 2 * cs) cs *= 2;
     const int rows = (p.L + cs - 1) / cs, items = rows * p.hpr;
