@@ -39,6 +39,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <atomic>
 #include <mutex>
 #include <type_traits>
 
@@ -486,34 +487,87 @@ __global__ void __launch_bounds__(kMaxThreads, 1) resident_kernel(const __grid_c
 
 __global__ void resident_flag_kernel() { g_resident_seen = atomicExch(&g_resident_error, 0); }
 
-template <int K, bool RAGGED>
-cudaError_t launch(const ResidentSweep &p, int cs, int threads, size_t smem, cudaStream_t s)
+// How a side is cut: half words per row, CTAs, half words per deciding thread and
+// colour, deciding threads and threads of a CTA, its shared memory.
+struct Plan {
+    int hpr, cs, k, deciders, threads;
+    size_t smem;
+};
+
+Plan plan_of(int L)
 {
-    auto kernel = resident_kernel<K, RAGGED>;
-    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    if (e == cudaSuccess && smem > 48 * 1024)
-        e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)cs);
-    cfg.blockDim = dim3((unsigned)threads);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = (unsigned)cs;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kernel, p);
+    Plan q;
+    const int half = L / 2;
+    q.hpr = (half + 7) / 8;
+    q.cs = 1;
+    while (q.cs < kMaxCluster && 2 * q.cs <= L && (int64_t)L * q.hpr >= kItems * 2 * q.cs) q.cs *= 2;
+    const int rows = (L + q.cs - 1) / q.cs, items = rows * q.hpr;
+    // at most 1024 half words per CTA on this route: one or two per thread
+    q.k = (items + kMaxThreads / 2 - 1) / (kMaxThreads / 2);
+    q.deciders = ((items + q.k - 1) / q.k + 31) / 32 * 32;
+    // as many threads draw, or twice as many where drawing takes longest and the
+    // block has room: at two half words per thread (384^2 1.64 -> 1.43 us per sweep)
+    // and with ragged rows, three Philox blocks per half word (100^2 0.89 -> 0.69; but
+    // 256^2, one word each, 0.80 -> 0.84)
+    q.threads = q.deciders * ((q.k > 1 || half % 8) && 3 * q.deciders <= kMaxThreads ? 3 : 2);
+    q.smem = ((2 + q.deciders / 32) * kTraceRows + 2 * (size_t)(rows + 2) * q.hpr + 4 * (size_t)items) * sizeof(uint32_t);
+    return q;
 }
 
-template <bool RAGGED>
-cudaError_t launch_k(const ResidentSweep &p, int k, int cs, int threads, size_t smem, cudaStream_t s)
+// Calls go(kernel) with the kernel of a plan.
+template <typename Go>
+auto with_kernel(const Plan &q, int L, Go go)
 {
-    // at most 1024 half words per CTA on this route: one or two per thread
-    return k == 1 ? launch<1, RAGGED>(p, cs, threads, smem, s) : launch<2, RAGGED>(p, cs, threads, smem, s);
+    if (L / 2 % 8) return q.k == 1 ? go(resident_kernel<1, true>) : go(resident_kernel<2, true>);
+    return q.k == 1 ? go(resident_kernel<1, false>) : go(resident_kernel<2, false>);
+}
+
+struct Config {
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[1];
+
+    Config(int cs, int threads, size_t smem, cudaStream_t s)
+    {
+        cfg.gridDim = dim3((unsigned)cs);
+        cfg.blockDim = dim3((unsigned)threads);
+        cfg.dynamicSmemBytes = smem;
+        cfg.stream = s;
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = (unsigned)cs;
+        attr[0].val.clusterDim.y = 1;
+        attr[0].val.clusterDim.z = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+    }
+};
+
+// Whether the device has the SMs of one graphics processing cluster that a plan's
+// CTAs need; a partition of it, or a limit on a process's SMs, may not.  A device on
+// which the largest cluster fits (asked once per kernel) has room for every other.
+constexpr size_t kMaxSmem = 40 * 1024;  // no plan takes more (512^2 36 KB)
+constexpr int kMaxDevices = 64;
+std::atomic<uint8_t> g_room[kMaxDevices][4];  // 0: not asked, 1: for any plan, 2: not for all
+
+bool cluster_fits(const Plan &q, int L)
+{
+    if (q.cs == 1) return true;
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return false;
+    std::atomic<uint8_t> &room = g_room[dev][(q.k - 1) * 2 + (L / 2 % 8 ? 1 : 0)];
+    if (room == 1) return true;
+    return with_kernel(q, L, [&](auto kernel) {
+        auto fits = [&](int cs, int threads, size_t smem) {
+            int n = 0;
+            Config c(cs, threads, smem, nullptr);
+            if (cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
+                cudaOccupancyMaxActiveClusters(&n, kernel, &c.cfg) == cudaSuccess)
+                return n > 0;
+            cudaGetLastError();
+            return false;
+        };
+        if (room == 0) room = fits(kMaxCluster, kMaxThreads, kMaxSmem) ? 1 : 2;
+        return room == 1 || fits(q.cs, q.threads, q.smem);
+    });
 }
 
 }  // namespace
@@ -523,7 +577,11 @@ cudaError_t launch_k(const ResidentSweep &p, int k, int cs, int threads, size_t 
 // ragged rows 430^2 2.7 / 3.6, 510^2 3.4 / 3.6, 530^2 4.9 / 3.6.  A single call of
 // few sweeps of ragged rows is no faster here from about 400^2 on (510^2, us per
 // call of 1 / 3 / 10 sweeps: 14.7 / 22.6 / 45.5 here, 12.5 / 21.3 / 50.5 launched).
-bool resident_fits(int64_t L, int64_t n_sweeps) { return L <= (L % 16 && n_sweeps < 6 ? 400 : 512); }
+// Where the cluster has no room the launches serve any side.
+bool resident_fits(int64_t L, int64_t n_sweeps)
+{
+    return L <= (L % 16 && n_sweeps < 6 ? 400 : 512) && cluster_fits(plan_of((int)L), (int)L);
+}
 
 cudaError_t resident_check(bool *gave_up, cudaStream_t s)
 {
@@ -540,25 +598,15 @@ cudaError_t resident_check(bool *gave_up, cudaStream_t s)
 
 cudaError_t resident_sweep(ResidentSweep p, int64_t n_sweeps, cudaStream_t s)
 {
-    const int half = p.L / 2;
-    p.hpr = (half + 7) / 8;
+    const Plan q = plan_of(p.L);
+    p.hpr = q.hpr;
+    p.deciders = q.deciders;
     p.wide = ((uintptr_t)p.plane[0] | (uintptr_t)p.plane[1] | (uint64_t)p.stride) % 8 == 0;
     if (p.wait_cycles == 0) p.wait_cycles = kWaitCycles;
-    int cs = 1;
-    while (cs < kMaxCluster && 2 * cs <= p.L && (int64_t)p.L * p.hpr >= kItems * 2 * cs) cs *= 2;
-    const int rows = (p.L + cs - 1) / cs, items = rows * p.hpr;
-    const int k = (items + kMaxThreads / 2 - 1) / (kMaxThreads / 2);
-    p.deciders = ((items + k - 1) / k + 31) / 32 * 32;
-    // as many threads draw, or twice as many where drawing takes longest and the
-    // block has room: at two half words per thread (384^2 1.64 -> 1.43 us per sweep)
-    // and with ragged rows, three Philox blocks per half word (100^2 0.89 -> 0.69; but
-    // 256^2, one word each, 0.80 -> 0.84)
-    const int threads = p.deciders * ((k > 1 || half % 8) && 3 * p.deciders <= kMaxThreads ? 3 : 2);
-    const size_t smem =
-        ((2 + p.deciders / 32) * kTraceRows + 2 * (size_t)(rows + 2) * p.hpr + 4 * (size_t)items) * sizeof(uint32_t);
+    Config c(q.cs, q.threads, q.smem, s);
     while (n_sweeps > 0) {
         p.n_sweeps = (int32_t)std::min<int64_t>(n_sweeps, kMaxSweeps);
-        cudaError_t e = half % 8 ? launch_k<true>(p, k, cs, threads, smem, s) : launch_k<false>(p, k, cs, threads, smem, s);
+        cudaError_t e = with_kernel(q, p.L, [&](auto kernel) { return cudaLaunchKernelEx(&c.cfg, kernel, p); });
         if (e != cudaSuccess) return e;
         n_sweeps -= p.n_sweeps;
         p.t0 += (uint64_t)p.n_sweeps;
