@@ -495,7 +495,7 @@ ISING_API int ising_sweep(const ising_lattice_t *lat, double beta, int64_t n_swe
         if (rc) return rc;
     }
     const RoundKeys rk = make_round_keys(seed);
-    if (resident_fits(lat->L, n_sweeps)) {
+    if (resident_fits(lat->L, n_sweeps, lat->layout == ISING_INT8)) {
         cudaError_t e = resident_sweep(resident_params(lat, acc, rk, sweep_offset, trace_dev), n_sweeps, s);
         return e == cudaSuccess ? ISING_OK : cuda_fail(e, "resident sweep launch");
     }
@@ -526,7 +526,7 @@ ISING_API int ising_sweep_wait_selftest(const ising_lattice_t *lat, ising_stream
     int rc = check_lattice(lat);
     if (rc) return rc;
     constexpr int64_t kSweeps = 8;
-    if (lat->L < 48 || !resident_fits(lat->L, kSweeps))
+    if (lat->L < 48 || !resident_fits(lat->L, kSweeps, lat->layout == ISING_INT8))
         return fail(ISING_EINVAL, "L = %lld: not a lattice that several CTAs of one cluster sweep", (long long)lat->L);
     Accept acc;
     uint64_t T[5];

@@ -52,7 +52,7 @@ cudaError_t int8_observables(const int8_t *black, const int8_t *white, int64_t L
 // Sweeps of a small lattice, either layout, all of a call's in launches of one
 // cluster; writes (not adds to) the trace.  resident_fits: the calls it is for, on a
 // device that has room for the cluster; asked before a sweep, since it prepares the kernel.
-bool resident_fits(int64_t L, int64_t n_sweeps);
+bool resident_fits(int64_t L, int64_t n_sweeps, bool bytes);
 cudaError_t resident_sweep(ResidentSweep p, int64_t n_sweeps, cudaStream_t s);
 // Synchronises s; whether a wait of such a launch on this device has given up since
 // the last question.

@@ -577,10 +577,16 @@ bool cluster_fits(const Plan &q, int L)
 // ragged rows 430^2 2.7 / 3.6, 510^2 3.4 / 3.6, 530^2 4.9 / 3.6.  A single call of
 // few sweeps of ragged rows is no faster here from about 400^2 on (510^2, us per
 // call of 1 / 3 / 10 sweeps: 14.7 / 22.6 / 45.5 here, 12.5 / 21.3 / 50.5 launched).
-// Where the cluster has no room the launches serve any side.
-bool resident_fits(int64_t L, int64_t n_sweeps)
+// One sweep of a one-byte lattice, us with nothing behind it / among others, here and
+// launched: 256^2 20.4 / 8.7 and 18.9 / 10.5, 512^2 23.2 / 8.8 and 19.2 / 10.5, ragged
+// 254^2 21.6 / 8.9 and 19.1 / 10.6, 398^2 24.5 / 10.3 and 19.3 / 10.6; a general kernel in
+// two launches 22.5 / 10.9 at any of these sides, which is where the line lies.  (One
+// MSC4 sweep 22.4 / 8.7 here at 512^2.)  Where the cluster has no room the launches serve any side.
+bool resident_fits(int64_t L, int64_t n_sweeps, bool bytes)
 {
-    return L <= (L % 16 && n_sweeps < 6 ? 400 : 512) && cluster_fits(plan_of((int)L), (int)L);
+    const bool ragged = L % 16 != 0, single = bytes && n_sweeps == 1;
+    const int64_t most = single ? (ragged ? 256 : 400) : ragged && n_sweeps < 6 ? 400 : 512;
+    return L <= most && cluster_fits(plan_of((int)L), (int)L);
 }
 
 cudaError_t resident_check(bool *gave_up, cudaStream_t s)

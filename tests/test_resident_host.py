@@ -30,12 +30,12 @@ static cudaError_t fake_clusters(int *n, const cudaLaunchConfig_t *cfg)
 #define cudaGetLastError() cudaSuccess
 #include "resident.cu"
 
-extern "C" __attribute__((visibility("default"))) int fits(int device, int limit, long long L, long long n, int *queries)
+extern "C" __attribute__((visibility("default"))) int fits(int device, int limit, long long L, long long n, int bytes, int *queries)
 {
     g_device = device;
     g_limit = limit;
     g_queries = 0;
-    const bool f = ising::resident_fits(L, n);
+    const bool f = ising::resident_fits(L, n, bytes != 0);
     *queries = g_queries;
     return f;
 }
@@ -52,11 +52,12 @@ def fits(tmp_path_factory):
     subprocess.run([nvcc, *_build.NVCC_FLAGS, f"-I{_build.CSRC}", "-shared", str(d / "fits.cu"), "-o", str(d / "fits.so")],
                    check=True)
     fn = ctypes.CDLL(str(d / "fits.so")).fits
-    fn.argtypes = [ctypes.c_int, ctypes.c_int, ctypes.c_longlong, ctypes.c_longlong, ctypes.c_void_p]
+    fn.argtypes = [ctypes.c_int, ctypes.c_int, ctypes.c_longlong, ctypes.c_longlong, ctypes.c_int,
+                   ctypes.c_void_p]
 
-    def ask(device, limit, L, n=100):
+    def ask(device, limit, L, n=100, layout="int8"):
         q = ctypes.c_int(0)
-        return bool(fn(device, limit, L, n, ctypes.byref(q))), q.value
+        return bool(fn(device, limit, L, n, layout == "int8", ctypes.byref(q))), q.value
 
     return ask
 
@@ -83,3 +84,13 @@ def test_a_device_without_room_for_the_cluster_takes_the_launches(fits, limit, f
         assert fits(device, limit, L)[0]
     for L in not_fit:
         assert not fits(device, limit, L)[0]
+
+
+def test_single_sweeps_of_large_one_byte_lattices_take_the_launches(fits):
+    """A cluster that loads, sweeps once and stores takes longer there than two
+    launches of whatever kernel."""
+    for L, n, layout, want in ((256, 1, "int8", True), (254, 1, "int8", True), (258, 1, "int8", False), (350, 1, "int8", False),
+                               (398, 1, "int8", False), (400, 1, "int8", True), (416, 1, "int8", False),
+                               (512, 1, "int8", False), (512, 1, "msc4", True), (512, 2, "int8", True),
+                               (398, 2, "int8", True), (402, 2, "int8", False), (402, 6, "int8", True)):
+        assert fits(30, 16, L, n, layout)[0] == want
