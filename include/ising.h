@@ -452,8 +452,9 @@ ISING_API int ising_net_wait_selftest(int64_t L, int64_t C, const void *black_de
 /* grad_dev = d(sum dlogits * logits)/d(params) for the last training forward
  * on the same chains and parameters (straight-through the bfloat16 rounding).
  * The data and weight gradients of the 32 -> 32 layers run on the tensor
- * cores (the weight gradients see the output gradient as two bfloat16 parts, its rounding and the rounding of the
- * remainder, which carry it to about 2^-17); a bounded wait that gives up there
+ * cores (the weight gradients see the output gradient as two bfloat16 parts, its
+ * rounding and the rounding of the remainder, which carry it to about 2^-17, for L
+ * a multiple of 128, else as three, which are all of it); a bounded wait that gives up there
  * is reported by the next ising_net_check.  Every weight gradient is a sum of
  * per-CTA partials in a fixed order: the result is deterministic. */
 ISING_API int ising_net_backward(int64_t L, int64_t C, const void *black_dev, const void *white_dev,

@@ -100,6 +100,14 @@ __device__ __forceinline__ void split_bf16(const float (&v)[8], uint32_t (&hi)[4
     }
 }
 
+// What the two parts leave (8 bits at most, so hi + lo + rest equals v).
+__device__ __forceinline__ void rest_bf16(const float (&v)[8], const uint32_t (&hi)[4], const uint32_t (&lo)[4], uint32_t (&rest)[4])
+{
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+        rest[j] = pack_bf16x2(v[2 * j] - bf16_lo(hi[j]) - bf16_lo(lo[j]), v[2 * j + 1] - bf16_hi(hi[j]) - bf16_hi(lo[j]));
+}
+
 __device__ __forceinline__ float rcp_approx(float x)
 {
     float r;
@@ -435,7 +443,7 @@ __device__ int g_tc_error;  // set to 1 when a tensor-core wait gives up
 // SBO = 128).  (Sides that are no multiple of 128 took a kernel that gathered all
 // 9 taps of every tile, im2col, from global memory and one that projected on the
 // CUDA cores: a forward of 256 chains of 96^2 892 us, here 343; a training step of
-// 40 chains of 96^2 1352, here 445.)
+// 40 chains of 96^2 1352, here 364.)
 // Warp roles, linked by mbarriers (every wait bounded):
 //   warp 0: loader -- lane 0 fetches each row with four tensor copies (TMA),
 //           one per channel group: a box of 8 channels x tw + 2 pixels of the
@@ -493,7 +501,7 @@ __device__ int g_tc_error;  // set to 1 when a tensor-core wait gives up
 // W[o][i][8 - k], since dz_prev(p)[i] = gelu'(z_prev(p)[i]) sum_k sum_o
 // W[o][i][k] dz(p - off_k)[o] and -off_k = off_{8-k}; the epilogue multiplies
 // by gelu'(z_prev) and writes dz_prev in FP32 (layer 1's, for its weight gradient)
-// or as two bfloat16 parts with halo columns, for what takes it from there.
+// or as its bfloat16 parts with halo columns, for what takes it from there.
 // Dependencies: the MMAs of staged row i wait on the epilogue of output rows
 // up to i + 1 - kAcc only, the epilogue of row t on the MMAs of staged rows up
 // to t + 1 only, so no wait can close a cycle.
@@ -651,6 +659,7 @@ struct RingConv {
     const __nv_bfloat16 *a_in;
     __nv_bfloat16 *a_out;  // nullable when PROJ
     __nv_bfloat16 *a_lo;   // BWD, nullable: bf16(dz_prev - bf16(dz_prev)) beside a_out (for the weight gradient)
+    __nv_bfloat16 *a_rest; // BWD, nullable, sides that are no multiple of 128: what these two leave
     float *z_out;          // nullable
     float *P;              // PROJ: 9 planes of C L^2
     const float *zg;       // BWD: z of the layer below (FP32, NHWC) for gelu', or, where that is layer 1,
@@ -1057,13 +1066,14 @@ __global__ void __launch_bounds__(ring_threads<PROJ, FUSED>(), 2) conv32_ring_ke
                     for (int i = 0; i < 16; ++i) v[i] *= gz[i];
                     if (p.d_out) tile_store_f32(p.d_out + q0 * kCh + 16 * half, stg, lane, v);
                     if (p.a_out) {
-                        uint32_t hb[2][4], rb[2][4];
+                        uint32_t hb[2][4], rb[2][4], sb[2][4];
 #pragma unroll
                         for (int h8 = 0; h8 < 2; ++h8) {
                             float v8[8];
 #pragma unroll
                             for (int i = 0; i < 8; ++i) v8[i] = v[8 * h8 + i];
                             split_bf16(v8, hb[h8], rb[h8]);
+                            if constexpr (!FULL) rest_bf16(v8, hb[h8], rb[h8], sb[h8]);
                         }
                         tile_store_bf16(p.a_out, L, w.c, y, w.x0 + xw, 16 * half, st16, lane,
                                         make_uint4(hb[0][0], hb[0][1], hb[0][2], hb[0][3]),
@@ -1072,6 +1082,11 @@ __global__ void __launch_bounds__(ring_threads<PROJ, FUSED>(), 2) conv32_ring_ke
                             tile_store_bf16(p.a_lo, L, w.c, y, w.x0 + xw, 16 * half, st16, lane,
                                             make_uint4(rb[0][0], rb[0][1], rb[0][2], rb[0][3]),
                                             make_uint4(rb[1][0], rb[1][1], rb[1][2], rb[1][3]));
+                        if constexpr (!FULL)
+                            if (p.a_rest)
+                                tile_store_bf16(p.a_rest, L, w.c, y, w.x0 + xw, 16 * half, st16, lane,
+                                                make_uint4(sb[0][0], sb[0][1], sb[0][2], sb[0][3]),
+                                                make_uint4(sb[1][0], sb[1][1], sb[1][2], sb[1][3]));
                     }
                 } else {
                     if (p.z_out) {
@@ -1250,7 +1265,8 @@ __global__ void __launch_bounds__(kPoolThreads) pool_rows_kernel(int L, int64_t 
 // ---------------------------------------------------------------------------
 // dz3 = gelu'(z3) * sum_k W4[i][k] * d4(p - off_k),  d4(p) = dlogit(block of p) / 64,
 // as bfloat16 with halo columns, the operand of the next data gradient on the
-// tensor cores, and the rounding of its remainder, for the weight gradient.
+// tensor cores, and the rounding of its remainder, for the weight gradient (REST:
+// and what these two leave).
 // Four threads per pixel, 8 channels each (a warp reads 8 pixels' 1 KB of z3
 // contiguously); a channel pair's weight is one 64-bit operand of a packed multiply-
 // add, and a tap's weights of 8 channels come from shared memory in two 16-byte
@@ -1260,9 +1276,11 @@ __global__ void __launch_bounds__(kPoolThreads) pool_rows_kernel(int L, int64_t 
 // here 68; it moves 270 MB.
 constexpr int kL4Threads = 256;
 
+template <bool REST>
 __global__ void __launch_bounds__(kL4Threads, 4) l4_bwd_data_kernel(int L, int64_t C, const float *params,
                                                                     const float *dlogits, const float *z3,
-                                                                    __nv_bfloat16 *dz3b, __nv_bfloat16 *dz3r)
+                                                                    __nv_bfloat16 *dz3b, __nv_bfloat16 *dz3r,
+                                                                    __nv_bfloat16 *dz3s)
 {
     const int nb1 = L / kBlk, i8 = (threadIdx.x & 3) * 8;
     const uint32_t LL = (uint32_t)L * (uint32_t)L;
@@ -1312,6 +1330,11 @@ __global__ void __launch_bounds__(kL4Threads, 4) l4_bwd_data_kernel(int L, int64
             split_bf16(v, hb, rb);
             store_act(dz3b, L, c, y, x, i8, make_uint4(hb[0], hb[1], hb[2], hb[3]));
             store_act(dz3r, L, c, y, x, i8, make_uint4(rb[0], rb[1], rb[2], rb[3]));
+            if constexpr (REST) {
+                uint32_t sb[4];
+                rest_bf16(v, hb, rb, sb);
+                store_act(dz3s, L, c, y, x, i8, make_uint4(sb[0], sb[1], sb[2], sb[3]));
+            }
         }
     }
 }
@@ -1543,6 +1566,15 @@ __global__ void __launch_bounds__(32 * kReduceWarps) reduce_partials_kernel(cons
 // and the FP32 accumulation sees the unrounded gradient to that accuracy
 // (dW = D[.][64 b + o] + D[.][64 b + 32 + o]).  tw / 16 MMAs of M128 x N192 x
 // K16 per input row segment.
+// Sides that are no multiple of 128, whose sums the CUDA cores took in FP32 before,
+// keep that: the gradient comes in three parts, which are all of its bits, added
+// one after the other (smallest first) onto N = 96 columns n = 32 b + o, and, since the
+// MMA's accumulation truncates where FP32 additions round, each input row has its
+// own sum, in two sets of columns in turn, which warps 2..4 add up in registers.
+// Largest error of layer 3's weight gradients against 64 bits, of the largest one,
+// FP32 on the CUDA cores / two parts in two sums per CTA / here: 40 chains of 96^2
+// 7.6e-7 / 1.9e-6 / 3.4e-7, 1024 of 32^2 2.7e-6 / 8.8e-6 / 6.3e-7, 40 of 160^2 5.0e-6 /
+// 1.5e-5 / 1.1e-6; us per training step of the first 1348 / 330 / 364.
 // Both operands are MN-major and come straight from the NHWC buffers: a
 // tensor copy of tw whole pixels (32 channels, 64 bytes each) with the
 // 64-byte swizzle is the MN-major 64-byte-swizzled operand form: 8 K rows
@@ -1562,41 +1594,43 @@ __global__ void __launch_bounds__(32 * kReduceWarps) reduce_partials_kernel(cons
 // gradient rows r0 - 2 .. r0 + n + 1, those outside the run as zeros (tensor
 // copies of a row past the lattice's last, which the copy fills with zeros),
 // so that every (input row, gradient row) pair is counted by exactly one CTA.
-// The accumulators (192 TMEM columns per set) collect the CTA's whole range; at the
-// end they are written as the CTA's partial sums in the weight-gradient
-// layout (e = (o CIN + i) 9 + k, then the biases).
+// The accumulators (192 TMEM columns, or the registers) collect the CTA's whole
+// range; at the end they are written as the CTA's partial sums in the weight-
+// gradient layout (e = (o CIN + i) 9 + k, then the biases).
 // Warp roles (bounded mbarrier waits): warp 0 lane 0 issues the tensor
 // copies; warp 1 the MMAs (one elected lane); warps 2..5 add up every staged gradient row
 // for the bias sums (fixed order; the zero rows add nothing) and, after the
-// last MMA, read the accumulators.  A gradient slot is free once the MMAs of
-// its last input row have completed and the four bias warps have read it.
+// last MMA (or behind each input row's), read the accumulators.  A gradient slot is
+// free once the MMAs of its last input row have completed and the four bias warps
+// have read it.  Where those warps wait for an input row's MMAs they have read every
+// gradient row that these need, so no wait closes a cycle.
 constexpr int kWgActSlots = 3;                      // staged input rows
 constexpr int kWgDzSlots = 4;                       // staged gradient rows (3 in use, 1 ahead)
 constexpr int kWgDzMirror = 2;                      // slots 0, 1 repeated after the last
 constexpr int kWgBiasWarps = 4;
 constexpr uint32_t kWgBox = kTileM * kCh * 2;      // 128 pixels x 32 channels, bfloat16, 64-byte swizzled
 constexpr uint32_t kWgActBytes = 3 * kWgBox;        // dx = 0, 1, 2
-constexpr uint32_t kWgDzBytes = 2 * kWgBox;         // hi, lo
 constexpr uint32_t kWgDz0 = kWgActSlots * kWgActBytes;
-constexpr uint32_t kWgBias = kWgDz0 + (kWgDzSlots + kWgDzMirror) * kWgDzBytes;  // per bias warp 32 sums
-constexpr uint32_t kWgBar = kWgBias + kWgBiasWarps * kCh * 4;
-constexpr uint32_t kWgSmem = kWgBar + (2 * kWgActSlots + 2 * kWgDzSlots + 1) * 8 + 16;
 constexpr int kWgThreads = 64 + 32 * kWgBiasWarps;
-constexpr int kWgN = 6 * kCh;                       // three gradient rows, hi and lo
-// accumulator sets of 192 (in 256) columns: the MMA's accumulation truncates, an
-// error that grows with the terms of a sum (1.6e-5 of the largest weight gradient
-// over 15000 pixels per CTA), so the input rows go to two sets in turn where the
-// CUDA cores' rounding sums had served before (sides that are no multiple of 128)
 template <bool FULL>
-constexpr int kWgSets = FULL ? 1 : 2;
-static_assert(kWgDz0 >= kWgActBytes + kWgBox && kWgSmem <= 227 * 1024 && kWgActBytes % 1024 == 0 &&
-                  kWgDz0 % 1024 == 0,
+struct WgLayout {
+    static constexpr int parts = FULL ? 2 : 3;               // of a gradient: its rounding, the remainder's, the rest
+    static constexpr uint32_t dz = parts * kWgBox;           // bytes of a gradient slot
+    static constexpr uint32_t bias = kWgDz0 + (kWgDzSlots + kWgDzMirror) * dz;  // per bias warp 32 sums
+    static constexpr uint32_t bar = bias + kWgBiasWarps * kCh * 4;
+    static constexpr uint32_t bytes = bar + (2 * kWgActSlots + 2 * kWgDzSlots + 5) * 8 + 16;
+    static constexpr int n = FULL ? 6 * kCh : 3 * kCh;       // columns: three gradient rows, hi and lo or their sum
+};
+constexpr uint32_t kWgCols = 256;  // TMEM: one set of 192, or two of 96, 128 apart
+static_assert(kWgDz0 >= kWgActBytes + kWgBox && WgLayout<false>::bytes <= 227 * 1024 && kWgActBytes % 1024 == 0 &&
+                  kWgDz0 % 1024 == 0 && kWgBox % 1024 == 0,
               "the unused M rows of the last input slot read the gradient slots; one CTA per SM");
 
 struct WgradTc {
     CUtensorMap act;  // a: (32 channels, L + 2 pixels, L rows, C chains), boxes 32 x tw x 1 x 1, 64-byte swizzle
     CUtensorMap hi;   // bf16(dz), the same without the last halo column (a box past pixel L reads zeros)
     CUtensorMap lo;   // bf16(dz - bf16(dz)), likewise
+    CUtensorMap rest; // what these leave, likewise (sides that are no multiple of 128)
     float *partial;   // [gridDim.x][kN2 + kCh]
     int L, segs, tw;
     int64_t lines;    // C segs L
@@ -1620,18 +1654,18 @@ template <bool FULL>
 __global__ void __launch_bounds__(kWgThreads, 1) wgrad_tc_kernel(const __grid_constant__ WgradTc p)
 {
     extern __shared__ __align__(1024) uint8_t wg_smem[];
-    float *bias_part = reinterpret_cast<float *>(wg_smem + kWgBias);
-    uint64_t *afull = reinterpret_cast<uint64_t *>(wg_smem + kWgBar);
+    using Lay = WgLayout<FULL>;
+    float *bias_part = reinterpret_cast<float *>(wg_smem + Lay::bias);
+    uint64_t *afull = reinterpret_cast<uint64_t *>(wg_smem + Lay::bar);
     uint64_t *aempty = afull + kWgActSlots, *dfull = aempty + kWgActSlots, *dempty = dfull + kWgDzSlots;
-    uint64_t *drain = dempty + kWgDzSlots;
-    uint32_t *tslot = reinterpret_cast<uint32_t *>(drain + 1);
+    uint64_t *drain = dempty + kWgDzSlots, *rowf = drain + 1, *rowe = rowf + 2;  // an input row's sums: there, read
+    uint32_t *tslot = reinterpret_cast<uint32_t *>(rowe + 2);
     const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
     const int L = p.L;
     const uint32_t box = (uint32_t)(FULL ? kTileM : p.tw) * kCh * 2;  // bytes of a staged row of tw pixels
     const int64_t begin = blockIdx.x * p.lines / gridDim.x, end = (blockIdx.x + 1) * p.lines / gridDim.x;
 
-    constexpr uint32_t kCols = 256 * kWgSets<FULL>;
-    if (warp == 1) tc::tmem_alloc(tslot, kCols);
+    if (warp == 1) tc::tmem_alloc(tslot, kWgCols);
     if (tid == 0) {
         for (int s = 0; s < kWgActSlots; ++s) {
             tc::mbar_init(&afull[s], 1);
@@ -1642,6 +1676,10 @@ __global__ void __launch_bounds__(kWgThreads, 1) wgrad_tc_kernel(const __grid_co
             tc::mbar_init(&dempty[s], 1 + kWgBiasWarps);
         }
         tc::mbar_init(drain, 1);
+        for (int s = 0; s < 2; ++s) {
+            tc::mbar_init(&rowf[s], 1);
+            tc::mbar_init(&rowe[s], kWgBiasWarps);
+        }
         tc::fence_mbar_init();
     }
     tc::fence_before_sync();
@@ -1649,6 +1687,7 @@ __global__ void __launch_bounds__(kWgThreads, 1) wgrad_tc_kernel(const __grid_co
     tc::fence_after_sync();
     const uint32_t tmem = *tslot;
     bool ok = true;
+    float rows[FULL ? 1 : 96];  // column n of this lane's TMEM row, over the input rows so far
 
     if (warp == 0) {
         if (lane == 0) {
@@ -1672,11 +1711,12 @@ __global__ void __launch_bounds__(kWgThreads, 1) wgrad_tc_kernel(const __grid_co
                     return false;
                 const int y = (r >= w.r0 && r < w.r0 + w.nrows) ? r : L;
                 const int copies = s < (uint32_t)kWgDzMirror ? 2 : 1;
-                tc::mbar_arrive_expect_tx(&dfull[s], (uint32_t)copies * 2 * box);
+                tc::mbar_arrive_expect_tx(&dfull[s], (uint32_t)copies * Lay::parts * box);
                 for (int k = 0; k < copies; ++k) {
-                    uint8_t *dst = wg_smem + kWgDz0 + (s + k * kWgDzSlots) * kWgDzBytes;
+                    uint8_t *dst = wg_smem + kWgDz0 + (s + k * kWgDzSlots) * Lay::dz;
                     tc::tma_load_4d(dst, &p.hi, 0, w.x0 + 1, y, (int)w.c, &dfull[s]);
                     tc::tma_load_4d(dst + kWgBox, &p.lo, 0, w.x0 + 1, y, (int)w.c, &dfull[s]);
+                    if (!FULL) tc::tma_load_4d(dst + 2 * kWgBox, &p.rest, 0, w.x0 + 1, y, (int)w.c, &dfull[s]);
                 }
                 ++nd;
                 return true;
@@ -1699,13 +1739,14 @@ __global__ void __launch_bounds__(kWgThreads, 1) wgrad_tc_kernel(const __grid_co
         __syncwarp();
     } else if (warp == 1) {
         {
-            const uint32_t idesc = tc::idesc_bf16_f32_mn(kTileM, kWgN);
+            const uint32_t idesc = tc::idesc_bf16_f32_mn(kTileM, Lay::n);
             const uint64_t a_desc0 = tc::smem_desc_sw64(tc::smem_u32(wg_smem), kWgBox, 512);
-            const uint64_t b_desc0 = tc::smem_desc_sw64(tc::smem_u32(wg_smem + kWgDz0), kWgBox, 512);
+            // the columns' groups of 32: hi and lo of one row after the other, or one part of each row
+            const uint64_t b_desc0 = tc::smem_desc_sw64(tc::smem_u32(wg_smem + kWgDz0), FULL ? kWgBox : Lay::dz, 512);
             const uint32_t a_lo0 = (uint32_t)a_desc0, a_hi = (uint32_t)(a_desc0 >> 32);
             const uint32_t b_lo0 = (uint32_t)b_desc0, b_hi = (uint32_t)(b_desc0 >> 32);
             uint32_t ma = 0, md = 0, dready = 0;  // input rows consumed; first gradient row of the run; gradient rows landed
-            uint32_t seen = 0;  // input rows so far: row `seen` goes to set seen % sets
+            uint32_t seen = 0;  // input rows so far (!FULL: row `seen` goes to set seen % 2)
             for (int64_t lin = begin; lin < end && ok;) {
                 const RingUnit w = wg_run(p, lin, end);
                 lin += w.nrows;
@@ -1719,16 +1760,29 @@ __global__ void __launch_bounds__(kWgThreads, 1) wgrad_tc_kernel(const __grid_co
                     }
                     const uint32_t as = ma % kWgActSlots;
                     if (ok && !__all_sync(0xffffffffu, tc::mbar_wait(&afull[as], (ma / kWgActSlots) & 1u, kWaitCycles))) ok = false;
+                    const uint32_t set = seen & 1;
+                    if (!FULL && ok && seen >= 2 &&
+                        !__all_sync(0xffffffffu, tc::mbar_wait(&rowe[set], ((seen >> 1) + 1) & 1u, kWaitCycles)))
+                        ok = false;
                     if (!ok) break;
                     tc::fence_after_sync();
                     const uint32_t a_row = a_lo0 + ((as * kWgActBytes) >> 4);
-                    const uint32_t b_row = b_lo0 + ((((md + (uint32_t)a) % kWgDzSlots) * kWgDzBytes) >> 4);
+                    const uint32_t b_row = b_lo0 + ((((md + (uint32_t)a) % kWgDzSlots) * Lay::dz) >> 4);
+                    if constexpr (FULL) {
 #pragma unroll
-                    for (int ks = 0; ks < kTileM / 16; ++ks)  // 16 pixels = two 512-byte atoms
-                        if (FULL || 16 * ks < p.tw)
-                            tc::mma_bf16_warp(tmem + 256 * (seen % kWgSets<FULL>), a_row + (uint32_t)(ks * 64), a_hi,
-                                           b_row + (uint32_t)(ks * 64), b_hi, idesc,
-                                           (seen < kWgSets<FULL> && ks == 0) ? 0u : 1u);
+                        for (int ks = 0; ks < kTileM / 16; ++ks)  // 16 pixels = two 512-byte atoms
+                            tc::mma_bf16_warp(tmem, a_row + (uint32_t)(ks * 64), a_hi, b_row + (uint32_t)(ks * 64), b_hi, idesc,
+                                              (seen == 0 && ks == 0) ? 0u : 1u);
+                    } else {
+                        for (int h = 2; h >= 0; --h)
+#pragma unroll
+                            for (int ks = 0; ks < kTileM / 16; ++ks)
+                                if (16 * ks < p.tw)
+                                    tc::mma_bf16_warp(tmem + 128 * set, a_row + (uint32_t)(ks * 64), a_hi,
+                                                      b_row + (uint32_t)(h * (kWgBox >> 4) + ks * 64), b_hi, idesc,
+                                                      (h == 2 && ks == 0) ? 0u : 1u);
+                        tc::mma_commit_warp(&rowf[set]);
+                    }
                     ++seen;
                     tc::mma_commit_warp(&aempty[as]);
                     ++ma;
@@ -1754,35 +1808,65 @@ __global__ void __launch_bounds__(kWgThreads, 1) wgrad_tc_kernel(const __grid_co
         float acc[8];
 #pragma unroll
         for (int j = 0; j < 8; ++j) acc[j] = 0.0f;
-        int64_t staged = 0;  // gradient rows staged for this CTA: n + 4 per run
-        for (int64_t lin = begin; lin < end;) {
+        if constexpr (!FULL) {
+#pragma unroll
+            for (int n = 0; n < 96; ++n) rows[n] = 0.0f;
+        }
+        int64_t md = 0, seen = 0;  // gradient rows and input rows so far
+        for (int64_t lin = begin; lin < end && ok;) {
             const RingUnit w = wg_run(p, lin, end);
             lin += w.nrows;
-            staged += w.nrows + 4;
-        }
-        for (int64_t md = 0; md < staged; ++md) {
-            const uint32_t ds = (uint32_t)(md % kWgDzSlots);
-            if (!__all_sync(0xffffffffu, tc::mbar_wait(&dfull[ds], (uint32_t)(md / kWgDzSlots) & 1u, kWaitCycles))) {
-                ok = false;
-                break;
-            }
-            const uint8_t *dz = wg_smem + kWgDz0 + ds * kWgDzBytes;
+            for (int j = 0; j < w.nrows + 4; ++j, ++md) {
+                const uint32_t ds = (uint32_t)(md % kWgDzSlots);
+                if (!__all_sync(0xffffffffu, tc::mbar_wait(&dfull[ds], (uint32_t)(md / kWgDzSlots) & 1u, kWaitCycles))) {
+                    ok = false;
+                    break;
+                }
+                const uint8_t *dz = wg_smem + kWgDz0 + ds * Lay::dz;
 #pragma unroll
-            for (int it = 0; it < 4; ++it) {
-                if (!FULL && 32 * q >= p.tw) break;  // no pixels of this warp's are staged
-                const int px = 32 * q + 8 * it + p8;
-                const uint32_t at = px * 64 + ((g ^ ((px >> 1) & 3)) << 4);
-                const uint4 h = *reinterpret_cast<const uint4 *>(dz + at);
-                const uint4 l = *reinterpret_cast<const uint4 *>(dz + kWgBox + at);
-                const uint32_t hw[4] = {h.x, h.y, h.z, h.w}, lw[4] = {l.x, l.y, l.z, l.w};
+                for (int it = 0; it < 4; ++it) {
+                    if (!FULL && 32 * q >= p.tw) break;  // no pixels of this warp's are staged
+                    const int px = 32 * q + 8 * it + p8;
+                    const uint32_t at = px * 64 + ((g ^ ((px >> 1) & 3)) << 4);
+                    const uint4 h = *reinterpret_cast<const uint4 *>(dz + at);
+                    const uint4 l = *reinterpret_cast<const uint4 *>(dz + kWgBox + at);
+                    const uint4 r = FULL ? uint4{} : *reinterpret_cast<const uint4 *>(dz + 2 * kWgBox + at);
+                    const uint32_t hw[4] = {h.x, h.y, h.z, h.w}, lw[4] = {l.x, l.y, l.z, l.w}, rw[4] = {r.x, r.y, r.z, r.w};
 #pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    acc[2 * j] += bf16_lo(hw[j]) + bf16_lo(lw[j]);
-                    acc[2 * j + 1] += bf16_hi(hw[j]) + bf16_hi(lw[j]);
+                    for (int i = 0; i < 4; ++i) {
+                        // hi + lo and, with the rest, the gradient itself are exact
+                        const float d0 = bf16_lo(hw[i]) + bf16_lo(lw[i]), d1 = bf16_hi(hw[i]) + bf16_hi(lw[i]);
+                        acc[2 * i] += FULL ? d0 : d0 + bf16_lo(rw[i]);
+                        acc[2 * i + 1] += FULL ? d1 : d1 + bf16_hi(rw[i]);
+                    }
+                }
+                __syncwarp();
+                if (lane == 0) tc::mbar_arrive(&dempty[ds]);
+                if constexpr (!FULL) {
+                    if (j < 2) continue;
+                    // input row r0 - 1 + j - 2 has met its last gradient row
+                    const uint32_t set = (uint32_t)seen & 1;
+                    if (!__all_sync(0xffffffffu, tc::mbar_wait(&rowf[set], (uint32_t)(seen >> 1) & 1u, kWaitCycles))) {
+                        ok = false;
+                        break;
+                    }
+                    ++seen;
+                    tc::fence_after_sync();
+                    const int quad = warp & 3;
+                    if (quad < 3) {
+#pragma unroll
+                        for (int k = 0; k < 6; ++k) {
+                            float v[16];
+                            tc::tmem_ld16(tmem + 128 * set + 16 * k + ((uint32_t)(quad * 32) << 16), v);
+#pragma unroll
+                            for (int i = 0; i < 16; ++i) rows[16 * k + i] += v[i];
+                        }
+                    }
+                    tc::fence_before_sync();
+                    __syncwarp();
+                    if (lane == 0) tc::mbar_arrive(&rowe[set]);
                 }
             }
-            __syncwarp();
-            if (lane == 0) tc::mbar_arrive(&dempty[ds]);
         }
         // lanes of one channel group (lane ^ 4, ^ 8, ^ 16), then the four warps in order
 #pragma unroll
@@ -1801,26 +1885,24 @@ __global__ void __launch_bounds__(kWgThreads, 1) wgrad_tc_kernel(const __grid_co
         // holds tap row dy = 2 - b.
         const int quad = warp & 3;
         float *out = p.partial + (int64_t)blockIdx.x * (kN2 + kCh);
+        if constexpr (FULL) {
 #pragma unroll 1
-        for (int b = 0; b < 3; ++b) {
+            for (int b = 0; b < 3; ++b) {
 #pragma unroll 1
-            for (int oh = 0; oh < 2; ++oh) {
-                float vh[16], vl[16];
-                const uint32_t ta = tmem + (uint32_t)(64 * b + 16 * oh) + ((uint32_t)(quad * 32) << 16);
-                tc::tmem_ld16(ta, vh);
-                tc::tmem_ld16(ta + (uint32_t)kCh, vl);
-                if constexpr (!FULL) {  // a CTA walks three input rows at least: both sets were written
-                    float uh[16], ul[16];
-                    tc::tmem_ld16(ta + 256u, uh);
-                    tc::tmem_ld16(ta + 256u + (uint32_t)kCh, ul);
+                for (int oh = 0; oh < 2; ++oh) {
+                    float vh[16], vl[16];
+                    const uint32_t ta = tmem + (uint32_t)(64 * b + 16 * oh) + ((uint32_t)(quad * 32) << 16);
+                    tc::tmem_ld16(ta, vh);
+                    tc::tmem_ld16(ta + (uint32_t)kCh, vl);
+                    if (quad < 3)
 #pragma unroll
-                    for (int j = 0; j < 16; ++j) vh[j] += uh[j], vl[j] += ul[j];
+                        for (int j = 0; j < 16; ++j)
+                            out[((16 * oh + j) * kCh + lane) * 9 + 3 * (2 - b) + quad] = vh[j] + vl[j];
                 }
-                if (quad < 3)
-#pragma unroll
-                    for (int j = 0; j < 16; ++j)
-                        out[((16 * oh + j) * kCh + lane) * 9 + 3 * (2 - b) + quad] = vh[j] + vl[j];
             }
+        } else if (quad < 3) {
+#pragma unroll
+            for (int n = 0; n < 96; ++n) out[((n & 31) * kCh + lane) * 9 + 3 * (2 - (n >> 5)) + quad] = rows[n];
         }
         if (warp == 2)
             out[kN2 + lane] = ((bias_part[lane] + bias_part[kCh + lane]) + bias_part[2 * kCh + lane]) +
@@ -1831,7 +1913,7 @@ __global__ void __launch_bounds__(kWgThreads, 1) wgrad_tc_kernel(const __grid_co
     __syncthreads();
     if (warp == 1) {
         tc::fence_after_sync();
-        tc::tmem_dealloc(tmem, kCols);
+        tc::tmem_dealloc(tmem, kWgCols);
     }
 }
 
@@ -2111,7 +2193,7 @@ int check_chains(int64_t L, int64_t C)
 }
 
 // Work layout: training keeps layer 1's patterns, z2 z3 (FP32), a1 a2 a3
-// (bfloat16), dz1 (FP32) and dz2, dz3 (as two bfloat16 parts), then the weight-gradient partials; inference keeps a2
+// (bfloat16), dz1 (FP32) and dz2, dz3 (as bfloat16 parts, two or three), then the weight-gradient partials; inference keeps a2
 // alone (bfloat16).  Both end with the row partials of z4, 9 values per row and
 // 8-pixel block column.
 struct NetWork {
@@ -2119,6 +2201,7 @@ struct NetWork {
     uint16_t *pat;
     __nv_bfloat16 *a1, *a2, *a3, *ta, *gb1, *gb2;  // gb: bfloat16 gradients with halo columns (training)
     __nv_bfloat16 *gr1, *gr2;                      // the bfloat16 roundings of their remainders
+    __nv_bfloat16 *gs1, *gs2;                      // and the rest, where L is no multiple of 128 (in da's place)
     int64_t n_cta;
     size_t bytes;
 };
@@ -2142,7 +2225,12 @@ NetWork net_layout(int64_t L, int64_t C, int train, char *base)
         w.pat = (uint16_t *)take(pix / kCh * 2);
         w.a1 = (__nv_bfloat16 *)take(apx * 2); w.a2 = (__nv_bfloat16 *)take(apx * 2);
         w.a3 = (__nv_bfloat16 *)take(apx * 2);
-        w.da = (float *)take(pix * 4);
+        // dz1 is written when the rests of dz3 and dz2 have been read
+        const size_t rest = L % kTileM ? (apx * 2 + 255) & ~size_t(255) : 0;
+        char *da = (char *)take(std::max(pix * 4, 2 * rest));
+        w.da = (float *)da;
+        w.gs1 = rest && da ? (__nv_bfloat16 *)da : nullptr;
+        w.gs2 = rest && da ? (__nv_bfloat16 *)(da + rest) : nullptr;
         w.gb1 = (__nv_bfloat16 *)take(apx * 2); w.gb2 = (__nv_bfloat16 *)take(apx * 2);
         w.gr1 = (__nv_bfloat16 *)take(apx * 2); w.gr2 = (__nv_bfloat16 *)take(apx * 2);
         DeviceInfo info{152};
@@ -2237,9 +2325,10 @@ void launch_ring(const RingConv &p, unsigned grid, cudaStream_t s)
 // cores: dz_prev = gelu'(z_prev) * conv^T(in), in the bfloat16 gradient with halo
 // columns, gelu'(z_prev) from zg = z_prev or from the patterns and their table;
 // writes what is given of d_out (FP32), a_out (bfloat16, halo columns) and a_lo
-// (the bfloat16 rounding of the remainder).
+// (the bfloat16 rounding of the remainder) and a_rest (what is left).
 int launch_ring_bwd(int L, int64_t C, const float *params, int w_off, const __nv_bfloat16 *in, const float *zg,
-                    const uint16_t *pat, const float *tg, float *d_out, __nv_bfloat16 *a_out, __nv_bfloat16 *a_lo, cudaStream_t s)
+                    const uint16_t *pat, const float *tg, float *d_out, __nv_bfloat16 *a_out, __nv_bfloat16 *a_lo,
+                    __nv_bfloat16 *a_rest, cudaStream_t s)
 {
     DeviceInfo info{152};
     device_info(&info);
@@ -2248,6 +2337,7 @@ int launch_ring_bwd(int L, int64_t C, const float *params, int w_off, const __nv
     p.a_in = in;
     p.a_out = a_out;
     p.a_lo = a_lo;
+    p.a_rest = a_rest;
     p.zg = zg;
     p.pat = pat;
     p.tg = tg;
@@ -2269,11 +2359,12 @@ int launch_ring_bwd(int L, int64_t C, const float *params, int w_off, const __nv
     return e == cudaSuccess ? ISING_OK : nfail(ISING_ECUDA, cudaGetErrorString(e));
 }
 
-// The weight gradients of a 32 -> 32 layer on the tensor cores: the layer's input a (bfloat16, halo columns) and its gradient as
-// hi = bf16(dz), lo = bf16(dz - hi) (same layout); one CTA per SM writes its
-// partial sums into partial[cta][kN2 + kCh].  Returns the number of CTAs.
+// The weight gradients of a 32 -> 32 layer on the tensor cores: the layer's input a
+// (bfloat16, halo columns) and its gradient as hi = bf16(dz), lo = bf16(dz - hi) and,
+// where L is no multiple of 128, rest = dz - hi - lo (same layout); one CTA per SM
+// writes its partial sums into partial[cta][kN2 + kCh].  Returns the number of CTAs.
 int launch_wgrad_tc(int L, int64_t C, const __nv_bfloat16 *a, const __nv_bfloat16 *hi, const __nv_bfloat16 *lo,
-                    float *partial, int64_t max_ctas, cudaStream_t s, int64_t *n_cta)
+                    const __nv_bfloat16 *rest, float *partial, int64_t max_ctas, cudaStream_t s, int64_t *n_cta)
 {
     EncodeTiledFn fn = encode_tiled_fn();
     if (fn == nullptr) return nfail(ISING_ECUDA, "cuTensorMapEncodeTiled is not available");
@@ -2284,9 +2375,10 @@ int launch_wgrad_tc(int L, int64_t C, const __nv_bfloat16 *a, const __nv_bfloat1
                                    (cuuint64_t)L * (L + 2) * kCh * 2};
     const cuuint32_t box[4] = {kCh, (cuuint32_t)seg_width(L), 1, 1};  // whole pixels, 64 bytes: the 64-byte swizzle
     const cuuint32_t estr[4] = {1, 1, 1, 1};
-    const __nv_bfloat16 *src[3] = {a, hi, lo};
-    CUtensorMap *maps[3] = {&p.act, &p.hi, &p.lo};
-    for (int t = 0; t < 3; ++t) {
+    const bool full = L % kTileM == 0;
+    const __nv_bfloat16 *src[4] = {a, hi, lo, rest};
+    CUtensorMap *maps[4] = {&p.act, &p.hi, &p.lo, &p.rest};
+    for (int t = 0; t < (full ? 3 : 4); ++t) {
         const cuuint64_t dims[4] = {(cuuint64_t)kCh, (cuuint64_t)L + (t == 0 ? 2 : 1), (cuuint64_t)L, (cuuint64_t)C};
         if (fn(maps[t], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, (void *)src[t], dims, strides, box, estr,
                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
@@ -2300,9 +2392,10 @@ int launch_wgrad_tc(int L, int64_t C, const __nv_bfloat16 *a, const __nv_bfloat1
     p.lines = C * p.segs * L;
     // every CTA gets at least one row, so every partial row is written
     const int64_t grid = std::max<int64_t>(1, std::min<int64_t>({(int64_t)info.sm_count, max_ctas, p.lines}));
-    auto kernel = L % kTileM == 0 ? wgrad_tc_kernel<true> : wgrad_tc_kernel<false>;
-    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kWgSmem);
-    kernel<<<(unsigned)grid, kWgThreads, kWgSmem, s>>>(p);
+    auto kernel = full ? wgrad_tc_kernel<true> : wgrad_tc_kernel<false>;
+    const uint32_t smem = full ? WgLayout<true>::bytes : WgLayout<false>::bytes;
+    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    kernel<<<(unsigned)grid, kWgThreads, smem, s>>>(p);
     *n_cta = grid;
     cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? ISING_OK : nfail(ISING_ECUDA, cudaGetErrorString(e));
@@ -2496,21 +2589,24 @@ ISING_API int ising_net_backward(int64_t L, int64_t C, const void *black_dev, co
     wgrad_l4_kernel<<<(unsigned)(2 * sms), 32 * kThinWarps, 0, s>>>((int)L, C, w.a3, dlogits_dev, part4);
     // the data and weight gradients of the 32 -> 32 layers run on the tensor
     // cores; their gradients are kept as bfloat16 parts (gb: the rounding, gr: the
-    // rounding of the remainder)
+    // rounding of the remainder, gs: what these leave)
     const int64_t steps = (L * L + kL4Threads / 4 - 1) / (kL4Threads / 4);
     const int64_t gx = std::min<int64_t>(steps, std::max<int64_t>(1, (8 * sms + C - 1) / C));
-    l4_bwd_data_kernel<<<dim3((unsigned)gx, (unsigned)std::min<int64_t>(C, 2 * sms)), kL4Threads, 0, s>>>(
-        (int)L, C, params_dev, dlogits_dev, w.z3, w.gb1, w.gr1);  // dz3
+    auto l4 = w.gs1 ? l4_bwd_data_kernel<true> : l4_bwd_data_kernel<false>;
+    l4<<<dim3((unsigned)gx, (unsigned)std::min<int64_t>(C, 2 * sms)), kL4Threads, 0, s>>>(
+        (int)L, C, params_dev, dlogits_dev, w.z3, w.gb1, w.gr1, w.gs1);  // dz3
     // layer 3
     int64_t n3 = 0, n2 = 0;
-    rc = launch_wgrad_tc((int)L, C, w.a2, w.gb1, w.gr1, part3, sms, s, &n3);
+    rc = launch_wgrad_tc((int)L, C, w.a2, w.gb1, w.gr1, w.gs1, part3, sms, s, &n3);
     if (rc) return rc;
-    rc = launch_ring_bwd((int)L, C, params_dev, kOffW3, w.gb1, w.z2, nullptr, nullptr, nullptr, w.gb2, w.gr2, s);  // dz2
+    rc = launch_ring_bwd((int)L, C, params_dev, kOffW3, w.gb1, w.z2, nullptr, nullptr, nullptr, w.gb2, w.gr2,
+                         w.gs2, s);  // dz2
     if (rc) return rc;
     // layer 2
-    rc = launch_wgrad_tc((int)L, C, w.a1, w.gb2, w.gr2, part2, sms, s, &n2);
+    rc = launch_wgrad_tc((int)L, C, w.a1, w.gb2, w.gr2, w.gs2, part2, sms, s, &n2);
     if (rc) return rc;
-    rc = launch_ring_bwd((int)L, C, params_dev, kOffW2, w.gb2, nullptr, w.pat, w.tg, w.da, nullptr, nullptr, s);  // dz1
+    rc = launch_ring_bwd((int)L, C, params_dev, kOffW2, w.gb2, nullptr, w.pat, w.tg, w.da, nullptr, nullptr,
+                         nullptr, s);  // dz1
     if (rc) return rc;
     // layer 1
     wgrad_l1_kernel<<<(unsigned)(2 * sms), 32 * kThinWarps, 0, s>>>(C * L * L, w.da, w.pat, part1);
