@@ -33,6 +33,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -925,17 +926,28 @@ int64_t deal(BatchParams &p, int owners)
         const BatchGroup &G = p.g[order[k]];
         const int64_t w = G.items / 32 * chunk_cost(G);
         auto room = [&](int o, int64_t level) { return level <= load[o] ? int64_t(0) : (level - load[o]) / w; };
-        // the largest level that does not take more than the group has
-        int64_t lo = 0, hi = *std::max_element(load, load + owners) + (G.count + 1) * w;
-        while (hi - lo > 1) {
-            const int64_t mid = lo + (hi - lo) / 2;
-            int64_t n = 0;
-            for (int o = 0; o < owners && n <= G.count; ++o) n += room(o, mid);
-            (n <= G.count ? lo : hi) = mid;
+        int64_t take[kMaxOwners] = {}, left = G.count;
+        if (left > 16) {
+            // a level that does not take more than the group has, with one a lattice higher that does
+            int64_t lo = 0, hi = *std::max_element(load, load + owners) + (G.count + 1) * w;
+            while (hi - lo > w) {
+                const int64_t mid = lo + (hi - lo) / 2;
+                int64_t n = 0;
+                for (int o = 0; o < owners && n <= G.count; ++o) n += room(o, mid);
+                (n <= G.count ? lo : hi) = mid;
+            }
+            for (int o = 0; o < owners; ++o) left -= take[o] = room(o, lo);
+            for (int o = 0; o < owners; ++o) load[o] += take[o] * w;
+            // those left, fewer than the owners below that level, go one each to the least loaded ones
+            int by_load[kMaxOwners];
+            for (int o = 0; o < owners; ++o) by_load[o] = o;
+            std::nth_element(by_load, by_load + left, by_load + owners,
+                             [&](int a, int b) { return load[a] != load[b] ? load[a] < load[b] : a < b; });
+            for (; left > 0; --left) {
+                ++take[by_load[left - 1]];
+                load[by_load[left - 1]] += w;
+            }
         }
-        int64_t take[kMaxOwners], left = G.count;
-        for (int o = 0; o < owners; ++o) left -= take[o] = room(o, lo);
-        for (int o = 0; o < owners; ++o) load[o] += take[o] * w;
         for (; left > 0; --left) {
             const int o = (int)(std::min_element(load, load + owners) - load);
             ++take[o];
@@ -952,9 +964,14 @@ int64_t deal(BatchParams &p, int owners)
 size_t smem_for(int threads) { return (size_t)(threads / 32) * sizeof(MarchRing); }
 
 // Clusters of cs blocks of 512 threads that are resident together, 0 if none are
-// (a graphics processing cluster's SMs need not be a multiple of cs).
+// (a graphics processing cluster's SMs need not be a multiple of cs).  Asked once
+// per device: the three questions of a call take 15 us.
 int resident_clusters(int cs)
 {
+    static std::atomic<int> known[64][5];  // the answer + 1
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
+    if (known[dev][cs] != 0) return known[dev][cs] - 1;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)cs);
     cfg.blockDim = dim3(512);
@@ -971,6 +988,7 @@ int resident_clusters(int cs)
         cudaGetLastError();
         return 0;
     }
+    known[dev][cs] = n + 1;
     return n;
 }
 
@@ -990,22 +1008,19 @@ void pick_owners(BatchParams &p, int blocks)
         total += p.g[g].count * (p.g[g].items / 32) * chunk_cost(p.g[g]);
     }
     int64_t best = total / blocks + kGridSync;
-    int pick = 0;
+    decltype(p.part) part;
     for (int cs : {1, 2, 4}) {
         const int owners = cs == 1 ? blocks : resident_clusters(cs);
         if (owners < 1 || owners > kMaxOwners) continue;
         const int64_t cost = deal(p, owners) / cs + (cs == 1 ? kBlockSync : kClusterSync);
         if (cost < best) {
             best = cost;
-            pick = cs;
+            p.cs = cs;
+            p.expect_blocks = owners * cs;
+            memcpy(part, p.part, sizeof(part));
         }
     }
-    if (pick > 0) {
-        const int owners = pick == 1 ? blocks : resident_clusters(pick);
-        deal(p, owners);
-        p.expect_blocks = owners * pick;
-    }
-    p.cs = pick;
+    if (p.cs > 0) memcpy(p.part, part, sizeof(part));
     p.sync_every = (int32_t)std::min<int64_t>(1 << 20, std::max<int64_t>(1, 100000000 / best));
 }
 
@@ -1646,7 +1661,10 @@ extern "C" ISING_API int ising_batch_run_noalloc(int64_t n, const int64_t *L, in
     if (rc) return rc;
     p.expect_blocks = blocks;
     if (n_sweeps > 0) {
-        pick_owners(p, blocks);
+        // the dealing takes the host some 10 us for a dozen lattices, where a sweep of theirs
+        // then gains 5: us per call of 1 / 2 / 10 sweeps of 12 lattices 83 / 94 / 172 shared by
+        // the grid, 94 / 101 / 132 dealt
+        if (n_sweeps >= 4) pick_owners(p, blocks);
         e = launch_coop(p, p.expect_blocks, 512, s);
         if (e != cudaSuccess) return bfail(ISING_ECUDA, cudaGetErrorString(e));
     }

@@ -44,3 +44,28 @@ def test_exchanges_after_every_sweep_stay_consistent(sides, per, S, n, traced):
                    [torch.from_numpy(slot.copy()), torch.from_numpy(at.copy())])
     for x, y in zip(*got):
         assert torch.equal(x, y)
+
+
+@pytest.mark.parametrize("sides,per,S", [([32, 64, 128], 4, 4), ([64], 160, 8)])
+def test_short_allocation_free_runs_equal_batch_runs(sides, per, S):
+    """Runs of a few sweeps, which the allocation-free call lets the grid share, and of
+    more, whose lattices it deals to SMs: the same planes, slot state and traces as
+    those of a batch that goes on from the same state."""
+    L = [x for x in sides for _ in range(per)]
+    beta = np.linspace(0.40, 0.46, S)
+    ref = ising.Batch(L, S, beta)
+    ref.init(ising.ISING_INIT_RANDOM, 4)
+    words = 8 * int(ref.word_off[-1])
+    parts = ((ref._black_off, words), (ref._white_off, words), (ref._slot_off, 4 * ref.n), (ref._at_off, 4 * ref.n))
+    torch.cuda.synchronize()
+    mine = [ref.ws[o:o + k].clone() for o, k in parts]
+    t = 0
+    for n in (1, 2, 3, 4, 5, 1):
+        a, b = (torch.zeros((n, ref.n, 2), dtype=torch.int64, device="cuda") for _ in range(2))
+        ref.run(n, 4, t, 1, True, a)
+        ref.check()
+        ising.ising_batch_run_noalloc(L, S, beta, *mine, n, 4, t, 1, True, b)
+        t += n
+        assert torch.equal(a, b)
+        for (o, k), m in zip(parts, mine):
+            assert torch.equal(ref.ws[o:o + k], m)
