@@ -185,15 +185,16 @@ __device__ __forceinline__ void store_half(const ResidentSweep &p, int colour, i
 template <bool RAGGED>
 __device__ __forceinline__ uint32_t marks8(uint32_t b, uint32_t o, const DrawCtx &dc, const RoundKeys &rk)
 {
-    uint32_t m[3] = {0, 0, 0}, unused = 0;
+    uint32_t m[3] = {0, 0, 0}, other[3] = {0, 0, 0};  // other stays 0 where mark_ge keeps one counter
 #pragma unroll
     for (int i = 0; i < (RAGGED ? 3 : 2); ++i) {
         if (i == 2 && o == 0) break;
         const uint4 u = philox(b + i, 0u, dc.c2, dc.c3, rk);
-        mark_ge(m[i], unused, u.x, dc.T3, dc.T4, 1u);
-        mark_ge(m[i], unused, u.y, dc.T3, dc.T4, 1u << 4);
-        mark_ge(m[i], unused, u.z, dc.T3, dc.T4, 1u << 8);
-        mark_ge(m[i], unused, u.w, dc.T3, dc.T4, 1u << 12);
+        mark_ge(m[i], other[i], u.x, dc.T3, dc.T4, 1u);
+        mark_ge(m[i], other[i], u.y, dc.T3, dc.T4, 1u << 4);
+        mark_ge(m[i], other[i], u.z, dc.T3, dc.T4, 1u << 8);
+        mark_ge(m[i], other[i], u.w, dc.T3, dc.T4, 1u << 12);
+        m[i] += other[i];
     }
     const uint32_t lo = m[0] | (m[1] << 16);
     return RAGGED ? __funnelshift_r(lo, m[2], 4 * o) : lo;
