@@ -134,7 +134,7 @@ ISING_API int ising_sweep_wait_selftest(const ising_lattice_t *lat, ising_stream
  * the trace (if trace_host is not NULL; trace_dev is then required as device
  * staging of n_sweeps x 2 int64) back.  Pinned host memory makes the copies
  * asynchronous; the call does not synchronise the stream.  One sweep of an
- * MSC4 lattice of a few MB or more runs in row bands (3 to 32 with the size,
+ * MSC4 lattice of a few MB or more runs in row bands (3 to 31 with the size,
  * smaller first and last bands) on streams of the library's own: plane bands are
  * copied in in the order the half-sweeps need them and each is copied out as
  * soon as it is final, so that both directions of the host link are busy

@@ -663,7 +663,7 @@ cudaError_t copy_plane(void *dst, size_t dpitch, const void *src, size_t spitch,
 // for the first copy in and the last one out (time / bands), each costs two
 // copies each way and a launch or two (about 10 us of the streams), so their
 // number goes with the root of the plane's size: 1.5 per root megabyte, at most
-// 32, measured best within 3% from 4 MB to 1 GB in either format.  us per
+// 31 (from 455 MB on), measured best within 3% from 4 MB to 1 GB in either format.  us per
 // sweep of bit planes with 3 / 8 / 12 / 16 / 32 bands: 8192^2 143 / 166 / 188 / 231 /
 // -, 16384^2 439 / 376 / 396 / 410 / 490, 32768^2 1592 / 1178 / 1140 / 1155 / 1215;
 // MSC4 planes of 65536^2 18831 / 15166 / 14424 / 14101 / 13837.  Below 3 the sweep

@@ -442,7 +442,7 @@ __device__ int g_tc_error;  // set to 1 when a tensor-core wait gives up
 // y + dy offset by (1 + dx) x 16 bytes (no-swizzle K-major, LBO = kRingPlane,
 // SBO = 128).  (Sides that are no multiple of 128 took a kernel that gathered all
 // 9 taps of every tile, im2col, from global memory and one that projected on the
-// CUDA cores: a forward of 256 chains of 96^2 892 us, here 343; a training step of
+// CUDA cores: a forward of 256 chains of 96^2 892 us, here 272; a training step of
 // 40 chains of 96^2 1352, here 364.)
 // Warp roles, linked by mbarriers (every wait bounded):
 //   warp 0: loader -- lane 0 fetches each row with four tensor copies (TMA),
@@ -661,7 +661,7 @@ struct RingConv {
     __nv_bfloat16 *a_lo;   // BWD, nullable: bf16(dz_prev - bf16(dz_prev)) beside a_out (for the weight gradient)
     __nv_bfloat16 *a_rest; // BWD, nullable, sides that are no multiple of 128: what these two leave
     float *z_out;          // nullable
-    float *P;              // PROJ: 9 planes of C L^2
+    float *P;              // PROJ: row partials of z4, 9 per row and block column (pool_rows_kernel)
     const float *zg;       // BWD: z of the layer below (FP32, NHWC) for gelu', or, where that is layer 1,
     const uint16_t *pat;   // the pixels' patterns and
     const float *tg;       // the table of gelu'(z1)
@@ -1151,7 +1151,7 @@ __global__ void __launch_bounds__(ring_threads<PROJ, FUSED>(), 2) conv32_ring_ke
     } else if (PROJ && warp > kRingExtra && warp <= kRingExtra + kProjWarps) {
         // P of every output row, pixel lane 32 quad + lane: waits for the
         // projection (pfull), reads its 16 TMEM columns, frees them (pempty,
-        // four arrivals) and stores the 9 taps as FP32 planes P[k][pixel]
+        // four arrivals) and writes the row's partial sums of z4 per block column
         const int quad = warp & 3, m = quad * 32 + lane;
         int64_t s = 0;
         for (int64_t lin = begin; lin < end && ok;) {

@@ -1,7 +1,7 @@
 // tc.cuh -- inline-PTX wrappers for the fifth-generation tensor cores of
 // sm_100-family GPUs (tcgen05): tensor-memory (TMEM) allocation, the
-// single-thread MMA issue with shared-memory operand descriptors, completion
-// through an mbarrier, the warp-wide TMEM loads of the epilogue, and the
+// MMA issue with shared-memory operand descriptors (by a whole warp, of which one
+// elected lane issues), completion through an mbarrier, the warp-wide TMEM loads of the epilogue, and the
 // tensor copies (TMA) that stage operands in shared memory.
 //
 // Operand layouts used here, both without swizzle.  A "core matrix" is 8 rows
