@@ -108,10 +108,10 @@ ISING_API int ising_half_sweep(const ising_lattice_t *lat, double beta, int32_t 
  * (Sec. 3.3: a step updates black, then white).  trace_dev, if not
  * NULL, receives n_sweeps x 2 int64 {sum of spins, sum over bonds} after each
  * sweep (the call zeroes it first).  Running a sweeps and then b sweeps with
- * offset a gives the same lattice as a + b sweeps in one call.  L <= 512 runs in
- * one cluster whose CTAs wait for one another, each wait bounded (~2 s): should
- * one give up, the lattice and the trace are not to be used and ising_sweep_check
- * says so. */
+ * offset a gives the same lattice as a + b sweeps in one call.  Most calls of
+ * L <= 512 run in one cluster whose CTAs wait for one another, each wait bounded
+ * (~2 s): should one give up, the lattice and the trace are not to be used and
+ * ising_sweep_check says so. */
 ISING_API int ising_sweep(const ising_lattice_t *lat, double beta, int64_t n_sweeps, uint64_t seed,
                           uint64_t sweep_offset, int64_t *trace_dev, ising_stream_t stream);
 
